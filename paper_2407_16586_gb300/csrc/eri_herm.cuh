@@ -1,0 +1,1018 @@
+// fp64 derivative-ERI class kernel: one warp per contracted shell quartet,
+// one primitive quartet per lane, the density folded into Hermite densities.
+//
+// Derivation.  With R = A - B, a^ = zeta_a / p, b^ = zeta_b / p, the expansion
+// coefficients of a function pair (eq. cartG) are polynomials in
+// P - A = -b^ R and P - B = a^ R:
+//   E^{ab}_h(p) = sum_{k,l} c^{ab}_{h,k,l} R^{la+lb-k-l} (-b^)^{la-k} a^^{lb-l} (1/2p)^{(k+l+|h|)/2}
+// (integer c; k, l: how much of a and b is expanded about P).  Everything that
+// depends on the function pair is in c R^(..), which all primitive pairs
+// share; a primitive pair enters through the few scalars
+// s_m = (-b^)^(la-k) a^^(lb-l) (1/2p)^((k+l+|h|)/2) only.  So the density of a
+// contracted quartet is transformed ONCE to the "monomials" m = (h, k, l),
+//   G'[m1][m2] = sum_{ab,cd} Gamma[ab][cd] c^{ab}_{m1} R^.. c^{cd}_{m2} S^..       (S = C - D)
+// ((pp|pp): 81 -> 14 x 14, (dd|dd): 1296 -> 76 x 76), and per operator
+//   F[h1][m2]   = sum_{m1 of h1} s_m1(p) G'[m1][m2]                 per bra primitive pair
+//   X[h]        = sum_{h1+h2=h} (-1)^|h2| s_m2(q) F[h1][m2]         per primitive quartet (lane)
+//   E, T_i      = sum_h X[h] R[h], sum_h X[h] R[h + 1_i]            per primitive quartet (lane)
+//   U[h1][m2]   = sum_q (-1)^|h2| s_m2(q) R[h1 + h2]                items over lanes, lanes' R from shared memory
+//   V[m1][m2]  += s_m1(p) U[h1][m2]                                 per bra primitive pair
+// With P = A - b^ R, exp(-mu R^2), and the polynomials in R, eq. deriv becomes
+//   d/dA = sum a^ T - 2 mu_ab R E + sum V dG'/dR
+//   d/dC = sum -c^ T - 2 mu_cd S E + sum V dG'/dS,   d/dA + d/dB = sum T,
+// and d/dB, d/dD follow from translational invariance (eq. ti).  Against
+// contracting E tables for every primitive quartet this needs 3 ((pp|pp)) to
+// 8 times ((dd|dd)) fewer fp64 operations.
+//
+// What bounds it: the fp64 pipe.  GB300 retires 2 DFMA per clock and SM, so a
+// warp instruction holds it for 16 clocks whether one lane or all 32 are
+// active, and everything else (shared-memory traffic, index arithmetic, even
+// one warp per scheduler) hides behind it.  Hence full lanes come first:
+// primitive quartets of a block of PB bra primitive pairs are flattened over
+// the 32 lanes, PB chosen per quartet to waste the fewest; the reverse sums U
+// are spread over (h1, m2) items, several lanes per item when there are few.
+#pragma once
+#include <utility>
+
+#include "eri_warp.cuh"
+
+namespace tg {
+
+// ------------------------------------------------------------ pair tables
+
+// Scalars of order n = |h|: (k, l) with k <= LA, l <= LB, k + l >= n of n's
+// parity, k ascending, then l.  nsig: how many; soff / moff: first scalar and
+// first monomial of an order.
+template <int LA, int LB>
+struct PairMono {
+    static constexpr int L = LA + LB, NA = ncart(LA), NB = ncart(LB), NAB = NA * NB, NH = nherm(L);
+    __host__ __device__ static constexpr int nsig(int n)
+    {
+        int c = 0;
+        for (int k = 0; k <= LA; ++k)
+            for (int l = 0; l <= LB; ++l) c += (k + l >= n && ((k + l - n) & 1) == 0) ? 1 : 0;
+        return c;
+    }
+    __host__ __device__ static constexpr int soff(int n)
+    {
+        int c = 0;
+        for (int i = 0; i < n; ++i) c += nsig(i);
+        return c;
+    }
+    __host__ __device__ static constexpr int moff(int n)
+    {
+        int c = 0;
+        for (int i = 0; i < n; ++i) c += nsig(i) * (i + 1) * (i + 2) / 2;
+        return c;
+    }
+    static constexpr int NS = soff(L + 1), NM = moff(L + 1);
+    static constexpr int choose2(int n, int k) { return (k == 0 || k == n) ? 1 : 2; }  // n <= 2
+    // (x - P)^n in Hermite functions: coefficient of Lambda_t over (1/2p)^((n+t)/2)
+    static constexpr int herm_coef(int n, int t)
+    {
+        int v = 1;
+        for (int i = t + 1; i <= n; ++i) v *= i;       // n! / t!
+        for (int i = 1; i <= (n - t) / 2; ++i) v /= 2 * i;
+        return v;
+    }
+    static constexpr int monomial(int h, int n, int k, int l)
+    {
+        int s = 0;
+        for (int kk = 0; kk <= LA; ++kk)
+            for (int ll = 0; ll <= LB; ++ll) {
+                if (kk == k && ll == l) return moff(n) + (h - nherm(n - 1)) * nsig(n) + s;
+                s += (kk + ll >= n && ((kk + ll - n) & 1) == 0) ? 1 : 0;
+            }
+        return -1;
+    }
+};
+
+// One term c^{ab}_m R_x^px R_y^py R_z^pz: ab | coef << 8 | px << 16 | py << 19 | pz << 22.
+constexpr int pair_entries(int la, int lb)
+{
+    // (ss) 1, (ps) 6, (pp) 39, (ds) 24, (dp) 159, (dd) 648; make_pair_tab counts them again
+    return la == 0 ? 1 : (la == 1 ? (lb == 0 ? 6 : 39) : (lb == 0 ? 24 : (lb == 1 ? 159 : 648)));
+}
+
+template <int LA, int LB>
+struct PairTab {
+    using M = PairMono<LA, LB>;
+    static constexpr int NE = pair_entries(LA, LB);
+    int n;                             // entries found
+    unsigned ent[NE];                  // by monomial
+    unsigned short own[NE];            // monomial of each entry
+    unsigned short start[M::NM + 1];   // entries of monomial m: start[m] .. start[m + 1]
+    unsigned short hm[M::NH];          // per Hermite index: first monomial | nsig << 8 | first scalar << 12
+};
+
+template <int LA, int LB>
+constexpr PairTab<LA, LB> make_pair_tab()
+{
+    using M = PairMono<LA, LB>;
+    PairTab<LA, LB> T{};
+    int ne = 0;
+    for (int n = 0; n <= M::L; ++n)
+        for (int t = n; t >= 0; --t)
+            for (int u = n - t; u >= 0; --u) {
+                const int v = n - t - u, h = hidx(t, u, v);
+                T.hm[h] = (unsigned short)((M::moff(n) + (h - nherm(n - 1)) * M::nsig(n)) | (M::nsig(n) << 8) |
+                                           (M::soff(n) << 12));
+                for (int k = 0; k <= LA; ++k)
+                    for (int l = 0; l <= LB; ++l) {
+                        if (!(k + l >= n && ((k + l - n) & 1) == 0)) continue;
+                        const int m = M::monomial(h, n, k, l);
+                        T.start[m] = (unsigned short)ne;
+                        for (int ia = 0; ia < M::NA; ++ia)
+                            for (int ib = 0; ib < M::NB; ++ib) {
+                                const int as = ia == 0 ? 0 : (ia < 3 ? 1 : 2), bs = ib == 0 ? 0 : (ib < 3 ? 1 : 2);
+                                const int az = ia - as * (as + 1) / 2, ay = as - az, ax = LA - as;
+                                const int bz = ib - bs * (bs + 1) / 2, by = bs - bz, bx = LB - bs;
+                                for (int kx = 0; kx <= ax; ++kx)
+                                    for (int ky = 0; ky <= ay; ++ky)
+                                        for (int lx = 0; lx <= bx; ++lx)
+                                            for (int ly = 0; ly <= by; ++ly) {
+                                                const int kz = k - kx - ky, lz = l - lx - ly;
+                                                if (kz < 0 || kz > az || lz < 0 || lz > bz) continue;
+                                                const int nx = kx + lx, ny = ky + ly, nz = kz + lz;
+                                                if (nx < t || ny < u || nz < v || ((nx - t) & 1) || ((ny - u) & 1) ||
+                                                    ((nz - v) & 1))
+                                                    continue;
+                                                const int c = M::choose2(ax, kx) * M::choose2(ay, ky) * M::choose2(az, kz) *
+                                                              M::choose2(bx, lx) * M::choose2(by, ly) * M::choose2(bz, lz) *
+                                                              M::herm_coef(nx, t) * M::herm_coef(ny, u) * M::herm_coef(nz, v);
+                                                const int px = ax + bx - nx, py = ay + by - ny, pz = az + bz - nz;
+                                                const unsigned w = (unsigned)(ia * M::NB + ib) | ((unsigned)px << 16) |
+                                                                   ((unsigned)py << 19) | ((unsigned)pz << 22);
+                                                int at = -1;  // terms of the same power add up
+                                                for (int e = T.start[m]; e < ne; ++e)
+                                                    if ((T.ent[e] & 0xffff00ffu) == w) at = e;
+                                                if (at >= 0) {
+                                                    T.ent[at] += (unsigned)c << 8;
+                                                } else {
+                                                    if (ne < PairTab<LA, LB>::NE) {
+                                                        T.ent[ne] = w | ((unsigned)c << 8);
+                                                        T.own[ne] = (unsigned short)m;
+                                                    }
+                                                    ++ne;
+                                                }
+                                            }
+                            }
+                    }
+            }
+    T.start[M::NM] = (unsigned short)ne;
+    T.n = ne;
+    return T;
+}
+
+static __device__ const PairTab<0, 0> kPair00 = make_pair_tab<0, 0>();
+static __device__ const PairTab<1, 0> kPair10 = make_pair_tab<1, 0>();
+static __device__ const PairTab<1, 1> kPair11 = make_pair_tab<1, 1>();
+static __device__ const PairTab<2, 0> kPair20 = make_pair_tab<2, 0>();
+static __device__ const PairTab<2, 1> kPair21 = make_pair_tab<2, 1>();
+static __device__ const PairTab<2, 2> kPair22 = make_pair_tab<2, 2>();
+
+template <int LA, int LB>
+__device__ __forceinline__ const PairTab<LA, LB> &pair_tab()
+{
+    if constexpr (LA == 0) return kPair00;
+    else if constexpr (LA == 1 && LB == 0) return kPair10;
+    else if constexpr (LA == 1) return kPair11;
+    else if constexpr (LB == 0) return kPair20;
+    else if constexpr (LB == 1) return kPair21;
+    else return kPair22;
+}
+
+// ------------------------------------------------------------ layout
+
+// One warp's slice of shared memory, in doubles.  Rows that lanes read at
+// different row numbers have an odd stride.  NO operators are resident at a
+// time; classes whose arrays are large take the operators one after the other
+// (the scalars of a primitive quartet are then formed twice, 3 % of the work
+// at (pp|pp)), which keeps at least four warps on an SM.
+template <int LA, int LB, int LC, int LD>
+struct HermLay {
+    using B = PairMono<LA, LB>;
+    using K = PairMono<LC, LD>;
+    static constexpr int NAB = B::NAB, NCD = K::NAB, L1 = B::L, L2 = K::L, L = L1 + L2, LM = L + 1;
+    static constexpr int NT1 = B::NH, NM1 = B::NM, NM2 = K::NM, NS1 = B::NS, NS2 = K::NS;
+    static constexpr int NABP = NAB | 1, NM2P = NM2 | 1;
+    static constexpr int RS = 33;                     // row stride of the per-lane columns
+    static constexpr int NRH = nherm(L);              // Hermite rows kept for the reverse sums
+    static constexpr bool RREG = LM <= 5;             // R tensor in registers, or in its shared-memory rows
+    static constexpr int NO = (NAB * NCD <= 27) ? 2 : 1;
+    // bra primitive pairs of a block: a budget of 1200 doubles for F, 1 to 16
+    static constexpr int PB_RAW = 1200 / (NT1 * NM2P * NO);
+    static constexpr int PB = PB_RAW < 1 ? 1 : (PB_RAW > 16 ? 16 : PB_RAW);
+    static constexpr int NE1 = pair_entries(LA, LB), NE2 = pair_entries(LC, LD);
+    // the transforms' half-way arrays share the space of the R rows
+    static constexpr int HALF = (NM2 * NABP > NM1 * NCD ? NM2 * NABP : NM1 * NCD) * NO + NE1 + NE2;
+    static constexpr int ROWS = NRH * RS + NS2 * RS;
+    static constexpr int RED = 9 * RS;
+    static constexpr int SHARED = HALF > ROWS ? (HALF > RED ? HALF : RED) : (ROWS > RED ? ROWS : RED);
+    static constexpr int NP1 = 5;                     // per bra primitive pair: a^, mu, K/p factor, p, spare
+    static constexpr int o_G = 0;                                  // [NO][NCD][NABP]
+    static constexpr int o_Gp = o_G + NO * NCD * NABP;             // [NO][NM1][NM2P]
+    static constexpr int o_V = o_Gp + NO * NM1 * NM2P;             // [NO][NM1][NM2P]
+    static constexpr int o_F = o_V + NO * NM1 * NM2P;              // [PB][NO][NT1][NM2P]
+    static constexpr int o_S1 = o_F + PB * NO * NT1 * NM2P;        // [PB][NS1]
+    static constexpr int o_P1 = o_S1 + PB * NS1;                   // [PB][NP1]
+    static constexpr int o_pw = o_P1 + PB * NP1;                   // [2][3][5] powers of R and S
+    static constexpr int o_X = o_pw + 30;                          // SHARED
+    static constexpr int TOTAL = (o_X + SHARED + 1) & ~1;
+    static constexpr size_t BYTES = sizeof(double) * (size_t)TOTAL;
+};
+
+// (h1, m2) items of the reverse sums: those whose V enters a derivative, i.e.
+// some monomial of h1 carries a power of R or m2 one of S.
+// R row | h1 << 8 | m2 << 14 | scalar of m2 << 21
+template <int LA, int LB, int LC, int LD>
+constexpr int herm_item_count()
+{
+    using B = PairMono<LA, LB>;
+    using K = PairMono<LC, LD>;
+    int n = 0;
+    for (int n2 = 0; n2 <= K::L; ++n2)
+        for (int k = 0; k <= LC; ++k)
+            for (int l = 0; l <= LD; ++l)
+                if (k + l >= n2 && ((k + l - n2) & 1) == 0)
+                    n += (n2 + 1) * (n2 + 2) / 2 * (k + l < K::L ? nherm(B::L) : nherm(B::L - 1));
+    return n;
+}
+
+template <int LA, int LB, int LC, int LD>
+struct HermItems {
+    static constexpr int N = herm_item_count<LA, LB, LC, LD>();
+    unsigned it[N > 0 ? N : 1];
+};
+
+template <int LA, int LB, int LC, int LD>
+constexpr HermItems<LA, LB, LC, LD> make_herm_items()
+{
+    using B = PairMono<LA, LB>;
+    using K = PairMono<LC, LD>;
+    HermItems<LA, LB, LC, LD> T{};
+    int n = 0;
+    for (int n1 = 0; n1 <= B::L; ++n1)
+        for (int t1 = n1; t1 >= 0; --t1)
+            for (int u1 = n1 - t1; u1 >= 0; --u1)
+                for (int n2 = 0; n2 <= K::L; ++n2)
+                    for (int t2 = n2; t2 >= 0; --t2)
+                        for (int u2 = n2 - t2; u2 >= 0; --u2) {
+                            const int v1 = n1 - t1 - u1, v2 = n2 - t2 - u2;
+                            int s = 0;
+                            for (int k = 0; k <= LC; ++k)
+                                for (int l = 0; l <= LD; ++l) {
+                                    if (!(k + l >= n2 && ((k + l - n2) & 1) == 0)) continue;
+                                    if (k + l < K::L || n1 < B::L)
+                                        T.it[n++] = (unsigned)hidx(t1 + t2, u1 + u2, v1 + v2) |
+                                                    ((unsigned)hidx(t1, u1, v1) << 8) |
+                                                    ((unsigned)K::monomial(hidx(t2, u2, v2), n2, k, l) << 14) |
+                                                    ((unsigned)(K::soff(n2) + s) << 21);
+                                    ++s;
+                                }
+                        }
+    return T;
+}
+
+// ------------------------------------------------------------ lane pieces
+
+// F_m(T), m = 0..M, one argument per lane.  T < 36: F_M and F_{M+1} by the
+// Taylor step of the table (shared d/k factors), e^-T = (2M+1) F_M - 2T F_{M+1}
+// (error below eps (2M+1) F_M, which the next order up divides by 2M-1), then
+// downward recursion: no exponential.  T >= 36: upward recursion, with e^-T
+// only below 64 (beyond, it is under 1e-14 of the smallest order's term).
+template <int M>
+__device__ __forceinline__ void boys_lane(double T, double (&F)[M + 1], const double *__restrict__ tab)
+{
+    if (T < BOYS_TMAX) {
+        const int i = __double2int_rn(T * (1.0 / BOYS_H));
+        const double d = i * BOYS_H - T;
+        const double *row = tab + i * (BOYS_M + 1) + M;
+        double hi = row[BOYS_TAYLOR + 1], lo = row[BOYS_TAYLOR];
+#pragma unroll
+        for (int k = BOYS_TAYLOR - 1; k >= 0; --k) {
+            const double dk = d * (1.0 / (k + 1));
+            hi = row[k + 1] + hi * dk;
+            lo = row[k] + lo * dk;
+        }
+        const double t2 = 2.0 * T;
+        const double et = (2 * M + 1) * lo - t2 * hi;
+        F[M] = lo;
+#pragma unroll
+        for (int m = M - 1; m >= 0; --m) F[m] = (t2 * F[m + 1] + et) * (1.0 / (2 * m + 1));
+    } else {
+        const double is = rsqrt(T), h = 0.5 * is * is;
+        const double et = T < 64.0 ? exp(-T) : 0.0;
+        F[0] = 0.88622692545275801365 * is;
+#pragma unroll
+        for (int m = 0; m < M; ++m) F[m + 1] = ((2 * m + 1) * F[m] - et) * h;
+    }
+}
+
+// s_m of one primitive pair: oo2 = 1/2p, a = zeta_a/p, b = zeta_b/p; the ket
+// carries the sign (-1)^|h|.
+template <int LA, int LB, bool KET>
+__device__ __forceinline__ void pair_scalars(double oo2, double a, double b, double (&s)[PairMono<LA, LB>::NS])
+{
+    double bp[LA + 1], ap[LB + 1], op[LA + LB + 1];
+    bp[0] = ap[0] = op[0] = 1.0;
+#pragma unroll
+    for (int i = 1; i <= LA; ++i) bp[i] = -b * bp[i - 1];
+#pragma unroll
+    for (int i = 1; i <= LB; ++i) ap[i] = a * ap[i - 1];
+#pragma unroll
+    for (int i = 1; i <= LA + LB; ++i) op[i] = oo2 * op[i - 1];
+    int c = 0;
+#pragma unroll
+    for (int n = 0; n <= LA + LB; ++n)
+#pragma unroll
+        for (int k = 0; k <= LA; ++k)
+#pragma unroll
+            for (int l = 0; l <= LB; ++l)
+                if (k + l >= n && ((k + l - n) & 1) == 0) {
+                    const double v = bp[LA - k] * ap[LB - l] * op[(k + l + n) / 2];
+                    s[c++] = (KET && (n & 1)) ? -v : v;
+                }
+}
+
+// f(integral_constant<int, 0>), ..., f(integral_constant<int, N - 1>)
+template <typename Fn, int... I>
+__device__ __forceinline__ void static_for_impl(Fn &&f, std::integer_sequence<int, I...>)
+{
+    (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, typename Fn>
+__device__ __forceinline__ void static_for(Fn &&f)
+{
+    static_for_impl(f, std::make_integer_sequence<int, N>{});
+}
+
+// Shared-memory load of the unrolled lane phases.  Volatile inline PTX: the
+// address is the warp's own slice and every write to it is ordered by
+// __syncwarp, while plain loads between this many stores make the compiler's
+// alias analysis take minutes per class.
+__device__ __forceinline__ double lds(const double *p)
+{
+    double v;
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"((unsigned)__cvta_generic_to_shared(p)));
+    return v;
+}
+
+// (t, u, v) of a compact Hermite index, at compile time
+struct Triple {
+    int t, u, v;
+};
+__host__ __device__ constexpr Triple herm_triple(int h)
+{
+    for (int n = 0;; ++n)
+        if (h < nherm(n)) {
+            int r = h - nherm(n - 1);
+            for (int t = n;; --t) {
+                if (r <= n - t) return Triple{t, n - t - r, r};
+                r -= n - t + 1;
+            }
+        }
+}
+
+// One row of the Hermite density: for the bra index h1, X[h1 + h2] gets every
+// ket monomial's s_m2 F[h1][m2].
+template <int LC, int LD>
+struct DensRow {
+    using K = PairMono<LC, LD>;
+    short h2[K::NM], s[K::NM];
+};
+template <int LC, int LD>
+__host__ __device__ constexpr DensRow<LC, LD> make_dens_row()
+{
+    using K = PairMono<LC, LD>;
+    DensRow<LC, LD> r{};
+    for (int h = 0; h < K::NH; ++h) {
+        const Triple x = herm_triple(h);
+        const int n = x.t + x.u + x.v;
+        for (int k = 0; k < K::nsig(n); ++k) {
+            const int m = K::moff(n) + (h - nherm(n - 1)) * K::nsig(n) + k;
+            r.h2[m] = (short)h;
+            r.s[m] = (short)(K::soff(n) + k);
+        }
+    }
+    return r;
+}
+__host__ __device__ constexpr int herm_sum(int h1, int h2)
+{
+    const Triple a = herm_triple(h1), b = herm_triple(h2);
+    return hidx(a.t + b.t, a.u + b.u, a.v + b.v);
+}
+
+// X[h] of one lane: sum over h1 and the ket monomials of s_m2 F[h1][m2]
+// (F: this lane's bra primitive pair).
+template <int LA, int LB, int LC, int LD>
+__device__ __forceinline__ void hermite_density(const double *F, const double (&s2)[PairMono<LC, LD>::NS],
+                                                double (&X)[nherm(LA + LB + LC + LD)])
+{
+    using Lay = HermLay<LA, LB, LC, LD>;
+#pragma unroll
+    for (int h = 0; h < nherm(Lay::L); ++h) X[h] = 0.0;
+    static_for<Lay::NT1>([&](auto H1) {
+        static_for<Lay::NM2>([&](auto M2) {
+            constexpr int h1 = decltype(H1)::value, m2 = decltype(M2)::value;
+            constexpr auto row = make_dens_row<LC, LD>();
+            constexpr int x = herm_sum(h1, row.h2[m2]), sc = row.s[m2];
+            X[x] += s2[sc] * lds(F + h1 * Lay::NM2P + m2);
+        });
+    });
+}
+
+// E += X[h] r and T_i += X[h - 1_i] r of Hermite entry h, where X holds the
+// orders up to L.
+template <int L, int H>
+__device__ __forceinline__ void energy_terms(double r, const double (&X)[nherm(L)], double &e, double (&T)[3])
+{
+    constexpr Triple x = herm_triple(H);
+    if constexpr (H < nherm(L)) e += X[H] * r;
+    if constexpr (x.t > 0) T[0] += X[hidx(x.t - 1, x.u, x.v)] * r;
+    if constexpr (x.u > 0) T[1] += X[hidx(x.t, x.u - 1, x.v)] * r;
+    if constexpr (x.v > 0) T[2] += X[hidx(x.t, x.u, x.v - 1)] * r;
+}
+
+// How Hermite entry h follows from the level above (hermite_R): direction,
+// first and second source, coefficient.  dir | src1 << 2 | src2 << 10 | coef << 18
+// (coef 0: no second term, src2 = 0).
+struct HermSteps {
+    unsigned w[nherm(9)];
+};
+constexpr HermSteps make_herm_steps()
+{
+    HermSteps s{};
+    for (int h = 1; h < nherm(9); ++h) {
+        const Triple x = herm_triple(h);
+        const int d = x.t > 0 ? 0 : (x.u > 0 ? 1 : 2), c = d == 0 ? x.t : (d == 1 ? x.u : x.v);
+        const int s1 = hidx(x.t - (d == 0), x.u - (d == 1), x.v - (d == 2));
+        const int s2 = c > 1 ? hidx(x.t - 2 * (d == 0), x.u - 2 * (d == 1), x.v - 2 * (d == 2)) : 0;
+        s.w[h] = (unsigned)d | ((unsigned)s1 << 2) | ((unsigned)s2 << 10) | ((unsigned)(c - 1) << 18);
+    }
+    return s;
+}
+static __device__ const HermSteps kHermSteps = make_herm_steps();
+
+// ------------------------------------------------------------ quartet
+
+// Gamma_op of the canonical quartet (the 8 permutation images of the pair
+// products, times scale), [cd][ab], for operators o0 .. o0 + NO - 1.
+template <int LA, int LB, int LC, int LD>
+__device__ __forceinline__ void herm_gamma(double *G, int lane, int o0, const DensArgs &den, int fa, int fb, int fc,
+                                           int fd, double scale)
+{
+    using Lay = HermLay<LA, LB, LC, LD>;
+    constexpr int NB = ncart(LB), ND = ncart(LD);
+    const int nbf = den.nbf;
+    for (int it = lane; it < Lay::NAB * Lay::NCD; it += 32) {
+        const int cd = it / Lay::NAB, ab = it % Lay::NAB;
+        const size_t m = fa + ab / NB, n = fb + ab % NB, l = fc + cd / ND, s = fd + cd % ND;
+        double g0 = 0.0, g1 = 0.0;
+        for (int p = 0; p < den.npair; ++p) {
+            const double *A = den.A[p], *B = den.B[p];
+            const double cj = den.cJ[p], ck = den.cK[p], cl = den.cKlr[p];
+            if (cj != 0.0 && (Lay::NO == 2 || o0 == 0))
+                g0 += cj * (den.S[p][m * nbf + n] * den.T[p][l * nbf + s] + den.S[p][l * nbf + s] * den.T[p][m * nbf + n]);
+            if (ck != 0.0 || cl != 0.0) {
+                const double kk = A[m * nbf + l] * B[n * nbf + s] + A[n * nbf + l] * B[m * nbf + s] +
+                                  A[m * nbf + s] * B[n * nbf + l] + A[n * nbf + s] * B[m * nbf + l] +
+                                  A[l * nbf + m] * B[s * nbf + n] + A[s * nbf + m] * B[l * nbf + n] +
+                                  A[l * nbf + n] * B[s * nbf + m] + A[s * nbf + n] * B[l * nbf + m];
+                g0 += ck * kk;
+                g1 += cl * kk;
+            }
+        }
+        if constexpr (Lay::NO == 2) {
+            G[cd * Lay::NABP + ab] = g0 * scale;
+            G[(Lay::NCD + cd) * Lay::NABP + ab] = g1 * scale;
+        } else {
+            G[cd * Lay::NABP + ab] = (o0 == 0 ? g0 : g1) * scale;
+        }
+    }
+}
+
+// c^{ab}_m R^.. of every table entry of a pair class.
+template <int LA, int LB>
+__device__ __forceinline__ void entry_values(double *out, int lane, const double *pw)
+{
+    const auto &T = pair_tab<LA, LB>();
+    for (int e = lane; e < PairTab<LA, LB>::NE; e += 32) {
+        const unsigned w = T.ent[e];
+        out[e] = double((int)((w >> 8) & 0xff)) * pw[(w >> 16) & 7] * pw[5 + ((w >> 19) & 7)] * pw[10 + ((w >> 22) & 7)];
+    }
+}
+
+// half[o][m2][ab] = sum_{entries of m2} value Gamma[cd][ab]
+template <int LA, int LB, int LC, int LD>
+__device__ __forceinline__ void half_ket(double *half, const double *G, const double *vk, int lane)
+{
+    using Lay = HermLay<LA, LB, LC, LD>;
+    const auto &T = pair_tab<LC, LD>();
+    for (int it = lane; it < Lay::NM2 * Lay::NAB; it += 32) {
+        const int m = it / Lay::NAB, ab = it % Lay::NAB;
+#pragma unroll
+        for (int o = 0; o < Lay::NO; ++o) {
+            double s = 0.0;
+            for (int e = T.start[m]; e < T.start[m + 1]; ++e)
+                s += vk[e] * G[(o * Lay::NCD + (T.ent[e] & 0xff)) * Lay::NABP + ab];
+            half[(o * Lay::NM2 + m) * Lay::NABP + ab] = s;
+        }
+    }
+}
+
+// One contracted quartet by one warp, bra primitive pairs ib0, ib0 + ibs, ...
+// acc[0..2] += d/dA, acc[3..5] += d/dA + d/dB, acc[6..8] += d/dC (this lane's
+// share; the caller sums the warp).
+template <int LA, int LB, int LC, int LD>
+__device__ void quartet_herm(double *sm, int lane, const unsigned *items, const GeoArgs &geo, const DensArgs &den,
+                             const PrimPairs &pp, int sa, int sb, int sc, int sd, int pb0, int nbp, int ib0, int ibs,
+                             int pk0, int nkp, double scale, const double *boys, double (&acc)[9])
+{
+    using Lay = HermLay<LA, LB, LC, LD>;
+    constexpr int NCD = Lay::NCD, L = Lay::L, LM = Lay::LM, NT1 = Lay::NT1;
+    constexpr int NM1 = Lay::NM1, NM2 = Lay::NM2, NM2P = Lay::NM2P, NS1 = Lay::NS1, NS2 = Lay::NS2, RS = Lay::RS;
+    constexpr int NO = Lay::NO, NP1 = Lay::NP1, NABP = Lay::NABP;
+    constexpr int NIT = HermItems<LA, LB, LC, LD>::N;
+    // lanes per item of the reverse sums: as many as fit
+    constexpr int SUB = NIT == 0 ? 1 : (NIT <= 4 ? 8 : (NIT <= 8 ? 4 : (NIT <= 16 ? 2 : 1)));
+    constexpr int ITL = 32 / SUB;
+    double *G = sm + Lay::o_G, *Gp = sm + Lay::o_Gp, *V = sm + Lay::o_V, *F = sm + Lay::o_F;
+    double *S1 = sm + Lay::o_S1, *P1 = sm + Lay::o_P1, *pw = sm + Lay::o_pw, *X1 = sm + Lay::o_X;
+    double *Rr = X1, *S2 = X1 + Lay::NRH * RS;                      // main loop
+    double *half = X1 + Lay::NE1 + Lay::NE2, *vb = X1, *vk = X1 + Lay::NE1;  // transforms
+    const auto &TBra = pair_tab<LA, LB>();
+    const auto &TKet = pair_tab<LC, LD>();
+    const int nops = den.use_lr ? 2 : 1;
+    const bool ominf = isinf(den.omega);
+    const double om = ominf ? 1.0 : den.omega;
+    const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xb = geo.xyz + 3 * geo.sh_atom[sb];
+    const double *xc = geo.xyz + 3 * geo.sh_atom[sc], *xd = geo.xyz + 3 * geo.sh_atom[sd];
+    if (lane < 6) {  // powers of R = A - B and S = C - D
+        const int d = lane % 3;
+        const double x = lane < 3 ? xa[d] - xb[d] : xc[d] - xd[d];
+        double p = 1.0;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            pw[(lane / 3) * 15 + d * 5 + k] = p;
+            p *= x;
+        }
+    }
+    const int nbra = (nbp - ib0 + ibs - 1) / ibs;  // bra primitive pairs of this call
+    // block size: the fewest idle lanes over whole blocks
+    int pb = 1;
+    {
+        int best = -1;
+        for (int c = 1; c <= (nbra < Lay::PB ? nbra : Lay::PB); ++c) {
+            const int n = c * nkp, use = n * 64 / ((n + 31) / 32);  // lanes in use per pass, times 64
+            if (use >= best) best = use, pb = c;
+        }
+    }
+    // this lane's sums over its primitive quartets: T, a^ T, c^ T, mu_ab E, mu_cd E
+    double aT[3] = {0.0, 0.0, 0.0}, aA[3] = {0.0, 0.0, 0.0}, aC[3] = {0.0, 0.0, 0.0}, eA = 0.0, eC = 0.0;
+    double gA[3] = {0.0, 0.0, 0.0}, gC[3] = {0.0, 0.0, 0.0};  // polynomial parts
+    __syncwarp();
+
+    for (int o0 = 0; o0 < nops; o0 += NO) {
+        // ---- Gamma -> G'[m1][m2]
+        herm_gamma<LA, LB, LC, LD>(G, lane, o0, den, geo.sh_bf[sa], geo.sh_bf[sb], geo.sh_bf[sc], geo.sh_bf[sd], scale);
+        entry_values<LA, LB>(vb, lane, pw);
+        entry_values<LC, LD>(vk, lane, pw + 15);
+        __syncwarp();
+        half_ket<LA, LB, LC, LD>(half, G, vk, lane);
+        __syncwarp();
+        for (int it = lane; it < NM1 * NM2; it += 32) {
+            const int m1 = it / NM2, m2 = it % NM2;
+#pragma unroll
+            for (int o = 0; o < NO; ++o) {
+                double s = 0.0;
+                for (int e = TBra.start[m1]; e < TBra.start[m1 + 1]; ++e)
+                    s += vb[e] * half[(o * NM2 + m2) * NABP + (TBra.ent[e] & 0xff)];
+                Gp[(o * NM1 + m1) * NM2P + m2] = s;
+                V[(o * NM1 + m1) * NM2P + m2] = 0.0;
+            }
+        }
+        __syncwarp();
+
+        for (int blk = 0; blk < nbra; blk += pb) {
+            const int np = min(pb, nbra - blk);
+            // ---- scalars of the block's bra primitive pairs, then F[p][h1][m2]
+            if (lane < np) {
+                const int ip = pb0 + ib0 + (blk + lane) * ibs;
+                const double p = pp.p[ip], za = pp.za[ip], oo2 = 0.5 / p;
+                const double a = 2.0 * oo2 * za, b = 2.0 * oo2 * (p - za);
+                double s[NS1];
+                pair_scalars<LA, LB, false>(oo2, a, b, s);
+#pragma unroll
+                for (int k = 0; k < NS1; ++k) S1[lane * NS1 + k] = s[k];
+                P1[lane * NP1] = a;
+                P1[lane * NP1 + 1] = za * b;
+                P1[lane * NP1 + 2] = pp.K[ip] * oo2 * 69.97367331049945;  // 4 pi^(5/2) K / 2p
+                P1[lane * NP1 + 3] = p;
+            }
+            __syncwarp();
+            for (int it = lane; it < np * NT1 * NM2; it += 32) {
+                const int pi = it / (NT1 * NM2), r = it % (NT1 * NM2), h = r / NM2, m2 = r % NM2;
+                const unsigned hm = TBra.hm[h];
+                const double *g = Gp + (hm & 0xff) * NM2P + m2, *s = S1 + pi * NS1 + (hm >> 12);
+                const int ns = (hm >> 8) & 0xf;
+#pragma unroll
+                for (int o = 0; o < NO; ++o) {
+                    double f = 0.0;
+                    for (int k = 0; k < ns; ++k) f += s[k] * g[(o * NM1 + k) * NM2P];
+                    F[((pi * NO + o) * NT1 + h) * NM2P + m2] = f;
+                }
+            }
+            __syncwarp();
+            const int ntot = np * nkp;
+            for (int j0 = 0; j0 < ntot; j0 += 32) {
+                // ---- this lane's primitive quartet
+                const int idx = min(j0 + lane, ntot - 1);
+                const int pi = idx / nkp;
+                const int ip = pb0 + ib0 + (blk + pi) * ibs, kp = pk0 + (idx - pi * nkp);
+                const double p = P1[pi * NP1 + 3], q = pp.p[kp], zc = pp.za[kp];
+                const double oo2q = 0.5 / q, c = 2.0 * oo2q * zc, d = 2.0 * oo2q * (q - zc);
+                const double ir = rsqrt(p + q);
+                const double rho = p * q * ir * ir;
+                const double X = pp.Px[ip] - pp.Px[kp], Y = pp.Py[ip] - pp.Py[kp], Z = pp.Pz[ip] - pp.Pz[kp];
+                const double T0 = rho * (X * X + Y * Y + Z * Z);
+                // lanes past the end repeat the last quartet with weight zero
+                const double pref = j0 + lane < ntot ? P1[pi * NP1 + 2] * pp.K[kp] * (2.0 * oo2q) * ir : 0.0;
+                double s2[NS2];
+                pair_scalars<LC, LD, true>(oo2q, c, d, s2);
+                if constexpr (NIT > 0)
+#pragma unroll
+                    for (int k = 0; k < NS2; ++k) S2[k * RS + lane] = s2[k];
+                double e = 0.0, T[3] = {0.0, 0.0, 0.0};
+#pragma unroll 1
+                for (int o = 0; o < NO; ++o) {
+                    if (o0 + o >= nops) break;
+                    double base[LM + 1];
+                    {
+                        double th = 1.0;
+                        if (o0 + o == 1 && !ominf) th = om * rsqrt(om * om + rho);
+                        double Fm[LM + 1];
+                        const double th2 = th * th;
+                        boys_lane<LM>(T0 * th2, Fm, boys);
+                        double f = pref * th;
+                        const double m2r = -2.0 * rho * th2;
+#pragma unroll
+                        for (int n = 0; n <= LM; ++n) {
+                            base[n] = f * Fm[n];
+                            f *= m2r;
+                        }
+                    }
+                    const double *Fl = F + (pi * NO + o) * NT1 * NM2P;
+                    double *Rl = Rr + lane;
+                    double Xd[nherm(L)];
+                    hermite_density<LA, LB, LC, LD>(Fl, s2, Xd);
+                    if constexpr (Lay::RREG) {
+                        double R[nherm(LM)];
+                        hermite_R<LM>(R, base, X, Y, Z);
+                        static_for<nherm(LM)>([&](auto H) {
+                            energy_terms<L, decltype(H)::value>(R[decltype(H)::value], Xd, e, T);
+                        });
+                        if constexpr (NIT > 0)
+#pragma unroll
+                            for (int h = 0; h < nherm(L); ++h) Rl[h * RS] = R[h];
+                    } else {
+                        // R in this lane's column, level by level in place: entries from high to
+                        // low, four at a time (their reads all precede their writes).  Before the
+                        // last level, the top order, which only T needs, is formed from level 1
+                        // and not stored.
+                        Rl[0] = base[LM];
+                        static_for<LM>([&](auto I) {
+                            constexpr int n = LM - 1 - decltype(I)::value;
+                            if constexpr (n == 0)
+                                static_for<nherm(LM) - nherm(L)>([&](auto J) {
+                                    constexpr int h = nherm(L) + decltype(J)::value;
+                                    constexpr Triple x = herm_triple(h);
+                                    constexpr int d = x.t > 0 ? 0 : (x.u > 0 ? 1 : 2);
+                                    constexpr int c = d == 0 ? x.t : (d == 1 ? x.u : x.v);
+                                    double r = (d == 0 ? X : (d == 1 ? Y : Z)) *
+                                               lds(Rl + hidx(x.t - (d == 0), x.u - (d == 1), x.v - (d == 2)) * RS);
+                                    if constexpr (c > 1)
+                                        r += double(c - 1) *
+                                             lds(Rl + hidx(x.t - 2 * (d == 0), x.u - 2 * (d == 1), x.v - 2 * (d == 2)) * RS);
+                                    energy_terms<L, h>(r, Xd, e, T);
+                                });
+                            constexpr int top = (LM - n < L ? LM - n : L);
+#pragma unroll 1
+                            for (int h = nherm(top) - 1; h >= 1; h -= 4) {
+                                double v[4];
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) {
+                                    const unsigned w = kHermSteps.w[h - k > 0 ? h - k : 1];
+                                    const unsigned dir = w & 3;
+                                    v[k] = (dir == 0 ? X : (dir == 1 ? Y : Z)) * Rl[((w >> 2) & 0xff) * RS] +
+                                           double((int)(w >> 18)) * Rl[((w >> 10) & 0xff) * RS];
+                                }
+#pragma unroll
+                                for (int k = 0; k < 4; ++k)
+                                    if (h - k > 0) Rl[(h - k) * RS] = v[k];
+                            }
+                            Rl[0] = base[n];
+                        });
+                        static_for<nherm(L)>([&](auto H) {
+                            constexpr int h = decltype(H)::value;
+                            energy_terms<L, h>(lds(Rl + h * RS), Xd, e, T);
+                        });
+                    }
+                    __syncwarp();
+                    // ---- reverse sums U[h1][m2], added to V with the bra scalars
+                    if constexpr (NIT > 0) {
+                        const int n = min(32, ntot - j0), pfirst = j0 / nkp, plast = (j0 + n - 1) / nkp;
+                        const int sub = lane / ITL;
+                        for (int i0 = 0; i0 < NIT; i0 += ITL) {
+                            const int it = i0 + lane % ITL;
+                            const unsigned w = items[min(it, NIT - 1)];
+                            const double *r = Rr + (w & 0xff) * RS, *s = S2 + (w >> 21) * RS;
+                            const unsigned hm = TBra.hm[(w >> 8) & 0x3f];
+                            double *v = V + (o * NM1 + (hm & 0xff)) * NM2P + ((w >> 14) & 0x7f);
+                            const int ns = (hm >> 8) & 0xf;
+                            for (int pj = pfirst; pj <= plast; ++pj) {
+                                const int lo = max(pj * nkp - j0, 0), hi = min((pj + 1) * nkp - j0, n);
+                                double u = 0.0;
+#pragma unroll 4
+                                for (int j = lo + sub; j < hi; j += SUB) u += s[j] * r[j];
+#pragma unroll
+                                for (int x = ITL; x < 32; x *= 2) u += __shfl_xor_sync(0xffffffffu, u, x);
+                                if (it < NIT && sub == 0) {
+                                    const double *s1 = S1 + pj * NS1 + (hm >> 12);
+                                    for (int k = 0; k < ns; ++k) v[k * NM2P] += s1[k] * u;
+                                }
+                            }
+                        }
+                        __syncwarp();
+                    }
+                }
+                const double a = P1[pi * NP1];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    aT[i] += T[i];
+                    aA[i] += a * T[i];
+                    aC[i] += c * T[i];
+                }
+                eA += P1[pi * NP1 + 1] * e;
+                eC += zc * d * e;
+            }
+            __syncwarp();  // S1, P1 and F are rewritten for the next block
+        }
+        // ---- polynomial parts: V with dG'/dR (ket half again) and dG'/dS (bra half)
+        if constexpr (NIT > 0) {
+            entry_values<LA, LB>(vb, lane, pw);
+            entry_values<LC, LD>(vk, lane, pw + 15);
+            __syncwarp();
+            if constexpr (Lay::L1 > 0) {
+                half_ket<LA, LB, LC, LD>(half, G, vk, lane);
+                __syncwarp();
+                for (int it = lane; it < Lay::NE1; it += 32) {
+                    const unsigned w = TBra.ent[it];
+                    const int px = (w >> 16) & 7, py = (w >> 19) & 7, pz = (w >> 22) & 7;
+                    if (px + py + pz == 0) continue;
+                    const int m1 = TBra.own[it], ab = w & 0xff;
+                    double s = 0.0;
+#pragma unroll
+                    for (int o = 0; o < NO; ++o)
+                        for (int m2 = 0; m2 < NM2; ++m2)
+                            s += half[(o * NM2 + m2) * NABP + ab] * V[(o * NM1 + m1) * NM2P + m2];
+                    s *= double((int)((w >> 8) & 0xff));
+                    const double qx = pw[px], qy = pw[5 + py], qz = pw[10 + pz];
+                    if (px) gA[0] += s * double(px) * pw[px - 1] * qy * qz;
+                    if (py) gA[1] += s * double(py) * qx * pw[5 + py - 1] * qz;
+                    if (pz) gA[2] += s * double(pz) * qx * qy * pw[10 + pz - 1];
+                }
+                __syncwarp();
+            }
+            if constexpr (Lay::L2 > 0) {
+                // bra half [m1][cd]
+                for (int it = lane; it < NM1 * NCD; it += 32) {
+                    const int m1 = it / NCD, cd = it % NCD;
+#pragma unroll
+                    for (int o = 0; o < NO; ++o) {
+                        double s = 0.0;
+                        for (int x = TBra.start[m1]; x < TBra.start[m1 + 1]; ++x)
+                            s += vb[x] * G[(o * NCD + cd) * NABP + (TBra.ent[x] & 0xff)];
+                        half[(o * NM1 + m1) * NCD + cd] = s;
+                    }
+                }
+                __syncwarp();
+                for (int it = lane; it < Lay::NE2; it += 32) {
+                    const unsigned w = TKet.ent[it];
+                    const int px = (w >> 16) & 7, py = (w >> 19) & 7, pz = (w >> 22) & 7;
+                    if (px + py + pz == 0) continue;
+                    const int m2 = TKet.own[it], cd = w & 0xff;
+                    double s = 0.0;
+#pragma unroll
+                    for (int o = 0; o < NO; ++o)
+                        for (int m1 = 0; m1 < NM1; ++m1)
+                            s += half[(o * NM1 + m1) * NCD + cd] * V[(o * NM1 + m1) * NM2P + m2];
+                    s *= double((int)((w >> 8) & 0xff));
+                    const double *pk = pw + 15;
+                    const double qx = pk[px], qy = pk[5 + py], qz = pk[10 + pz];
+                    if (px) gC[0] += s * double(px) * pk[px - 1] * qy * qz;
+                    if (py) gC[1] += s * double(py) * qx * pk[5 + py - 1] * qz;
+                    if (pz) gC[2] += s * double(pz) * qx * qy * pk[10 + pz - 1];
+                }
+            }
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        acc[i] += aA[i] - 2.0 * pw[i * 5 + 1] * eA + gA[i];
+        acc[3 + i] += aT[i];
+        acc[6 + i] += -aC[i] - 2.0 * pw[15 + i * 5 + 1] * eC + gC[i];
+    }
+}
+
+// items table of the class this translation unit compiles
+template <int LA, int LB, int LC, int LD>
+__device__ const HermItems<LA, LB, LC, LD> kHermItems = make_herm_items<LA, LB, LC, LD>();
+
+// CTAs per SM the registers are limited to
+template <int LA, int LB, int LC, int LD>
+constexpr int herm_min_ctas()
+{
+    return LA + LB + LC + LD <= 2 ? 4 : (LA + LB + LC + LD <= 3 ? 3 : (LA + LB + LC + LD <= 4 ? 2 : 1));
+}
+
+// Persistent class kernel, four warps per CTA; units, screening, staging and
+// the fixed-order tile reduction as in k_grad.
+template <int LA, int LB, int LC, int LD>
+__global__ void __launch_bounds__(TILE, (herm_min_ctas<LA, LB, LC, LD>()))
+    k_grad_herm(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out, const double *__restrict__ boys)
+{
+    using Lay = HermLay<LA, LB, LC, LD>;
+    constexpr int NG = TILE / 32;
+    extern __shared__ double smem[];
+    const int nacc3 = out.use_smem ? out.natom_max * 3 : 0;
+    double *sg = smem;
+    double *stg = smem + nacc3;
+    int *sat = reinterpret_cast<int *>(stg + TILE * 12);
+    double *tred = reinterpret_cast<double *>(sat + TILE * 4);
+    int *ratom = reinterpret_cast<int *>(tred + 6 * (TB + TK));
+    const int grp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    double *wsm = reinterpret_cast<double *>(ratom + 2 * (TB + TK)) + (size_t)grp * Lay::TOTAL;
+    const unsigned *items = kHermItems<LA, LB, LC, LD>.it;
+    double *slab = out.partials + (size_t)blockIdx.x * out.natom_total * 3;
+    int cur = -1, cur_off3 = 0, cur_n3 = 0;
+    unsigned long long nq = 0, npq = 0, nbv = 0;
+    const int S = cl.nsplit, C = cl.nchunk, QPC = TILE / C;
+    for (long long it = blockIdx.x; it < cl.ntiles * C * S; it += gridDim.x) {
+        const long long tile = it / (C * S);
+        const int chunk = (int)((it / S) % C), split = (int)(it % S);
+        const uint4 tl = cl.tiles[tile * cl.stride];
+        const int mol = (int)tl.x;
+        if (mol != cur) {
+            if (out.use_smem) {
+                if (cur >= 0)
+                    for (int k = threadIdx.x; k < cur_n3; k += blockDim.x) slab[cur_off3 + k] += sg[k];
+                __syncthreads();
+                for (int k = threadIdx.x; k < nacc3; k += blockDim.x) sg[k] = 0.0;
+                __syncthreads();
+            }
+            cur = mol;
+            cur_off3 = mols[mol].atom_off * 3;
+            cur_n3 = mols[mol].geo.natom * 3;
+        }
+        const MolDesc &md = mols[mol];
+        const PairSet bra = md.sets[cl.P], ket = md.sets[cl.Q];
+        const ScreenArgs scr = md.scr;
+        const bool same = cl.P == cl.Q;
+        if (C > 1 && !out.dump) {
+            for (int k = threadIdx.x; k < TILE * 12; k += blockDim.x) stg[k] = 0.0;
+            for (int k = threadIdx.x; k < TILE * 4; k += blockDim.x) sat[k] = -1;
+            __syncthreads();
+        }
+        for (int qi = chunk * QPC + grp; qi < (chunk + 1) * QPC; qi += NG) {
+            const int bi = tl.y * TB + qi / TK;
+            const int ki = tl.z * TK + qi % TK;
+            double g = 0.0;
+            bool ok = bi < bra.n && ki < ket.n && (!same || bi >= ki);
+            if (ok) ok = split < bra.np[bi];
+            int sa = 0, sb = 0, sc = 0, sd = 0;
+            if (ok) {
+                sa = bra.sa[bi];
+                sb = bra.sb[bi];
+                sc = ket.sa[ki];
+                sd = ket.sb[ki];
+                ok = keep_quartet(scr, bra, ket, bi, ki, sa, sb, sc, sd);
+            }
+            if (ok) {  // uniform across the warp
+                double scale = 1.0;
+                if (sa == sb) scale *= 0.5;
+                if (sc == sd) scale *= 0.5;
+                if (same && bi == ki) scale *= 0.5;
+                const int nbp = bra.np[bi], nkp = ket.np[ki];
+                double acc[9];
+#pragma unroll
+                for (int k = 0; k < 9; ++k) acc[k] = 0.0;
+                if (nkp > 0)
+                    quartet_herm<LA, LB, LC, LD>(wsm, lane, items, md.geo, md.den, md.pp, sa, sb, sc, sd, bra.poff[bi],
+                                                 nbp, split, S, ket.poff[ki], nkp, scale, boys, acc);
+                // the nine sums over the warp through shared memory: three lanes a sum
+                double *red = wsm + Lay::o_X;
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < 9; ++k) red[k * Lay::RS + lane] = acc[k];
+                __syncwarp();
+                double s = 0.0;
+                const int k = lane / 3 < 9 ? lane / 3 : 8, part = lane % 3;
+                for (int j = part; j < 32; j += 3) s += red[k * Lay::RS + j];
+                const double s1 = __shfl_down_sync(0xffffffffu, s, 1), s2 = __shfl_down_sync(0xffffffffu, s, 2);
+                s = s + s1 + s2;  // valid on lanes 3k
+                const int X = lane / 3, i = lane % 3;  // lanes 0..11: output component X * 3 + i
+                const double dA = __shfl_sync(0xffffffffu, s, 3 * i), dT = __shfl_sync(0xffffffffu, s, 3 * (3 + i));
+                const double dC = __shfl_sync(0xffffffffu, s, 3 * (6 + i));
+                g = X == 0 ? dA : (X == 1 ? dT - dA : (X == 2 ? dC : -dT - dC));
+                __syncwarp();
+                if (lane == 0) {
+                    if (split == 0) nq += 1;
+                    npq += (unsigned long long)((nbp - split + S - 1) / S) * nkp;
+                    nbv += (unsigned long long)((nbp - split + S - 1) / S);
+                }
+            }
+            if (out.dump) {  // one unit per tile
+                if (lane < 12) out.dump[((size_t)tile * TILE + qi) * 12 + lane] = g;
+            } else {
+                if (lane < 12) stg[qi * 12 + lane] = g;
+                if (lane < 4) sat[qi * 4 + lane] = ok ? md.geo.sh_atom[lane == 0 ? sa : (lane == 1 ? sb : (lane == 2 ? sc : sd))] : -1;
+            }
+        }
+        __syncthreads();
+        if (!out.dump) tile_reduce(stg, sat, tred, ratom, out.use_smem ? sg : slab + cur_off3);
+        __syncthreads();
+    }
+    if (out.use_smem && cur >= 0)
+        for (int k = threadIdx.x; k < cur_n3; k += blockDim.x) slab[cur_off3 + k] += sg[k];
+    if (lane == 0 && (nq || npq)) {  // a split unit may hold primitives only
+        atomicAdd(out.counters + 0, nq);
+        atomicAdd(out.counters + 1, npq);
+        atomicAdd(out.counters + 4, nbv);
+    }
+}
+
+// Launch of the class kernel.  smem holds the tile staging and, with use_smem,
+// one molecule's gradient; where that gradient no longer fits beside the warps'
+// arrays the CTAs add to their slabs in device memory instead.
+template <int LA, int LB, int LC, int LD>
+cudaError_t launch_herm(int gcap, size_t smem, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl,
+                        const OutArgs &out, const double *boys)
+{
+    constexpr size_t warps = (TILE / 32) * HermLay<LA, LB, LC, LD>::BYTES;
+    static_assert(PairTab<LA, LB>::NE > 0 && warps + 16384 <= 227 * 1024, "four warps' arrays fit beside the staging");
+    OutArgs o = out;
+    if (o.use_smem && smem + warps > 227 * 1024) {
+        o.use_smem = 0;
+        smem -= sizeof(double) * 3 * (size_t)o.natom_max;
+    }
+    return launch_units(k_grad_herm<LA, LB, LC, LD>, TILE / 32, gcap, smem + warps, st, mols, cl, o, boys);
+}
+
+// Kernel forms per class.  fp64: the Hermite-density kernel wherever four
+// warps' arrays fit beside the staging, else the group kernel ((dd|dp),
+// (dd|dd)).  fp32: the thread kernel below 648 function quartets (above, its
+// per-thread arrays run to tens of KB of local memory), the group kernel from
+// 648, the warp kernel wherever four warps' arrays fit (all but (dd|dd)).
+// ClassLaunch::kind 1 / 2 / 3 asks for the thread / group / warp kernel; a form
+// not compiled for the class and precision falls back to the default.
+template <int LA, int LB, int LC, int LD>
+struct ClassForms {
+    static constexpr int nfq = ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD);
+    static constexpr size_t kStageMax = 200 * 1024;  // warp arrays + tile staging (16 KB) per CTA
+    static constexpr bool herm = (TILE / 32) * HermLay<LA, LB, LC, LD>::BYTES + 16384 <= 227 * 1024;
+    static constexpr bool thread32 = nfq < 648;
+    static constexpr bool group32 = nfq >= 648;
+    static constexpr bool warp32 = warp_kernel_smem<LA, LB, LC, LD, float>() + 16384 <= kStageMax;
+    // default fp32 form per class (1 thread, 2 group, 3 warp)
+    static constexpr int qc = pair_class(LA, LB) * (pair_class(LA, LB) + 1) / 2 + pair_class(LC, LD);
+    static constexpr int default32 = kDefaultForm32[qc];
+    static_assert((default32 != 1 || thread32) && (default32 != 2 || group32) && (default32 != 3 || warp32),
+                  "default fp32 form not compiled");
+};
+
+template <int LA, int LB, int LC, int LD>
+cudaError_t launch_class_kernel(int fp32, int gcap, size_t smem, cudaStream_t st, const MolDesc *mols,
+                                const ClassLaunch &cl, const OutArgs &out, const double *boys)
+{
+    using K = ClassForms<LA, LB, LC, LD>;
+    if (!fp32) {
+        if constexpr (K::herm)
+            return launch_herm<LA, LB, LC, LD>(gcap, smem, st, mols, cl, out, boys);
+        else
+            return launch_coop<LA, LB, LC, LD, double>(gcap, smem, st, mols, cl, out, boys);
+    }
+    int kind = cl.kind;
+    if ((kind == 1 && !K::thread32) || (kind == 2 && !K::group32) || (kind == 3 && !K::warp32) || kind < 1 || kind > 3)
+        kind = K::default32;
+    if constexpr (K::warp32)
+        if (kind == 3) return launch_warp<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
+    if constexpr (K::group32)
+        if (kind == 2) return launch_coop<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
+    if constexpr (K::thread32)
+        if (kind == 1) return launch_units(k_grad<LA, LB, LC, LD, true>, 0, gcap, smem, st, mols, cl, out, boys);
+    return cudaErrorInvalidValue;  // not reached: every class compiles its default form
+}
+
+}  // namespace tg

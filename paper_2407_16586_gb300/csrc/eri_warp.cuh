@@ -821,62 +821,6 @@ cudaError_t launch_warp(int gcap, size_t smem, cudaStream_t st, const MolDesc *m
 // kernel times of the mixed route on the 32-atom chain (the fp64 lists there
 // hold the largest, most contracted tiles) and of the all-fp64 route; where
 // the two disagree by little, the mixed route's choice is kept.
-constexpr int kDefaultForm64[NQC] = {1, 1, 1, 1, 1, 3, 1, 1, 1, 3, 1, 3, 3, 3, 3, 3, 3, 3, 3, 2, 2};
 constexpr int kDefaultForm32[NQC] = {1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 3, 3, 2, 2};
-
-// Kernel forms per class.  The thread kernel is compiled below 648 function
-// quartets (above, its per-thread arrays run to tens of KB of local memory),
-// the group kernel for fp64 from 54 and fp32 from 648 function quartets, and
-// the warp kernel wherever four warps' arrays fit in shared memory next to
-// the tile staging (all classes but (dd|dp) and (dd|dd) in fp64, all but
-// (dd|dd) in fp32).  ClassLaunch::kind 1 / 2 / 3 asks for the thread / group /
-// warp kernel; a form not compiled for the class falls back to the default.
-template <int LA, int LB, int LC, int LD>
-struct ClassForms {
-    static constexpr int nfq = ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD);
-    static constexpr size_t kStageMax = 200 * 1024;  // warp arrays + tile staging (16 KB) per CTA
-    static constexpr bool thread = nfq < 648;
-    static constexpr bool group64 = nfq >= 54;
-    static constexpr bool group32 = nfq >= 648;
-    static constexpr bool warp64 = warp_kernel_smem<LA, LB, LC, LD, double>() + 16384 <= kStageMax;
-    static constexpr bool warp32 = warp_kernel_smem<LA, LB, LC, LD, float>() + 16384 <= kStageMax;
-    // default form per class (1 thread, 2 group, 3 warp): the fastest form
-    // measured on GB300 for the 32-atom chain workload, per precision
-    static constexpr int qc = pair_class(LA, LB) * (pair_class(LA, LB) + 1) / 2 + pair_class(LC, LD);
-    static constexpr int default64 = kDefaultForm64[qc];
-    static constexpr int default32 = kDefaultForm32[qc];
-    static_assert((default64 != 1 || thread) && (default64 != 2 || group64) && (default64 != 3 || warp64),
-                  "default fp64 form not compiled");
-    static_assert((default32 != 1 || thread) && (default32 != 2 || group32) && (default32 != 3 || warp32),
-                  "default fp32 form not compiled");
-};
-
-template <int LA, int LB, int LC, int LD>
-cudaError_t launch_class_kernel(int fp32, int gcap, size_t smem, cudaStream_t st, const MolDesc *mols,
-                                const ClassLaunch &cl, const OutArgs &out, const double *boys)
-{
-    using K = ClassForms<LA, LB, LC, LD>;
-    int kind = cl.kind;
-    if (fp32) {
-        if ((kind == 1 && !K::thread) || (kind == 2 && !K::group32) || (kind == 3 && !K::warp32) || kind < 1 || kind > 3)
-            kind = K::default32;
-        if constexpr (K::warp32)
-            if (kind == 3) return launch_warp<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
-        if constexpr (K::group32)
-            if (kind == 2) return launch_coop<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
-        if constexpr (K::thread)
-            if (kind == 1) return launch_units(k_grad<LA, LB, LC, LD, true>, 0, gcap, smem, st, mols, cl, out, boys);
-    } else {
-        if ((kind == 1 && !K::thread) || (kind == 2 && !K::group64) || (kind == 3 && !K::warp64) || kind < 1 || kind > 3)
-            kind = K::default64;
-        if constexpr (K::warp64)
-            if (kind == 3) return launch_warp<LA, LB, LC, LD, double>(gcap, smem, st, mols, cl, out, boys);
-        if constexpr (K::group64)
-            if (kind == 2) return launch_coop<LA, LB, LC, LD, double>(gcap, smem, st, mols, cl, out, boys);
-        if constexpr (K::thread)
-            if (kind == 1) return launch_units(k_grad<LA, LB, LC, LD, false>, 0, gcap, smem, st, mols, cl, out, boys);
-    }
-    return cudaErrorInvalidValue;  // not reached: every class compiles its default form
-}
 
 }  // namespace tg
