@@ -197,8 +197,11 @@ struct HermLay {
     static constexpr int NT1 = B::NH, NM1 = B::NM, NM2 = K::NM, NS1 = B::NS, NS2 = K::NS;
     static constexpr int NABP = NAB | 1, NM2P = NM2 | 1;
     static constexpr int RS = 33;                     // row stride of the per-lane columns
-    static constexpr int NRH = nherm(L);              // Hermite rows kept for the reverse sums
-    static constexpr bool RREG = LM <= 5;             // R tensor in registers, or in its shared-memory rows
+    // The R tensor: in registers up to LM = 5, else in shared-memory rows; X in
+    // registers, from L = 7 (120 entries) in passes over ranges of Hermite
+    // orders, which need R's top order stored too.
+    static constexpr bool RREG = LM <= 5, PASSES = L >= 7;
+    static constexpr int NRH = nherm(PASSES ? LM : L);  // Hermite rows
     static constexpr int NO = (NAB * NCD <= 27) ? 2 : 1;
     // bra primitive pairs of a block: a budget of 1200 doubles for F, 1 to 16
     static constexpr int PB_RAW = 1200 / (NT1 * NM2P * NO);
@@ -347,15 +350,20 @@ __device__ __forceinline__ void static_for(Fn &&f)
     static_for_impl(f, std::make_integer_sequence<int, N>{});
 }
 
-// Shared-memory load of the unrolled lane phases.  Volatile inline PTX: the
-// address is the warp's own slice and every write to it is ordered by
-// __syncwarp, while plain loads between this many stores make the compiler's
-// alias analysis take minutes per class.
+// Shared-memory load of the unrolled lane phases.  Inline PTX: plain loads
+// between this many stores make the compiler's alias analysis take minutes per
+// class.  The compiler does not see that it reads memory, so lds_fence() (or
+// __syncwarp) stands between it and plain accesses to the same rows.
 __device__ __forceinline__ double lds(const double *p)
 {
     double v;
     asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"((unsigned)__cvta_generic_to_shared(p)));
     return v;
+}
+
+__device__ __forceinline__ void lds_fence()
+{
+    asm volatile("" ::: "memory");
 }
 
 // (t, u, v) of a compact Hermite index, at compile time
@@ -403,22 +411,42 @@ __host__ __device__ constexpr int herm_sum(int h1, int h2)
     return hidx(a.t + b.t, a.u + b.u, a.v + b.v);
 }
 
-// X[h] of one lane: sum over h1 and the ket monomials of s_m2 F[h1][m2]
-// (F: this lane's bra primitive pair).
-template <int LA, int LB, int LC, int LD>
+// X[h] of one lane for the Hermite orders HLO .. HHI: sum over h1 and the ket
+// monomials of s_m2 F[h1][m2] (F: this lane's bra primitive pair).
+template <int LA, int LB, int LC, int LD, int HLO, int HHI>
 __device__ __forceinline__ void hermite_density(const double *F, const double (&s2)[PairMono<LC, LD>::NS],
-                                                double (&X)[nherm(LA + LB + LC + LD)])
+                                                double (&X)[nherm(HHI) - nherm(HLO - 1)])
 {
     using Lay = HermLay<LA, LB, LC, LD>;
+    constexpr int H0 = nherm(HLO - 1), H1 = nherm(HHI);
 #pragma unroll
-    for (int h = 0; h < nherm(Lay::L); ++h) X[h] = 0.0;
-    static_for<Lay::NT1>([&](auto H1) {
+    for (int h = 0; h < H1 - H0; ++h) X[h] = 0.0;
+    static_for<Lay::NT1>([&](auto B) {
         static_for<Lay::NM2>([&](auto M2) {
-            constexpr int h1 = decltype(H1)::value, m2 = decltype(M2)::value;
+            constexpr int h1 = decltype(B)::value, m2 = decltype(M2)::value;
             constexpr auto row = make_dens_row<LC, LD>();
             constexpr int x = herm_sum(h1, row.h2[m2]), sc = row.s[m2];
-            X[x] += s2[sc] * lds(F + h1 * Lay::NM2P + m2);
+            if constexpr (x >= H0 && x < H1) X[x - H0] += s2[sc] * lds(F + h1 * Lay::NM2P + m2);
         });
+    });
+}
+
+// One pass over a range of orders: E += X[h] R[h], T_i += X[h] R[h + 1_i], R
+// from this lane's column.
+template <int LA, int LB, int LC, int LD, int HLO, int HHI>
+__device__ __forceinline__ void density_pass(const double *F, const double (&s2)[PairMono<LC, LD>::NS],
+                                             const double *Rl, double &e, double (&T)[3])
+{
+    constexpr int RS = HermLay<LA, LB, LC, LD>::RS, H0 = nherm(HLO - 1);
+    double X[nherm(HHI) - H0];
+    hermite_density<LA, LB, LC, LD, HLO, HHI>(F, s2, X);
+    static_for<nherm(HHI) - H0>([&](auto J) {
+        constexpr int j = decltype(J)::value;
+        constexpr Triple x = herm_triple(H0 + j);
+        e += X[j] * lds(Rl + (H0 + j) * RS);
+        T[0] += X[j] * lds(Rl + hidx(x.t + 1, x.u, x.v) * RS);
+        T[1] += X[j] * lds(Rl + hidx(x.t, x.u + 1, x.v) * RS);
+        T[2] += X[j] * lds(Rl + hidx(x.t, x.u, x.v + 1) * RS);
     });
 }
 
@@ -453,6 +481,29 @@ constexpr HermSteps make_herm_steps()
     return s;
 }
 static __device__ const HermSteps kHermSteps = make_herm_steps();
+
+// Entries 1 .. n - 1 of one level in this lane's column, in place, from high
+// to low: every entry reads lower ones, and of four at a time all reads
+// precede the writes.
+template <int RS>
+__device__ __forceinline__ void hermite_level(double *Rl, int n, double X, double Y, double Z)
+{
+#pragma unroll 1
+    for (int h = n - 1; h >= 1; h -= 4) {
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned w = kHermSteps.w[h - k > 0 ? h - k : 1];
+            const unsigned dir = w & 3;
+            v[k] = (dir == 0 ? X : (dir == 1 ? Y : Z)) * Rl[((w >> 2) & 0xff) * RS];
+            const int c = (int)(w >> 18);  // the same for all lanes
+            if (c > 0) v[k] += double(c) * Rl[((w >> 10) & 0xff) * RS];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (h - k > 0) Rl[(h - k) * RS] = v[k];
+    }
+}
 
 // ------------------------------------------------------------ quartet
 
@@ -664,9 +715,9 @@ __device__ void quartet_herm(double *sm, int lane, const unsigned *items, const 
                     }
                     const double *Fl = F + (pi * NO + o) * NT1 * NM2P;
                     double *Rl = Rr + lane;
-                    double Xd[nherm(L)];
-                    hermite_density<LA, LB, LC, LD>(Fl, s2, Xd);
                     if constexpr (Lay::RREG) {
+                        double Xd[nherm(L)];
+                        hermite_density<LA, LB, LC, LD, 0, L>(Fl, s2, Xd);
                         double R[nherm(LM)];
                         hermite_R<LM>(R, base, X, Y, Z);
                         static_for<nherm(LM)>([&](auto H) {
@@ -675,15 +726,16 @@ __device__ void quartet_herm(double *sm, int lane, const unsigned *items, const 
                         if constexpr (NIT > 0)
 #pragma unroll
                             for (int h = 0; h < nherm(L); ++h) Rl[h * RS] = R[h];
-                    } else {
-                        // R in this lane's column, level by level in place: entries from high to
-                        // low, four at a time (their reads all precede their writes).  Before the
-                        // last level, the top order, which only T needs, is formed from level 1
-                        // and not stored.
+                    } else if constexpr (!Lay::PASSES) {
+                        double Xd[nherm(L)];
+                        hermite_density<LA, LB, LC, LD, 0, L>(Fl, s2, Xd);
+                        // R in this lane's column, level by level.  Before the last level, the
+                        // top order, which only T needs, is formed from level 1 and not stored.
                         Rl[0] = base[LM];
                         static_for<LM>([&](auto I) {
                             constexpr int n = LM - 1 - decltype(I)::value;
-                            if constexpr (n == 0)
+                            if constexpr (n == 0) {
+                                lds_fence();
                                 static_for<nherm(LM) - nherm(L)>([&](auto J) {
                                     constexpr int h = nherm(L) + decltype(J)::value;
                                     constexpr Triple x = herm_triple(h);
@@ -696,27 +748,27 @@ __device__ void quartet_herm(double *sm, int lane, const unsigned *items, const 
                                              lds(Rl + hidx(x.t - 2 * (d == 0), x.u - 2 * (d == 1), x.v - 2 * (d == 2)) * RS);
                                     energy_terms<L, h>(r, Xd, e, T);
                                 });
-                            constexpr int top = (LM - n < L ? LM - n : L);
-#pragma unroll 1
-                            for (int h = nherm(top) - 1; h >= 1; h -= 4) {
-                                double v[4];
-#pragma unroll
-                                for (int k = 0; k < 4; ++k) {
-                                    const unsigned w = kHermSteps.w[h - k > 0 ? h - k : 1];
-                                    const unsigned dir = w & 3;
-                                    v[k] = (dir == 0 ? X : (dir == 1 ? Y : Z)) * Rl[((w >> 2) & 0xff) * RS] +
-                                           double((int)(w >> 18)) * Rl[((w >> 10) & 0xff) * RS];
-                                }
-#pragma unroll
-                                for (int k = 0; k < 4; ++k)
-                                    if (h - k > 0) Rl[(h - k) * RS] = v[k];
+                                lds_fence();
                             }
+                            hermite_level<RS>(Rl, nherm(LM - n < L ? LM - n : L), X, Y, Z);
                             Rl[0] = base[n];
                         });
+                        lds_fence();
                         static_for<nherm(L)>([&](auto H) {
                             constexpr int h = decltype(H)::value;
                             energy_terms<L, h>(lds(Rl + h * RS), Xd, e, T);
                         });
+                    } else {
+                        Rl[0] = base[LM];
+                        static_for<LM>([&](auto I) {
+                            constexpr int n = LM - 1 - decltype(I)::value;
+                            hermite_level<RS>(Rl, nherm(LM - n), X, Y, Z);
+                            Rl[0] = base[n];
+                        });
+                        lds_fence();
+                        density_pass<LA, LB, LC, LD, 0, 5>(Fl, s2, Rl, e, T);
+                        density_pass<LA, LB, LC, LD, 6, 7>(Fl, s2, Rl, e, T);
+                        if constexpr (L == 8) density_pass<LA, LB, LC, LD, 8, 8>(Fl, s2, Rl, e, T);
                     }
                     __syncwarp();
                     // ---- reverse sums U[h1][m2], added to V with the bra scalars
@@ -830,62 +882,54 @@ __device__ void quartet_herm(double *sm, int lane, const unsigned *items, const 
 template <int LA, int LB, int LC, int LD>
 __device__ const HermItems<LA, LB, LC, LD> kHermItems = make_herm_items<LA, LB, LC, LD>();
 
-// CTAs per SM the registers are limited to
+// Warps of a CTA and resident CTAs the registers are limited to: 16 warps at
+// 128 registers up to L = 2, 12 at 168 for L = 3, 8 at 255 above.  One warp per
+// scheduler already covers most of the fp64 pipe; the second and third fill
+// the gaps left by the transforms' loads and by dependent steps.
 template <int LA, int LB, int LC, int LD>
-constexpr int herm_min_ctas()
-{
-    return LA + LB + LC + LD <= 2 ? 4 : (LA + LB + LC + LD <= 3 ? 3 : (LA + LB + LC + LD <= 4 ? 2 : 1));
-}
+struct HermWarps {
+    static constexpr int L = LA + LB + LC + LD;
+    static constexpr int max_warps = L == 3 ? 12 : 8;
+    static constexpr int min_ctas = L <= 2 ? 2 : 1;
+};
 
-// Persistent class kernel, four warps per CTA; units, screening, staging and
-// the fixed-order tile reduction as in k_grad.
+// Persistent class kernel; every warp works alone.  Warp w of W takes the
+// units (tile, chunk of cl.nchunk per tile, split) w, 2W - 1 - w, 2W + w, ...:
+// the tile list is in decreasing cost, so the alternating order evens the
+// sums out.  A quartet's 12 components are added to the warp's own gradient
+// (shared memory, or with out.use_smem = 0 the warp's slab), so the schedule
+// and the order of all sums are fixed and results are bitwise reproducible.
 template <int LA, int LB, int LC, int LD>
-__global__ void __launch_bounds__(TILE, (herm_min_ctas<LA, LB, LC, LD>()))
+__global__ void __launch_bounds__((32 * HermWarps<LA, LB, LC, LD>::max_warps), (HermWarps<LA, LB, LC, LD>::min_ctas))
     k_grad_herm(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out, const double *__restrict__ boys)
 {
     using Lay = HermLay<LA, LB, LC, LD>;
-    constexpr int NG = TILE / 32;
     extern __shared__ double smem[];
-    const int nacc3 = out.use_smem ? out.natom_max * 3 : 0;
-    double *sg = smem;
-    double *stg = smem + nacc3;
-    int *sat = reinterpret_cast<int *>(stg + TILE * 12);
-    double *tred = reinterpret_cast<double *>(sat + TILE * 4);
-    int *ratom = reinterpret_cast<int *>(tred + 6 * (TB + TK));
-    const int grp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    double *wsm = reinterpret_cast<double *>(ratom + 2 * (TB + TK)) + (size_t)grp * Lay::TOTAL;
+    const int nw = blockDim.x / 32, grp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int n3 = out.natom_total * 3;
+    double *wsm = smem + (size_t)grp * Lay::TOTAL;
+    double *grad = out.use_smem ? smem + (size_t)nw * Lay::TOTAL + (size_t)grp * n3
+                                : out.partials + (size_t)(blockIdx.x * nw + grp) * n3;
     const unsigned *items = kHermItems<LA, LB, LC, LD>.it;
-    double *slab = out.partials + (size_t)blockIdx.x * out.natom_total * 3;
-    int cur = -1, cur_off3 = 0, cur_n3 = 0;
+    if (out.use_smem) {
+        for (int k = lane; k < n3; k += 32) grad[k] = 0.0;
+        __syncwarp();
+    }
     unsigned long long nq = 0, npq = 0, nbv = 0;
     const int S = cl.nsplit, C = cl.nchunk, QPC = TILE / C;
-    for (long long it = blockIdx.x; it < cl.ntiles * C * S; it += gridDim.x) {
+    const bool same = cl.P == cl.Q;
+    const long long units = cl.ntiles * C * S, W = (long long)gridDim.x * nw;
+    // neighbouring warps sit on different CTAs, so a short list spreads over the SMs
+    const long long w0 = (long long)grp * gridDim.x + blockIdx.x;
+    for (long long r = 0; r * W < units; ++r) {
+        const long long it = r * W + ((r & 1) ? W - 1 - w0 : w0);
+        if (it >= units) continue;
         const long long tile = it / (C * S);
         const int chunk = (int)((it / S) % C), split = (int)(it % S);
         const uint4 tl = cl.tiles[tile * cl.stride];
-        const int mol = (int)tl.x;
-        if (mol != cur) {
-            if (out.use_smem) {
-                if (cur >= 0)
-                    for (int k = threadIdx.x; k < cur_n3; k += blockDim.x) slab[cur_off3 + k] += sg[k];
-                __syncthreads();
-                for (int k = threadIdx.x; k < nacc3; k += blockDim.x) sg[k] = 0.0;
-                __syncthreads();
-            }
-            cur = mol;
-            cur_off3 = mols[mol].atom_off * 3;
-            cur_n3 = mols[mol].geo.natom * 3;
-        }
-        const MolDesc &md = mols[mol];
-        const PairSet bra = md.sets[cl.P], ket = md.sets[cl.Q];
-        const ScreenArgs scr = md.scr;
-        const bool same = cl.P == cl.Q;
-        if (C > 1 && !out.dump) {
-            for (int k = threadIdx.x; k < TILE * 12; k += blockDim.x) stg[k] = 0.0;
-            for (int k = threadIdx.x; k < TILE * 4; k += blockDim.x) sat[k] = -1;
-            __syncthreads();
-        }
-        for (int qi = chunk * QPC + grp; qi < (chunk + 1) * QPC; qi += NG) {
+        const MolDesc &md = mols[tl.x];
+        const PairSet &bra = md.sets[cl.P], &ket = md.sets[cl.Q];
+        for (int qi = chunk * QPC; qi < (chunk + 1) * QPC; ++qi) {
             const int bi = tl.y * TB + qi / TK;
             const int ki = tl.z * TK + qi % TK;
             double g = 0.0;
@@ -897,7 +941,7 @@ __global__ void __launch_bounds__(TILE, (herm_min_ctas<LA, LB, LC, LD>()))
                 sb = bra.sb[bi];
                 sc = ket.sa[ki];
                 sd = ket.sb[ki];
-                ok = keep_quartet(scr, bra, ket, bi, ki, sa, sb, sc, sd);
+                ok = keep_quartet(md.scr, bra, ket, bi, ki, sa, sb, sc, sd);
             }
             if (ok) {  // uniform across the warp
                 double scale = 1.0;
@@ -926,6 +970,14 @@ __global__ void __launch_bounds__(TILE, (herm_min_ctas<LA, LB, LC, LD>()))
                 const double dA = __shfl_sync(0xffffffffu, s, 3 * i), dT = __shfl_sync(0xffffffffu, s, 3 * (3 + i));
                 const double dC = __shfl_sync(0xffffffffu, s, 3 * (6 + i));
                 g = X == 0 ? dA : (X == 1 ? dT - dA : (X == 2 ? dC : -dT - dC));
+                if (!out.dump && lane < 3) {  // lane i owns component i of every atom
+                    const int *at = md.geo.sh_atom;
+                    double *gi = grad + md.atom_off * 3 + lane;
+                    gi[at[sa] * 3] += dA;
+                    gi[at[sb] * 3] += dT - dA;
+                    gi[at[sc] * 3] += dC;
+                    gi[at[sd] * 3] += -dT - dC;
+                }
                 __syncwarp();
                 if (lane == 0) {
                     if (split == 0) nq += 1;
@@ -933,19 +985,19 @@ __global__ void __launch_bounds__(TILE, (herm_min_ctas<LA, LB, LC, LD>()))
                     nbv += (unsigned long long)((nbp - split + S - 1) / S);
                 }
             }
-            if (out.dump) {  // one unit per tile
-                if (lane < 12) out.dump[((size_t)tile * TILE + qi) * 12 + lane] = g;
-            } else {
-                if (lane < 12) stg[qi * 12 + lane] = g;
-                if (lane < 4) sat[qi * 4 + lane] = ok ? md.geo.sh_atom[lane == 0 ? sa : (lane == 1 ? sb : (lane == 2 ? sc : sd))] : -1;
-            }
+            if (out.dump && lane < 12) out.dump[((size_t)tile * TILE + qi) * 12 + lane] = g;
         }
-        __syncthreads();
-        if (!out.dump) tile_reduce(stg, sat, tred, ratom, out.use_smem ? sg : slab + cur_off3);
-        __syncthreads();
     }
-    if (out.use_smem && cur >= 0)
-        for (int k = threadIdx.x; k < cur_n3; k += blockDim.x) slab[cur_off3 + k] += sg[k];
+    if (out.use_smem && !out.dump) {
+        __syncthreads();
+        double *slab = out.partials + (size_t)blockIdx.x * n3;
+        const double *all = smem + (size_t)nw * Lay::TOTAL;
+        for (int k = threadIdx.x; k < n3; k += blockDim.x) {
+            double s = 0.0;
+            for (int w = 0; w < nw; ++w) s += all[(size_t)w * n3 + k];
+            slab[k] += s;
+        }
+    }
     if (lane == 0 && (nq || npq)) {  // a split unit may hold primitives only
         atomicAdd(out.counters + 0, nq);
         atomicAdd(out.counters + 1, npq);
@@ -953,35 +1005,66 @@ __global__ void __launch_bounds__(TILE, (herm_min_ctas<LA, LB, LC, LD>()))
     }
 }
 
-// Launch of the class kernel.  smem holds the tile staging and, with use_smem,
-// one molecule's gradient; where that gradient no longer fits beside the warps'
-// arrays the CTAs add to their slabs in device memory instead.
+// Shared memory a CTA may take (227 KB), and an SM's (228 KB with 1 KB per CTA).
+constexpr size_t kCtaSmem = 227 * 1024;
+
+// Launch of the class kernel with at most gcap slabs of partial gradients.
+// Tiles are cut into chunks down to single quartets until every warp has 32
+// units (with 4, the heaviest unit alone left (pp|pp) SMs idle 57 % of the
+// time on a 1/16 shard of the 32-atom workload), then along the bra primitive
+// pairs (which repeats the density transform) while warps have fewer than 4.
 template <int LA, int LB, int LC, int LD>
-cudaError_t launch_herm(int gcap, size_t smem, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl,
-                        const OutArgs &out, const double *boys)
+cudaError_t launch_herm(int gcap, cudaStream_t st, const MolDesc *mols, ClassLaunch cl, const OutArgs &out,
+                        const double *boys)
 {
-    constexpr size_t warps = (TILE / 32) * HermLay<LA, LB, LC, LD>::BYTES;
-    static_assert(PairTab<LA, LB>::NE > 0 && warps + 16384 <= 227 * 1024, "four warps' arrays fit beside the staging");
+    using Wp = HermWarps<LA, LB, LC, LD>;
+    constexpr size_t bytes = HermLay<LA, LB, LC, LD>::BYTES;
+    static_assert(bytes <= kCtaSmem, "one warp's arrays fit in a CTA");
     OutArgs o = out;
-    if (o.use_smem && smem + warps > 227 * 1024) {
-        o.use_smem = 0;
-        smem -= sizeof(double) * 3 * (size_t)o.natom_max;
+    auto kern = k_grad_herm<LA, LB, LC, LD>;
+    int dev = 0, nsm = 1, per = 1;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    // each warp's gradient beside its arrays while that leaves four warps (or what fits without), else per-warp slabs
+    const size_t grad = sizeof(double) * 3 * (size_t)o.natom_total;
+    const int fit = (int)(kCtaSmem / bytes), fit_g = (int)(kCtaSmem / (bytes + grad));
+    o.use_smem = fit_g >= (fit < 4 ? fit : 4);
+    const size_t per_warp = bytes + (o.use_smem ? grad : 0);
+    int nw = o.use_smem ? fit_g : fit;
+    if (nw > Wp::max_warps) nw = Wp::max_warps;
+    const int slabs = o.use_smem ? gcap : (gcap > nw ? gcap / nw : 1);  // CTAs the partials have room for
+    if (nw > gcap && !o.use_smem) nw = gcap;
+    const size_t sm = per_warp * nw;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * nw, sm)) != cudaSuccess) return e;
+    long long gmax = (long long)(per > 0 ? per : 1) * nsm;
+    if (gmax > slabs) gmax = slabs;
+    cl.nchunk = 1;
+    cl.nsplit = 1;
+    const long long warps = gmax * nw;
+    while (cl.ntiles * cl.nchunk < 32 * warps && cl.nchunk < TILE) cl.nchunk *= 2;
+    if (!o.dump) {
+        while (cl.ntiles * cl.nchunk * cl.nsplit < 4 * warps && cl.nsplit < 8) ++cl.nsplit;
+        if (cl.split_req > 0) cl.nsplit = cl.split_req;
     }
-    return launch_units(k_grad_herm<LA, LB, LC, LD>, TILE / 32, gcap, smem + warps, st, mols, cl, o, boys);
+    const long long units = cl.ntiles * cl.nchunk * cl.nsplit;
+    const int grid = (int)(units < gmax ? units : gmax);
+    if (units < grid * (long long)nw) nw = (int)((units + grid - 1) / grid);
+    kern<<<grid, 32 * nw, per_warp * nw, st>>>(mols, cl, o, boys);
+    return cudaGetLastError();
 }
 
-// Kernel forms per class.  fp64: the Hermite-density kernel wherever four
-// warps' arrays fit beside the staging, else the group kernel ((dd|dp),
-// (dd|dd)).  fp32: the thread kernel below 648 function quartets (above, its
-// per-thread arrays run to tens of KB of local memory), the group kernel from
-// 648, the warp kernel wherever four warps' arrays fit (all but (dd|dd)).
-// ClassLaunch::kind 1 / 2 / 3 asks for the thread / group / warp kernel; a form
-// not compiled for the class and precision falls back to the default.
+// Kernel forms per class.  fp64: the Hermite-density kernel.  fp32: the thread
+// kernel below 648 function quartets (above, its per-thread arrays run to tens
+// of KB of local memory), the group kernel from 648, the warp kernel wherever
+// four warps' arrays fit (all but (dd|dd)).  ClassLaunch::kind 1 / 2 / 3 asks
+// for the thread / group / warp kernel; a form not compiled for the class and
+// precision falls back to the default.
 template <int LA, int LB, int LC, int LD>
 struct ClassForms {
     static constexpr int nfq = ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD);
     static constexpr size_t kStageMax = 200 * 1024;  // warp arrays + tile staging (16 KB) per CTA
-    static constexpr bool herm = (TILE / 32) * HermLay<LA, LB, LC, LD>::BYTES + 16384 <= 227 * 1024;
     static constexpr bool thread32 = nfq < 648;
     static constexpr bool group32 = nfq >= 648;
     static constexpr bool warp32 = warp_kernel_smem<LA, LB, LC, LD, float>() + 16384 <= kStageMax;
@@ -997,12 +1080,7 @@ cudaError_t launch_class_kernel(int fp32, int gcap, size_t smem, cudaStream_t st
                                 const ClassLaunch &cl, const OutArgs &out, const double *boys)
 {
     using K = ClassForms<LA, LB, LC, LD>;
-    if (!fp32) {
-        if constexpr (K::herm)
-            return launch_herm<LA, LB, LC, LD>(gcap, smem, st, mols, cl, out, boys);
-        else
-            return launch_coop<LA, LB, LC, LD, double>(gcap, smem, st, mols, cl, out, boys);
-    }
+    if (!fp32) return launch_herm<LA, LB, LC, LD>(gcap, st, mols, cl, out, boys);
     int kind = cl.kind;
     if ((kind == 1 && !K::thread32) || (kind == 2 && !K::group32) || (kind == 3 && !K::warp32) || kind < 1 || kind > 3)
         kind = K::default32;
