@@ -15,7 +15,7 @@
 // Each target block is summed over the quartet on the warp and added to F
 // with fp64 atomics.
 #pragma once
-#include "eri_herm.cuh"
+#include "eri_lane32.cuh"
 
 namespace tg {
 

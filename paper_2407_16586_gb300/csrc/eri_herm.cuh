@@ -102,6 +102,8 @@ struct PairTab {
     unsigned ent[NE];                  // by monomial
     unsigned short own[NE];            // monomial of each entry
     unsigned short start[M::NM + 1];   // entries of monomial m: start[m] .. start[m + 1]
+    unsigned short fstart[M::NAB + 1]; // entries of function pair ab: fent[fstart[ab]] .. fent[fstart[ab + 1] - 1]
+    unsigned short fent[NE];
     unsigned short hm[M::NH];          // per Hermite index: first monomial | nsig << 8 | first scalar << 12
 };
 
@@ -161,6 +163,13 @@ constexpr PairTab<LA, LB> make_pair_tab()
             }
     T.start[M::NM] = (unsigned short)ne;
     T.n = ne;
+    int nf = 0;
+    for (int ab = 0; ab < M::NAB; ++ab) {
+        T.fstart[ab] = (unsigned short)nf;
+        for (int e = 0; e < ne && e < PairTab<LA, LB>::NE; ++e)
+            if ((int)(T.ent[e] & 0xff) == ab) T.fent[nf++] = (unsigned short)e;
+    }
+    T.fstart[M::NAB] = (unsigned short)nf;
     return T;
 }
 
@@ -225,10 +234,10 @@ struct HermLay {
     static constexpr size_t BYTES = sizeof(double) * (size_t)TOTAL;
 };
 
-// (h1, m2) items of the reverse sums: those whose V enters a derivative, i.e.
-// some monomial of h1 carries a power of R or m2 one of S.
+// (h1, m2) items of the reverse sums: ALL, or those whose V enters a
+// derivative, i.e. some monomial of h1 carries a power of R or m2 one of S.
 // R row | h1 << 8 | m2 << 14 | scalar of m2 << 21
-template <int LA, int LB, int LC, int LD>
+template <int LA, int LB, int LC, int LD, bool ALL>
 constexpr int herm_item_count()
 {
     using B = PairMono<LA, LB>;
@@ -238,22 +247,22 @@ constexpr int herm_item_count()
         for (int k = 0; k <= LC; ++k)
             for (int l = 0; l <= LD; ++l)
                 if (k + l >= n2 && ((k + l - n2) & 1) == 0)
-                    n += (n2 + 1) * (n2 + 2) / 2 * (k + l < K::L ? nherm(B::L) : nherm(B::L - 1));
+                    n += (n2 + 1) * (n2 + 2) / 2 * (ALL || k + l < K::L ? nherm(B::L) : nherm(B::L - 1));
     return n;
 }
 
-template <int LA, int LB, int LC, int LD>
+template <int LA, int LB, int LC, int LD, bool ALL>
 struct HermItems {
-    static constexpr int N = herm_item_count<LA, LB, LC, LD>();
+    static constexpr int N = herm_item_count<LA, LB, LC, LD, ALL>();
     unsigned it[N > 0 ? N : 1];
 };
 
-template <int LA, int LB, int LC, int LD>
-constexpr HermItems<LA, LB, LC, LD> make_herm_items()
+template <int LA, int LB, int LC, int LD, bool ALL>
+constexpr HermItems<LA, LB, LC, LD, ALL> make_herm_items()
 {
     using B = PairMono<LA, LB>;
     using K = PairMono<LC, LD>;
-    HermItems<LA, LB, LC, LD> T{};
+    HermItems<LA, LB, LC, LD, ALL> T{};
     int n = 0;
     for (int n1 = 0; n1 <= B::L; ++n1)
         for (int t1 = n1; t1 >= 0; --t1)
@@ -266,7 +275,7 @@ constexpr HermItems<LA, LB, LC, LD> make_herm_items()
                             for (int k = 0; k <= LC; ++k)
                                 for (int l = 0; l <= LD; ++l) {
                                     if (!(k + l >= n2 && ((k + l - n2) & 1) == 0)) continue;
-                                    if (k + l < K::L || n1 < B::L)
+                                    if (ALL || k + l < K::L || n1 < B::L)
                                         T.it[n++] = (unsigned)hidx(t1 + t2, u1 + u2, v1 + v2) |
                                                     ((unsigned)hidx(t1, u1, v1) << 8) |
                                                     ((unsigned)K::monomial(hidx(t2, u2, v2), n2, k, l) << 14) |
@@ -572,11 +581,64 @@ __device__ __forceinline__ void half_ket(double *half, const double *G, const do
     }
 }
 
+// Bra primitive pairs taken at a time (1 .. cap, at most nbra): the block of
+// pb * nkp primitive quartets that leaves the fewest of its lanes idle.
+__device__ __forceinline__ int block_pairs(int nbra, int nkp, int cap)
+{
+    int pb = 1, best = -1;
+    for (int c = 1; c <= (nbra < cap ? nbra : cap); ++c) {
+        const int n = c * nkp, use = n * 64 / ((n + 31) / 32);  // primitive quartets per pass, times 64
+        if (use >= best) best = use, pb = c;
+    }
+    return pb;
+}
+
+// items table of the class a translation unit compiles
+template <int LA, int LB, int LC, int LD, bool ALL>
+__device__ const HermItems<LA, LB, LC, LD, ALL> kHermItems = make_herm_items<LA, LB, LC, LD, ALL>();
+
+// Reverse sums of one pass (primitive quartets j0 .. j0 + n - 1 of the block, n
+// <= 32, lane j - j0's R in column j - j0 of Rr): per bra primitive pair,
+// U[h1][m2] = sum_q s_m2 R[h1 + h2], added to V[m1][m2] with its scalars.
+template <int LA, int LB, int LC, int LD, bool ALL>
+__device__ __forceinline__ void reverse_sums(double *V, const double *Rr, const double *S2, const double *S1, int j0,
+                                             int n, int nkp, int lane)
+{
+    using B = PairMono<LA, LB>;
+    constexpr int NIT = HermItems<LA, LB, LC, LD, ALL>::N, RS = 33, NM2P = PairMono<LC, LD>::NM | 1;
+    // lanes per item: as many as fit
+    constexpr int SUB = NIT <= 1 ? 16 : (NIT <= 4 ? 8 : (NIT <= 8 ? 4 : (NIT <= 16 ? 2 : 1)));
+    constexpr int ITL = 32 / SUB;
+    const auto &TBra = pair_tab<LA, LB>();
+    const unsigned *items = kHermItems<LA, LB, LC, LD, ALL>.it;
+    const int pfirst = j0 / nkp, plast = (j0 + n - 1) / nkp, sub = lane / ITL;
+    for (int i0 = 0; i0 < NIT; i0 += ITL) {
+        const int it = i0 + lane % ITL;
+        const unsigned w = items[it < NIT ? it : NIT - 1];
+        const double *r = Rr + (w & 0xff) * RS, *s = S2 + (w >> 21) * RS;
+        const unsigned hm = TBra.hm[(w >> 8) & 0x3f];
+        double *v = V + (hm & 0xff) * NM2P + ((w >> 14) & 0x7f);
+        const int ns = (hm >> 8) & 0xf;
+        for (int pj = pfirst; pj <= plast; ++pj) {
+            const int lo = max(pj * nkp - j0, 0), hi = min((pj + 1) * nkp - j0, n);
+            double u = 0.0;
+#pragma unroll 4
+            for (int j = lo + sub; j < hi; j += SUB) u += s[j] * r[j];
+#pragma unroll
+            for (int x = ITL; x < 32; x *= 2) u += __shfl_xor_sync(0xffffffffu, u, x);
+            if (it < NIT && sub == 0) {
+                const double *s1 = S1 + pj * B::NS + (hm >> 12);
+                for (int k = 0; k < ns; ++k) v[k * NM2P] += s1[k] * u;
+            }
+        }
+    }
+}
+
 // One contracted quartet by one warp, bra primitive pairs ib0, ib0 + ibs, ...
 // acc[0..2] += d/dA, acc[3..5] += d/dA + d/dB, acc[6..8] += d/dC (this lane's
 // share; the caller sums the warp).
 template <int LA, int LB, int LC, int LD>
-__device__ void quartet_herm(double *sm, int lane, const unsigned *items, const GeoArgs &geo, const DensArgs &den,
+__device__ void quartet_herm(double *sm, int lane, const GeoArgs &geo, const DensArgs &den,
                              const PrimPairs &pp, int sa, int sb, int sc, int sd, int pb0, int nbp, int ib0, int ibs,
                              int pk0, int nkp, double scale, const double *boys, double (&acc)[9])
 {
@@ -584,10 +646,7 @@ __device__ void quartet_herm(double *sm, int lane, const unsigned *items, const 
     constexpr int NCD = Lay::NCD, L = Lay::L, LM = Lay::LM, NT1 = Lay::NT1;
     constexpr int NM1 = Lay::NM1, NM2 = Lay::NM2, NM2P = Lay::NM2P, NS1 = Lay::NS1, NS2 = Lay::NS2, RS = Lay::RS;
     constexpr int NO = Lay::NO, NP1 = Lay::NP1, NABP = Lay::NABP;
-    constexpr int NIT = HermItems<LA, LB, LC, LD>::N;
-    // lanes per item of the reverse sums: as many as fit
-    constexpr int SUB = NIT == 0 ? 1 : (NIT <= 4 ? 8 : (NIT <= 8 ? 4 : (NIT <= 16 ? 2 : 1)));
-    constexpr int ITL = 32 / SUB;
+    constexpr int NIT = HermItems<LA, LB, LC, LD, false>::N;
     double *G = sm + Lay::o_G, *Gp = sm + Lay::o_Gp, *V = sm + Lay::o_V, *F = sm + Lay::o_F;
     double *S1 = sm + Lay::o_S1, *P1 = sm + Lay::o_P1, *pw = sm + Lay::o_pw, *X1 = sm + Lay::o_X;
     double *Rr = X1, *S2 = X1 + Lay::NRH * RS;                      // main loop
@@ -610,15 +669,7 @@ __device__ void quartet_herm(double *sm, int lane, const unsigned *items, const 
         }
     }
     const int nbra = (nbp - ib0 + ibs - 1) / ibs;  // bra primitive pairs of this call
-    // block size: the fewest idle lanes over whole blocks
-    int pb = 1;
-    {
-        int best = -1;
-        for (int c = 1; c <= (nbra < Lay::PB ? nbra : Lay::PB); ++c) {
-            const int n = c * nkp, use = n * 64 / ((n + 31) / 32);  // lanes in use per pass, times 64
-            if (use >= best) best = use, pb = c;
-        }
-    }
+    const int pb = block_pairs(nbra, nkp, Lay::PB);
     // this lane's sums over its primitive quartets: T, a^ T, c^ T, mu_ab E, mu_cd E
     double aT[3] = {0.0, 0.0, 0.0}, aA[3] = {0.0, 0.0, 0.0}, aC[3] = {0.0, 0.0, 0.0}, eA = 0.0, eC = 0.0;
     double gA[3] = {0.0, 0.0, 0.0}, gC[3] = {0.0, 0.0, 0.0};  // polynomial parts
@@ -773,28 +824,8 @@ __device__ void quartet_herm(double *sm, int lane, const unsigned *items, const 
                     __syncwarp();
                     // ---- reverse sums U[h1][m2], added to V with the bra scalars
                     if constexpr (NIT > 0) {
-                        const int n = min(32, ntot - j0), pfirst = j0 / nkp, plast = (j0 + n - 1) / nkp;
-                        const int sub = lane / ITL;
-                        for (int i0 = 0; i0 < NIT; i0 += ITL) {
-                            const int it = i0 + lane % ITL;
-                            const unsigned w = items[min(it, NIT - 1)];
-                            const double *r = Rr + (w & 0xff) * RS, *s = S2 + (w >> 21) * RS;
-                            const unsigned hm = TBra.hm[(w >> 8) & 0x3f];
-                            double *v = V + (o * NM1 + (hm & 0xff)) * NM2P + ((w >> 14) & 0x7f);
-                            const int ns = (hm >> 8) & 0xf;
-                            for (int pj = pfirst; pj <= plast; ++pj) {
-                                const int lo = max(pj * nkp - j0, 0), hi = min((pj + 1) * nkp - j0, n);
-                                double u = 0.0;
-#pragma unroll 4
-                                for (int j = lo + sub; j < hi; j += SUB) u += s[j] * r[j];
-#pragma unroll
-                                for (int x = ITL; x < 32; x *= 2) u += __shfl_xor_sync(0xffffffffu, u, x);
-                                if (it < NIT && sub == 0) {
-                                    const double *s1 = S1 + pj * NS1 + (hm >> 12);
-                                    for (int k = 0; k < ns; ++k) v[k * NM2P] += s1[k] * u;
-                                }
-                            }
-                        }
+                        reverse_sums<LA, LB, LC, LD, false>(V + o * NM1 * NM2P, Rr, S2, S1, j0, min(32, ntot - j0), nkp,
+                                                            lane);
                         __syncwarp();
                     }
                 }
@@ -878,19 +909,24 @@ __device__ void quartet_herm(double *sm, int lane, const unsigned *items, const 
     }
 }
 
-// items table of the class this translation unit compiles
-template <int LA, int LB, int LC, int LD>
-__device__ const HermItems<LA, LB, LC, LD> kHermItems = make_herm_items<LA, LB, LC, LD>();
-
 // Warps of a CTA and resident CTAs the registers are limited to: 16 warps at
 // 128 registers up to L = 2, 12 at 168 for L = 3, 8 at 255 above.  One warp per
 // scheduler already covers most of the fp64 pipe; the second and third fill
 // the gaps left by the transforms' loads and by dependent steps.
 template <int LA, int LB, int LC, int LD>
-struct HermWarps {
+struct HermOp {
+    using Lay = HermLay<LA, LB, LC, LD>;
+    static constexpr bool FP32 = false;
     static constexpr int L = LA + LB + LC + LD;
     static constexpr int max_warps = L == 3 ? 12 : 8;
     static constexpr int min_ctas = L <= 2 ? 2 : 1;
+    static __device__ __forceinline__ void quartet(double *sm, int lane, const MolDesc &md, int sa, int sb, int sc,
+                                                   int sd, int pb0, int nbp, int ib0, int ibs, int pk0, int nkp,
+                                                   double scale, const double *boys, double (&acc)[9])
+    {
+        quartet_herm<LA, LB, LC, LD>(sm, lane, md.geo, md.den, md.pp, sa, sb, sc, sd,
+                                     pb0, nbp, ib0, ibs, pk0, nkp, scale, boys, acc);
+    }
 };
 
 // Persistent class kernel; every warp works alone.  Warp w of W takes the
@@ -899,18 +935,17 @@ struct HermWarps {
 // sums out.  A quartet's 12 components are added to the warp's own gradient
 // (shared memory, or with out.use_smem = 0 the warp's slab), so the schedule
 // and the order of all sums are fixed and results are bitwise reproducible.
-template <int LA, int LB, int LC, int LD>
-__global__ void __launch_bounds__((32 * HermWarps<LA, LB, LC, LD>::max_warps), (HermWarps<LA, LB, LC, LD>::min_ctas))
-    k_grad_herm(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out, const double *__restrict__ boys)
+template <class Op>
+__global__ void __launch_bounds__(32 * Op::max_warps, Op::min_ctas)
+    k_grad_lanes(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out, const double *__restrict__ boys)
 {
-    using Lay = HermLay<LA, LB, LC, LD>;
+    using Lay = typename Op::Lay;
     extern __shared__ double smem[];
     const int nw = blockDim.x / 32, grp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int n3 = out.natom_total * 3;
     double *wsm = smem + (size_t)grp * Lay::TOTAL;
     double *grad = out.use_smem ? smem + (size_t)nw * Lay::TOTAL + (size_t)grp * n3
                                 : out.partials + (size_t)(blockIdx.x * nw + grp) * n3;
-    const unsigned *items = kHermItems<LA, LB, LC, LD>.it;
     if (out.use_smem) {
         for (int k = lane; k < n3; k += 32) grad[k] = 0.0;
         __syncwarp();
@@ -953,8 +988,8 @@ __global__ void __launch_bounds__((32 * HermWarps<LA, LB, LC, LD>::max_warps), (
 #pragma unroll
                 for (int k = 0; k < 9; ++k) acc[k] = 0.0;
                 if (nkp > 0)
-                    quartet_herm<LA, LB, LC, LD>(wsm, lane, items, md.geo, md.den, md.pp, sa, sb, sc, sd, bra.poff[bi],
-                                                 nbp, split, S, ket.poff[ki], nkp, scale, boys, acc);
+                    Op::quartet(wsm, lane, md, sa, sb, sc, sd, bra.poff[bi], nbp, split, S, ket.poff[ki], nkp, scale,
+                                boys, acc);
                 // the nine sums over the warp through shared memory: three lanes a sum
                 double *red = wsm + Lay::o_X;
                 __syncwarp();
@@ -1000,97 +1035,66 @@ __global__ void __launch_bounds__((32 * HermWarps<LA, LB, LC, LD>::max_warps), (
     }
     if (lane == 0 && (nq || npq)) {  // a split unit may hold primitives only
         atomicAdd(out.counters + 0, nq);
-        atomicAdd(out.counters + 1, npq);
-        atomicAdd(out.counters + 4, nbv);
+        atomicAdd(out.counters + (Op::FP32 ? 3 : 1), npq);
+        atomicAdd(out.counters + (Op::FP32 ? 5 : 4), nbv);
+        if (Op::FP32) atomicAdd(out.counters + 2, nq);
     }
 }
 
 // Shared memory a CTA may take (227 KB), and an SM's (228 KB with 1 KB per CTA).
 constexpr size_t kCtaSmem = 227 * 1024;
 
-// Launch of the class kernel with at most gcap slabs of partial gradients.
-// Tiles are cut into chunks down to single quartets until every warp has 32
-// units (with 4, the heaviest unit alone left (pp|pp) SMs idle 57 % of the
-// time on a 1/16 shard of the 32-atom workload), then along the bra primitive
-// pairs (which repeats the density transform) while warps have fewer than 4.
-template <int LA, int LB, int LC, int LD>
-cudaError_t launch_herm(int gcap, cudaStream_t st, const MolDesc *mols, ClassLaunch cl, const OutArgs &out,
-                        const double *boys)
+// Launch of a kernel over warp units (tile, chunk, split) with at most gmax
+// CTAs of nw warps.  Tiles are cut into chunks down to single quartets until
+// every warp has 32 units (with 4, the heaviest unit alone left (pp|pp) SMs
+// idle 57 % of the time on a 1/16 shard of the 32-atom workload), then along
+// the bra primitive pairs (which repeats the density transform) while warps
+// have fewer than 4.
+template <typename K>
+cudaError_t launch_warp_units(K kern, int nw, size_t per_warp, long long gmax, cudaStream_t st, const MolDesc *mols,
+                              ClassLaunch cl, const OutArgs &out, const double *boys)
 {
-    using Wp = HermWarps<LA, LB, LC, LD>;
-    constexpr size_t bytes = HermLay<LA, LB, LC, LD>::BYTES;
-    static_assert(bytes <= kCtaSmem, "one warp's arrays fit in a CTA");
-    OutArgs o = out;
-    auto kern = k_grad_herm<LA, LB, LC, LD>;
     int dev = 0, nsm = 1, per = 1;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    // each warp's gradient beside its arrays while that leaves four warps (or what fits without), else per-warp slabs
-    const size_t grad = sizeof(double) * 3 * (size_t)o.natom_total;
-    const int fit = (int)(kCtaSmem / bytes), fit_g = (int)(kCtaSmem / (bytes + grad));
-    o.use_smem = fit_g >= (fit < 4 ? fit : 4);
-    const size_t per_warp = bytes + (o.use_smem ? grad : 0);
-    int nw = o.use_smem ? fit_g : fit;
-    if (nw > Wp::max_warps) nw = Wp::max_warps;
-    const int slabs = o.use_smem ? gcap : (gcap > nw ? gcap / nw : 1);  // CTAs the partials have room for
-    if (nw > gcap && !o.use_smem) nw = gcap;
     const size_t sm = per_warp * nw;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * nw, sm)) != cudaSuccess) return e;
-    long long gmax = (long long)(per > 0 ? per : 1) * nsm;
-    if (gmax > slabs) gmax = slabs;
+    if (gmax > (long long)(per > 0 ? per : 1) * nsm) gmax = (long long)(per > 0 ? per : 1) * nsm;
     cl.nchunk = 1;
     cl.nsplit = 1;
     const long long warps = gmax * nw;
     while (cl.ntiles * cl.nchunk < 32 * warps && cl.nchunk < TILE) cl.nchunk *= 2;
-    if (!o.dump) {
+    if (!out.dump) {
         while (cl.ntiles * cl.nchunk * cl.nsplit < 4 * warps && cl.nsplit < 8) ++cl.nsplit;
         if (cl.split_req > 0) cl.nsplit = cl.split_req;
     }
     const long long units = cl.ntiles * cl.nchunk * cl.nsplit;
     const int grid = (int)(units < gmax ? units : gmax);
     if (units < grid * (long long)nw) nw = (int)((units + grid - 1) / grid);
-    kern<<<grid, 32 * nw, per_warp * nw, st>>>(mols, cl, o, boys);
+    kern<<<grid, 32 * nw, per_warp * nw, st>>>(mols, cl, out, boys);
     return cudaGetLastError();
 }
 
-// Kernel forms per class.  fp64: the Hermite-density kernel.  fp32: the thread
-// kernel below 648 function quartets (above, its per-thread arrays run to tens
-// of KB of local memory), the group kernel from 648, the warp kernel wherever
-// four warps' arrays fit (all but (dd|dd)).  ClassLaunch::kind 1 / 2 / 3 asks
-// for the thread / group / warp kernel; a form not compiled for the class and
-// precision falls back to the default.
-template <int LA, int LB, int LC, int LD>
-struct ClassForms {
-    static constexpr int nfq = ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD);
-    static constexpr size_t kStageMax = 200 * 1024;  // warp arrays + tile staging (16 KB) per CTA
-    static constexpr bool thread32 = nfq < 648;
-    static constexpr bool group32 = nfq >= 648;
-    static constexpr bool warp32 = warp_kernel_smem<LA, LB, LC, LD, float>() + 16384 <= kStageMax;
-    // default fp32 form per class (1 thread, 2 group, 3 warp)
-    static constexpr int qc = pair_class(LA, LB) * (pair_class(LA, LB) + 1) / 2 + pair_class(LC, LD);
-    static constexpr int default32 = kDefaultForm32[qc];
-    static_assert((default32 != 1 || thread32) && (default32 != 2 || group32) && (default32 != 3 || warp32),
-                  "default fp32 form not compiled");
-};
-
-template <int LA, int LB, int LC, int LD>
-cudaError_t launch_class_kernel(int fp32, int gcap, size_t smem, cudaStream_t st, const MolDesc *mols,
-                                const ClassLaunch &cl, const OutArgs &out, const double *boys)
+// Launch of a gradient kernel with at most gcap slabs of partial gradients.
+// Each warp's gradient lies beside its arrays while that leaves four warps (or
+// what fits without), else every warp adds to a slab of its own.
+template <class Op>
+cudaError_t launch_lanes(int gcap, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl, const OutArgs &out,
+                         const double *boys)
 {
-    using K = ClassForms<LA, LB, LC, LD>;
-    if (!fp32) return launch_herm<LA, LB, LC, LD>(gcap, st, mols, cl, out, boys);
-    int kind = cl.kind;
-    if ((kind == 1 && !K::thread32) || (kind == 2 && !K::group32) || (kind == 3 && !K::warp32) || kind < 1 || kind > 3)
-        kind = K::default32;
-    if constexpr (K::warp32)
-        if (kind == 3) return launch_warp<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
-    if constexpr (K::group32)
-        if (kind == 2) return launch_coop<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
-    if constexpr (K::thread32)
-        if (kind == 1) return launch_units(k_grad<LA, LB, LC, LD, true>, 0, gcap, smem, st, mols, cl, out, boys);
-    return cudaErrorInvalidValue;  // not reached: every class compiles its default form
+    constexpr size_t bytes = Op::Lay::BYTES;
+    static_assert(bytes <= kCtaSmem, "one warp's arrays fit in a CTA");
+    OutArgs o = out;
+    const size_t grad = sizeof(double) * 3 * (size_t)o.natom_total;
+    const int fit = (int)(kCtaSmem / bytes), fit_g = (int)(kCtaSmem / (bytes + grad));
+    o.use_smem = fit_g >= (fit < 4 ? fit : 4);
+    int nw = o.use_smem ? fit_g : fit;
+    if (nw > Op::max_warps) nw = Op::max_warps;
+    if (nw > gcap && !o.use_smem) nw = gcap;
+    return launch_warp_units(k_grad_lanes<Op>, nw, bytes + (o.use_smem ? grad : 0), o.use_smem ? gcap : gcap / nw, st,
+                             mols, cl, o, boys);
 }
 
 }  // namespace tg

@@ -815,12 +815,9 @@ cudaError_t launch_warp(int gcap, size_t smem, cudaStream_t st, const MolDesc *m
                         st, mols, cl, out, boys);
 }
 
-// Default class-kernel form per angular class (ssss, psss, psps, ppss, ppps,
+// Default fp32 kernel form per angular class (ssss, psss, psps, ppss, ppps,
 // pppp, dsss, dsps, dspp, dsds, dpss, dpps, dppp, dpds, dpdp, ddss, ddps, ddpp,
-// ddds, dddp, dddd): 1 = thread, 2 = group, 3 = warp.  Picked from per-class
-// kernel times of the mixed route on the 32-atom chain (the fp64 lists there
-// hold the largest, most contracted tiles) and of the all-fp64 route; where
-// the two disagree by little, the mixed route's choice is kept.
-constexpr int kDefaultForm32[NQC] = {1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 3, 3, 2, 2};
+// ddds, dddp, dddd): 0 = lane, 2 = group, 3 = warp.
+constexpr int kDefaultForm32[NQC] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 3, 3, 2, 2};
 
 }  // namespace tg
