@@ -1,49 +1,46 @@
 // Fock-type build (Sec. II.B, the two-electron part of eqs. G_2e and zfock):
-// one warp per canonical shell quartet, as the warp gradient kernel.
+// one warp per canonical shell quartet, one primitive quartet per lane.
 //
 // The density pairs are combined beforehand (the result is linear in them)
 // into S_J = sum_p c_J (B_p + B_p^T), B_K = sum_p c_K B_p and B_lr =
-// sum_p c_K_lr B_p.  Per canonical quartet (a b|c d) with integrals
-// I_s(m n|l s) of both operators s (McMurchie-Davidson, W form over the
-// ket primitive pairs and index boxes, as in eri_warp.cuh, without
-// derivatives), the 8 permutation images of every integral give
+// sum_p c_K_lr B_p.  Per canonical quartet (a b|c d) the integrals
+// I_s(m n|l s) of both operators s come from the monomial sums of
+// eri_herm.cuh: V_s[m1][m2] = sum_pq s_m1(p) s_m2(q) (-1)^|h2| R_s[h1 + h2]
+// over the primitive quartets, and once per contracted quartet
+// I_s[ab][cd] = sum_m1m2 c^{ab}_{m1} R^.. V_s[m1][m2] c^{cd}_{m2} S^...  The 8
+// permutation images of every integral give
 //   Coulomb:  F[m][n], F[n][m] += I_0 S_J[l][s];   F[l][s], F[s][l] += I_0 S_J[m][n]
 //   exchange: F[m][l] += I.B[n][s]   F[n][l] += I.B[m][s]   F[m][s] += I.B[n][l]
 //             F[n][s] += I.B[m][l]   F[l][m] += I.B[s][n]   F[s][m] += I.B[l][n]
 //             F[l][n] += I.B[s][m]   F[s][n] += I.B[l][m]
 // with I.B = I_0 B_K + I_1 B_lr, all times 1/|stabiliser| of the quartet.
 // Each target block is summed over the quartet on the warp and added to F
-// with fp64 atomics.
+// with fp64 atomics.  Bound: the fp64 pipe, as the gradient kernel.
 #pragma once
 #include "eri_lane32.cuh"
 
 namespace tg {
 
+// One warp's slice of shared memory, in doubles (as HermLay).
 template <int LA, int LB, int LC, int LD>
-struct FockLayout {
+struct FockLay {
+    using B = PairMono<LA, LB>;
+    using K = PairMono<LC, LD>;
     static constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD);
-    static constexpr int NAB = NA * NB, NCD = NC * ND;
-    static constexpr int L1 = LA + LB, L2 = LC + LD, L = L1 + L2;
-    static constexpr int NH1 = nherm(L1), NH2 = nherm(L2), NR = nherm(L);
-    static constexpr int BJ = LB + 1, BT = L1 + 2, KJ = LD + 1, KT = L2 + 2;
-    static constexpr int EBN = (LA + 2) * BJ * BT;  // pair_table layout (one row beyond what the build needs)
-    static constexpr int EKN = (LC + 2) * KJ * KT;
-    static constexpr int SC_X = 0, SC_T = 3, SC_TH2 = 4, SC_PW = 5;
-    static constexpr int NSC = SC_PW + 2 * (L + 1);
-    static constexpr int QT_RAW = (int)((6144 / sizeof(double)) / (3 * EKN + NSC));
-    static constexpr int QT = QT_RAW < 4 ? 4 : (QT_RAW > 32 ? 32 : QT_RAW);
-    static constexpr int KW = (NCD * NH1 + 31) / 32;
-    static constexpr int o_I = 0;                       // [2][NAB][NCD]
-    static constexpr int o_W = o_I + 2 * NAB * NCD;     // [2][NCD][NH1]
-    static constexpr int o_E3b = o_W + 2 * NCD * NH1;   // [NAB][NH1]
-    static constexpr int o_E3k = o_E3b + NAB * NH1;     // [NCD][NH2]
-    static constexpr int o_R = o_E3k + NCD * NH2;       // [2][NR]
-    static constexpr int o_base = o_R + 2 * NR;         // [2][L+1]
-    static constexpr int o_Eb = o_base + 2 * (L + 1);   // [3][EBN]
-    static constexpr int o_Ek = o_Eb + 3 * EBN;         // [QT][3][EKN]
-    static constexpr int o_sc = o_Ek + QT * 3 * EKN;    // [QT][NSC]
-    static constexpr int TOTAL = o_sc + QT * NSC;
-    static constexpr size_t BYTES = (sizeof(double) * (size_t)TOTAL + 15) & ~(size_t)15;
+    static constexpr int NAB = NA * NB, NCD = NC * ND, L = B::L + K::L;
+    static constexpr int NM1 = B::NM, NM2 = K::NM, NS1 = B::NS, NS2 = K::NS, NM2P = NM2 | 1, RS = 33;
+    static constexpr int NRH = nherm(L), PB = 16, NP1 = 2;
+    static constexpr int NE1 = pair_entries(LA, LB), NE2 = pair_entries(LC, LD);
+    static constexpr int NO = (NAB * NCD <= 81) ? 2 : 1;  // operators at a time
+    static constexpr int HALF = NE1 + NE2 + NO * NM1 * NCD, ROWS = (NRH + NS2) * RS;
+    static constexpr int o_I = 0;                            // [2][NAB][NCD]
+    static constexpr int o_V = o_I + 2 * NAB * NCD;          // [NO][NM1][NM2P]
+    static constexpr int o_S1 = o_V + NO * NM1 * NM2P;       // [PB][NS1]
+    static constexpr int o_P1 = o_S1 + PB * NS1;             // [PB][NP1]: p, 4 pi^(5/2) K / 2p
+    static constexpr int o_pw = o_P1 + PB * NP1;             // [2][3][5] powers of R and S
+    static constexpr int o_X = o_pw + 30;
+    static constexpr int TOTAL = (o_X + (HALF > ROWS ? HALF : ROWS) + 1) & ~1;
+    static constexpr size_t BYTES = sizeof(double) * (size_t)TOTAL;
 };
 
 // Per-quartet Fock bound: 8 Q_ab Q_cd M_q (see tg_fock2e in tdgrad.h).
@@ -64,199 +61,137 @@ __device__ __forceinline__ bool keep_quartet_fock(const ScreenArgs &scr, const P
     return true;
 }
 
-// Integrals of one canonical quartet (both operators) into I[2][NAB][NCD].
+// Integrals of one canonical quartet (both operators) into I[2][NAB][NCD],
+// summed over bra primitive pairs ib0, ib0 + ibs, ...
 template <int LA, int LB, int LC, int LD>
 __device__ void quartet_fock_ints(double *sm, int lane, const GeoArgs &geo, const PrimPairs &pp, int nops,
                                   double omega, int sa, int sb, int sc, int sd, int pb0, int nbp, int ib0, int ibs,
                                   int pk0, int nkp, const double *boys)
 {
-    using Lay = FockLayout<LA, LB, LC, LD>;
-    constexpr int NB = Lay::NB, ND = Lay::ND, NAB = Lay::NAB, NCD = Lay::NCD;
-    constexpr int L = Lay::L, NH1 = Lay::NH1, NH2 = Lay::NH2, NR = Lay::NR;
-    constexpr int BJ = Lay::BJ, BT = Lay::BT, KJ = Lay::KJ, KT = Lay::KT, EBN = Lay::EBN, EKN = Lay::EKN;
-    constexpr int QT = Lay::QT, NSC = Lay::NSC, KW = Lay::KW;
-    double *I = sm + Lay::o_I, *W = sm + Lay::o_W, *E3b = sm + Lay::o_E3b, *E3k = sm + Lay::o_E3k;
-    double *R = sm + Lay::o_R, *base = sm + Lay::o_base, *Eb = sm + Lay::o_Eb, *Ekall = sm + Lay::o_Ek;
-    double *scall = sm + Lay::o_sc;
-    const double om2 = omega * omega;
+    using Lay = FockLay<LA, LB, LC, LD>;
+    constexpr int NAB = Lay::NAB, NCD = Lay::NCD, L = Lay::L, NM1 = Lay::NM1, NM2P = Lay::NM2P;
+    constexpr int NS1 = Lay::NS1, NS2 = Lay::NS2, RS = Lay::RS, NO = Lay::NO, NP1 = Lay::NP1;
+    double *I = sm + Lay::o_I, *V = sm + Lay::o_V, *S1 = sm + Lay::o_S1, *P1 = sm + Lay::o_P1, *pw = sm + Lay::o_pw;
+    double *Rr = sm + Lay::o_X, *S2 = Rr + Lay::NRH * RS;
+    double *vb = sm + Lay::o_X, *vk = vb + Lay::NE1, *half = vk + Lay::NE2;
+    const auto &TBra = pair_tab<LA, LB>();
+    const auto &TKet = pair_tab<LC, LD>();
     const bool ominf = isinf(omega);
+    const double om = ominf ? 1.0 : omega;
     const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xb = geo.xyz + 3 * geo.sh_atom[sb];
     const double *xc = geo.xyz + 3 * geo.sh_atom[sc], *xd = geo.xyz + 3 * geo.sh_atom[sd];
-    for (int it = lane; it < 2 * NAB * NCD; it += 32) I[it] = 0.0;
-    const bool ket_once = nkp <= QT;
-    if (ket_once)
-        for (int it = lane; it < 3 * nkp; it += 32) {
-            const int j = it / 3, dir = it % 3;
-            pair_table<LC, LD, double>(Ekall + (j * 3 + dir) * EKN, pp, pk0 + j, dir, xc[dir], xd[dir]);
+    if (lane < 6) {
+        const int d = lane % 3;
+        const double x = lane < 3 ? xa[d] - xb[d] : xc[d] - xd[d];
+        double p = 1.0;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            pw[(lane / 3) * 15 + d * 5 + k] = p;
+            p *= x;
         }
-    __syncwarp();
-    for (int ib = ib0; ib < nbp; ib += ibs) {
-        const int ip = pb0 + ib;
-        if (lane < 3) pair_table<LA, LB, double>(Eb + lane * EBN, pp, ip, lane, xa[lane], xb[lane]);
+    }
+    const int nbra = (nbp - ib0 + ibs - 1) / ibs, pb = block_pairs(nbra, nkp, Lay::PB);
+    if (nops == 1)
+        for (int it = lane; it < NAB * NCD; it += 32) I[NAB * NCD + it] = 0.0;
+    for (int o0 = 0; o0 < nops; o0 += NO) {
+        for (int it = lane; it < NO * NM1 * NM2P; it += 32) V[it] = 0.0;
         __syncwarp();
-        for (int it = lane; it < NAB * NH1; it += 32) {
-            const int ab = it / NH1, h = it % NH1;
-            int t, u, v, ax, ay, az, bx, by, bz;
-            herm_tuv(h, t, u, v);
-            cart_xyz(LA, ab / NB, ax, ay, az);
-            cart_xyz(LB, ab % NB, bx, by, bz);
-            double e = 0.0;
-            if (t <= ax + bx && u <= ay + by && v <= az + bz)
-                e = Eb[(ax * BJ + bx) * BT + t] * Eb[EBN + (ay * BJ + by) * BT + u] *
-                    Eb[2 * EBN + (az * BJ + bz) * BT + v];
-            E3b[it] = e;
-        }
-        double w0r[KW], w1r[KW];
+        for (int blk = 0; blk < nbra; blk += pb) {
+            const int np = min(pb, nbra - blk);
+            if (lane < np) {
+                const int ip = pb0 + ib0 + (blk + lane) * ibs;
+                const double p = pp.p[ip], za = pp.za[ip], oo2 = 0.5 / p;
+                double s[NS1];
+                pair_scalars<LA, LB, false>(oo2, 2.0 * oo2 * za, 2.0 * oo2 * (p - za), s);
 #pragma unroll
-        for (int k = 0; k < KW; ++k) w0r[k] = w1r[k] = 0.0;
-        for (int q0 = 0; q0 < nkp; q0 += QT) {
-            const int nq = min(QT, nkp - q0);
-            if (!ket_once)
-                for (int it = lane; it < 3 * nq; it += 32) {
-                    const int j = it / 3, dir = it % 3;
-                    pair_table<LC, LD, double>(Ekall + (j * 3 + dir) * EKN, pp, pk0 + q0 + j, dir, xc[dir], xd[dir]);
-                }
-            if (lane < nq) {
-                double *sc_ = scall + lane * NSC;
-                const int kp = pk0 + q0 + lane;
-                const double p = pp.p[ip], q = pp.p[kp], pq = p + q, rho = p * q / pq;
-                const double X = pp.Px[ip] - pp.Px[kp], Y = pp.Py[ip] - pp.Py[kp], Z = pp.Pz[ip] - pp.Pz[kp];
-                const double th2 = (nops == 2) ? (ominf ? 1.0 : om2 / (om2 + rho)) : 1.0;
-                const double pref = 34.986836655249725 / (p * q * sqrt(pq)) * pp.K[ip] * pp.K[kp];
-                sc_[0] = X;
-                sc_[1] = Y;
-                sc_[2] = Z;
-                sc_[Lay::SC_T] = rho * (X * X + Y * Y + Z * Z);
-                sc_[Lay::SC_TH2] = th2;
-                double b0 = pref, b1 = pref * sqrt(th2);
-                const double m0 = -2.0 * rho, m1 = -2.0 * rho * th2;
-#pragma unroll
-                for (int m = 0; m <= L; ++m) {
-                    sc_[Lay::SC_PW + m] = b0;
-                    sc_[Lay::SC_PW + L + 1 + m] = b1;
-                    b0 *= m0;
-                    b1 *= m1;
-                }
+                for (int k = 0; k < NS1; ++k) S1[lane * NS1 + k] = s[k];
+                P1[lane * NP1] = p;
+                P1[lane * NP1 + 1] = pp.K[ip] * oo2 * 69.97367331049945;
             }
             __syncwarp();
-            for (int j = 0; j < nq; ++j) {
-                const double *sc_ = scall + j * NSC;
-                const double *Ek = Ekall + (ket_once ? (q0 + j) : j) * 3 * EKN;
+            const int ntot = np * nkp;
+            for (int j0 = 0; j0 < ntot; j0 += 32) {
+                const int idx = min(j0 + lane, ntot - 1);
+                const int pi = idx / nkp;
+                const int ip = pb0 + ib0 + (blk + pi) * ibs, kp = pk0 + (idx - pi * nkp);
+                const double p = P1[pi * NP1], q = pp.p[kp], zc = pp.za[kp], oo2q = 0.5 / q;
+                const double ir = rsqrt(p + q), rho = p * q * ir * ir;
+                const double X = pp.Px[ip] - pp.Px[kp], Y = pp.Py[ip] - pp.Py[kp], Z = pp.Pz[ip] - pp.Pz[kp];
+                const double T0 = rho * (X * X + Y * Y + Z * Z);
+                const double pref = j0 + lane < ntot ? P1[pi * NP1 + 1] * pp.K[kp] * (2.0 * oo2q) * ir : 0.0;
                 {
-                    const int op = lane >> 4, m = lane & 15;
-                    if (op < nops && m <= L) {
-                        const double T = sc_[Lay::SC_T] * (op ? sc_[Lay::SC_TH2] : 1.0);
-                        base[op * (L + 1) + m] = sc_[Lay::SC_PW + op * (L + 1) + m] * boys_order_fp64(T, m, boys);
-                    }
-                }
-                __syncwarp();
-                {
-                    const double X = sc_[0], Y = sc_[1], Z = sc_[2];
-                    if (lane < nops) R[lane * NR] = base[lane * (L + 1) + L];
-                    __syncwarp();
-#pragma unroll 1
-                    for (int n = L - 1; n >= 0; --n) {
-                        const int ne = nherm(L - n) - 1;
-                        const int items = nops * ne;
-#pragma unroll 1
-                        for (int i0 = 0; i0 < items; i0 += 32) {
-                            const int it = i0 + lane;
-                            double val = 0.0;
-                            int dst = -1;
-                            if (it < items) {
-                                const int op = it / ne, idx = ne - it % ne;
-                                int t, u, v;
-                                herm_tuv(idx, t, u, v);
-                                const double *c = R + op * NR;
-                                if (t > 0) {
-                                    val = X * c[hidx(t - 1, u, v)];
-                                    if (t > 1) val += double(t - 1) * c[hidx(t - 2, u, v)];
-                                } else if (u > 0) {
-                                    val = Y * c[hidx(t, u - 1, v)];
-                                    if (u > 1) val += double(u - 1) * c[hidx(t, u - 2, v)];
-                                } else {
-                                    val = Z * c[hidx(t, u, v - 1)];
-                                    if (v > 1) val += double(v - 1) * c[hidx(t, u, v - 2)];
-                                }
-                                dst = op * NR + idx;
-                            }
-                            __syncwarp();
-                            if (dst >= 0) R[dst] = val;
-                            __syncwarp();
-                        }
-                        if (lane < nops) R[lane * NR] = base[lane * (L + 1) + n];
-                        __syncwarp();
-                    }
-                }
-                for (int it = lane; it < NCD * NH2; it += 32) {
-                    const int cd = it / NH2, h = it % NH2;
-                    int t, u, v, cx, cy, cz, dx, dy, dz;
-                    herm_tuv(h, t, u, v);
-                    cart_xyz(LC, cd / ND, cx, cy, cz);
-                    cart_xyz(LD, cd % ND, dx, dy, dz);
-                    double e = 0.0;
-                    if (t <= cx + dx && u <= cy + dy && v <= cz + dz) {
-                        e = Ek[(cx * KJ + dx) * KT + t] * Ek[EKN + (cy * KJ + dy) * KT + u] *
-                            Ek[2 * EKN + (cz * KJ + dz) * KT + v];
-                        e = flip_if(e, t + u + v);
-                    }
-                    E3k[it] = e;
-                }
-                __syncwarp();
-                const double *R0 = R, *R1 = R + NR;
+                    double s2[NS2];
+                    pair_scalars<LC, LD, true>(oo2q, 2.0 * oo2q * zc, 2.0 * oo2q * (q - zc), s2);
 #pragma unroll
-                for (int k = 0; k < KW; ++k) {
-                    const int it = lane + 32 * k;
-                    if (it >= NCD * NH1) break;
-                    const int cd = it / NH1, h1 = it % NH1;
-                    int t1, u1, v1, cx, cy, cz, dx, dy, dz;
-                    herm_tuv(h1, t1, u1, v1);
-                    cart_xyz(LC, cd / ND, cx, cy, cz);
-                    cart_xyz(LD, cd % ND, dx, dy, dz);
-                    const int nx = cx + dx, ny = cy + dy, nz = cz + dz;
-                    const double *e = E3k + cd * NH2;
-                    double a0 = 0.0, a1 = 0.0;
-                    for (int t2 = 0; t2 <= nx; ++t2)
-                        for (int u2 = 0; u2 <= ny; ++u2)
-                            for (int v2 = 0; v2 <= nz; ++v2) {
-                                const double ev = e[hidx(t2, u2, v2)];
-                                const int r = hidx(t1 + t2, u1 + u2, v1 + v2);
-                                a0 += ev * R0[r];
-                                a1 += ev * R1[r];
-                            }
-                    w0r[k] += a0;
-                    w1r[k] += a1;
+                    for (int k = 0; k < NS2; ++k) S2[k * RS + lane] = s2[k];
                 }
-                __syncwarp();
+#pragma unroll 1
+                for (int o = 0; o < NO; ++o) {
+                    if (o0 + o >= nops) break;
+                    double base[L + 1];
+                    {
+                        double th = 1.0;
+                        if (o0 + o == 1 && !ominf) th = om * rsqrt(om * om + rho);
+                        double Fm[L + 1];
+                        const double th2 = th * th;
+                        boys_lane<L>(T0 * th2, Fm, boys);
+                        double f = pref * th;
+                        const double m2r = -2.0 * rho * th2;
+#pragma unroll
+                        for (int n = 0; n <= L; ++n) {
+                            base[n] = f * Fm[n];
+                            f *= m2r;
+                        }
+                    }
+                    double *Rl = Rr + lane;
+                    if constexpr (L <= 5) {
+                        double R[nherm(L)];
+                        hermite_R<L>(R, base, X, Y, Z);
+#pragma unroll
+                        for (int h = 0; h < nherm(L); ++h) Rl[h * RS] = R[h];
+                    } else {
+                        Rl[0] = base[L];
+                        static_for<L>([&](auto N) {
+                            constexpr int n = L - 1 - decltype(N)::value;
+                            hermite_level<RS>(Rl, nherm(L - n), X, Y, Z);
+                            Rl[0] = base[n];
+                        });
+                    }
+                    __syncwarp();
+                    reverse_sums<LA, LB, LC, LD, true>(V + o * NM1 * NM2P, Rr, S2, S1, j0, min(32, ntot - j0), nkp, lane);
+                    __syncwarp();
+                }
             }
         }
+        // ---- V -> I: ket functions, then bra functions
+        entry_values<LA, LB>(vb, lane, pw);
+        entry_values<LC, LD>(vk, lane, pw + 15);
+        __syncwarp();
+        for (int it = lane; it < NM1 * NCD; it += 32) {
+            const int m1 = it / NCD, cd = it % NCD;
 #pragma unroll
-        for (int k = 0; k < KW; ++k) {
-            const int it = lane + 32 * k;
-            if (it < NCD * NH1) {
-                W[it] = w0r[k];
-                W[NCD * NH1 + it] = w1r[k];
+            for (int o = 0; o < NO; ++o) {
+                double s = 0.0;
+                for (int k = TKet.fstart[cd]; k < TKet.fstart[cd + 1]; ++k) {
+                    const int e = TKet.fent[k];
+                    s += vk[e] * V[(o * NM1 + m1) * NM2P + TKet.own[e]];
+                }
+                half[(o * NM1 + m1) * NCD + cd] = s;
             }
         }
         __syncwarp();
-        // I_s[ab][cd] += sum_{h1 in box(ab)} E^{ab}_{h1} W_s[cd][h1]
         for (int it = lane; it < NAB * NCD; it += 32) {
             const int ab = it / NCD, cd = it % NCD;
-            int ax, ay, az, bx, by, bz;
-            cart_xyz(LA, ab / NB, ax, ay, az);
-            cart_xyz(LB, ab % NB, bx, by, bz);
-            const int nx = ax + bx, ny = ay + by, nz = az + bz;
-            const double *e = E3b + ab * NH1, *w0 = W + cd * NH1, *w1 = W + NCD * NH1 + cd * NH1;
-            double i0 = 0.0, i1 = 0.0;
-            for (int t = 0; t <= nx; ++t)
-                for (int u = 0; u <= ny; ++u)
-                    for (int v = 0; v <= nz; ++v) {
-                        const int h = hidx(t, u, v);
-                        i0 += e[h] * w0[h];
-                        i1 += e[h] * w1[h];
-                    }
-            I[it] += i0;
-            I[NAB * NCD + it] += i1;
+#pragma unroll
+            for (int o = 0; o < NO; ++o) {
+                if (o0 + o >= nops) break;
+                double s = 0.0;
+                for (int k = TBra.fstart[ab]; k < TBra.fstart[ab + 1]; ++k) {
+                    const int e = TBra.fent[k];
+                    s += vb[e] * half[(o * NM1 + TBra.own[e]) * NCD + cd];
+                }
+                I[(o0 + o) * NAB * NCD + it] = s;
+            }
         }
         __syncwarp();
     }
@@ -268,7 +203,7 @@ __device__ void quartet_fock_scatter(const double *I, int lane, int nops, const 
                                      const double *BL, int nbf, int fa, int fb, int fc, int fd, double scale,
                                      double *F)
 {
-    using Lay = FockLayout<LA, LB, LC, LD>;
+    using Lay = FockLay<LA, LB, LC, LD>;
     constexpr int NA = Lay::NA, NB = Lay::NB, NC = Lay::NC, ND = Lay::ND, NCD = Lay::NCD, NAB = Lay::NAB;
     const double *I1 = I + NAB * NCD;
     auto ix = [&](int ia, int ib, int ic, int id) { return (ia * NB + ib) * NCD + ic * ND + id; };
@@ -322,27 +257,30 @@ __device__ void quartet_fock_scatter(const double *I, int lane, int nops, const 
     }
 }
 
-// Persistent Fock class kernel over tile units (as k_grad_warp).  The
+// Persistent Fock class kernel over warp units (as k_grad_lanes).  The
 // combined matrices are den.A[0] = S_J, den.B[0] = B_K, den.A[1] = B_lr.
 template <int LA, int LB, int LC, int LD>
-__global__ void __launch_bounds__(TILE, 2) k_fock_warp(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out,
-                                                       const double *__restrict__ boys)
+__global__ void __launch_bounds__(256, (LA + LB + LC + LD <= 2 ? 2 : 1))
+    k_fock_lanes(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out, const double *__restrict__ boys)
 {
-    using Lay = FockLayout<LA, LB, LC, LD>;
-    const int NG = blockDim.x / 32;
+    using Lay = FockLay<LA, LB, LC, LD>;
     extern __shared__ double smem[];
-    const int grp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    double *wsm = smem + (size_t)grp * (Lay::BYTES / sizeof(double));
+    const int nw = blockDim.x / 32, grp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    double *wsm = smem + (size_t)grp * Lay::TOTAL;
     unsigned long long nq = 0, npq = 0, nbv = 0;
     const int S = cl.nsplit, C = cl.nchunk, QPC = TILE / C;
-    for (long long it = blockIdx.x; it < cl.ntiles * C * S; it += gridDim.x) {
+    const bool same = cl.P == cl.Q;
+    const long long units = cl.ntiles * C * S, W = (long long)gridDim.x * nw;
+    const long long w0 = (long long)grp * gridDim.x + blockIdx.x;
+    for (long long r = 0; r * W < units; ++r) {
+        const long long it = r * W + ((r & 1) ? W - 1 - w0 : w0);
+        if (it >= units) continue;
         const long long tile = it / (C * S);
         const int chunk = (int)((it / S) % C), split = (int)(it % S);
         const uint4 tl = cl.tiles[tile * cl.stride];
         const MolDesc &md = mols[tl.x];
-        const PairSet bra = md.sets[cl.P], ket = md.sets[cl.Q];
-        const bool same = cl.P == cl.Q;
-        for (int qi = chunk * QPC + grp; qi < (chunk + 1) * QPC; qi += NG) {
+        const PairSet &bra = md.sets[cl.P], &ket = md.sets[cl.Q];
+        for (int qi = chunk * QPC; qi < (chunk + 1) * QPC; ++qi) {
             const int bi = tl.y * TB + qi / TK;
             const int ki = tl.z * TK + qi % TK;
             bool ok = bi < bra.n && ki < ket.n && (!same || bi >= ki);
@@ -361,13 +299,15 @@ __global__ void __launch_bounds__(TILE, 2) k_fock_warp(const MolDesc *__restrict
             if (sc == sd) scale *= 0.5;
             if (same && bi == ki) scale *= 0.5;
             const int nbp = bra.np[bi], nkp = ket.np[ki];
-            const int nops = md.den.use_lr ? 2 : 1;
-            quartet_fock_ints<LA, LB, LC, LD>(wsm, lane, md.geo, md.pp, nops, md.den.omega, sa, sb, sc, sd,
-                                              bra.poff[bi], nbp, split, S, ket.poff[ki], nkp, boys);
-            const int *bf = md.geo.sh_bf;
-            quartet_fock_scatter<LA, LB, LC, LD>(wsm + Lay::o_I, lane, nops, md.den.A[0], md.den.B[0], md.den.A[1],
-                                                 md.den.nbf, bf[sa], bf[sb], bf[sc], bf[sd], scale, out.fock);
-            __syncwarp();
+            if (nkp > 0) {
+                const int nops = md.den.use_lr ? 2 : 1;
+                quartet_fock_ints<LA, LB, LC, LD>(wsm, lane, md.geo, md.pp, nops, md.den.omega, sa, sb, sc, sd,
+                                                  bra.poff[bi], nbp, split, S, ket.poff[ki], nkp, boys);
+                const int *bf = md.geo.sh_bf;
+                quartet_fock_scatter<LA, LB, LC, LD>(wsm + Lay::o_I, lane, nops, md.den.A[0], md.den.B[0], md.den.A[1],
+                                                     md.den.nbf, bf[sa], bf[sb], bf[sc], bf[sd], scale, out.fock);
+                __syncwarp();
+            }
             if (lane == 0) {
                 if (split == 0) nq += 1;
                 npq += (unsigned long long)((nbp - split + S - 1) / S) * nkp;
@@ -382,20 +322,15 @@ __global__ void __launch_bounds__(TILE, 2) k_fock_warp(const MolDesc *__restrict
     }
 }
 
-// Warps per CTA: four, or two where four warps' arrays would pass 200 KB ((dd|dd)).
-template <int LA, int LB, int LC, int LD>
-constexpr int fock_warps()
-{
-    return 4 * FockLayout<LA, LB, LC, LD>::BYTES <= 200 * 1024 ? 4 : 2;
-}
-
+// At most 8 warps a CTA; units as in launch_lanes.
 template <int LA, int LB, int LC, int LD>
 cudaError_t launch_fock_class(int gcap, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl,
                               const OutArgs &out, const double *boys)
 {
-    constexpr int nw = fock_warps<LA, LB, LC, LD>();
-    return launch_units(k_fock_warp<LA, LB, LC, LD>, nw, gcap, (size_t)nw * FockLayout<LA, LB, LC, LD>::BYTES, st,
-                        mols, cl, out, boys, 32 * nw);
+    constexpr size_t bytes = FockLay<LA, LB, LC, LD>::BYTES;
+    static_assert(bytes <= kCtaSmem, "one warp's arrays fit in a CTA");
+    constexpr int nw = (int)(kCtaSmem / bytes) < 8 ? (int)(kCtaSmem / bytes) : 8;
+    return launch_warp_units(k_fock_lanes<LA, LB, LC, LD>, nw, bytes, gcap, st, mols, cl, out, boys);
 }
 
 }  // namespace tg
