@@ -65,6 +65,59 @@ inline size_t al(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
 
 }  // namespace
 
+// Streams the class launches of one call are spread over.  The 42 lists of a
+// call are independent, and most lists of a small molecule end in a tail of a
+// few long quartets on a few SMs (c1: 21 launches of 0.3 to 3.6 ms each, 27 ms
+// one after the other, with about 5 ms of fp64 work).  Owned by the handle
+// whose work areas the launches use; every call forks from the caller's
+// stream and joins it again, also on an error.
+struct SideStreams {
+    static constexpr int N = 6;
+    cudaStream_t s[N] = {};
+    cudaEvent_t fork = nullptr, join[N] = {};
+    bool ready = false;
+    cudaError_t create()
+    {
+        if (ready) return cudaSuccess;
+        cudaError_t e = cudaSuccess;
+        if (!fork) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+        for (int i = 0; i < N && e == cudaSuccess; ++i) {
+            if (!s[i]) e = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking);
+            if (e == cudaSuccess && !join[i]) e = cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
+        }
+        ready = e == cudaSuccess;
+        return e;
+    }
+    cudaError_t begin(cudaStream_t st)
+    {
+        cudaError_t e = cudaEventRecord(fork, st);
+        for (int i = 0; i < N && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(s[i], fork, 0);
+        return e;
+    }
+    cudaError_t end(cudaStream_t st)
+    {
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < N; ++i) {
+            cudaError_t f = cudaEventRecord(join[i], s[i]);
+            if (f == cudaSuccess) f = cudaStreamWaitEvent(st, join[i], 0);
+            if (e == cudaSuccess) e = f;
+        }
+        return e;
+    }
+    void destroy()
+    {
+        for (int i = 0; i < N; ++i) {
+            if (s[i]) cudaStreamDestroy(s[i]);
+            if (join[i]) cudaEventDestroy(join[i]);
+        }
+        if (fork) cudaEventDestroy(fork);
+        *this = SideStreams();
+    }
+};
+// sets of partial-gradient slabs: one per side stream, so that concurrent
+// launches never add to the same slab and every sum keeps a fixed order
+constexpr int kSlabSets = SideStreams::N;
+
 struct tg_router {
     float params[NPARAM];
     float mu[NFEAT], sd[NFEAT];
@@ -98,6 +151,7 @@ struct tg_basis {
     int nsph = 0;
     std::vector<int> cmap;
     DevArena ws6;  // tg_grad2e_sph: spherical and Cartesian densities, gradient
+    SideStreams side;
 };
 
 namespace {
@@ -139,6 +193,7 @@ void free_basis(tg_basis *b)
     b->ws4.release();
     b->ws5.release();
     b->ws6.release();
+    b->side.destroy();
 }
 
 int basis_setup(tg_basis *b, const double *xyz, const double *exps, const double *coefs)
@@ -532,7 +587,7 @@ int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &op
     // primitive-pair offsets are int32 on the device
     if (npp_max > 0x7fffffffLL) return TG_EUNSUPPORTED;
     // ---- arena 2: pair arrays, primitive-pair records, tiles, features, partials
-    pl.G = std::max(1, 4 * b->nsm);  // partial slabs: up to 4 resident CTAs per SM
+    pl.G = std::max(1, 8 * b->nsm);  // partial slabs: up to 8 resident CTAs per SM
     {
         const size_t np_k = (size_t)std::max<long long>(nk_all, 1);
         const size_t npp = (size_t)std::max<long long>(npp_max, 1);
@@ -546,7 +601,7 @@ int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &op
                              6 * al(sizeof(double) * npp) + 12 * al(sizeof(float) * npp) + al(sizeof(uint4) * ntl) +
                              al(sizeof(MolDesc)) +
                              al(sizeof(TileRef) * ntl) + al(sizeof(float) * ntl * (NFEAT + 1)) +
-                             al(sizeof(double) * (size_t)pl.G * 3 * natom) + 8192;
+                             al(sizeof(double) * (size_t)kSlabSets * pl.G * 3 * natom) + 8192;
         DevArena &V = b->ws2;
         TG_CUDA(V.reserve(need2));
         V.used = 0;
@@ -1120,11 +1175,14 @@ void build_exec(const std::vector<const Plan *> &plans, const std::vector<std::v
 
 // Class launches over an uploaded Exec.  grids[k] (nullable) overrides the
 // persistent grid of list k; with dump != nullptr every quartet's 12
-// components go to dump[(list position * TILE + thread) * 12 + c].
+// components go to dump[(list position * TILE + thread) * 12 + c].  With side
+// streams the lists are launched over them, the classes with the longest
+// quartets first, list i on stream i mod N into slab set i mod N (the caller
+// has cleared all sets); without, on st into the first set.
 int launch_exec(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, double *d_part,
                 unsigned long long *dcnt, double *dump, const double *boys, int G, const int *grids, bool timing,
                 cudaStream_t st, tg_stats *stats, int &launches, const int *kinds = nullptr, int kind_all = 0,
-                int tile_rank = 0, int tile_nranks = 1, const int *splits = nullptr)
+                int tile_rank = 0, int tile_nranks = 1, const int *splits = nullptr, SideStreams *side = nullptr)
 {
     OutArgs out;
     out.partials = d_part;
@@ -1139,8 +1197,13 @@ int launch_exec(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, dou
     EventPair ev;
     if (timing) TG_CUDA(ev.create());
     cudaEvent_t e0 = ev.a, e1 = ev.b;
-    int rc = TG_OK;
-    for (int qc = 0; qc < NQC && rc == TG_OK; ++qc) {
+    int rc = TG_OK, nlist = 0;
+    if (side) {
+        TG_CUDA(side->create());
+        TG_CUDA(side->begin(st));
+    }
+    for (int i = 0; i < NQC && rc == TG_OK; ++i) {
+        const int qc = side ? NQC - 1 - i : i;
         for (int r = 0; r < 2; ++r) {
             const int k = 2 * qc + r;
             // tile-cyclic shard: tiles tile_rank, tile_rank + tile_nranks, ... of the list
@@ -1165,10 +1228,13 @@ int launch_exec(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, dou
             cl.split_req = splits ? splits[k] : 0;
             OutArgs o = out;
             o.counters = dcnt + NCNT * qc;
+            const int on = nlist++ % SideStreams::N;
+            cudaStream_t ls = side ? side->s[on] : st;
+            if (side) o.partials = d_part + (size_t)on * G * 3 * ex.natom_total;
             if (dump) o.dump = dump + (size_t)ex.off[k] * TILE * 12;
             const int grid = std::min(G, (grids && grids[k] > 0) ? grids[k] : G);  // cap; the launcher sizes it
             if (timing) cudaEventRecord(e0, st);
-            cudaError_t e = kClassLaunchers[qc](r, grid, smem, st, d_mols, cl, o, boys);
+            cudaError_t e = kClassLaunchers[qc](r, grid, smem, ls, d_mols, cl, o, boys);
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 rc = TG_ECUDA;
@@ -1183,6 +1249,10 @@ int launch_exec(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, dou
                 if (stats) (r ? stats->class_ms_fp32 : stats->class_ms)[qc] += ms;
             }
         }
+    }
+    if (side && side->end(st) != cudaSuccess) {
+        cudaGetLastError();
+        rc = TG_ECUDA;
     }
     return rc;
 }
@@ -1206,9 +1276,9 @@ void alu_peaks(double &p64, double &p32)
 // with more than nsm tiles, time a sample of 2 to 4 x nsm tiles taken at a
 // fixed stride over the whole list (whose tiles run from the costliest to
 // the cheapest) and search the kernel form (thread, group,
-// warp), the grid cap (1, 2 or 4 CTAs per SM) and the unit shape (bra
+// warp), the grid cap (8, 4 or 2 CTAs per SM) and the unit shape (bra
 // primitive splits per tile: automatic, 1 or 4) one coordinate at a time
-// from (form 1, 2 CTAs per SM, automatic splits): the
+// from (form 1, 8 CTAs per SM, automatic splits): the
 // fastest form, then the fastest grid cap for it, then the fastest split
 // (7 timed launches per list).  Lists left untimed keep kinds[k] = 0 (the
 // default form), grids[k] = 0 (the persistent grid) and splits[k] = 0.
@@ -1245,7 +1315,7 @@ int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, doub
             cudaEventElapsedTime(&ms, e0, e1);
             return TG_OK;
         };
-        int bk = 1, bm = 2, bs = 0;
+        int bk = 1, bm = 8, bs = 0;
         float best = -1.f;
         for (int kind = 1; kind <= 3; ++kind) {
             float ms;
@@ -1253,7 +1323,7 @@ int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, doub
             if (rc != TG_OK) return rc;
             if (best < 0.f || ms < best) best = ms, bk = kind;
         }
-        for (int mult : {1, 4}) {
+        for (int mult : {4, 2}) {
             float ms;
             const int rc = time_cfg(bk, mult, bs, ms);
             if (rc != TG_OK) return rc;
@@ -1332,6 +1402,7 @@ struct tg_batch {
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
+    SideStreams side;
     long long pairs = 0;
     int launches = 0;
     std::vector<int> atom_off;
@@ -1356,7 +1427,10 @@ int tg_grad2e(const tg_basis *cb, int npair, const tg_pair *pairs, const tg_opti
     const int natom = b->natom;
     int launches = pl.launches;
     DevArena &V = b->ws2;
-    double *d_part = V.take<double>((size_t)pl.G * 3 * natom);
+    // with per-class timing the lists run one after the other, in one slab set
+    SideStreams *side = opt.timing ? nullptr : &b->side;
+    const size_t nslab = (size_t)(side ? kSlabSets : 1) * pl.G;
+    double *d_part = V.take<double>((size_t)kSlabSets * pl.G * 3 * natom);
     MolDesc *d_mol = V.take<MolDesc>(1);
     // the screened tile lists, routed and split per (class, precision), built on the device
     DevTiles dt;
@@ -1386,7 +1460,7 @@ int tg_grad2e(const tg_basis *cb, int npair, const tg_pair *pairs, const tg_opti
             sp[k] = b->tune_split[k];
         }
     }
-    TG_CUDA(cudaMemsetAsync(d_part, 0, sizeof(double) * (size_t)pl.G * 3 * natom, st));
+    TG_CUDA(cudaMemsetAsync(d_part, 0, sizeof(double) * nslab * 3 * natom, st));
     TG_CUDA(cudaMemsetAsync(pl.dcnt, 0, sizeof(unsigned long long) * NCNT * NQC, st));
     if (stats)
         for (int qc = 0; qc < NQC; ++qc) stats->class_ms[qc] = stats->class_ms_fp32[qc] = 0.0;
@@ -1394,9 +1468,9 @@ int tg_grad2e(const tg_basis *cb, int npair, const tg_pair *pairs, const tg_opti
     // (a tile shard is already in the lists)
     rc = launch_exec(ex, d_mol, d_tiles, d_part, pl.dcnt, nullptr, b->d_boys, pl.G, tune ? gr : nullptr,
                      opt.timing != 0, st, stats, launches, tune ? kd : nullptr, opt.kernel_kind, 0, 1,
-                     tune ? sp : nullptr);
+                     tune ? sp : nullptr, side);
     if (rc != TG_OK) return rc;
-    k_reduce<<<(3 * natom + 127) / 128, 128, 0, st>>>(3 * natom, pl.G, d_part, pl.dgrad);
+    k_reduce<<<(3 * natom + 31) / 32, 1024, 0, st>>>(3 * natom, (int)nslab, d_part, pl.dgrad);
     ++launches;
     TG_CUDA(cudaGetLastError());
     unsigned long long hc[NCNT * NQC];
@@ -1557,7 +1631,13 @@ int tg_fock2e(const tg_basis *cb, int npair, const tg_fpair *fpairs, const tg_op
     const double plan_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     EventPair ev;
     if (opt.timing) TG_CUDA(ev.create());
-    for (int qc = 0; qc < NQC; ++qc) {
+    SideStreams *side = opt.timing ? nullptr : &b->side;
+    if (side) {
+        TG_CUDA(side->create());
+        TG_CUDA(side->begin(st));
+    }
+    int nlist = 0;
+    for (int qc = NQC - 1; qc >= 0 && rc == TG_OK; --qc) {
         const long long nt = dt.off[2 * qc + 1] - dt.off[2 * qc];
         if (nt <= 0) continue;
         ClassLaunch cl;
@@ -1574,10 +1654,12 @@ int tg_fock2e(const tg_basis *cb, int npair, const tg_fpair *fpairs, const tg_op
         o.natom_total = o.natom_max = natom;
         o.fock = dF;
         if (opt.timing) cudaEventRecord(ev.a, st);
-        cudaError_t e = kFockLaunchers[qc](pl.G, st, d_mol, cl, o, b->d_boys);
+        cudaStream_t ls = side ? side->s[nlist++ % SideStreams::N] : st;
+        cudaError_t e = kFockLaunchers[qc](pl.G, ls, d_mol, cl, o, b->d_boys);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            return TG_ECUDA;
+            rc = TG_ECUDA;
+            break;
         }
         ++launches;
         if (opt.timing) {
@@ -1588,6 +1670,11 @@ int tg_fock2e(const tg_basis *cb, int npair, const tg_fpair *fpairs, const tg_op
             if (stats) stats->class_ms[qc] += ms;
         }
     }
+    if (side && side->end(st) != cudaSuccess) {
+        cudaGetLastError();
+        rc = TG_ECUDA;
+    }
+    if (rc != TG_OK) return rc;
     unsigned long long hc[NCNT * NQC];
     TG_CUDA(cudaMemcpyAsync(hc, pl.dcnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
     TG_CUDA(cudaMemcpyAsync(F, dF, sizeof(double) * nbf2,
@@ -1761,13 +1848,13 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
     bt->G = G;
     const size_t ntl = std::max<size_t>(bt->ex.tiles.size(), 1);
     const size_t need = al(sizeof(MolDesc) * nmol) + al(sizeof(uint4) * ntl) +
-                        al(sizeof(double) * (size_t)G * 3 * natom_total) + al(sizeof(double) * 3 * natom_total) +
+                        al(sizeof(double) * (size_t)kSlabSets * G * 3 * natom_total) + al(sizeof(double) * 3 * natom_total) +
                         al(sizeof(unsigned long long) * NCNT * NQC) + 4096;
     TG_CUDA(bt->arena.reserve(need));
     bt->arena.used = 0;
     bt->d_mols = bt->arena.take<MolDesc>(nmol);
     bt->d_tiles = bt->arena.take<uint4>(ntl);
-    bt->d_part = bt->arena.take<double>((size_t)G * 3 * natom_total);
+    bt->d_part = bt->arena.take<double>((size_t)kSlabSets * G * 3 * natom_total);
     bt->d_grad = bt->arena.take<double>(3 * natom_total);
     bt->d_cnt = bt->arena.take<unsigned long long>(NCNT * NQC);
     std::vector<MolDesc> mds(nmol);
@@ -1799,13 +1886,13 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
         // re-carve with the larger slab count
         bt->arena.release();
         const size_t need2 = al(sizeof(MolDesc) * nmol) + al(sizeof(uint4) * ntl) +
-                             al(sizeof(double) * (size_t)G * 3 * natom_total) + al(sizeof(double) * 3 * natom_total) +
+                             al(sizeof(double) * (size_t)kSlabSets * G * 3 * natom_total) + al(sizeof(double) * 3 * natom_total) +
                              al(sizeof(unsigned long long) * NCNT * NQC) + 4096;
         TG_CUDA(bt->arena.reserve(need2));
         bt->arena.used = 0;
         bt->d_mols = bt->arena.take<MolDesc>(nmol);
         bt->d_tiles = bt->arena.take<uint4>(ntl);
-        bt->d_part = bt->arena.take<double>((size_t)G * 3 * natom_total);
+        bt->d_part = bt->arena.take<double>((size_t)kSlabSets * G * 3 * natom_total);
         bt->d_grad = bt->arena.take<double>(3 * natom_total);
         bt->d_cnt = bt->arena.take<unsigned long long>(NCNT * NQC);
         TG_CUDA(cudaMemcpy(bt->d_mols, mds.data(), sizeof(MolDesc) * nmol, cudaMemcpyHostToDevice));
@@ -1819,12 +1906,13 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
     for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) TG_CUDA(cudaStreamBeginCapture(bt->cap, cudaStreamCaptureModeThreadLocal));
         int n = 0;
-        cudaMemsetAsync(bt->d_part, 0, sizeof(double) * (size_t)G * 3 * natom_total, bt->cap);
+        cudaMemsetAsync(bt->d_part, 0, sizeof(double) * (size_t)kSlabSets * G * 3 * natom_total, bt->cap);
         cudaMemsetAsync(bt->d_cnt, 0, sizeof(unsigned long long) * NCNT * NQC, bt->cap);
         int rc = launch_exec(bt->ex, bt->d_mols, bt->d_tiles, bt->d_part, bt->d_cnt, nullptr, boys, G,
                              bt->grids.data(), false, bt->cap, nullptr, n, bt->kinds.data(), 0, 0, 1,
-                             bt->splits.data());
-        k_reduce<<<(3 * natom_total + 127) / 128, 128, 0, bt->cap>>>(3 * natom_total, G, bt->d_part, bt->d_grad);
+                             bt->splits.data(), &bt->side);
+        k_reduce<<<(3 * natom_total + 31) / 32, 1024, 0, bt->cap>>>(3 * natom_total, kSlabSets * G, bt->d_part,
+                                                                   bt->d_grad);
         ++n;
         if (pass == 1) {
             cudaError_t e = cudaStreamEndCapture(bt->cap, &bt->graph);
@@ -1879,6 +1967,7 @@ void tg_batch_destroy(tg_batch *bt)
     if (bt->gexec) cudaGraphExecDestroy(bt->gexec);
     if (bt->graph) cudaGraphDestroy(bt->graph);
     if (bt->cap) cudaStreamDestroy(bt->cap);
+    bt->side.destroy();
     bt->arena.release();
     delete bt;
 }

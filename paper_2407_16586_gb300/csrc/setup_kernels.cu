@@ -350,14 +350,23 @@ __global__ void k_fock_combine(int nbf, DensArgs den, double *SJ, double *BK, do
     BL[id] = bl;
 }
 
-// grad[k] = sum_c partials[c][k] in the fixed order c = 0..nslab-1
-__global__ void k_reduce(int n, int nslab, const double *partials, double *grad)
+// grad[k] = sum_c partials[c][k] in a fixed order: 32 components per block, warp
+// w adds slabs w, w + 32, ..., then the 32 sums of a component are added in
+// order.  (One thread per component walked all slabs one load after the other.)
+__global__ void __launch_bounds__(1024) k_reduce(int n, int nslab, const double *partials, double *grad)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+    __shared__ double part[32][33];
+    const int tx = threadIdx.x % 32, ty = threadIdx.x / 32, k = blockIdx.x * 32 + tx;
     double s = 0.0;
-    for (int c = 0; c < nslab; ++c) s += partials[(size_t)c * n + k];
-    grad[k] = s;
+    if (k < n)
+        for (int c = ty; c < nslab; c += 32) s += partials[(size_t)c * n + k];
+    part[ty][tx] = s;
+    __syncthreads();
+    if (ty == 0 && k < n) {
+        s = 0.0;
+        for (int w = 0; w < 32; ++w) s += part[w][tx];
+        grad[k] = s;
+    }
 }
 
 // Spherical shells (Sec. II.C: the 2l+1 spherical functions of a shell are a
