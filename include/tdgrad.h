@@ -263,7 +263,7 @@ int tg_fock2e(const tg_basis *b, int npair, const tg_fpair *pairs, const tg_opti
  * are copied at creation.  opt->autotune = 1 autotunes every class list
  * on a sample of 2 to 4 x (SM count) of its tiles taken at a fixed stride
  * over the whole list: the kernel form (thread, group or
- * warp), the persistent grid (1, 2 or 4 CTAs per SM) and the work-unit shape
+ * warp), the persistent grid (8, 4 or 2 CTAs per SM) and the work-unit shape
  * (bra primitive splits per tile: automatic, 1 or 4), searched one
  * coordinate at a time (form, then grid, then splits; 7 timed launches per
  * list), keeping the fastest.

@@ -164,8 +164,8 @@ __device__ void quartet_fock_ints(double *sm, int lane, const GeoArgs &geo, cons
             }
         }
         // ---- V -> I: ket functions, then bra functions
-        entry_values<LA, LB>(vb, lane, pw);
-        entry_values<LC, LD>(vk, lane, pw + 15);
+        entry_values<LA, LB>(vb, lane, pw, 1);
+        entry_values<LC, LD>(vk, lane, pw + 15, 1);
         __syncwarp();
         for (int it = lane; it < NM1 * NCD; it += 32) {
             const int m1 = it / NCD, cd = it % NCD;
@@ -260,7 +260,7 @@ __device__ void quartet_fock_scatter(const double *I, int lane, int nops, const 
 // Persistent Fock class kernel over warp units (as k_grad_lanes).  The
 // combined matrices are den.A[0] = S_J, den.B[0] = B_K, den.A[1] = B_lr.
 template <int LA, int LB, int LC, int LD>
-__global__ void __launch_bounds__(256, (LA + LB + LC + LD <= 2 ? 2 : 1))
+__global__ void __launch_bounds__(32, LA + LB + LC + LD <= 3 ? 16 : 8)
     k_fock_lanes(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out, const double *__restrict__ boys)
 {
     using Lay = FockLay<LA, LB, LC, LD>;
@@ -322,15 +322,14 @@ __global__ void __launch_bounds__(256, (LA + LB + LC + LD <= 2 ? 2 : 1))
     }
 }
 
-// At most 8 warps a CTA; units as in launch_lanes.
+// CTAs of one warp (see HermOp); F takes atomic adds, so no slab limits the grid.
 template <int LA, int LB, int LC, int LD>
-cudaError_t launch_fock_class(int gcap, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl,
-                              const OutArgs &out, const double *boys)
+cudaError_t launch_fock_class(int, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl, const OutArgs &out,
+                              const double *boys)
 {
     constexpr size_t bytes = FockLay<LA, LB, LC, LD>::BYTES;
     static_assert(bytes <= kCtaSmem, "one warp's arrays fit in a CTA");
-    constexpr int nw = (int)(kCtaSmem / bytes) < 8 ? (int)(kCtaSmem / bytes) : 8;
-    return launch_warp_units(k_fock_lanes<LA, LB, LC, LD>, nw, bytes, gcap, st, mols, cl, out, boys);
+    return launch_warp_units(k_fock_lanes<LA, LB, LC, LD>, 1, bytes, 1, 1 << 20, st, mols, cl, out, boys);
 }
 
 }  // namespace tg

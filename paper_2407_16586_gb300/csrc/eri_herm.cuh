@@ -193,15 +193,17 @@ __device__ __forceinline__ const PairTab<LA, LB> &pair_tab()
 
 // ------------------------------------------------------------ layout
 
-// One warp's slice of shared memory, in doubles.  Rows that lanes read at
-// different row numbers have an odd stride.  NO operators are resident at a
-// time; classes whose arrays are large take the operators one after the other
-// (the scalars of a primitive quartet are then formed twice, 3 % of the work
-// at (pp|pp)), which keeps at least four warps on an SM.
-template <int LA, int LB, int LC, int LD>
-struct HermLay {
+// One warp's slice of shared memory, in doubles, for KQ ket pairs at a time.
+// Rows that lanes read at different row numbers have an odd stride.  NO
+// operators are resident at a time; classes whose arrays are large take the
+// operators one after the other (the scalars of a primitive quartet are then
+// formed twice, 3 % of the work at (pp|pp)), which keeps at least four warps on
+// an SM.
+template <int LA, int LB, int LC, int LD, int KQ_>
+struct HermLayK {
     using B = PairMono<LA, LB>;
     using K = PairMono<LC, LD>;
+    static constexpr int KQ = KQ_;
     static constexpr int NAB = B::NAB, NCD = K::NAB, L1 = B::L, L2 = K::L, L = L1 + L2, LM = L + 1;
     static constexpr int NT1 = B::NH, NM1 = B::NM, NM2 = K::NM, NS1 = B::NS, NS2 = K::NS;
     static constexpr int NABP = NAB | 1, NM2P = NM2 | 1;
@@ -213,25 +215,56 @@ struct HermLay {
     static constexpr int NRH = nherm(PASSES ? LM : L);  // Hermite rows
     static constexpr int NO = (NAB * NCD <= 27) ? 2 : 1;
     // bra primitive pairs of a block: a budget of 1200 doubles for F, 1 to 16
-    static constexpr int PB_RAW = 1200 / (NT1 * NM2P * NO);
+    // (700 buys (dp|pp) a sixth warp, but its half-filled passes cost more:
+    // 23.4 -> 29.3 ms on a 1/8 shard of the 32-atom workload)
+    static constexpr int PB_RAW = 1200 / (NT1 * NM2P * NO * KQ);
     static constexpr int PB = PB_RAW < 1 ? 1 : (PB_RAW > 16 ? 16 : PB_RAW);
     static constexpr int NE1 = pair_entries(LA, LB), NE2 = pair_entries(LC, LD);
+    static constexpr int GS = NO * NCD * NABP, MS = NO * NM1 * NM2P, FS = NO * NT1 * NM2P;  // per ket pair
+    static constexpr int HS = (NM2 * NABP > NM1 * NCD ? NM2 * NABP : NM1 * NCD) * NO;
     // the transforms' half-way arrays share the space of the R rows
-    static constexpr int HALF = (NM2 * NABP > NM1 * NCD ? NM2 * NABP : NM1 * NCD) * NO + NE1 + NE2;
-    static constexpr int ROWS = NRH * RS + NS2 * RS;
-    static constexpr int RED = 9 * RS;
+    static constexpr int HALF = NE1 + KQ * (NE2 + HS), ROWS = (NRH + NS2) * RS, RED = 9 * RS;
     static constexpr int SHARED = HALF > ROWS ? (HALF > RED ? HALF : RED) : (ROWS > RED ? ROWS : RED);
-    static constexpr int NP1 = 5;                     // per bra primitive pair: a^, mu, K/p factor, p, spare
-    static constexpr int o_G = 0;                                  // [NO][NCD][NABP]
-    static constexpr int o_Gp = o_G + NO * NCD * NABP;             // [NO][NM1][NM2P]
-    static constexpr int o_V = o_Gp + NO * NM1 * NM2P;             // [NO][NM1][NM2P]
-    static constexpr int o_F = o_V + NO * NM1 * NM2P;              // [PB][NO][NT1][NM2P]
-    static constexpr int o_S1 = o_F + PB * NO * NT1 * NM2P;        // [PB][NS1]
-    static constexpr int o_P1 = o_S1 + PB * NS1;                   // [PB][NP1]
-    static constexpr int o_pw = o_P1 + PB * NP1;                   // [2][3][5] powers of R and S
-    static constexpr int o_X = o_pw + 30;                          // SHARED
+    static constexpr int NP1 = 4;                     // per bra primitive pair: a^, mu, 4 pi^(5/2) K / 2p, p
+    static constexpr int o_G = 0;                              // [KQ][NO][NCD][NABP]
+    static constexpr int o_Gp = o_G + KQ * GS;                 // [KQ][NO][NM1][NM2P]
+    static constexpr int o_V = o_Gp + KQ * MS;                 // [KQ][NO][NM1][NM2P]
+    static constexpr int o_F = o_V + KQ * MS;                  // [PB][KQ][NO][NT1][NM2P]
+    static constexpr int o_S1 = o_F + PB * KQ * FS;            // [PB][NS1]
+    static constexpr int o_P1 = o_S1 + PB * NS1;               // [PB][NP1]
+    static constexpr int o_pw = o_P1 + PB * NP1;               // [1 + KQ][3][5] powers of R, then of each S
+    static constexpr int o_X = o_pw + (1 + KQ) * 15;           // SHARED
     static constexpr int TOTAL = (o_X + SHARED + 1) & ~1;
     static constexpr size_t BYTES = sizeof(double) * (size_t)TOTAL;
+};
+
+// Ket pairs of one bra pair that may be taken together: the most (8, 4, 2, 1)
+// with which 16 warps still fit an SM's shared memory, up to L = 2 ((ps|ss):
+// 16.7 -> 11.5 ms on a 1/8 shard of the 32-atom workload).  Above, a group costs
+// warps and gains nothing ((pp|ps): 23.9 -> 27.6 ms, (dp|pp): 23.4 -> 30.4 ms).
+template <int LA, int LB, int LC, int LD>
+constexpr int herm_kets()
+{
+    constexpr size_t cap = (223 * 1024) / 16;
+    if (LA + LB + LC + LD > 2) return 1;
+    if (HermLayK<LA, LB, LC, LD, 8>::BYTES <= cap) return 8;
+    if (HermLayK<LA, LB, LC, LD, 4>::BYTES <= cap) return 4;
+    if (HermLayK<LA, LB, LC, LD, 2>::BYTES <= cap) return 2;
+    return 1;
+}
+
+template <int LA, int LB, int LC, int LD>
+using HermLay = HermLayK<LA, LB, LC, LD, herm_kets<LA, LB, LC, LD>()>;
+
+// The valid ket pairs of one bra pair among up to KQ neighbours, in shared
+// memory; entries past them have nk = 0 and a valid pk0.  A group is the
+// entries k0 .. k0 + kg - 1.
+struct GroupInfo {
+    static constexpr int CAP = 8;
+    int n;                       // valid ket pairs of the whole record
+    int sc[8], sd[8];            // shells
+    int pk0[8], nk[8];           // primitive pairs
+    double scale[8];             // 1/|stabiliser|
 };
 
 // (h1, m2) items of the reverse sums: ALL, or those whose V enters a
@@ -516,81 +549,80 @@ __device__ __forceinline__ void hermite_level(double *Rl, int n, double X, doubl
 
 // ------------------------------------------------------------ quartet
 
-// Gamma_op of the canonical quartet (the 8 permutation images of the pair
-// products, times scale), [cd][ab], for operators o0 .. o0 + NO - 1.
+// Gamma_op of the group's quartets (the 8 permutation images of the pair
+// products, times scale), [ket][op][cd][ab], for operators o0 .. o0 + NO - 1.
 template <int LA, int LB, int LC, int LD>
-__device__ __forceinline__ void herm_gamma(double *G, int lane, int o0, const DensArgs &den, int fa, int fb, int fc,
-                                           int fd, double scale)
+__device__ __forceinline__ void herm_gamma(double *G, int lane, int kg, const GroupInfo &gi, int k0, int o0, const DensArgs &den,
+                                           const int *sh_bf, int fa, int fb)
 {
     using Lay = HermLay<LA, LB, LC, LD>;
-    constexpr int NB = ncart(LB), ND = ncart(LD);
+    constexpr int NB = ncart(LB), ND = ncart(LD), NFQ = Lay::NAB * Lay::NCD;
     const int nbf = den.nbf;
-    for (int it = lane; it < Lay::NAB * Lay::NCD; it += 32) {
-        const int cd = it / Lay::NAB, ab = it % Lay::NAB;
-        const size_t m = fa + ab / NB, n = fb + ab % NB, l = fc + cd / ND, s = fd + cd % ND;
+    for (int x = lane; x < kg * NFQ; x += 32) {
+        const int kq = x / NFQ, it = x % NFQ, cd = it / Lay::NAB, ab = it % Lay::NAB;
+        double *g = G + kq * Lay::GS + cd * Lay::NABP + ab;
         double g0 = 0.0, g1 = 0.0;
-        for (int p = 0; p < den.npair; ++p) {
-            const double *A = den.A[p], *B = den.B[p];
-            const double cj = den.cJ[p], ck = den.cK[p], cl = den.cKlr[p];
-            if (cj != 0.0 && (Lay::NO == 2 || o0 == 0))
-                g0 += cj * (den.S[p][m * nbf + n] * den.T[p][l * nbf + s] + den.S[p][l * nbf + s] * den.T[p][m * nbf + n]);
-            if (ck != 0.0 || cl != 0.0) {
-                const double kk = A[m * nbf + l] * B[n * nbf + s] + A[n * nbf + l] * B[m * nbf + s] +
-                                  A[m * nbf + s] * B[n * nbf + l] + A[n * nbf + s] * B[m * nbf + l] +
-                                  A[l * nbf + m] * B[s * nbf + n] + A[s * nbf + m] * B[l * nbf + n] +
-                                  A[l * nbf + n] * B[s * nbf + m] + A[s * nbf + n] * B[l * nbf + m];
-                g0 += ck * kk;
-                g1 += cl * kk;
+        if (k0 + kq < gi.n) {
+            const size_t m = fa + ab / NB, n = fb + ab % NB;
+            const size_t l = sh_bf[gi.sc[k0 + kq]] + cd / ND, s = sh_bf[gi.sd[k0 + kq]] + cd % ND;
+            for (int p = 0; p < den.npair; ++p) {
+                const double *A = den.A[p], *B = den.B[p];
+                const double cj = den.cJ[p], ck = den.cK[p], cl = den.cKlr[p];
+                if (cj != 0.0 && (Lay::NO == 2 || o0 == 0))
+                    g0 += cj * (den.S[p][m * nbf + n] * den.T[p][l * nbf + s] + den.S[p][l * nbf + s] * den.T[p][m * nbf + n]);
+                if (ck != 0.0 || cl != 0.0) {
+                    const double kk = A[m * nbf + l] * B[n * nbf + s] + A[n * nbf + l] * B[m * nbf + s] +
+                                      A[m * nbf + s] * B[n * nbf + l] + A[n * nbf + s] * B[m * nbf + l] +
+                                      A[l * nbf + m] * B[s * nbf + n] + A[s * nbf + m] * B[l * nbf + n] +
+                                      A[l * nbf + n] * B[s * nbf + m] + A[s * nbf + n] * B[l * nbf + m];
+                    g0 += ck * kk;
+                    g1 += cl * kk;
+                }
             }
+            g0 *= gi.scale[k0 + kq];
+            g1 *= gi.scale[k0 + kq];
         }
         if constexpr (Lay::NO == 2) {
-            G[cd * Lay::NABP + ab] = g0 * scale;
-            G[(Lay::NCD + cd) * Lay::NABP + ab] = g1 * scale;
+            g[0] = g0;
+            g[Lay::NCD * Lay::NABP] = g1;
         } else {
-            G[cd * Lay::NABP + ab] = (o0 == 0 ? g0 : g1) * scale;
+            g[0] = o0 == 0 ? g0 : g1;
         }
     }
 }
 
-// c^{ab}_m R^.. of every table entry of a pair class.
+// c^{ab}_m R^.. of every table entry of a pair class, for n pairs (powers pw,
+// 15 apart).
 template <int LA, int LB>
-__device__ __forceinline__ void entry_values(double *out, int lane, const double *pw)
+__device__ __forceinline__ void entry_values(double *out, int lane, const double *pw, int n)
 {
     const auto &T = pair_tab<LA, LB>();
-    for (int e = lane; e < PairTab<LA, LB>::NE; e += 32) {
-        const unsigned w = T.ent[e];
-        out[e] = double((int)((w >> 8) & 0xff)) * pw[(w >> 16) & 7] * pw[5 + ((w >> 19) & 7)] * pw[10 + ((w >> 22) & 7)];
+    constexpr int NE = PairTab<LA, LB>::NE;
+    for (int x = lane; x < n * NE; x += 32) {
+        const unsigned w = T.ent[x % NE];
+        const double *q = pw + x / NE * 15;
+        out[x] = double((int)((w >> 8) & 0xff)) * q[(w >> 16) & 7] * q[5 + ((w >> 19) & 7)] * q[10 + ((w >> 22) & 7)];
     }
 }
 
-// half[o][m2][ab] = sum_{entries of m2} value Gamma[cd][ab]
+// half[ket][o][m2][ab] = sum_{entries of m2} value Gamma[cd][ab]
 template <int LA, int LB, int LC, int LD>
-__device__ __forceinline__ void half_ket(double *half, const double *G, const double *vk, int lane)
+__device__ __forceinline__ void half_ket(double *half, const double *G, const double *vk, int lane, int kg)
 {
     using Lay = HermLay<LA, LB, LC, LD>;
     const auto &T = pair_tab<LC, LD>();
-    for (int it = lane; it < Lay::NM2 * Lay::NAB; it += 32) {
-        const int m = it / Lay::NAB, ab = it % Lay::NAB;
+    constexpr int N = Lay::NM2 * Lay::NAB;
+    for (int x = lane; x < kg * N; x += 32) {
+        const int kq = x / N, it = x % N, m = it / Lay::NAB, ab = it % Lay::NAB;
+        const double *v = vk + kq * Lay::NE2;
 #pragma unroll
         for (int o = 0; o < Lay::NO; ++o) {
+            const double *g = G + kq * Lay::GS + o * Lay::NCD * Lay::NABP + ab;
             double s = 0.0;
-            for (int e = T.start[m]; e < T.start[m + 1]; ++e)
-                s += vk[e] * G[(o * Lay::NCD + (T.ent[e] & 0xff)) * Lay::NABP + ab];
-            half[(o * Lay::NM2 + m) * Lay::NABP + ab] = s;
+            for (int e = T.start[m]; e < T.start[m + 1]; ++e) s += v[e] * g[(T.ent[e] & 0xff) * Lay::NABP];
+            half[kq * Lay::HS + (o * Lay::NM2 + m) * Lay::NABP + ab] = s;
         }
     }
-}
-
-// Bra primitive pairs taken at a time (1 .. cap, at most nbra): the block of
-// pb * nkp primitive quartets that leaves the fewest of its lanes idle.
-__device__ __forceinline__ int block_pairs(int nbra, int nkp, int cap)
-{
-    int pb = 1, best = -1;
-    for (int c = 1; c <= (nbra < cap ? nbra : cap); ++c) {
-        const int n = c * nkp, use = n * 64 / ((n + 31) / 32);  // primitive quartets per pass, times 64
-        if (use >= best) best = use, pb = c;
-    }
-    return pb;
 }
 
 // items table of the class a translation unit compiles
@@ -634,42 +666,98 @@ __device__ __forceinline__ void reverse_sums(double *V, const double *Rr, const 
     }
 }
 
-// One contracted quartet by one warp, bra primitive pairs ib0, ib0 + ibs, ...
-// acc[0..2] += d/dA, acc[3..5] += d/dA + d/dB, acc[6..8] += d/dC (this lane's
-// share; the caller sums the warp).
+// The same for a group of kg > 1 ket pairs, whose lanes are kq LG .. kq LG +
+// LG - 1 with the primitive quartets it0 .. it0 + LG - 1 of its own list of np
+// * nks[kq]; V of ket pair kq at V + kq * vs.
 template <int LA, int LB, int LC, int LD>
-__device__ void quartet_herm(double *sm, int lane, const GeoArgs &geo, const DensArgs &den,
-                             const PrimPairs &pp, int sa, int sb, int sc, int sd, int pb0, int nbp, int ib0, int ibs,
-                             int pk0, int nkp, double scale, const double *boys, double (&acc)[9])
+__device__ __forceinline__ void reverse_sums_group(double *V, int vs, const double *Rr, const double *S2,
+                                                   const double *S1, int it0, int np, int kg, int LG,
+                                                   const int *nks, int lane)
+{
+    using B = PairMono<LA, LB>;
+    constexpr int NIT = HermItems<LA, LB, LC, LD, false>::N, RS = 33, NM2P = PairMono<LC, LD>::NM | 1;
+    const auto &TBra = pair_tab<LA, LB>();
+    const unsigned *items = kHermItems<LA, LB, LC, LD, false>.it;
+    for (int x = lane; x < kg * NIT; x += 32) {
+        const int kq = x / NIT, nk = nks[kq];
+        const int n = min(LG, np * nk - it0);
+        if (n <= 0) continue;
+        const unsigned w = items[x % NIT];
+        const double *r = Rr + (w & 0xff) * RS + kq * LG, *s = S2 + (w >> 21) * RS + kq * LG;
+        const unsigned hm = TBra.hm[(w >> 8) & 0x3f];
+        double *v = V + kq * vs + (hm & 0xff) * NM2P + ((w >> 14) & 0x7f);
+        const int ns = (hm >> 8) & 0xf;
+        int pj = it0 / nk, j = 0;
+        while (j < n) {
+            const int hi = min((pj + 1) * nk - it0, n);
+            double u = 0.0;
+#pragma unroll 4
+            for (; j < hi; ++j) u += s[j] * r[j];
+            const double *s1 = S1 + pj * B::NS + (hm >> 12);
+            for (int k = 0; k < ns; ++k) v[k * NM2P] += s1[k] * u;
+            ++pj;
+        }
+    }
+}
+
+// Bra primitive pairs taken at a time (1 .. cap, at most nbra): the block of
+// pb * nkp primitive quartets that leaves the fewest of its lanes idle.
+__device__ __forceinline__ int block_pairs(int nbra, int nkp, int cap, int lanes = 32)
+{
+    int pb = 1, best = -1;
+    for (int c = 1; c <= (nbra < cap ? nbra : cap); ++c) {
+        const int n = c * nkp, use = n * 64 / ((n + lanes - 1) / lanes);  // primitive quartets per pass, times 64
+        if (use >= best) best = use, pb = c;
+    }
+    return pb;
+}
+
+// A group of kg (1, 2, 4, 8; at most KQ) ket pairs with one bra pair by one
+// warp, bra primitive pairs ib0, ib0 + ibs, ...  Lanes kq LG .. kq LG + LG - 1
+// (LG = 32 / kg) take the primitive quartets of ket pair kq: the density
+// transform, its loads and the closing sums, which a few lanes of a single
+// quartet would leave half empty in the small classes, run over all ket pairs
+// at once.  acc[0..2] += d/dA, acc[3..5] += d/dA + d/dB, acc[6..8] += d/dC
+// (this lane's share; d/dA of all ket pairs may sit on any lane, the others on
+// their ket pair's lanes).
+template <int LA, int LB, int LC, int LD>
+__device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo &gi, const GeoArgs &geo, const DensArgs &den,
+                           const PrimPairs &pp, int sa, int sb, int pb0, int nbp, int ib0, int ibs, const double *boys,
+                           double (&acc)[9])
 {
     using Lay = HermLay<LA, LB, LC, LD>;
     constexpr int NCD = Lay::NCD, L = Lay::L, LM = Lay::LM, NT1 = Lay::NT1;
     constexpr int NM1 = Lay::NM1, NM2 = Lay::NM2, NM2P = Lay::NM2P, NS1 = Lay::NS1, NS2 = Lay::NS2, RS = Lay::RS;
-    constexpr int NO = Lay::NO, NP1 = Lay::NP1, NABP = Lay::NABP;
+    constexpr int NO = Lay::NO, NP1 = Lay::NP1, NABP = Lay::NABP, KQ = Lay::KQ;
     constexpr int NIT = HermItems<LA, LB, LC, LD, false>::N;
     double *G = sm + Lay::o_G, *Gp = sm + Lay::o_Gp, *V = sm + Lay::o_V, *F = sm + Lay::o_F;
     double *S1 = sm + Lay::o_S1, *P1 = sm + Lay::o_P1, *pw = sm + Lay::o_pw, *X1 = sm + Lay::o_X;
-    double *Rr = X1, *S2 = X1 + Lay::NRH * RS;                      // main loop
-    double *half = X1 + Lay::NE1 + Lay::NE2, *vb = X1, *vk = X1 + Lay::NE1;  // transforms
+    double *Rr = X1, *S2 = X1 + Lay::NRH * RS;                                    // main loop
+    double *vb = X1, *vk = X1 + Lay::NE1, *half = vk + KQ * Lay::NE2;              // transforms
     const auto &TBra = pair_tab<LA, LB>();
     const auto &TKet = pair_tab<LC, LD>();
     const int nops = den.use_lr ? 2 : 1;
     const bool ominf = isinf(den.omega);
     const double om = ominf ? 1.0 : den.omega;
-    const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xb = geo.xyz + 3 * geo.sh_atom[sb];
-    const double *xc = geo.xyz + 3 * geo.sh_atom[sc], *xd = geo.xyz + 3 * geo.sh_atom[sd];
-    if (lane < 6) {  // powers of R = A - B and S = C - D
-        const int d = lane % 3;
-        const double x = lane < 3 ? xa[d] - xb[d] : xc[d] - xd[d];
+    if constexpr (KQ == 1) kg = 1;
+    const int LG = 32 / kg, kq = lane / LG, sl = lane % LG;
+    if (lane < 3 + 3 * kg) {  // powers of R = A - B and of every S = C - D
+        const int d = lane % 3, w = lane / 3;
+        const int k = min(k0 + w - 1, gi.n - 1);
+        const int s0 = w == 0 ? sa : gi.sc[k], s1 = w == 0 ? sb : gi.sd[k];
+        const double x = geo.xyz[3 * geo.sh_atom[s0] + d] - geo.xyz[3 * geo.sh_atom[s1] + d];
         double p = 1.0;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            pw[(lane / 3) * 15 + d * 5 + k] = p;
+        for (int i = 0; i < 5; ++i) {
+            pw[w * 15 + d * 5 + i] = p;
             p *= x;
         }
     }
-    const int nbra = (nbp - ib0 + ibs - 1) / ibs;  // bra primitive pairs of this call
-    const int pb = block_pairs(nbra, nkp, Lay::PB);
+    int nkmax = gi.nk[k0];
+    for (int k = 1; k < kg; ++k) nkmax = max(nkmax, gi.nk[k0 + k]);
+    const int nk = gi.nk[k0 + kq], nkd = max(nk, 1), pk0 = gi.pk0[k0 + kq];  // this lane's ket pair
+    const int nbra = (nbp - ib0 + ibs - 1) / ibs;                  // bra primitive pairs of this call
+    const int pb = block_pairs(nbra, nkmax, Lay::PB, LG);
     // this lane's sums over its primitive quartets: T, a^ T, c^ T, mu_ab E, mu_cd E
     double aT[3] = {0.0, 0.0, 0.0}, aA[3] = {0.0, 0.0, 0.0}, aC[3] = {0.0, 0.0, 0.0}, eA = 0.0, eC = 0.0;
     double gA[3] = {0.0, 0.0, 0.0}, gC[3] = {0.0, 0.0, 0.0};  // polynomial parts
@@ -677,28 +765,28 @@ __device__ void quartet_herm(double *sm, int lane, const GeoArgs &geo, const Den
 
     for (int o0 = 0; o0 < nops; o0 += NO) {
         // ---- Gamma -> G'[m1][m2]
-        herm_gamma<LA, LB, LC, LD>(G, lane, o0, den, geo.sh_bf[sa], geo.sh_bf[sb], geo.sh_bf[sc], geo.sh_bf[sd], scale);
-        entry_values<LA, LB>(vb, lane, pw);
-        entry_values<LC, LD>(vk, lane, pw + 15);
+        herm_gamma<LA, LB, LC, LD>(G, lane, kg, gi, k0, o0, den, geo.sh_bf, geo.sh_bf[sa], geo.sh_bf[sb]);
+        entry_values<LA, LB>(vb, lane, pw, 1);
+        entry_values<LC, LD>(vk, lane, pw + 15, kg);
         __syncwarp();
-        half_ket<LA, LB, LC, LD>(half, G, vk, lane);
+        half_ket<LA, LB, LC, LD>(half, G, vk, lane, kg);
         __syncwarp();
-        for (int it = lane; it < NM1 * NM2; it += 32) {
-            const int m1 = it / NM2, m2 = it % NM2;
+        for (int x = lane; x < kg * NM1 * NM2; x += 32) {
+            const int q = x / (NM1 * NM2), it = x % (NM1 * NM2), m1 = it / NM2, m2 = it % NM2;
 #pragma unroll
             for (int o = 0; o < NO; ++o) {
+                const double *h = half + q * Lay::HS + (o * NM2 + m2) * NABP;
                 double s = 0.0;
-                for (int e = TBra.start[m1]; e < TBra.start[m1 + 1]; ++e)
-                    s += vb[e] * half[(o * NM2 + m2) * NABP + (TBra.ent[e] & 0xff)];
-                Gp[(o * NM1 + m1) * NM2P + m2] = s;
-                V[(o * NM1 + m1) * NM2P + m2] = 0.0;
+                for (int e = TBra.start[m1]; e < TBra.start[m1 + 1]; ++e) s += vb[e] * h[TBra.ent[e] & 0xff];
+                Gp[q * Lay::MS + (o * NM1 + m1) * NM2P + m2] = s;
+                V[q * Lay::MS + (o * NM1 + m1) * NM2P + m2] = 0.0;
             }
         }
         __syncwarp();
 
         for (int blk = 0; blk < nbra; blk += pb) {
             const int np = min(pb, nbra - blk);
-            // ---- scalars of the block's bra primitive pairs, then F[p][h1][m2]
+            // ---- scalars of the block's bra primitive pairs, then F[p][ket][h1][m2]
             if (lane < np) {
                 const int ip = pb0 + ib0 + (blk + lane) * ibs;
                 const double p = pp.p[ip], za = pp.za[ip], oo2 = 0.5 / p;
@@ -713,33 +801,34 @@ __device__ void quartet_herm(double *sm, int lane, const GeoArgs &geo, const Den
                 P1[lane * NP1 + 3] = p;
             }
             __syncwarp();
-            for (int it = lane; it < np * NT1 * NM2; it += 32) {
-                const int pi = it / (NT1 * NM2), r = it % (NT1 * NM2), h = r / NM2, m2 = r % NM2;
+            for (int x = lane; x < np * kg * NT1 * NM2; x += 32) {
+                const int pq = x / (NT1 * NM2), r = x % (NT1 * NM2), h = r / NM2, m2 = r % NM2;
+                const int pi = pq / kg, q = pq % kg;
                 const unsigned hm = TBra.hm[h];
-                const double *g = Gp + (hm & 0xff) * NM2P + m2, *s = S1 + pi * NS1 + (hm >> 12);
+                const double *g = Gp + q * Lay::MS + (hm & 0xff) * NM2P + m2, *s = S1 + pi * NS1 + (hm >> 12);
                 const int ns = (hm >> 8) & 0xf;
 #pragma unroll
                 for (int o = 0; o < NO; ++o) {
                     double f = 0.0;
                     for (int k = 0; k < ns; ++k) f += s[k] * g[(o * NM1 + k) * NM2P];
-                    F[((pi * NO + o) * NT1 + h) * NM2P + m2] = f;
+                    F[(pi * KQ + q) * Lay::FS + (o * NT1 + h) * NM2P + m2] = f;
                 }
             }
             __syncwarp();
-            const int ntot = np * nkp;
-            for (int j0 = 0; j0 < ntot; j0 += 32) {
+            const int ntot = np * nk, nmax = np * nkmax;
+            for (int it0 = 0; it0 < nmax; it0 += LG) {
                 // ---- this lane's primitive quartet
-                const int idx = min(j0 + lane, ntot - 1);
-                const int pi = idx / nkp;
-                const int ip = pb0 + ib0 + (blk + pi) * ibs, kp = pk0 + (idx - pi * nkp);
+                const int idx = max(min(it0 + sl, ntot - 1), 0);
+                const int pi = idx / nkd;
+                const int ip = pb0 + ib0 + (blk + pi) * ibs, kp = pk0 + (idx - pi * nkd);
                 const double p = P1[pi * NP1 + 3], q = pp.p[kp], zc = pp.za[kp];
                 const double oo2q = 0.5 / q, c = 2.0 * oo2q * zc, d = 2.0 * oo2q * (q - zc);
                 const double ir = rsqrt(p + q);
                 const double rho = p * q * ir * ir;
                 const double X = pp.Px[ip] - pp.Px[kp], Y = pp.Py[ip] - pp.Py[kp], Z = pp.Pz[ip] - pp.Pz[kp];
                 const double T0 = rho * (X * X + Y * Y + Z * Z);
-                // lanes past the end repeat the last quartet with weight zero
-                const double pref = j0 + lane < ntot ? P1[pi * NP1 + 2] * pp.K[kp] * (2.0 * oo2q) * ir : 0.0;
+                // lanes past the end repeat a quartet with weight zero
+                const double pref = it0 + sl < ntot ? P1[pi * NP1 + 2] * pp.K[kp] * (2.0 * oo2q) * ir : 0.0;
                 double s2[NS2];
                 pair_scalars<LC, LD, true>(oo2q, c, d, s2);
                 if constexpr (NIT > 0)
@@ -764,7 +853,7 @@ __device__ void quartet_herm(double *sm, int lane, const GeoArgs &geo, const Den
                             f *= m2r;
                         }
                     }
-                    const double *Fl = F + (pi * NO + o) * NT1 * NM2P;
+                    const double *Fl = F + (pi * KQ + kq) * Lay::FS + o * NT1 * NM2P;
                     double *Rl = Rr + lane;
                     if constexpr (Lay::RREG) {
                         double Xd[nherm(L)];
@@ -824,8 +913,12 @@ __device__ void quartet_herm(double *sm, int lane, const GeoArgs &geo, const Den
                     __syncwarp();
                     // ---- reverse sums U[h1][m2], added to V with the bra scalars
                     if constexpr (NIT > 0) {
-                        reverse_sums<LA, LB, LC, LD, false>(V + o * NM1 * NM2P, Rr, S2, S1, j0, min(32, ntot - j0), nkp,
-                                                            lane);
+                        if (kg == 1)
+                            reverse_sums<LA, LB, LC, LD, false>(V + o * NM1 * NM2P, Rr, S2, S1, it0, min(32, ntot - it0),
+                                                                nkd, lane);
+                        else if constexpr (KQ > 1)
+                            reverse_sums_group<LA, LB, LC, LD>(V + o * NM1 * NM2P, Lay::MS, Rr, S2, S1, it0, np, kg, LG,
+                                                               gi.nk + k0, lane);
                         __syncwarp();
                     }
                 }
@@ -843,22 +936,25 @@ __device__ void quartet_herm(double *sm, int lane, const GeoArgs &geo, const Den
         }
         // ---- polynomial parts: V with dG'/dR (ket half again) and dG'/dS (bra half)
         if constexpr (NIT > 0) {
-            entry_values<LA, LB>(vb, lane, pw);
-            entry_values<LC, LD>(vk, lane, pw + 15);
+            entry_values<LA, LB>(vb, lane, pw, 1);
+            if constexpr (Lay::L1 > 0) entry_values<LC, LD>(vk, lane, pw + 15, kg);
             __syncwarp();
             if constexpr (Lay::L1 > 0) {
-                half_ket<LA, LB, LC, LD>(half, G, vk, lane);
+                half_ket<LA, LB, LC, LD>(half, G, vk, lane, kg);
                 __syncwarp();
-                for (int it = lane; it < Lay::NE1; it += 32) {
+                for (int x = lane; x < kg * Lay::NE1; x += 32) {
+                    const int q = x / Lay::NE1, it = x % Lay::NE1;
                     const unsigned w = TBra.ent[it];
                     const int px = (w >> 16) & 7, py = (w >> 19) & 7, pz = (w >> 22) & 7;
                     if (px + py + pz == 0) continue;
                     const int m1 = TBra.own[it], ab = w & 0xff;
                     double s = 0.0;
 #pragma unroll
-                    for (int o = 0; o < NO; ++o)
-                        for (int m2 = 0; m2 < NM2; ++m2)
-                            s += half[(o * NM2 + m2) * NABP + ab] * V[(o * NM1 + m1) * NM2P + m2];
+                    for (int o = 0; o < NO; ++o) {
+                        const double *h = half + q * Lay::HS + o * NM2 * NABP + ab;
+                        const double *v = V + q * Lay::MS + (o * NM1 + m1) * NM2P;
+                        for (int m2 = 0; m2 < NM2; ++m2) s += h[m2 * NABP] * v[m2];
+                    }
                     s *= double((int)((w >> 8) & 0xff));
                     const double qx = pw[px], qy = pw[5 + py], qz = pw[10 + pz];
                     if (px) gA[0] += s * double(px) * pw[px - 1] * qy * qz;
@@ -868,30 +964,32 @@ __device__ void quartet_herm(double *sm, int lane, const GeoArgs &geo, const Den
                 __syncwarp();
             }
             if constexpr (Lay::L2 > 0) {
-                // bra half [m1][cd]
-                for (int it = lane; it < NM1 * NCD; it += 32) {
-                    const int m1 = it / NCD, cd = it % NCD;
+                // bra half [ket][o][m1][cd]
+                for (int x = lane; x < kg * NM1 * NCD; x += 32) {
+                    const int q = x / (NM1 * NCD), it = x % (NM1 * NCD), m1 = it / NCD, cd = it % NCD;
 #pragma unroll
                     for (int o = 0; o < NO; ++o) {
+                        const double *g = G + q * Lay::GS + (o * NCD + cd) * NABP;
                         double s = 0.0;
-                        for (int x = TBra.start[m1]; x < TBra.start[m1 + 1]; ++x)
-                            s += vb[x] * G[(o * NCD + cd) * NABP + (TBra.ent[x] & 0xff)];
-                        half[(o * NM1 + m1) * NCD + cd] = s;
+                        for (int k = TBra.start[m1]; k < TBra.start[m1 + 1]; ++k) s += vb[k] * g[TBra.ent[k] & 0xff];
+                        half[q * Lay::HS + (o * NM1 + m1) * NCD + cd] = s;
                     }
                 }
                 __syncwarp();
-                for (int it = lane; it < Lay::NE2; it += 32) {
+                const double *pk = pw + (1 + kq) * 15;
+                for (int it = sl; it < Lay::NE2; it += LG) {
                     const unsigned w = TKet.ent[it];
                     const int px = (w >> 16) & 7, py = (w >> 19) & 7, pz = (w >> 22) & 7;
                     if (px + py + pz == 0) continue;
                     const int m2 = TKet.own[it], cd = w & 0xff;
                     double s = 0.0;
 #pragma unroll
-                    for (int o = 0; o < NO; ++o)
-                        for (int m1 = 0; m1 < NM1; ++m1)
-                            s += half[(o * NM1 + m1) * NCD + cd] * V[(o * NM1 + m1) * NM2P + m2];
+                    for (int o = 0; o < NO; ++o) {
+                        const double *h = half + kq * Lay::HS + o * NM1 * NCD + cd;
+                        const double *v = V + kq * Lay::MS + o * NM1 * NM2P + m2;
+                        for (int m1 = 0; m1 < NM1; ++m1) s += h[m1 * NCD] * v[m1 * NM2P];
+                    }
                     s *= double((int)((w >> 8) & 0xff));
-                    const double *pk = pw + 15;
                     const double qx = pk[px], qy = pk[5 + py], qz = pk[10 + pz];
                     if (px) gC[0] += s * double(px) * pk[px - 1] * qy * qz;
                     if (py) gC[1] += s * double(py) * qx * pk[5 + py - 1] * qz;
@@ -905,53 +1003,63 @@ __device__ void quartet_herm(double *sm, int lane, const GeoArgs &geo, const Den
     for (int i = 0; i < 3; ++i) {
         acc[i] += aA[i] - 2.0 * pw[i * 5 + 1] * eA + gA[i];
         acc[3 + i] += aT[i];
-        acc[6 + i] += -aC[i] - 2.0 * pw[15 + i * 5 + 1] * eC + gC[i];
+        acc[6 + i] += -aC[i] - 2.0 * pw[(1 + kq) * 15 + i * 5 + 1] * eC + gC[i];
     }
 }
 
-// Warps of a CTA and resident CTAs the registers are limited to: 16 warps at
-// 128 registers up to L = 2, 12 at 168 for L = 3, 8 at 255 above.  One warp per
-// scheduler already covers most of the fp64 pipe; the second and third fill
-// the gaps left by the transforms' loads and by dependent steps.
+// Warps of a CTA and CTAs an SM the registers are limited to: 16 warps at 128
+// registers up to L = 2, 12 at 168 for L = 3, 8 at 255 above.  One warp per
+// scheduler already covers most of the fp64 pipe; the others fill the gaps left
+// by the transforms' loads and by dependent steps.  CTAs are small (one or two
+// warps) because a CTA gives its shared memory back only when its last warp
+// ends: with 8 to 16 warps a single long quartet kept a whole SM from the next
+// class's launch.
 template <int LA, int LB, int LC, int LD>
 struct HermOp {
     using Lay = HermLay<LA, LB, LC, LD>;
     static constexpr bool FP32 = false;
-    static constexpr int L = LA + LB + LC + LD;
-    static constexpr int max_warps = L == 3 ? 12 : 8;
-    static constexpr int min_ctas = L <= 2 ? 2 : 1;
-    static __device__ __forceinline__ void quartet(double *sm, int lane, const MolDesc &md, int sa, int sb, int sc,
-                                                   int sd, int pb0, int nbp, int ib0, int ibs, int pk0, int nkp,
-                                                   double scale, const double *boys, double (&acc)[9])
+    static constexpr int L = LA + LB + LC + LD, KQ = Lay::KQ;
+    static constexpr int cta_warps = L <= 3 ? 2 : 1, min_ctas = L == 3 ? 6 : 8;
+    // primitive quartets of a contracted one up to which ket pairs are grouped
+    // (kg times it stays below): the smaller the class, the more of a quartet's
+    // work is the density transform that a group shares
+    static constexpr int group_below = L == 0 ? 512 : (L == 1 ? 256 : (L == 2 ? 128 : 64));
+    static __device__ __forceinline__ void group(double *sm, int lane, int k0, int kg, const GroupInfo &gi,
+                                                 const MolDesc &md, int sa, int sb, int pb0, int nbp, int ib0, int ibs, const double *boys,
+                                                 double (&acc)[9])
     {
-        quartet_herm<LA, LB, LC, LD>(sm, lane, md.geo, md.den, md.pp, sa, sb, sc, sd,
-                                     pb0, nbp, ib0, ibs, pk0, nkp, scale, boys, acc);
+        group_herm<LA, LB, LC, LD>(sm, lane, k0, kg, gi, md.geo, md.den, md.pp, sa, sb, pb0, nbp, ib0, ibs, boys, acc);
     }
 };
 
 // Persistent class kernel; every warp works alone.  Warp w of W takes the
 // units (tile, chunk of cl.nchunk per tile, split) w, 2W - 1 - w, 2W + w, ...:
 // the tile list is in decreasing cost, so the alternating order evens the
-// sums out.  A quartet's 12 components are added to the warp's own gradient
-// (shared memory, or with out.use_smem = 0 the warp's slab), so the schedule
-// and the order of all sums are fixed and results are bitwise reproducible.
+// sums out.  A unit's quartets are taken in groups of up to KQ ket pairs of one
+// bra pair.  Their components are added to the warp's own gradient (shared
+// memory, or with out.use_smem = 0 the warp's slab), so the schedule and the
+// order of all sums are fixed and results are bitwise reproducible.
 template <class Op>
-__global__ void __launch_bounds__(32 * Op::max_warps, Op::min_ctas)
+__global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
     k_grad_lanes(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out, const double *__restrict__ boys)
 {
     using Lay = typename Op::Lay;
+    constexpr int RS = Lay::RS, KQ = Op::KQ;
     extern __shared__ double smem[];
+    __shared__ GroupInfo ginfo[Op::cta_warps];
     const int nw = blockDim.x / 32, grp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int n3 = out.natom_total * 3;
     double *wsm = smem + (size_t)grp * Lay::TOTAL;
+    GroupInfo &gi = ginfo[grp];
     double *grad = out.use_smem ? smem + (size_t)nw * Lay::TOTAL + (size_t)grp * n3
                                 : out.partials + (size_t)(blockIdx.x * nw + grp) * n3;
     if (out.use_smem) {
         for (int k = lane; k < n3; k += 32) grad[k] = 0.0;
         __syncwarp();
     }
-    unsigned long long nq = 0, npq = 0, nbv = 0;
+    unsigned long long nq = 0, npq = 0, nbv = 0;  // of this lane's ket pair
     const int S = cl.nsplit, C = cl.nchunk, QPC = TILE / C;
+    const int KG = out.dump ? 1 : (QPC < KQ ? QPC : KQ);
     const bool same = cl.P == cl.Q;
     const long long units = cl.ntiles * C * S, W = (long long)gridDim.x * nw;
     // neighbouring warps sit on different CTAs, so a short list spreads over the SMs
@@ -964,11 +1072,11 @@ __global__ void __launch_bounds__(32 * Op::max_warps, Op::min_ctas)
         const uint4 tl = cl.tiles[tile * cl.stride];
         const MolDesc &md = mols[tl.x];
         const PairSet &bra = md.sets[cl.P], &ket = md.sets[cl.Q];
-        for (int qi = chunk * QPC; qi < (chunk + 1) * QPC; ++qi) {
+        for (int qi = chunk * QPC; qi < (chunk + 1) * QPC; qi += KG) {
             const int bi = tl.y * TB + qi / TK;
-            const int ki = tl.z * TK + qi % TK;
-            double g = 0.0;
-            bool ok = bi < bra.n && ki < ket.n && (!same || bi >= ki);
+            // lane k < KG: ket pair k of the group
+            const int ki = tl.z * TK + qi % TK + lane;
+            bool ok = lane < KG && bi < bra.n && ki < ket.n && (!same || bi >= ki);
             if (ok) ok = split < bra.np[bi];
             int sa = 0, sb = 0, sc = 0, sd = 0;
             if (ok) {
@@ -978,47 +1086,92 @@ __global__ void __launch_bounds__(32 * Op::max_warps, Op::min_ctas)
                 sd = ket.sb[ki];
                 ok = keep_quartet(md.scr, bra, ket, bi, ki, sa, sb, sc, sd);
             }
-            if (ok) {  // uniform across the warp
-                double scale = 1.0;
-                if (sa == sb) scale *= 0.5;
-                if (sc == sd) scale *= 0.5;
-                if (same && bi == ki) scale *= 0.5;
-                const int nbp = bra.np[bi], nkp = ket.np[ki];
-                double acc[9];
-#pragma unroll
-                for (int k = 0; k < 9; ++k) acc[k] = 0.0;
-                if (nkp > 0)
-                    Op::quartet(wsm, lane, md, sa, sb, sc, sd, bra.poff[bi], nbp, split, S, ket.poff[ki], nkp, scale,
-                                boys, acc);
-                // the nine sums over the warp through shared memory: three lanes a sum
-                double *red = wsm + Lay::o_X;
-                __syncwarp();
-#pragma unroll
-                for (int k = 0; k < 9; ++k) red[k * Lay::RS + lane] = acc[k];
-                __syncwarp();
-                double s = 0.0;
-                const int k = lane / 3 < 9 ? lane / 3 : 8, part = lane % 3;
-                for (int j = part; j < 32; j += 3) s += red[k * Lay::RS + j];
-                const double s1 = __shfl_down_sync(0xffffffffu, s, 1), s2 = __shfl_down_sync(0xffffffffu, s, 2);
-                s = s + s1 + s2;  // valid on lanes 3k
-                const int X = lane / 3, i = lane % 3;  // lanes 0..11: output component X * 3 + i
-                const double dA = __shfl_sync(0xffffffffu, s, 3 * i), dT = __shfl_sync(0xffffffffu, s, 3 * (3 + i));
-                const double dC = __shfl_sync(0xffffffffu, s, 3 * (6 + i));
-                g = X == 0 ? dA : (X == 1 ? dT - dA : (X == 2 ? dC : -dT - dC));
-                if (!out.dump && lane < 3) {  // lane i owns component i of every atom
-                    const int *at = md.geo.sh_atom;
-                    double *gi = grad + md.atom_off * 3 + lane;
-                    gi[at[sa] * 3] += dA;
-                    gi[at[sb] * 3] += dT - dA;
-                    gi[at[sc] * 3] += dC;
-                    gi[at[sd] * 3] += -dT - dC;
+            if (ok) {
+                const int nbs = (bra.np[bi] - split + S - 1) / S;
+                if (split == 0) nq += 1;
+                npq += (unsigned long long)nbs * ket.np[ki];
+                nbv += (unsigned long long)nbs;
+                ok = ket.np[ki] > 0;  // all screened: counted, nothing to add
+            }
+            const unsigned mask = __ballot_sync(0xffffffffu, ok);
+            double g = 0.0;
+            if (mask) {
+                const int n = __popc(mask), first = __ffs(mask) - 1;
+                sa = __shfl_sync(0xffffffffu, sa, first);
+                sb = __shfl_sync(0xffffffffu, sb, first);
+                const int nbp = bra.np[bi], nbs = (nbp - split + S - 1) / S;
+                if (ok) {
+                    const int k = __popc(mask & ((1u << lane) - 1));
+                    double scale = 1.0;
+                    if (sa == sb) scale *= 0.5;
+                    if (sc == sd) scale *= 0.5;
+                    if (same && bi == ki) scale *= 0.5;
+                    gi.sc[k] = sc;
+                    gi.sd[k] = sd;
+                    gi.pk0[k] = ket.poff[ki];
+                    gi.nk[k] = ket.np[ki];
+                    gi.scale[k] = scale;
+                    if (k == 0) {
+                        gi.n = n;
+                        for (int j = n; j < GroupInfo::CAP; ++j) gi.nk[j] = 0, gi.pk0[j] = ket.poff[ki];
+                    }
                 }
                 __syncwarp();
-                if (lane == 0) {
-                    if (split == 0) nq += 1;
-                    npq += (unsigned long long)((nbp - split + S - 1) / S) * nkp;
-                    nbv += (unsigned long long)((nbp - split + S - 1) / S);
+                int kg = 1;
+                if (KQ > 1) {
+                    int nkmax = gi.nk[0];
+                    for (int k = 1; k < n; ++k) nkmax = max(nkmax, gi.nk[k]);
+                    while (kg < n && 2 * kg <= KQ && 2 * kg * nbs * nkmax <= Op::group_below) kg *= 2;
                 }
+                for (int k0 = 0; k0 < n; k0 += kg) {
+                    double acc[9];
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) acc[k] = 0.0;
+                    Op::group(wsm, lane, k0, kg, gi, md, sa, sb, bra.poff[bi], nbp, split, S, boys, acc);
+                    // the nine sums of every ket pair over its 32 / kg lanes, through shared memory
+                    double *red = wsm + Lay::o_X;
+                    __syncwarp();
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) red[k * RS + lane] = acc[k];
+                    __syncwarp();
+                    if (kg == 1) {  // three lanes a sum
+                        double s = 0.0;
+                        const int k = lane / 3 < 9 ? lane / 3 : 8, part = lane % 3;
+                        for (int j = part; j < 32; j += 3) s += red[k * RS + j];
+                        const double s1 = __shfl_down_sync(0xffffffffu, s, 1), s2 = __shfl_down_sync(0xffffffffu, s, 2);
+                        if (part == 0 && lane < 27) red[k * RS] = s + s1 + s2;
+                    } else {
+                        const int lg = 32 / kg;
+                        for (int x = lane; x < 9 * kg; x += 32) {
+                            double *p = red + (x % 9) * RS + x / 9 * lg;
+                            double s = p[0];
+                            for (int j = 1; j < lg; ++j) s += p[j];
+                            p[0] = s;
+                        }
+                    }
+                    __syncwarp();
+                    const int i = lane % 3, lg = 32 / kg;
+                    if (out.dump) {  // one ket pair; lanes 0..11: output component X * 3 + i
+                        const int X = lane / 3;
+                        const double dA = red[i * RS], dT = red[(3 + i) * RS], dC = red[(6 + i) * RS];
+                        g = X == 0 ? dA : (X == 1 ? dT - dA : (X == 2 ? dC : -dT - dC));
+                    } else if (lane < 3) {  // lane i owns component i of every atom
+                        const int *at = md.geo.sh_atom;
+                        double *gr = grad + md.atom_off * 3 + i;
+                        double dA = 0.0, dT = 0.0;
+                        for (int k = 0; k < kg && k0 + k < n; ++k) {
+                            const double t = red[(3 + i) * RS + k * lg], c = red[(6 + i) * RS + k * lg];
+                            gr[at[gi.sc[k0 + k]] * 3] += c;
+                            gr[at[gi.sd[k0 + k]] * 3] += -t - c;
+                            dT += t;
+                        }
+                        for (int k = 0; k < kg; ++k) dA += red[i * RS + k * lg];
+                        gr[at[sa] * 3] += dA;
+                        gr[at[sb] * 3] += dT - dA;
+                    }
+                    __syncwarp();
+                }
+                __syncwarp();
             }
             if (out.dump && lane < 12) out.dump[((size_t)tile * TILE + qi) * 12 + lane] = g;
         }
@@ -1033,6 +1186,12 @@ __global__ void __launch_bounds__(32 * Op::max_warps, Op::min_ctas)
             slab[k] += s;
         }
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        nq += __shfl_xor_sync(0xffffffffu, nq, o);
+        npq += __shfl_xor_sync(0xffffffffu, npq, o);
+        nbv += __shfl_xor_sync(0xffffffffu, nbv, o);
+    }
     if (lane == 0 && (nq || npq)) {  // a split unit may hold primitives only
         atomicAdd(out.counters + 0, nq);
         atomicAdd(out.counters + (Op::FP32 ? 3 : 1), npq);
@@ -1041,18 +1200,19 @@ __global__ void __launch_bounds__(32 * Op::max_warps, Op::min_ctas)
     }
 }
 
-// Shared memory a CTA may take (227 KB), and an SM's (228 KB with 1 KB per CTA).
-constexpr size_t kCtaSmem = 227 * 1024;
+// Dynamic shared memory a CTA may take beside the static group records.
+constexpr size_t kCtaSmem = 223 * 1024;
 
 // Launch of a kernel over warp units (tile, chunk, split) with at most gmax
-// CTAs of nw warps.  Tiles are cut into chunks down to single quartets until
-// every warp has 32 units (with 4, the heaviest unit alone left (pp|pp) SMs
-// idle 57 % of the time on a 1/16 shard of the 32-atom workload), then along
-// the bra primitive pairs (which repeats the density transform) while warps
-// have fewer than 4.
+// CTAs of nw warps, whose warps take groups of up to kets ket pairs.  Tiles are
+// cut into chunks of whole groups until every warp has 32 units (with 4, the
+// heaviest units left (pp|pp) SMs idle 57 % of the time on a 1/16 shard of the
+// 32-atom workload; 8 instead of 32 cost the fp32 lists of a 1/8 shard 7 %),
+// into smaller ones while it has fewer than 4, down to single quartets, and
+// then along the bra primitive pairs (which repeats the density transform).
 template <typename K>
-cudaError_t launch_warp_units(K kern, int nw, size_t per_warp, long long gmax, cudaStream_t st, const MolDesc *mols,
-                              ClassLaunch cl, const OutArgs &out, const double *boys)
+cudaError_t launch_warp_units(K kern, int nw, size_t per_warp, int kets, long long gmax, cudaStream_t st,
+                              const MolDesc *mols, ClassLaunch cl, const OutArgs &out, const double *boys)
 {
     int dev = 0, nsm = 1, per = 1;
     cudaError_t e;
@@ -1065,9 +1225,10 @@ cudaError_t launch_warp_units(K kern, int nw, size_t per_warp, long long gmax, c
     cl.nchunk = 1;
     cl.nsplit = 1;
     const long long warps = gmax * nw;
-    while (cl.ntiles * cl.nchunk < 32 * warps && cl.nchunk < TILE) cl.nchunk *= 2;
+    while (cl.ntiles * cl.nchunk < 32 * warps && cl.nchunk * kets < TILE) cl.nchunk *= 2;
+    while (cl.ntiles * cl.nchunk < 4 * warps && cl.nchunk < TILE) cl.nchunk *= 2;
     if (!out.dump) {
-        while (cl.ntiles * cl.nchunk * cl.nsplit < 4 * warps && cl.nsplit < 8) ++cl.nsplit;
+        while (cl.ntiles * cl.nchunk * cl.nsplit < 4 * warps && cl.nsplit < 32) ++cl.nsplit;
         if (cl.split_req > 0) cl.nsplit = cl.split_req;
     }
     const long long units = cl.ntiles * cl.nchunk * cl.nsplit;
@@ -1078,8 +1239,8 @@ cudaError_t launch_warp_units(K kern, int nw, size_t per_warp, long long gmax, c
 }
 
 // Launch of a gradient kernel with at most gcap slabs of partial gradients.
-// Each warp's gradient lies beside its arrays while that leaves four warps (or
-// what fits without), else every warp adds to a slab of its own.
+// Each warp's gradient lies beside its arrays while that leaves an SM four warps
+// (or what fits without), else every warp adds to a slab of its own.
 template <class Op>
 cudaError_t launch_lanes(int gcap, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl, const OutArgs &out,
                          const double *boys)
@@ -1090,11 +1251,9 @@ cudaError_t launch_lanes(int gcap, cudaStream_t st, const MolDesc *mols, const C
     const size_t grad = sizeof(double) * 3 * (size_t)o.natom_total;
     const int fit = (int)(kCtaSmem / bytes), fit_g = (int)(kCtaSmem / (bytes + grad));
     o.use_smem = fit_g >= (fit < 4 ? fit : 4);
-    int nw = o.use_smem ? fit_g : fit;
-    if (nw > Op::max_warps) nw = Op::max_warps;
-    if (nw > gcap && !o.use_smem) nw = gcap;
-    return launch_warp_units(k_grad_lanes<Op>, nw, bytes + (o.use_smem ? grad : 0), o.use_smem ? gcap : gcap / nw, st,
-                             mols, cl, o, boys);
+    const int have = o.use_smem ? fit_g : fit, nw = have < Op::cta_warps ? have : Op::cta_warps;
+    return launch_warp_units(k_grad_lanes<Op>, nw, bytes + (o.use_smem ? grad : 0), Op::KQ,
+                             o.use_smem ? gcap : (gcap > nw ? gcap / nw : 1), st, mols, cl, o, boys);
 }
 
 }  // namespace tg

@@ -361,14 +361,14 @@ struct Lane32Op {
     using Lay = Lane32Lay<LA, LB, LC, LD>;
     static constexpr bool FP32 = true;
     static constexpr int L = LA + LB + LC + LD;
-    static constexpr int max_warps = L == 3 ? 12 : 8;
-    static constexpr int min_ctas = L <= 2 ? 2 : 1;
-    static __device__ __forceinline__ void quartet(double *sm, int lane, const MolDesc &md, int sa, int sb, int sc,
-                                                   int sd, int pb0, int nbp, int ib0, int ibs, int pk0, int nkp,
-                                                   double scale, const double *boys, double (&acc)[9])
+    static constexpr int KQ = 1, cta_warps = L <= 3 ? 2 : 1, min_ctas = L == 3 ? 6 : 8;
+    static constexpr int group_below = 0;
+    static __device__ __forceinline__ void group(double *sm, int lane, int k0, int, const GroupInfo &gi, const MolDesc &md,
+                                                 int sa, int sb, int pb0, int nbp, int ib0, int ibs, const double *boys,
+                                                 double (&acc)[9])
     {
-        quartet_lane32<LA, LB, LC, LD>(sm, lane, md.geo, md.den, md.pp, sa, sb, sc, sd, pb0, nbp, ib0, ibs, pk0, nkp,
-                                       scale, boys, acc);
+        quartet_lane32<LA, LB, LC, LD>(sm, lane, md.geo, md.den, md.pp, sa, sb, gi.sc[k0], gi.sd[k0], pb0, nbp, ib0, ibs,
+                                       gi.pk0[k0], gi.nk[k0], gi.scale[k0], boys, acc);
     }
 };
 
