@@ -598,7 +598,7 @@ int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &op
                 ntl_max += (long long)((pl.cls[P].size() + TB - 1) / TB) * ((pl.cls[Qc].size() + TK - 1) / TK);
         const size_t ntl = host_tiles ? (size_t)std::max<long long>(ntl_max, 1) : 1;
         const size_t need2 = 6 * al(sizeof(int) * np_k) + 2 * al(sizeof(double) * np_k) +
-                             6 * al(sizeof(double) * npp) + 12 * al(sizeof(float) * npp) + al(sizeof(uint4) * ntl) +
+                             10 * al(sizeof(double) * npp) + 12 * al(sizeof(float) * npp) + al(sizeof(uint4) * ntl) +
                              al(sizeof(MolDesc)) +
                              al(sizeof(TileRef) * ntl) + al(sizeof(float) * ntl * (NFEAT + 1)) +
                              al(sizeof(double) * (size_t)kSlabSets * pl.G * 3 * natom) + 8192;
@@ -717,7 +717,9 @@ int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &op
     DevArena &V = b->ws2;
     const size_t npp = (size_t)std::max<long long>(pl.nprimpairs, 1);
     double *pp_p = V.take<double>(npp), *pp_x = V.take<double>(npp), *pp_y = V.take<double>(npp),
-           *pp_z = V.take<double>(npp), *pp_K = V.take<double>(npp), *pp_za = V.take<double>(npp);
+           *pp_z = V.take<double>(npp), *pp_K = V.take<double>(npp), *pp_za = V.take<double>(npp),
+           *pp_oo2 = V.take<double>(npp), *pp_fa = V.take<double>(npp), *pp_fb = V.take<double>(npp),
+           *pp_kop = V.take<double>(npp);
     float *fp_p = V.take<float>(npp), *fp_x = V.take<float>(npp), *fp_y = V.take<float>(npp),
           *fp_z = V.take<float>(npp), *fp_K = V.take<float>(npp), *fp_za = V.take<float>(npp);
     float *fp_PA = V.take<float>(3 * npp), *fp_PB = V.take<float>(3 * npp);
@@ -732,8 +734,8 @@ int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &op
         TG_CUDA(cudaMemcpyAsync(pl.d_Qd, h_Qd.data(), sizeof(double) * nk, cudaMemcpyHostToDevice, st));
         k_prim_pairs<<<(unsigned)((nk + 127) / 128), 128, 0, st>>>(
             (int)nk, pl.d_sa, pl.d_sb, pl.d_poff, pl.d_key, b->d_xyz, b->d_sh_atom, b->d_sh_nprim, b->d_sh_poff,
-            b->d_exps, b->d_cn, b->d_bpoff, b->d_bp, scale, qq, Mp, eps_p, pp_p, pp_x, pp_y, pp_z, pp_K, pp_za, fp_p,
-            fp_x, fp_y, fp_z, fp_K, fp_za, fp_PA, fp_PB, (long long)npp);
+            b->d_exps, b->d_cn, b->d_bpoff, b->d_bp, scale, qq, Mp, eps_p, pp_p, pp_x, pp_y, pp_z, pp_K, pp_za,
+            pp_oo2, pp_fa, pp_fb, pp_kop, fp_p, fp_x, fp_y, fp_z, fp_K, fp_za, fp_PA, fp_PB, (long long)npp);
         ++pl.launches;
         TG_CUDA(cudaGetLastError());
         // the host pair vectors must outlive the asynchronous copies
@@ -745,6 +747,10 @@ int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &op
     pl.pp.Pz = pp_z;
     pl.pp.K = pp_K;
     pl.pp.za = pp_za;
+    pl.pp.oo2 = pp_oo2;
+    pl.pp.fa = pp_fa;
+    pl.pp.fb = pp_fb;
+    pl.pp.kop = pp_kop;
     pl.pp.fp = fp_p;
     pl.pp.fPx = fp_x;
     pl.pp.fPy = fp_y;

@@ -36,7 +36,7 @@ struct FockLay {
     static constexpr int o_I = 0;                            // [2][NAB][NCD]
     static constexpr int o_V = o_I + 2 * NAB * NCD;          // [NO][NM1][NM2P]
     static constexpr int o_S1 = o_V + NO * NM1 * NM2P;       // [PB][NS1]
-    static constexpr int o_P1 = o_S1 + PB * NS1;             // [PB][NP1]: p, 4 pi^(5/2) K / 2p
+    static constexpr int o_P1 = o_S1 + PB * NS1;             // [PB][NP1]: p, 2 pi^(5/2) K / p
     static constexpr int o_pw = o_P1 + PB * NP1;             // [2][3][5] powers of R and S
     static constexpr int o_X = o_pw + 30;
     static constexpr int TOTAL = (o_X + (HALF > ROWS ? HALF : ROWS) + 1) & ~1;
@@ -100,13 +100,12 @@ __device__ void quartet_fock_ints(double *sm, int lane, const GeoArgs &geo, cons
             const int np = min(pb, nbra - blk);
             if (lane < np) {
                 const int ip = pb0 + ib0 + (blk + lane) * ibs;
-                const double p = pp.p[ip], za = pp.za[ip], oo2 = 0.5 / p;
                 double s[NS1];
-                pair_scalars<LA, LB, false>(oo2, 2.0 * oo2 * za, 2.0 * oo2 * (p - za), s);
+                pair_scalars<LA, LB, false>(pp.oo2[ip], pp.fa[ip], pp.fb[ip], s);
 #pragma unroll
                 for (int k = 0; k < NS1; ++k) S1[lane * NS1 + k] = s[k];
-                P1[lane * NP1] = p;
-                P1[lane * NP1 + 1] = pp.K[ip] * oo2 * 69.97367331049945;
+                P1[lane * NP1] = pp.p[ip];
+                P1[lane * NP1 + 1] = pp.kop[ip] * 34.986836655249725;
             }
             __syncwarp();
             const int ntot = np * nkp;
@@ -114,14 +113,14 @@ __device__ void quartet_fock_ints(double *sm, int lane, const GeoArgs &geo, cons
                 const int idx = min(j0 + lane, ntot - 1);
                 const int pi = idx / nkp;
                 const int ip = pb0 + ib0 + (blk + pi) * ibs, kp = pk0 + (idx - pi * nkp);
-                const double p = P1[pi * NP1], q = pp.p[kp], zc = pp.za[kp], oo2q = 0.5 / q;
+                const double p = P1[pi * NP1], q = pp.p[kp];
                 const double ir = rsqrt(p + q), rho = p * q * ir * ir;
                 const double X = pp.Px[ip] - pp.Px[kp], Y = pp.Py[ip] - pp.Py[kp], Z = pp.Pz[ip] - pp.Pz[kp];
                 const double T0 = rho * (X * X + Y * Y + Z * Z);
-                const double pref = j0 + lane < ntot ? P1[pi * NP1 + 1] * pp.K[kp] * (2.0 * oo2q) * ir : 0.0;
+                const double pref = j0 + lane < ntot ? P1[pi * NP1 + 1] * pp.kop[kp] * ir : 0.0;
                 {
                     double s2[NS2];
-                    pair_scalars<LC, LD, true>(oo2q, 2.0 * oo2q * zc, 2.0 * oo2q * (q - zc), s2);
+                    pair_scalars<LC, LD, true>(pp.oo2[kp], pp.fa[kp], pp.fb[kp], s2);
 #pragma unroll
                     for (int k = 0; k < NS2; ++k) S2[k * RS + lane] = s2[k];
                 }

@@ -212,7 +212,9 @@ struct HermLayK {
     // registers, from L = 7 (120 entries) in passes over ranges of Hermite
     // orders, which need R's top order stored too.
     static constexpr bool RREG = LM <= 5, PASSES = L >= 7;
-    static constexpr int NRH = nherm(PASSES ? LM : L);  // Hermite rows
+    // Hermite rows: the reverse sums reach order L - 1 (their items leave out the
+    // top order of both sides at once), the recursion in rows needs L
+    static constexpr int NRH = nherm(PASSES ? LM : (RREG ? L - 1 : L));
     static constexpr int NO = (NAB * NCD <= 27) ? 2 : 1;
     // bra primitive pairs of a block: a budget of 1200 doubles for F, 1 to 16
     // (700 buys (dp|pp) a sixth warp, but its half-filled passes cost more:
@@ -225,7 +227,7 @@ struct HermLayK {
     // the transforms' half-way arrays share the space of the R rows
     static constexpr int HALF = NE1 + KQ * (NE2 + HS), ROWS = (NRH + NS2) * RS, RED = 9 * RS;
     static constexpr int SHARED = HALF > ROWS ? (HALF > RED ? HALF : RED) : (ROWS > RED ? ROWS : RED);
-    static constexpr int NP1 = 4;                     // per bra primitive pair: a^, mu, 4 pi^(5/2) K / 2p, p
+    static constexpr int NP1 = 4;                     // per bra primitive pair: a^, mu, 2 pi^(5/2) K / p, p
     static constexpr int o_G = 0;                              // [KQ][NO][NCD][NABP]
     static constexpr int o_Gp = o_G + KQ * GS;                 // [KQ][NO][NM1][NM2P]
     static constexpr int o_V = o_Gp + KQ * MS;                 // [KQ][NO][NM1][NM2P]
@@ -321,15 +323,15 @@ constexpr HermItems<LA, LB, LC, LD, ALL> make_herm_items()
 
 // ------------------------------------------------------------ lane pieces
 
-// F_m(T), m = 0..M, one argument per lane.  T < 36: F_M and F_{M+1} by the
+// F_m(T), m = 0..M, one argument per lane.  T < 64: F_M and F_{M+1} by the
 // Taylor step of the table (shared d/k factors), e^-T = (2M+1) F_M - 2T F_{M+1}
 // (error below eps (2M+1) F_M, which the next order up divides by 2M-1), then
-// downward recursion: no exponential.  T >= 36: upward recursion, with e^-T
-// only below 64 (beyond, it is under 1e-14 of the smallest order's term).
+// downward recursion: no exponential.  T >= 64: upward recursion without e^-T,
+// which is under 1e-14 of the smallest order's term there.
 template <int M>
 __device__ __forceinline__ void boys_lane(double T, double (&F)[M + 1], const double *__restrict__ tab)
 {
-    if (T < BOYS_TMAX) {
+    if (T < BOYS_TFAR) {
         const int i = __double2int_rn(T * (1.0 / BOYS_H));
         const double d = i * BOYS_H - T;
         const double *row = tab + i * (BOYS_M + 1) + M;
@@ -347,10 +349,9 @@ __device__ __forceinline__ void boys_lane(double T, double (&F)[M + 1], const do
         for (int m = M - 1; m >= 0; --m) F[m] = (t2 * F[m + 1] + et) * (1.0 / (2 * m + 1));
     } else {
         const double is = rsqrt(T), h = 0.5 * is * is;
-        const double et = T < 64.0 ? exp(-T) : 0.0;
         F[0] = 0.88622692545275801365 * is;
 #pragma unroll
-        for (int m = 0; m < M; ++m) F[m + 1] = ((2 * m + 1) * F[m] - et) * h;
+        for (int m = 0; m < M; ++m) F[m + 1] = (2 * m + 1) * h * F[m];
     }
 }
 
@@ -789,16 +790,15 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
             // ---- scalars of the block's bra primitive pairs, then F[p][ket][h1][m2]
             if (lane < np) {
                 const int ip = pb0 + ib0 + (blk + lane) * ibs;
-                const double p = pp.p[ip], za = pp.za[ip], oo2 = 0.5 / p;
-                const double a = 2.0 * oo2 * za, b = 2.0 * oo2 * (p - za);
+                const double a = pp.fa[ip], b = pp.fb[ip];
                 double s[NS1];
-                pair_scalars<LA, LB, false>(oo2, a, b, s);
+                pair_scalars<LA, LB, false>(pp.oo2[ip], a, b, s);
 #pragma unroll
                 for (int k = 0; k < NS1; ++k) S1[lane * NS1 + k] = s[k];
                 P1[lane * NP1] = a;
-                P1[lane * NP1 + 1] = za * b;
-                P1[lane * NP1 + 2] = pp.K[ip] * oo2 * 69.97367331049945;  // 4 pi^(5/2) K / 2p
-                P1[lane * NP1 + 3] = p;
+                P1[lane * NP1 + 1] = pp.za[ip] * b;
+                P1[lane * NP1 + 2] = pp.kop[ip] * 34.986836655249725;  // 2 pi^(5/2) K / p
+                P1[lane * NP1 + 3] = pp.p[ip];
             }
             __syncwarp();
             for (int x = lane; x < np * kg * NT1 * NM2; x += 32) {
@@ -821,16 +821,15 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                 const int idx = max(min(it0 + sl, ntot - 1), 0);
                 const int pi = idx / nkd;
                 const int ip = pb0 + ib0 + (blk + pi) * ibs, kp = pk0 + (idx - pi * nkd);
-                const double p = P1[pi * NP1 + 3], q = pp.p[kp], zc = pp.za[kp];
-                const double oo2q = 0.5 / q, c = 2.0 * oo2q * zc, d = 2.0 * oo2q * (q - zc);
+                const double p = P1[pi * NP1 + 3], q = pp.p[kp], c = pp.fa[kp], d = pp.fb[kp];
                 const double ir = rsqrt(p + q);
                 const double rho = p * q * ir * ir;
                 const double X = pp.Px[ip] - pp.Px[kp], Y = pp.Py[ip] - pp.Py[kp], Z = pp.Pz[ip] - pp.Pz[kp];
                 const double T0 = rho * (X * X + Y * Y + Z * Z);
                 // lanes past the end repeat a quartet with weight zero
-                const double pref = it0 + sl < ntot ? P1[pi * NP1 + 2] * pp.K[kp] * (2.0 * oo2q) * ir : 0.0;
+                const double pref = it0 + sl < ntot ? P1[pi * NP1 + 2] * pp.kop[kp] * ir : 0.0;
                 double s2[NS2];
-                pair_scalars<LC, LD, true>(oo2q, c, d, s2);
+                pair_scalars<LC, LD, true>(pp.oo2[kp], c, d, s2);
                 if constexpr (NIT > 0)
 #pragma unroll
                     for (int k = 0; k < NS2; ++k) S2[k * RS + lane] = s2[k];
@@ -865,7 +864,7 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                         });
                         if constexpr (NIT > 0)
 #pragma unroll
-                            for (int h = 0; h < nherm(L); ++h) Rl[h * RS] = R[h];
+                            for (int h = 0; h < Lay::NRH; ++h) Rl[h * RS] = R[h];
                     } else if constexpr (!Lay::PASSES) {
                         double Xd[nherm(L)];
                         hermite_density<LA, LB, LC, LD, 0, L>(Fl, s2, Xd);
@@ -930,7 +929,7 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                     aC[i] += c * T[i];
                 }
                 eA += P1[pi * NP1 + 1] * e;
-                eC += zc * d * e;
+                eC += pp.za[kp] * d * e;
             }
             __syncwarp();  // S1, P1 and F are rewritten for the next block
         }

@@ -276,12 +276,14 @@ __global__ void k_prim_count(int npairs, const int *psa, const int *psb, const i
     np_out[ip] = n;
 }
 
-// Primitive-pair records: p, P, K = c_a c_b exp(-za zb/p |AB|^2), za.
+// Primitive-pair records: p, P, K = c_a c_b exp(-za zb/p |AB|^2), za, and the
+// quotients by p.
 __global__ void k_prim_pairs(int npairs, const int *psa, const int *psb, const int *poff, const int *key,
                              const double *xyz, const int *sh_atom, const int *sh_nprim, const int *sh_poff,
                              const double *exps, const double *cn, const long long *bpoff, const double *bp,
                              double scale, double qq, double mmax, double eps_p, double *p_, double *Px, double *Py,
-                             double *Pz, double *K, double *za_, float *fp, float *fPx, float *fPy, float *fPz,
+                             double *Pz, double *K, double *za_, double *oo2_, double *fa_, double *fb_,
+                             double *kop_, float *fp, float *fPx, float *fPy, float *fPz,
                              float *fK, float *fza, float *fPA, float *fPB, long long nrec)
 {
     const int ip = blockIdx.x * blockDim.x + threadIdx.x;
@@ -307,6 +309,10 @@ __global__ void k_prim_pairs(int npairs, const int *psa, const int *psb, const i
             Pz[o] = pz;
             K[o] = k;
             za_[o] = za;
+            oo2_[o] = 0.5 / p;
+            fa_[o] = za / p;
+            fb_[o] = zb / p;
+            kop_[o] = k / p;
             fp[o] = (float)p;
             fPx[o] = (float)px;
             fPy[o] = (float)py;

@@ -19,7 +19,8 @@ __global__ void k_prim_pairs(int npairs, const int *psa, const int *psb, const i
                              const double *xyz, const int *sh_atom, const int *sh_nprim, const int *sh_poff,
                              const double *exps, const double *cn, const long long *bpoff, const double *bp,
                              double scale, double qq, double mmax, double eps_p, double *p_, double *Px, double *Py,
-                             double *Pz, double *K, double *za_, float *fp, float *fPx, float *fPy, float *fPz,
+                             double *Pz, double *K, double *za_, double *oo2_, double *fa_, double *fb_,
+                             double *kop_, float *fp, float *fPx, float *fPy, float *fPz,
                              float *fK, float *fza, float *fPA, float *fPB, long long nrec);
 __global__ void k_symm(int nbf, const double *A, double *S);
 __global__ void k_fock_combine(int nbf, DensArgs den, double *SJ, double *BK, double *BL);

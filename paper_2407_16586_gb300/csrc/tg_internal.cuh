@@ -18,11 +18,14 @@ constexpr int TILE = TB * TK;
 // pairs visited (one per quartet and bra primitive pair of a unit)
 constexpr int NCNT = 6;
 
-// Boys table: F_m(T0) on T0 = 0, 0.05, ..., 36 for m = 0..BOYS_M.
+// Boys table: F_m(T0) on T0 = 0, 0.05, ..., 64 for m = 0..BOYS_M.  Most readers
+// take it up to BOYS_TMAX = 36; the fp64 lane kernels up to BOYS_TFAR, where
+// e^-T no longer enters the upward recursion (an exponential costs a warp more
+// fp64 instructions than the whole Taylor step).
 constexpr int BOYS_M = 16;
-constexpr int BOYS_NG = 721;
+constexpr int BOYS_NG = 1281;
 constexpr double BOYS_H = 0.05;
-constexpr double BOYS_TMAX = 36.0;
+constexpr double BOYS_TMAX = 36.0, BOYS_TFAR = 64.0;
 constexpr int BOYS_TAYLOR = 6;
 // the fp32 copy of the table follows the fp64 one in the same allocation
 constexpr int BOYS_TAB = BOYS_NG * (BOYS_M + 1);
@@ -51,9 +54,11 @@ struct PairSet {
     const int *key;          // canonical pair key X(X+1)/2 + Y
 };
 
-// Primitive pairs (SoA).  K = c_a c_b exp(-za zb/p |AB|^2).
+// Primitive pairs (SoA).  K = c_a c_b exp(-za zb/p |AB|^2).  oo2 = 1/2p, fa =
+// za/p, fb = zb/p and kop = K/p are kept too: a division costs a warp of the
+// fp64 kernels about ten instructions on a pipe of 2 lanes a clock.
 struct PrimPairs {
-    const double *p, *Px, *Py, *Pz, *K, *za;
+    const double *p, *Px, *Py, *Pz, *K, *za, *oo2, *fa, *fb, *kop;
     const float *fp, *fPx, *fPy, *fPz, *fK, *fza;  // fp32 mirrors
     const float *fPA, *fPB;                        // fp32 P - A and P - B, [3][n] (x, y, z planes)
     long long n;                                   // records (plane stride of fPA / fPB)
