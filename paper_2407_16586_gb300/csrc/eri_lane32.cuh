@@ -1,14 +1,28 @@
-// fp32 derivative-ERI class kernel with one primitive quartet per lane.
+// fp32 derivative-ERI class kernel: one warp per contracted quartet, one
+// primitive quartet per lane.
 //
-// The arithmetic of a primitive quartet is that of quartet_fp32r, operation by
-// operation (same scaled Hermite basis, same order of the sums), and every
-// primitive quartet's contribution is added in fp64, so the routed result
-// equals the thread form's to fp64 rounding.  What changes is the mapping:
-// quartet_fp32r keeps a contracted quartet's Gamma and F rows (15.6 KB for
-// (dp|dp)) in per-thread local memory and walks its up to 36 x 36 primitive
-// quartets one after the other; here a warp shares them in shared memory
-// (2.6 KB and 2.9 KB a bra primitive pair) and the lanes take the primitive
-// quartets, so a list of a few hundred contracted quartets fills the GPU.
+// Algebra (McMurchie-Davidson, both operators s = 1/r and erf(w r)/r), for a bra
+// primitive pair p and a ket primitive pair q:
+//   F_s[cd][h1] = sum_ab Gamma_s[ab][cd] E^{ab}_{h1}(p)                       (per p, on the warp)
+//   y[ab][h1]   = sum_h2 (-1)^|h2| [sum_cd Gamma_s[ab][cd] E^{cd}_{h2}(q)] R_s[h1+h2]
+//   z[cd][h2]   = (-1)^|h2| sum_h1 F_s[cd][h1] R_s[h1+h2]
+// d/dA and d/dA + d/dB are short dot products with y (eq. deriv, the R-tensor
+// shift), d/dC with z; d/dB and d/dD follow from translational invariance
+// (eq. ti).  The scaled Hermite basis R'_h = R_h / s^{|h|}, s = sqrt(2 rho),
+// keeps every intermediate within fp32 range for any exponent; the factors
+// s^{|h|} move onto the short Hermite vectors.  Every primitive quartet's
+// contribution is added in fp64, so the result does not depend on how primitive
+// quartets are dealt to lanes, up to fp64 rounding.
+//
+// Why lanes: one thread per contracted quartet kept its Gamma and F rows (15.6 KB
+// for (dp|dp)) in local memory and walked up to 36 x 36 primitive quartets one
+// after the other; the warp shares them in shared memory (2.6 KB, and 2.9 KB a bra
+// primitive pair), and a list of a few hundred contracted quartets fills the GPU
+// (fp32 lists of the 6-atom workload on the learned route: 114.5 -> 16.8 ms; of a
+// 1/8 shard of the 32-atom workload: 178.6 -> 127.8 ms).  Bound: instruction
+// supply -- the unrolled y and z loops of a warp are 16 KB of code, walked by each
+// warp on its own ((dp|pp): 6.5 of 9.6 cycles per instruction wait for it, FMA pipe
+// 13 %) -- and in the classes up to (pp|ps) the fp64 pipe of the Boys recursion.
 #pragma once
 #include "eri_herm.cuh"
 
@@ -373,41 +387,24 @@ struct Lane32Op {
 };
 
 // Kernel forms per class.  fp64: the Hermite-density kernel.  fp32: the lane
-// kernel or, where the thread kernel's values come from another form, that
-// form: the warp kernel for (dd|pp) and (dd|ds), the group kernel for (dd|dp)
-// and (dd|dd), so that the routed results stay what they were.
-// ClassLaunch::kind 1 / 2 / 3 asks for the thread / group / warp kernel; a form
-// not compiled for the class and precision falls back to the default.
-template <int LA, int LB, int LC, int LD>
-struct ClassForms {
-    static constexpr int nfq = ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD);
-    static constexpr size_t kStageMax = 200 * 1024;  // warp arrays + tile staging (16 KB) per CTA
-    static constexpr bool thread32 = nfq < 648;
-    static constexpr bool group32 = nfq >= 648;
-    static constexpr bool warp32 = warp_kernel_smem<LA, LB, LC, LD, float>() + 16384 <= kStageMax;
-    // default fp32 form per class (0 lane, 2 group, 3 warp)
-    static constexpr int qc = pair_class(LA, LB) * (pair_class(LA, LB) + 1) / 2 + pair_class(LC, LD);
-    static constexpr int default32 = kDefaultForm32[qc];
-    static_assert((default32 != 2 || group32) && (default32 != 3 || warp32), "default fp32 form not compiled");
-};
-
+// kernel, but the warp kernel for (dd|pp) and (dd|ds) and the group kernel for
+// (dd|dp) and (dd|dd), whose order of fp32 sums differs from the lane kernel's:
+// the routed results stay what they were.  ClassLaunch::kind 2 / 3 asks for the
+// group / warp kernel; a form not compiled for the class and precision (the
+// thread form is compiled for none) falls back to the default.
 template <int LA, int LB, int LC, int LD>
 cudaError_t launch_class_kernel(int fp32, int gcap, size_t smem, cudaStream_t st, const MolDesc *mols,
                                 const ClassLaunch &cl, const OutArgs &out, const double *boys)
 {
-    using K = ClassForms<LA, LB, LC, LD>;
+    constexpr int nfq = ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD);
+    constexpr bool group = nfq >= 648, warp = (LA + LB == 4) && nfq >= 216 && nfq < 648;
     if (!fp32) return launch_lanes<HermOp<LA, LB, LC, LD>>(gcap, st, mols, cl, out, boys);
-    int kind = cl.kind;
-    if ((kind == 1 && !K::thread32) || (kind == 2 && !K::group32) || (kind == 3 && !K::warp32) || kind < 1 || kind > 3)
-        kind = K::default32;
-    if constexpr (K::warp32)
-        if (kind == 3) return launch_warp<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
-    if constexpr (K::group32)
-        if (kind == 2) return launch_coop<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
-    if constexpr (K::thread32)
-        if (kind == 1) return launch_units(k_grad<LA, LB, LC, LD, true>, 0, gcap, smem, st, mols, cl, out, boys);
-    if constexpr (K::default32 == 0) return launch_lanes<Lane32Op<LA, LB, LC, LD>>(gcap, st, mols, cl, out, boys);
-    return cudaErrorInvalidValue;  // not reached: every class compiles its default form
+    if constexpr (warp)
+        return launch_warp<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
+    else if constexpr (group)
+        return launch_coop<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
+    else
+        return launch_lanes<Lane32Op<LA, LB, LC, LD>>(gcap, st, mols, cl, out, boys);
 }
 
 }  // namespace tg

@@ -815,9 +815,4 @@ cudaError_t launch_warp(int gcap, size_t smem, cudaStream_t st, const MolDesc *m
                         st, mols, cl, out, boys);
 }
 
-// Default fp32 kernel form per angular class (ssss, psss, psps, ppss, ppps,
-// pppp, dsss, dsps, dspp, dsds, dpss, dpps, dppp, dpds, dpdp, ddss, ddps, ddpp,
-// ddds, dddp, dddd): 0 = lane, 2 = group, 3 = warp.
-constexpr int kDefaultForm32[NQC] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 3, 3, 2, 2};
-
 }  // namespace tg
