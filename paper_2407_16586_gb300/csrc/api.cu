@@ -1022,7 +1022,20 @@ int device_tiles(tg_basis *b, const Plan &pl, const tg_options &opt, cudaStream_
     const long long nch = std::min(ntl, RCHUNK);
     size_t needB = al(sizeof(uint4) * ntl) + al(sizeof(uint4) * nout) + al(sizeof(float) * ntl) +
                    al(sizeof(int) * ntl) + 4096;
-    if (learned) needB += al(sizeof(TileRef) * nch) + al(sizeof(float) * nch * NFEAT) + al(sizeof(float) * nch);
+    // feature tables per pair class; the rows of density maxima (nshell doubles a
+    // bra tile: 94 MB for 300 atoms, 6.6 GB for 1500) only up to 16 GB, beyond
+    // which every tile gathers its block factors itself
+    size_t mxbytes = 0;
+    for (int c = 0; c < NPC; ++c) mxbytes += al(sizeof(double) * (size_t)ra.t[c].nbt * b->nshell);
+    const bool tables = learned && mxbytes <= ((size_t)16 << 30);
+    if (learned) needB += al(sizeof(float) * nch * NFEAT) + al(sizeof(float) * nch);
+    if (learned && !tables) needB += al(sizeof(TileRef) * nch);
+    if (tables) {
+        needB += mxbytes;
+        for (int c = 0; c < NPC; ++c)
+            needB += al(sizeof(SideFeature) * ra.t[c].nbt) + al(sizeof(SideFeature) * ra.t[c].nkt) +
+                     al(sizeof(double) * 3 * pl.cls[c].size());
+    }
     DevArena &B = b->ws4;
     TG_CUDA(B.reserve(needB));
     B.used = 0;
@@ -1045,7 +1058,32 @@ int device_tiles(tg_basis *b, const Plan &pl, const tg_options &opt, cudaStream_
             k_route_bins<<<gbin, 128, hbytes, st>>>(ntl, d_raw, d_bnd, 0, kEps32Bound * TILE, 0.0, ra, d_bin, d_hist);
             ++launches;
         } else {
-            TileRef *d_ref = B.take<TileRef>(nch);
+            const FeatureArgs fa = feature_args(b, pl);
+            FeatureTables ft;
+            std::memset(&ft, 0, sizeof(ft));
+            TileRef *d_ref = tables ? nullptr : B.take<TileRef>(nch);
+            if (tables) {
+                for (int qc = 0; qc < NQC; ++qc) {
+                    ft.P[qc] = pl.qc_P[qc];
+                    ft.Q[qc] = pl.qc_Q[qc];
+                }
+                for (int c = 0; c < NPC; ++c) {
+                    const PairSet ps = fa.sets[c];
+                    const int nbt = ra.t[c].nbt, nkt = ra.t[c].nkt;
+                    SideFeature *fb = B.take<SideFeature>(nbt), *fk = B.take<SideFeature>(nkt);
+                    double *cen = B.take<double>(3 * (size_t)ps.n), *mx = B.take<double>((size_t)nbt * b->nshell);
+                    ft.bra[c] = fb;
+                    ft.ket[c] = fk;
+                    ft.cen[c] = cen;
+                    ft.mx[c] = mx;
+                    if (!ps.n) continue;
+                    k_side_features<<<(nbt + 63) / 64, 64, 0, st>>>(TB, ps, fa, fb);
+                    k_side_features<<<(nkt + 63) / 64, 64, 0, st>>>(TK, ps, fa, fk);
+                    k_pair_centres<<<(ps.n + 127) / 128, 128, 0, st>>>(ps, b->d_xyz, b->d_sh_atom, cen);
+                    k_bra_density_max<<<nbt, 256, 0, st>>>(ps, pl.dM, b->nshell, mx);
+                    launches += 4;
+                }
+            }
             float *d_feat = B.take<float>(nch * NFEAT), *d_pred = B.take<float>(nch);
             const tg_router *r = opt.router;
             float *dparams = b->d_router;
@@ -1057,13 +1095,18 @@ int device_tiles(tg_basis *b, const Plan &pl, const tg_options &opt, cudaStream_
                 const long long n = std::min(RCHUNK, ntl - c0);
                 const unsigned g = (unsigned)((n + 127) / 128);
                 const unsigned gb = (unsigned)std::min<long long>(g, 8LL * b->nsm);
-                k_tile_refs<<<g, 128, 0, st>>>(n, d_raw + c0, ra, d_ref);
-                k_tile_features<<<g, 128, 0, st>>>((int)n, d_ref, feature_args(b, pl), d_feat);
+                if (tables) {
+                    k_tile_features_tab<<<g, 128, 0, st>>>(n, d_raw + c0, fa, ft, d_feat);
+                } else {
+                    k_tile_refs<<<g, 128, 0, st>>>(n, d_raw + c0, ra, d_ref);
+                    k_tile_features<<<g, 128, 0, st>>>((int)n, d_ref, fa, d_feat);
+                    ++launches;
+                }
                 k_mlp_predict<<<g, 128, 0, st>>>((int)n, d_feat, dparams + NPARAM, dparams + NPARAM + NFEAT, dparams,
                                                  d_pred);
                 k_route_bins<<<gb, 128, hbytes, st>>>(n, d_raw + c0, d_pred, 1, (double)r->eps_rel,
                                                       (double)r->margin, ra, d_bin + c0, d_hist);
-                launches += 4;
+                launches += 3;
             }
         }
         TG_CUDA(cudaGetLastError());
