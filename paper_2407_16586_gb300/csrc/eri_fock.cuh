@@ -328,7 +328,7 @@ cudaError_t launch_fock_class(int, cudaStream_t st, const MolDesc *mols, const C
 {
     constexpr size_t bytes = FockLay<LA, LB, LC, LD>::BYTES;
     static_assert(bytes <= kCtaSmem, "one warp's arrays fit in a CTA");
-    return launch_warp_units(k_fock_lanes<LA, LB, LC, LD>, 1, bytes, 1, 1 << 20, st, mols, cl, out, boys);
+    return launch_warp_units(k_fock_lanes<LA, LB, LC, LD>, 1, 32, bytes, 1, 1 << 20, st, mols, cl, out, boys);
 }
 
 }  // namespace tg

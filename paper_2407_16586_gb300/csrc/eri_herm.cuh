@@ -212,6 +212,11 @@ struct HermLayK {
     // registers, from L = 7 (120 entries) in passes over ranges of Hermite
     // orders, which need R's top order stored too.
     static constexpr bool RREG = LM <= 5, PASSES = L >= 7;
+    // warps per quartet: with PASSES one warp's arrays take 104 ((dd|dp)) or 188 KB
+    // ((dd|dd)), so four warps work on one quartet: the recursion's and the
+    // transforms' entries and the reverse items dealt over them, one range of orders
+    // of X each
+    static constexpr int NW = PASSES ? 4 : 1;
     // Hermite rows: the reverse sums reach order L - 1 (their items leave out the
     // top order of both sides at once), the recursion in rows needs L
     static constexpr int NRH = nherm(PASSES ? LM : (RREG ? L - 1 : L));
@@ -225,7 +230,7 @@ struct HermLayK {
     static constexpr int GS = NO * NCD * NABP, MS = NO * NM1 * NM2P, FS = NO * NT1 * NM2P;  // per ket pair
     static constexpr int HS = (NM2 * NABP > NM1 * NCD ? NM2 * NABP : NM1 * NCD) * NO;
     // the transforms' half-way arrays share the space of the R rows
-    static constexpr int HALF = NE1 + KQ * (NE2 + HS), ROWS = (NRH + NS2) * RS, RED = 9 * RS;
+    static constexpr int HALF = NE1 + KQ * (NE2 + HS), ROWS = (NRH + NS2) * RS, RED = 9 * RS * NW;
     static constexpr int SHARED = HALF > ROWS ? (HALF > RED ? HALF : RED) : (ROWS > RED ? ROWS : RED);
     static constexpr int NP1 = 4;                     // per bra primitive pair: a^, mu, 2 pi^(5/2) K / p, p
     static constexpr int o_G = 0;                              // [KQ][NO][NCD][NABP]
@@ -525,6 +530,42 @@ constexpr HermSteps make_herm_steps()
 }
 static __device__ const HermSteps kHermSteps = make_herm_steps();
 
+// Barrier of the NW warps that share a quartet.
+template <int NW>
+__device__ __forceinline__ void quartet_sync()
+{
+    if constexpr (NW == 1) __syncwarp();
+    else __syncthreads();
+}
+
+// The entries of one level (totals up to top) in the columns of 32 primitive
+// quartets by NW warps: total by total from the top, whose entries read the two
+// totals below only, so one barrier a total orders reads and writes.
+template <int RS, int NW>
+__device__ __forceinline__ void hermite_level_warps(double *Rl, int warp, int top, double X, double Y, double Z)
+{
+#pragma unroll 1
+    for (int k = top; k >= 1; --k) {
+        const int end = nherm(k);
+#pragma unroll 1
+        for (int h = nherm(k - 1) + warp; h < end; h += 4 * NW) {
+            double v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const unsigned w = kHermSteps.w[h + j * NW < end ? h + j * NW : h];
+                const unsigned dir = w & 3;
+                v[j] = (dir == 0 ? X : (dir == 1 ? Y : Z)) * Rl[((w >> 2) & 0xff) * RS];
+                const int c = (int)(w >> 18);
+                if (c > 0) v[j] += double(c) * Rl[((w >> 10) & 0xff) * RS];
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (h + j * NW < end) Rl[(h + j * NW) * RS] = v[j];
+        }
+        quartet_sync<NW>();
+    }
+}
+
 // Entries 1 .. n - 1 of one level in this lane's column, in place, from high
 // to low: every entry reads lower ones, and of four at a time all reads
 // precede the writes.
@@ -553,13 +594,13 @@ __device__ __forceinline__ void hermite_level(double *Rl, int n, double X, doubl
 // Gamma_op of the group's quartets (the 8 permutation images of the pair
 // products, times scale), [ket][op][cd][ab], for operators o0 .. o0 + NO - 1.
 template <int LA, int LB, int LC, int LD>
-__device__ __forceinline__ void herm_gamma(double *G, int lane, int kg, const GroupInfo &gi, int k0, int o0, const DensArgs &den,
+__device__ __forceinline__ void herm_gamma(double *G, int tid, int kg, const GroupInfo &gi, int k0, int o0, const DensArgs &den,
                                            const int *sh_bf, int fa, int fb)
 {
     using Lay = HermLay<LA, LB, LC, LD>;
     constexpr int NB = ncart(LB), ND = ncart(LD), NFQ = Lay::NAB * Lay::NCD;
     const int nbf = den.nbf;
-    for (int x = lane; x < kg * NFQ; x += 32) {
+    for (int x = tid; x < kg * NFQ; x += 32 * Lay::NW) {
         const int kq = x / NFQ, it = x % NFQ, cd = it / Lay::NAB, ab = it % Lay::NAB;
         double *g = G + kq * Lay::GS + cd * Lay::NABP + ab;
         double g0 = 0.0, g1 = 0.0;
@@ -594,12 +635,12 @@ __device__ __forceinline__ void herm_gamma(double *G, int lane, int kg, const Gr
 
 // c^{ab}_m R^.. of every table entry of a pair class, for n pairs (powers pw,
 // 15 apart).
-template <int LA, int LB>
-__device__ __forceinline__ void entry_values(double *out, int lane, const double *pw, int n)
+template <int LA, int LB, int NT = 32>
+__device__ __forceinline__ void entry_values(double *out, int tid, const double *pw, int n)
 {
     const auto &T = pair_tab<LA, LB>();
     constexpr int NE = PairTab<LA, LB>::NE;
-    for (int x = lane; x < n * NE; x += 32) {
+    for (int x = tid; x < n * NE; x += NT) {
         const unsigned w = T.ent[x % NE];
         const double *q = pw + x / NE * 15;
         out[x] = double((int)((w >> 8) & 0xff)) * q[(w >> 16) & 7] * q[5 + ((w >> 19) & 7)] * q[10 + ((w >> 22) & 7)];
@@ -608,12 +649,12 @@ __device__ __forceinline__ void entry_values(double *out, int lane, const double
 
 // half[ket][o][m2][ab] = sum_{entries of m2} value Gamma[cd][ab]
 template <int LA, int LB, int LC, int LD>
-__device__ __forceinline__ void half_ket(double *half, const double *G, const double *vk, int lane, int kg)
+__device__ __forceinline__ void half_ket(double *half, const double *G, const double *vk, int tid, int kg)
 {
     using Lay = HermLay<LA, LB, LC, LD>;
     const auto &T = pair_tab<LC, LD>();
     constexpr int N = Lay::NM2 * Lay::NAB;
-    for (int x = lane; x < kg * N; x += 32) {
+    for (int x = tid; x < kg * N; x += 32 * Lay::NW) {
         const int kq = x / N, it = x % N, m = it / Lay::NAB, ab = it % Lay::NAB;
         const double *v = vk + kq * Lay::NE2;
 #pragma unroll
@@ -633,9 +674,9 @@ __device__ const HermItems<LA, LB, LC, LD, ALL> kHermItems = make_herm_items<LA,
 // Reverse sums of one pass (primitive quartets j0 .. j0 + n - 1 of the block, n
 // <= 32, lane j - j0's R in column j - j0 of Rr): per bra primitive pair,
 // U[h1][m2] = sum_q s_m2 R[h1 + h2], added to V[m1][m2] with its scalars.
-template <int LA, int LB, int LC, int LD, bool ALL>
+template <int LA, int LB, int LC, int LD, bool ALL, int NW = 1>
 __device__ __forceinline__ void reverse_sums(double *V, const double *Rr, const double *S2, const double *S1, int j0,
-                                             int n, int nkp, int lane)
+                                             int n, int nkp, int tid)
 {
     using B = PairMono<LA, LB>;
     constexpr int NIT = HermItems<LA, LB, LC, LD, ALL>::N, RS = 33, NM2P = PairMono<LC, LD>::NM | 1;
@@ -644,9 +685,10 @@ __device__ __forceinline__ void reverse_sums(double *V, const double *Rr, const 
     constexpr int ITL = 32 / SUB;
     const auto &TBra = pair_tab<LA, LB>();
     const unsigned *items = kHermItems<LA, LB, LC, LD, ALL>.it;
-    const int pfirst = j0 / nkp, plast = (j0 + n - 1) / nkp, sub = lane / ITL;
-    for (int i0 = 0; i0 < NIT; i0 += ITL) {
-        const int it = i0 + lane % ITL;
+    static_assert(NW == 1 || SUB == 1, "several warps: one lane an item");
+    const int pfirst = j0 / nkp, plast = (j0 + n - 1) / nkp, sub = NW == 1 ? tid / ITL : 0;
+    for (int i0 = 0; i0 < NIT; i0 += ITL * NW) {
+        const int it = i0 + tid % (ITL * NW);
         const unsigned w = items[it < NIT ? it : NIT - 1];
         const double *r = Rr + (w & 0xff) * RS, *s = S2 + (w >> 21) * RS;
         const unsigned hm = TBra.hm[(w >> 8) & 0x3f];
@@ -722,7 +764,7 @@ __device__ __forceinline__ int block_pairs(int nbra, int nkp, int cap, int lanes
 // (this lane's share; d/dA of all ket pairs may sit on any lane, the others on
 // their ket pair's lanes).
 template <int LA, int LB, int LC, int LD>
-__device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo &gi, const GeoArgs &geo, const DensArgs &den,
+__device__ void group_herm(double *sm, int tid, int k0, int kg, const GroupInfo &gi, const GeoArgs &geo, const DensArgs &den,
                            const PrimPairs &pp, int sa, int sb, int pb0, int nbp, int ib0, int ibs, const double *boys,
                            double (&acc)[9])
 {
@@ -730,6 +772,8 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
     constexpr int NCD = Lay::NCD, L = Lay::L, LM = Lay::LM, NT1 = Lay::NT1;
     constexpr int NM1 = Lay::NM1, NM2 = Lay::NM2, NM2P = Lay::NM2P, NS1 = Lay::NS1, NS2 = Lay::NS2, RS = Lay::RS;
     constexpr int NO = Lay::NO, NP1 = Lay::NP1, NABP = Lay::NABP, KQ = Lay::KQ;
+    constexpr int NW = Lay::NW, NT = 32 * NW;  // warps and threads that share the group
+    const int lane = tid % 32, warp = tid / 32;
     constexpr int NIT = HermItems<LA, LB, LC, LD, false>::N;
     double *G = sm + Lay::o_G, *Gp = sm + Lay::o_Gp, *V = sm + Lay::o_V, *F = sm + Lay::o_F;
     double *S1 = sm + Lay::o_S1, *P1 = sm + Lay::o_P1, *pw = sm + Lay::o_pw, *X1 = sm + Lay::o_X;
@@ -742,7 +786,7 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
     const double om = ominf ? 1.0 : den.omega;
     if constexpr (KQ == 1) kg = 1;
     const int LG = 32 / kg, kq = lane / LG, sl = lane % LG;
-    if (lane < 3 + 3 * kg) {  // powers of R = A - B and of every S = C - D
+    if (tid < 3 + 3 * kg) {  // powers of R = A - B and of every S = C - D
         const int d = lane % 3, w = lane / 3;
         const int k = min(k0 + w - 1, gi.n - 1);
         const int s0 = w == 0 ? sa : gi.sc[k], s1 = w == 0 ? sb : gi.sd[k];
@@ -762,17 +806,17 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
     // this lane's sums over its primitive quartets: T, a^ T, c^ T, mu_ab E, mu_cd E
     double aT[3] = {0.0, 0.0, 0.0}, aA[3] = {0.0, 0.0, 0.0}, aC[3] = {0.0, 0.0, 0.0}, eA = 0.0, eC = 0.0;
     double gA[3] = {0.0, 0.0, 0.0}, gC[3] = {0.0, 0.0, 0.0};  // polynomial parts
-    __syncwarp();
+    quartet_sync<NW>();
 
     for (int o0 = 0; o0 < nops; o0 += NO) {
         // ---- Gamma -> G'[m1][m2]
-        herm_gamma<LA, LB, LC, LD>(G, lane, kg, gi, k0, o0, den, geo.sh_bf, geo.sh_bf[sa], geo.sh_bf[sb]);
-        entry_values<LA, LB>(vb, lane, pw, 1);
-        entry_values<LC, LD>(vk, lane, pw + 15, kg);
-        __syncwarp();
-        half_ket<LA, LB, LC, LD>(half, G, vk, lane, kg);
-        __syncwarp();
-        for (int x = lane; x < kg * NM1 * NM2; x += 32) {
+        herm_gamma<LA, LB, LC, LD>(G, tid, kg, gi, k0, o0, den, geo.sh_bf, geo.sh_bf[sa], geo.sh_bf[sb]);
+        entry_values<LA, LB, NT>(vb, tid, pw, 1);
+        entry_values<LC, LD, NT>(vk, tid, pw + 15, kg);
+        quartet_sync<NW>();
+        half_ket<LA, LB, LC, LD>(half, G, vk, tid, kg);
+        quartet_sync<NW>();
+        for (int x = tid; x < kg * NM1 * NM2; x += NT) {
             const int q = x / (NM1 * NM2), it = x % (NM1 * NM2), m1 = it / NM2, m2 = it % NM2;
 #pragma unroll
             for (int o = 0; o < NO; ++o) {
@@ -783,25 +827,25 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                 V[q * Lay::MS + (o * NM1 + m1) * NM2P + m2] = 0.0;
             }
         }
-        __syncwarp();
+        quartet_sync<NW>();
 
         for (int blk = 0; blk < nbra; blk += pb) {
             const int np = min(pb, nbra - blk);
             // ---- scalars of the block's bra primitive pairs, then F[p][ket][h1][m2]
-            if (lane < np) {
-                const int ip = pb0 + ib0 + (blk + lane) * ibs;
+            if (tid < np) {
+                const int ip = pb0 + ib0 + (blk + tid) * ibs;
                 const double a = pp.fa[ip], b = pp.fb[ip];
                 double s[NS1];
                 pair_scalars<LA, LB, false>(pp.oo2[ip], a, b, s);
 #pragma unroll
-                for (int k = 0; k < NS1; ++k) S1[lane * NS1 + k] = s[k];
-                P1[lane * NP1] = a;
-                P1[lane * NP1 + 1] = pp.za[ip] * b;
-                P1[lane * NP1 + 2] = pp.kop[ip] * 34.986836655249725;  // 2 pi^(5/2) K / p
-                P1[lane * NP1 + 3] = pp.p[ip];
+                for (int k = 0; k < NS1; ++k) S1[tid * NS1 + k] = s[k];
+                P1[tid * NP1] = a;
+                P1[tid * NP1 + 1] = pp.za[ip] * b;
+                P1[tid * NP1 + 2] = pp.kop[ip] * 34.986836655249725;  // 2 pi^(5/2) K / p
+                P1[tid * NP1 + 3] = pp.p[ip];
             }
-            __syncwarp();
-            for (int x = lane; x < np * kg * NT1 * NM2; x += 32) {
+            quartet_sync<NW>();
+            for (int x = tid; x < np * kg * NT1 * NM2; x += NT) {
                 const int pq = x / (NT1 * NM2), r = x % (NT1 * NM2), h = r / NM2, m2 = r % NM2;
                 const int pi = pq / kg, q = pq % kg;
                 const unsigned hm = TBra.hm[h];
@@ -814,7 +858,7 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                     F[(pi * KQ + q) * Lay::FS + (o * NT1 + h) * NM2P + m2] = f;
                 }
             }
-            __syncwarp();
+            quartet_sync<NW>();
             const int ntot = np * nk, nmax = np * nkmax;
             for (int it0 = 0; it0 < nmax; it0 += LG) {
                 // ---- this lane's primitive quartet
@@ -830,7 +874,7 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                 const double pref = it0 + sl < ntot ? P1[pi * NP1 + 2] * pp.kop[kp] * ir : 0.0;
                 double s2[NS2];
                 pair_scalars<LC, LD, true>(pp.oo2[kp], c, d, s2);
-                if constexpr (NIT > 0)
+                if (NIT > 0 && warp == 0)
 #pragma unroll
                     for (int k = 0; k < NS2; ++k) S2[k * RS + lane] = s2[k];
                 double e = 0.0, T[3] = {0.0, 0.0, 0.0};
@@ -898,27 +942,32 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                             energy_terms<L, h>(lds(Rl + h * RS), Xd, e, T);
                         });
                     } else {
-                        Rl[0] = base[LM];
+                        // every warp forms the scalars; then (0,0,0) of a level is written after
+                        // its entries, which read the level above
+                        if (warp == 0) Rl[0] = base[LM];
+                        quartet_sync<NW>();
                         static_for<LM>([&](auto I) {
                             constexpr int n = LM - 1 - decltype(I)::value;
-                            hermite_level<RS>(Rl, nherm(LM - n), X, Y, Z);
-                            Rl[0] = base[n];
+                            hermite_level_warps<RS, NW>(Rl, warp, LM - n, X, Y, Z);
+                            if (warp == 0) Rl[0] = base[n];
+                            quartet_sync<NW>();
                         });
-                        lds_fence();
-                        density_pass<LA, LB, LC, LD, 0, 5>(Fl, s2, Rl, e, T);
-                        density_pass<LA, LB, LC, LD, 6, 7>(Fl, s2, Rl, e, T);
-                        if constexpr (L == 8) density_pass<LA, LB, LC, LD, 8, 8>(Fl, s2, Rl, e, T);
+                        // a quarter of the density's products each ((dd|dd): 750, 585, 650, 675)
+                        if (warp == 0) density_pass<LA, LB, LC, LD, 0, 4>(Fl, s2, Rl, e, T);
+                        else if (warp == 1) density_pass<LA, LB, LC, LD, 5, 5>(Fl, s2, Rl, e, T);
+                        else if (warp == 2) density_pass<LA, LB, LC, LD, 6, 6>(Fl, s2, Rl, e, T);
+                        else density_pass<LA, LB, LC, LD, 7, L>(Fl, s2, Rl, e, T);
                     }
-                    __syncwarp();
+                    quartet_sync<NW>();
                     // ---- reverse sums U[h1][m2], added to V with the bra scalars
                     if constexpr (NIT > 0) {
                         if (kg == 1)
-                            reverse_sums<LA, LB, LC, LD, false>(V + o * NM1 * NM2P, Rr, S2, S1, it0, min(32, ntot - it0),
-                                                                nkd, lane);
+                            reverse_sums<LA, LB, LC, LD, false, NW>(V + o * NM1 * NM2P, Rr, S2, S1, it0,
+                                                                    min(32, ntot - it0), nkd, tid);
                         else if constexpr (KQ > 1)
                             reverse_sums_group<LA, LB, LC, LD>(V + o * NM1 * NM2P, Lay::MS, Rr, S2, S1, it0, np, kg, LG,
                                                                gi.nk + k0, lane);
-                        __syncwarp();
+                        quartet_sync<NW>();
                     }
                 }
                 const double a = P1[pi * NP1];
@@ -931,17 +980,17 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                 eA += P1[pi * NP1 + 1] * e;
                 eC += pp.za[kp] * d * e;
             }
-            __syncwarp();  // S1, P1 and F are rewritten for the next block
+            quartet_sync<NW>();  // S1, P1 and F are rewritten for the next block
         }
         // ---- polynomial parts: V with dG'/dR (ket half again) and dG'/dS (bra half)
         if constexpr (NIT > 0) {
-            entry_values<LA, LB>(vb, lane, pw, 1);
-            if constexpr (Lay::L1 > 0) entry_values<LC, LD>(vk, lane, pw + 15, kg);
-            __syncwarp();
+            entry_values<LA, LB, NT>(vb, tid, pw, 1);
+            if constexpr (Lay::L1 > 0) entry_values<LC, LD, NT>(vk, tid, pw + 15, kg);
+            quartet_sync<NW>();
             if constexpr (Lay::L1 > 0) {
-                half_ket<LA, LB, LC, LD>(half, G, vk, lane, kg);
-                __syncwarp();
-                for (int x = lane; x < kg * Lay::NE1; x += 32) {
+                half_ket<LA, LB, LC, LD>(half, G, vk, tid, kg);
+                quartet_sync<NW>();
+                for (int x = tid; x < kg * Lay::NE1; x += NT) {
                     const int q = x / Lay::NE1, it = x % Lay::NE1;
                     const unsigned w = TBra.ent[it];
                     const int px = (w >> 16) & 7, py = (w >> 19) & 7, pz = (w >> 22) & 7;
@@ -960,11 +1009,11 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                     if (py) gA[1] += s * double(py) * qx * pw[5 + py - 1] * qz;
                     if (pz) gA[2] += s * double(pz) * qx * qy * pw[10 + pz - 1];
                 }
-                __syncwarp();
+                quartet_sync<NW>();
             }
             if constexpr (Lay::L2 > 0) {
                 // bra half [ket][o][m1][cd]
-                for (int x = lane; x < kg * NM1 * NCD; x += 32) {
+                for (int x = tid; x < kg * NM1 * NCD; x += NT) {
                     const int q = x / (NM1 * NCD), it = x % (NM1 * NCD), m1 = it / NCD, cd = it % NCD;
 #pragma unroll
                     for (int o = 0; o < NO; ++o) {
@@ -974,9 +1023,9 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                         half[q * Lay::HS + (o * NM1 + m1) * NCD + cd] = s;
                     }
                 }
-                __syncwarp();
+                quartet_sync<NW>();
                 const double *pk = pw + (1 + kq) * 15;
-                for (int it = sl; it < Lay::NE2; it += LG) {
+                for (int it = sl + 32 * warp; it < Lay::NE2; it += LG * NW) {
                     const unsigned w = TKet.ent[it];
                     const int px = (w >> 16) & 7, py = (w >> 19) & 7, pz = (w >> 22) & 7;
                     if (px + py + pz == 0) continue;
@@ -996,7 +1045,7 @@ __device__ void group_herm(double *sm, int lane, int k0, int kg, const GroupInfo
                 }
             }
         }
-        __syncwarp();
+        quartet_sync<NW>();
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -1018,16 +1067,17 @@ struct HermOp {
     using Lay = HermLay<LA, LB, LC, LD>;
     static constexpr bool FP32 = false;
     static constexpr int L = LA + LB + LC + LD, KQ = Lay::KQ;
-    static constexpr int cta_warps = L <= 3 ? 2 : 1, min_ctas = L == 3 ? 6 : 8;
+    static constexpr int NW = Lay::NW;  // warps per worker (a worker takes units alone)
+    static constexpr int cta_workers = L <= 3 ? 2 : 1, min_ctas = L == 3 ? 6 : (NW == 1 ? 8 : 10 - L);
     // primitive quartets of a contracted one up to which ket pairs are grouped
     // (kg times it stays below): the smaller the class, the more of a quartet's
     // work is the density transform that a group shares
     static constexpr int group_below = L == 0 ? 512 : (L == 1 ? 256 : (L == 2 ? 128 : 64));
-    static __device__ __forceinline__ void group(double *sm, int lane, int k0, int kg, const GroupInfo &gi,
+    static __device__ __forceinline__ void group(double *sm, int tid, int k0, int kg, const GroupInfo &gi,
                                                  const MolDesc &md, int sa, int sb, int pb0, int nbp, int ib0, int ibs, const double *boys,
                                                  double (&acc)[9])
     {
-        group_herm<LA, LB, LC, LD>(sm, lane, k0, kg, gi, md.geo, md.den, md.pp, sa, sb, pb0, nbp, ib0, ibs, boys, acc);
+        group_herm<LA, LB, LC, LD>(sm, tid, k0, kg, gi, md.geo, md.den, md.pp, sa, sb, pb0, nbp, ib0, ibs, boys, acc);
     }
 };
 
@@ -1039,22 +1089,23 @@ struct HermOp {
 // memory, or with out.use_smem = 0 the warp's slab), so the schedule and the
 // order of all sums are fixed and results are bitwise reproducible.
 template <class Op>
-__global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
+__global__ void __launch_bounds__(32 * Op::NW * Op::cta_workers, Op::min_ctas)
     k_grad_lanes(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out, const double *__restrict__ boys)
 {
     using Lay = typename Op::Lay;
-    constexpr int RS = Lay::RS, KQ = Op::KQ;
+    constexpr int RS = Lay::RS, KQ = Op::KQ, NW = Op::NW, NT = 32 * NW;
     extern __shared__ double smem[];
-    __shared__ GroupInfo ginfo[Op::cta_warps];
-    const int nw = blockDim.x / 32, grp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    __shared__ GroupInfo ginfo[Op::cta_workers];
+    // nw workers of NW warps each; every warp of a worker walks the same units
+    const int nw = blockDim.x / NT, grp = threadIdx.x / NT, tid = threadIdx.x % NT, lane = tid % 32;
     const int n3 = out.natom_total * 3;
     double *wsm = smem + (size_t)grp * Lay::TOTAL;
     GroupInfo &gi = ginfo[grp];
     double *grad = out.use_smem ? smem + (size_t)nw * Lay::TOTAL + (size_t)grp * n3
                                 : out.partials + (size_t)(blockIdx.x * nw + grp) * n3;
     if (out.use_smem) {
-        for (int k = lane; k < n3; k += 32) grad[k] = 0.0;
-        __syncwarp();
+        for (int k = tid; k < n3; k += NT) grad[k] = 0.0;
+        quartet_sync<NW>();
     }
     unsigned long long nq = 0, npq = 0, nbv = 0;  // of this lane's ket pair
     const int S = cl.nsplit, C = cl.nchunk, QPC = TILE / C;
@@ -1087,7 +1138,7 @@ __global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
             }
             if (ok) {
                 const int nbs = (bra.np[bi] - split + S - 1) / S;
-                if (split == 0) nq += 1;
+                if (split == 0) nq += 1;  // (only a worker's first warp reports)
                 npq += (unsigned long long)nbs * ket.np[ki];
                 nbv += (unsigned long long)nbs;
                 ok = ket.np[ki] > 0;  // all screened: counted, nothing to add
@@ -1099,7 +1150,7 @@ __global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
                 sa = __shfl_sync(0xffffffffu, sa, first);
                 sb = __shfl_sync(0xffffffffu, sb, first);
                 const int nbp = bra.np[bi], nbs = (nbp - split + S - 1) / S;
-                if (ok) {
+                if (ok && tid < 32) {
                     const int k = __popc(mask & ((1u << lane) - 1));
                     double scale = 1.0;
                     if (sa == sb) scale *= 0.5;
@@ -1115,7 +1166,7 @@ __global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
                         for (int j = n; j < GroupInfo::CAP; ++j) gi.nk[j] = 0, gi.pk0[j] = ket.poff[ki];
                     }
                 }
-                __syncwarp();
+                quartet_sync<NW>();
                 int kg = 1;
                 if (KQ > 1) {
                     int nkmax = gi.nk[0];
@@ -1126,19 +1177,22 @@ __global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
                     double acc[9];
 #pragma unroll
                     for (int k = 0; k < 9; ++k) acc[k] = 0.0;
-                    Op::group(wsm, lane, k0, kg, gi, md, sa, sb, bra.poff[bi], nbp, split, S, boys, acc);
+                    Op::group(wsm, tid, k0, kg, gi, md, sa, sb, bra.poff[bi], nbp, split, S, boys, acc);
                     // the nine sums of every ket pair over its 32 / kg lanes, through shared memory
                     double *red = wsm + Lay::o_X;
-                    __syncwarp();
+                    quartet_sync<NW>();
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) red[k * RS + lane] = acc[k];
-                    __syncwarp();
+                    for (int k = 0; k < 9; ++k) red[(tid / 32 * 9 + k) * RS + lane] = acc[k];
+                    quartet_sync<NW>();
                     if (kg == 1) {  // three lanes a sum
                         double s = 0.0;
                         const int k = lane / 3 < 9 ? lane / 3 : 8, part = lane % 3;
-                        for (int j = part; j < 32; j += 3) s += red[k * RS + j];
+#pragma unroll
+                        for (int w = 0; w < NW; ++w)
+                            for (int j = part; j < 32; j += 3) s += red[(w * 9 + k) * RS + j];
                         const double s1 = __shfl_down_sync(0xffffffffu, s, 1), s2 = __shfl_down_sync(0xffffffffu, s, 2);
-                        if (part == 0 && lane < 27) red[k * RS] = s + s1 + s2;
+                        if (NW > 1) quartet_sync<NW>();  // all have read
+                        if (part == 0 && lane < 27 && tid < 32) red[k * RS] = s + s1 + s2;
                     } else {
                         const int lg = 32 / kg;
                         for (int x = lane; x < 9 * kg; x += 32) {
@@ -1148,13 +1202,13 @@ __global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
                             p[0] = s;
                         }
                     }
-                    __syncwarp();
+                    quartet_sync<NW>();
                     const int i = lane % 3, lg = 32 / kg;
                     if (out.dump) {  // one ket pair; lanes 0..11: output component X * 3 + i
                         const int X = lane / 3;
                         const double dA = red[i * RS], dT = red[(3 + i) * RS], dC = red[(6 + i) * RS];
                         g = X == 0 ? dA : (X == 1 ? dT - dA : (X == 2 ? dC : -dT - dC));
-                    } else if (lane < 3) {  // lane i owns component i of every atom
+                    } else if (tid < 3) {  // lane i owns component i of every atom
                         const int *at = md.geo.sh_atom;
                         double *gr = grad + md.atom_off * 3 + i;
                         double dA = 0.0, dT = 0.0;
@@ -1168,11 +1222,11 @@ __global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
                         gr[at[sa] * 3] += dA;
                         gr[at[sb] * 3] += dT - dA;
                     }
-                    __syncwarp();
+                    quartet_sync<NW>();
                 }
-                __syncwarp();
+                quartet_sync<NW>();
             }
-            if (out.dump && lane < 12) out.dump[((size_t)tile * TILE + qi) * 12 + lane] = g;
+            if (out.dump && tid < 12) out.dump[((size_t)tile * TILE + qi) * 12 + lane] = g;
         }
     }
     if (out.use_smem && !out.dump) {
@@ -1191,7 +1245,7 @@ __global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
         npq += __shfl_xor_sync(0xffffffffu, npq, o);
         nbv += __shfl_xor_sync(0xffffffffu, nbv, o);
     }
-    if (lane == 0 && (nq || npq)) {  // a split unit may hold primitives only
+    if (tid == 0 && (nq || npq)) {  // a split unit may hold primitives only
         atomicAdd(out.counters + 0, nq);
         atomicAdd(out.counters + (Op::FP32 ? 3 : 1), npq);
         atomicAdd(out.counters + (Op::FP32 ? 5 : 4), nbv);
@@ -1203,14 +1257,15 @@ __global__ void __launch_bounds__(32 * Op::cta_warps, Op::min_ctas)
 constexpr size_t kCtaSmem = 223 * 1024;
 
 // Launch of a kernel over warp units (tile, chunk, split) with at most gmax
-// CTAs of nw warps, whose warps take groups of up to kets ket pairs.  Tiles are
+// CTAs of nw workers (warps, or teams of threads / 32 warps), which take groups of
+// up to kets ket pairs.  Tiles are
 // cut into chunks of whole groups until every warp has 32 units (with 4, the
 // heaviest units left (pp|pp) SMs idle 57 % of the time on a 1/16 shard of the
 // 32-atom workload; 8 instead of 32 cost the fp32 lists of a 1/8 shard 7 %),
 // into smaller ones while it has fewer than 4, down to single quartets, and
 // then along the bra primitive pairs (which repeats the density transform).
 template <typename K>
-cudaError_t launch_warp_units(K kern, int nw, size_t per_warp, int kets, long long gmax, cudaStream_t st,
+cudaError_t launch_warp_units(K kern, int nw, int threads, size_t per_warp, int kets, long long gmax, cudaStream_t st,
                               const MolDesc *mols, ClassLaunch cl, const OutArgs &out, const double *boys)
 {
     int dev = 0, nsm = 1, per = 1;
@@ -1219,7 +1274,7 @@ cudaError_t launch_warp_units(K kern, int nw, size_t per_warp, int kets, long lo
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const size_t sm = per_warp * nw;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * nw, sm)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads * nw, sm)) != cudaSuccess) return e;
     if (gmax > (long long)(per > 0 ? per : 1) * nsm) gmax = (long long)(per > 0 ? per : 1) * nsm;
     cl.nchunk = 1;
     cl.nsplit = 1;
@@ -1233,7 +1288,7 @@ cudaError_t launch_warp_units(K kern, int nw, size_t per_warp, int kets, long lo
     const long long units = cl.ntiles * cl.nchunk * cl.nsplit;
     const int grid = (int)(units < gmax ? units : gmax);
     if (units < grid * (long long)nw) nw = (int)((units + grid - 1) / grid);
-    kern<<<grid, 32 * nw, per_warp * nw, st>>>(mols, cl, out, boys);
+    kern<<<grid, threads * nw, per_warp * nw, st>>>(mols, cl, out, boys);
     return cudaGetLastError();
 }
 
@@ -1250,8 +1305,8 @@ cudaError_t launch_lanes(int gcap, cudaStream_t st, const MolDesc *mols, const C
     const size_t grad = sizeof(double) * 3 * (size_t)o.natom_total;
     const int fit = (int)(kCtaSmem / bytes), fit_g = (int)(kCtaSmem / (bytes + grad));
     o.use_smem = fit_g >= (fit < 4 ? fit : 4);
-    const int have = o.use_smem ? fit_g : fit, nw = have < Op::cta_warps ? have : Op::cta_warps;
-    return launch_warp_units(k_grad_lanes<Op>, nw, bytes + (o.use_smem ? grad : 0), Op::KQ,
+    const int have = o.use_smem ? fit_g : fit, nw = have < Op::cta_workers ? have : Op::cta_workers;
+    return launch_warp_units(k_grad_lanes<Op>, nw, 32 * Op::NW, bytes + (o.use_smem ? grad : 0), Op::KQ,
                              o.use_smem ? gcap : (gcap > nw ? gcap / nw : 1), st, mols, cl, o, boys);
 }
 

@@ -375,7 +375,7 @@ struct Lane32Op {
     using Lay = Lane32Lay<LA, LB, LC, LD>;
     static constexpr bool FP32 = true;
     static constexpr int L = LA + LB + LC + LD;
-    static constexpr int KQ = 1, cta_warps = L <= 3 ? 2 : 1, min_ctas = L == 3 ? 6 : 8;
+    static constexpr int KQ = 1, NW = 1, cta_workers = L <= 3 ? 2 : 1, min_ctas = L == 3 ? 6 : 8;
     static constexpr int group_below = 0;
     static __device__ __forceinline__ void group(double *sm, int lane, int k0, int, const GroupInfo &gi, const MolDesc &md,
                                                  int sa, int sb, int pb0, int nbp, int ib0, int ibs, const double *boys,
