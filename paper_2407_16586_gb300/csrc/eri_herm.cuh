@@ -209,17 +209,19 @@ struct HermLayK {
     static constexpr int NABP = NAB | 1, NM2P = NM2 | 1;
     static constexpr int RS = 33;                     // row stride of the per-lane columns
     // The R tensor: in registers up to LM = 5, else in shared-memory rows; X in
-    // registers, from L = 7 (120 entries) in passes over ranges of Hermite
-    // orders, which need R's top order stored too.
-    static constexpr bool RREG = LM <= 5, PASSES = L >= 7;
-    // warps per quartet: with PASSES one warp's arrays take 104 ((dd|dp)) or 188 KB
-    // ((dd|dd)), so four warps work on one quartet: the recursion's and the
-    // transforms' entries and the reverse items dealt over them, one range of orders
-    // of X each
-    static constexpr int NW = PASSES ? 4 : 1;
+    // registers, from L = 5 in passes over ranges of Hermite orders (one a warp),
+    // which need R's top order stored too.
+    static constexpr bool RREG = LM <= 5, PASSES = !RREG;
+    // Warps per quartet: one warp's arrays take 104 ((dd|dp)) or 188 KB ((dd|dd)),
+    // so four warps work on one quartet there: transforms, recursion entries and
+    // reverse items dealt over them, one range of orders of X each (on a 1/8 shard of
+    // the 32-atom workload 22.2 -> 11.3 and 13.9 -> 4.2 ms).  Two at L = 5, 6 (40 to 60
+    // KB): 6 to 8 warps an SM instead of 4 or 5 and half the tails (all classes of
+    // that shard together 205.9 -> 198.4 ms, 6 atoms 16.0 -> 15.3 ms).
+    static constexpr int NW = L >= 7 ? 4 : (PASSES ? 2 : 1);
     // Hermite rows: the reverse sums reach order L - 1 (their items leave out the
-    // top order of both sides at once), the recursion in rows needs L
-    static constexpr int NRH = nherm(PASSES ? LM : (RREG ? L - 1 : L));
+    // top order of both sides at once), the recursion in rows needs all
+    static constexpr int NRH = nherm(PASSES ? LM : L - 1);
     static constexpr int NO = (NAB * NCD <= 27) ? 2 : 1;
     // bra primitive pairs of a block: a budget of 1200 doubles for F, 1 to 16
     // (700 buys (dp|pp) a sixth warp, but its half-filled passes cost more:
@@ -400,18 +402,13 @@ __device__ __forceinline__ void static_for(Fn &&f)
 
 // Shared-memory load of the unrolled lane phases.  Inline PTX: plain loads
 // between this many stores make the compiler's alias analysis take minutes per
-// class.  The compiler does not see that it reads memory, so lds_fence() (or
-// __syncwarp) stands between it and plain accesses to the same rows.
+// class.  The compiler does not see that it reads memory, so a barrier of the
+// warp or CTA stands between it and plain accesses to the same rows.
 __device__ __forceinline__ double lds(const double *p)
 {
     double v;
     asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"((unsigned)__cvta_generic_to_shared(p)));
     return v;
-}
-
-__device__ __forceinline__ void lds_fence()
-{
-    asm volatile("" ::: "memory");
 }
 
 // (t, u, v) of a compact Hermite index, at compile time
@@ -909,38 +906,6 @@ __device__ void group_herm(double *sm, int tid, int k0, int kg, const GroupInfo 
                         if constexpr (NIT > 0)
 #pragma unroll
                             for (int h = 0; h < Lay::NRH; ++h) Rl[h * RS] = R[h];
-                    } else if constexpr (!Lay::PASSES) {
-                        double Xd[nherm(L)];
-                        hermite_density<LA, LB, LC, LD, 0, L>(Fl, s2, Xd);
-                        // R in this lane's column, level by level.  Before the last level, the
-                        // top order, which only T needs, is formed from level 1 and not stored.
-                        Rl[0] = base[LM];
-                        static_for<LM>([&](auto I) {
-                            constexpr int n = LM - 1 - decltype(I)::value;
-                            if constexpr (n == 0) {
-                                lds_fence();
-                                static_for<nherm(LM) - nherm(L)>([&](auto J) {
-                                    constexpr int h = nherm(L) + decltype(J)::value;
-                                    constexpr Triple x = herm_triple(h);
-                                    constexpr int d = x.t > 0 ? 0 : (x.u > 0 ? 1 : 2);
-                                    constexpr int c = d == 0 ? x.t : (d == 1 ? x.u : x.v);
-                                    double r = (d == 0 ? X : (d == 1 ? Y : Z)) *
-                                               lds(Rl + hidx(x.t - (d == 0), x.u - (d == 1), x.v - (d == 2)) * RS);
-                                    if constexpr (c > 1)
-                                        r += double(c - 1) *
-                                             lds(Rl + hidx(x.t - 2 * (d == 0), x.u - 2 * (d == 1), x.v - 2 * (d == 2)) * RS);
-                                    energy_terms<L, h>(r, Xd, e, T);
-                                });
-                                lds_fence();
-                            }
-                            hermite_level<RS>(Rl, nherm(LM - n < L ? LM - n : L), X, Y, Z);
-                            Rl[0] = base[n];
-                        });
-                        lds_fence();
-                        static_for<nherm(L)>([&](auto H) {
-                            constexpr int h = decltype(H)::value;
-                            energy_terms<L, h>(lds(Rl + h * RS), Xd, e, T);
-                        });
                     } else {
                         // every warp forms the scalars; then (0,0,0) of a level is written after
                         // its entries, which read the level above
@@ -952,8 +917,12 @@ __device__ void group_herm(double *sm, int tid, int k0, int kg, const GroupInfo 
                             if (warp == 0) Rl[0] = base[n];
                             quartet_sync<NW>();
                         });
-                        // a quarter of the density's products each ((dd|dd): 750, 585, 650, 675)
-                        if (warp == 0) density_pass<LA, LB, LC, LD, 0, 4>(Fl, s2, Rl, e, T);
+                        // a quarter of the density's products each ((dd|dd): 750, 585, 650, 675) or
+                        // a half ((dp|dp): 400 and 280 with more sums to close)
+                        if constexpr (NW == 2) {
+                            if (warp == 0) density_pass<LA, LB, LC, LD, 0, L - 2>(Fl, s2, Rl, e, T);
+                            else density_pass<LA, LB, LC, LD, L - 1, L>(Fl, s2, Rl, e, T);
+                        } else if (warp == 0) density_pass<LA, LB, LC, LD, 0, 4>(Fl, s2, Rl, e, T);
                         else if (warp == 1) density_pass<LA, LB, LC, LD, 5, 5>(Fl, s2, Rl, e, T);
                         else if (warp == 2) density_pass<LA, LB, LC, LD, 6, 6>(Fl, s2, Rl, e, T);
                         else density_pass<LA, LB, LC, LD, 7, L>(Fl, s2, Rl, e, T);
@@ -1068,7 +1037,7 @@ struct HermOp {
     static constexpr bool FP32 = false;
     static constexpr int L = LA + LB + LC + LD, KQ = Lay::KQ;
     static constexpr int NW = Lay::NW;  // warps per worker (a worker takes units alone)
-    static constexpr int cta_workers = L <= 3 ? 2 : 1, min_ctas = L == 3 ? 6 : (NW == 1 ? 8 : 10 - L);
+    static constexpr int cta_workers = L <= 3 ? 2 : 1, min_ctas = L == 3 ? 6 : (NW == 1 ? 8 : (NW == 2 ? 4 : 10 - L));
     // primitive quartets of a contracted one up to which ket pairs are grouped
     // (kg times it stays below): the smaller the class, the more of a quartet's
     // work is the density transform that a group shares
