@@ -1261,9 +1261,11 @@ cudaError_t launch_warp_units(K kern, int nw, int threads, size_t per_warp, int 
     return cudaGetLastError();
 }
 
-// Launch of a gradient kernel with at most gcap slabs of partial gradients.
-// Each warp's gradient lies beside its arrays while that leaves an SM four warps
-// (or what fits without), else every warp adds to a slab of its own.
+// Launch of a gradient kernel with at most gcap slabs (8 an SM) of partial
+// gradients.  Each worker's gradient lies beside its arrays while that leaves an SM
+// three quarters of the workers that fit without it (or of the 8 there are slabs
+// for), else every worker adds to a slab of its own: 36 KB a warp at 1500 atoms
+// left the fp32 kernels 4 of 8 warps.
 template <class Op>
 cudaError_t launch_lanes(int gcap, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl, const OutArgs &out,
                          const double *boys)
@@ -1273,7 +1275,7 @@ cudaError_t launch_lanes(int gcap, cudaStream_t st, const MolDesc *mols, const C
     OutArgs o = out;
     const size_t grad = sizeof(double) * 3 * (size_t)o.natom_total;
     const int fit = (int)(kCtaSmem / bytes), fit_g = (int)(kCtaSmem / (bytes + grad));
-    o.use_smem = fit_g >= (fit < 4 ? fit : 4);
+    o.use_smem = 4 * fit_g >= 3 * (fit < 8 ? fit : 8);
     const int have = o.use_smem ? fit_g : fit, nw = have < Op::cta_workers ? have : Op::cta_workers;
     return launch_warp_units(k_grad_lanes<Op>, nw, 32 * Op::NW, bytes + (o.use_smem ? grad : 0), Op::KQ,
                              o.use_smem ? gcap : (gcap > nw ? gcap / nw : 1), st, mols, cl, o, boys);
