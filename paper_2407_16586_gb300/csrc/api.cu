@@ -1077,8 +1077,8 @@ int device_tiles(tg_basis *b, const Plan &pl, const tg_options &opt, cudaStream_
                     ft.cen[c] = cen;
                     ft.mx[c] = mx;
                     if (!ps.n) continue;
-                    k_side_features<<<(nbt + 63) / 64, 64, 0, st>>>(TB, ps, fa, fb);
-                    k_side_features<<<(nkt + 63) / 64, 64, 0, st>>>(TK, ps, fa, fk);
+                    k_side_features<<<(nbt * TB + 127) / 128, 128, 0, st>>>(TB, ps, fa, fb);
+                    k_side_features<<<(nkt * TK + 127) / 128, 128, 0, st>>>(TK, ps, fa, fk);
                     k_pair_centres<<<(ps.n + 127) / 128, 128, 0, st>>>(ps, b->d_xyz, b->d_sh_atom, cen);
                     k_bra_density_max<<<nbt, 256, 0, st>>>(ps, pl.dM, b->nshell, mx);
                     launches += 4;
@@ -1324,13 +1324,11 @@ void alu_peaks(double &p64, double &p32)
 // Autotuner of the class launches: for every (class, precision) list of ex
 // with more than nsm tiles, time a sample of 2 to 4 x nsm tiles taken at a
 // fixed stride over the whole list (whose tiles run from the costliest to
-// the cheapest) and search the kernel form (thread, group,
-// warp), the grid cap (8, 4 or 2 CTAs per SM) and the unit shape (bra
-// primitive splits per tile: automatic, 1 or 4) one coordinate at a time
-// from (form 1, 8 CTAs per SM, automatic splits): the
-// fastest form, then the fastest grid cap for it, then the fastest split
-// (7 timed launches per list).  Lists left untimed keep kinds[k] = 0 (the
-// default form), grids[k] = 0 (the persistent grid) and splits[k] = 0.
+// the cheapest) and search the grid cap (8, 4 or 2 CTAs per SM) and the unit
+// shape (bra primitive splits per tile: automatic, 1 or 4) one coordinate at a
+// time from (8 CTAs per SM, automatic splits); 6 timed launches per list.  Every
+// class and precision has one kernel form, so kinds[k] stays 0 (the default);
+// lists left untimed keep grids[k] = 0 (the persistent grid) and splits[k] = 0.
 // The sample launches write into d_part and d_cnt, which the caller clears
 // afterwards.
 int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, double *d_part,
@@ -1364,27 +1362,25 @@ int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, doub
             cudaEventElapsedTime(&ms, e0, e1);
             return TG_OK;
         };
-        int bk = 1, bm = 8, bs = 0;
+        const int kind = 0;
+        int bm = 8, bs = 0;
         float best = -1.f;
-        for (int kind = 1; kind <= 3; ++kind) {
-            float ms;
-            const int rc = time_cfg(kind, bm, bs, ms);
+        for (int rep = 0; rep < 2; ++rep) {  // the first one loads the kernel
+            const int rc = time_cfg(kind, bm, bs, best);
             if (rc != TG_OK) return rc;
-            if (best < 0.f || ms < best) best = ms, bk = kind;
         }
         for (int mult : {4, 2}) {
             float ms;
-            const int rc = time_cfg(bk, mult, bs, ms);
+            const int rc = time_cfg(kind, mult, bs, ms);
             if (rc != TG_OK) return rc;
             if (ms < best) best = ms, bm = mult;
         }
         for (int split : {1, 4}) {
             float ms;
-            const int rc = time_cfg(bk, bm, split, ms);
+            const int rc = time_cfg(kind, bm, split, ms);
             if (rc != TG_OK) return rc;
             if (ms < best) best = ms, bs = split;
         }
-        kinds[k] = bk;
         grids[k] = std::min(G, bm * nsm);
         splits[k] = bs;
     }

@@ -86,21 +86,29 @@ __global__ void k_tile_features(int ntiles, const TileRef *tiles, FeatureArgs fa
 // Bound: the fp64 pipe (the 128 centre distances, 6 instructions each).  The plan
 // of the 300-atom workload (3.1e7 tiles), of which features took 184 ms, went
 // from 231 to 97 ms.
+// One pair per thread, bsz (8 or 16) threads a tile: a thread that walks the up to
+// 16 x 36 primitive pairs of a tile alone waits 30 us for its loads.
 __global__ void k_side_features(int bsz, PairSet ps, FeatureArgs fa, SideFeature *out)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t * bsz >= ps.n) return;
-    const int lo = t * bsz, hi = min(ps.n, lo + bsz);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, t = i / bsz, lo = t * bsz;
     double q = 0, qd = 0, m = 0, e2 = 0, p = 1e300;
-    for (int i = lo; i < hi; ++i) {
-        q = fmax(q, ps.Q[i]);
-        qd = fmax(qd, ps.Qd[i]);
+    if (i < ps.n) {
+        q = ps.Q[i];
+        qd = ps.Qd[i];
         const int a = ps.sa[i], b = ps.sb[i];
-        m = fmax(m, fa.M[(size_t)a * fa.nshell + b]);
+        m = fa.M[(size_t)a * fa.nshell + b];
         const double *A = fa.xyz + 3 * fa.sh_atom[a], *B = fa.xyz + 3 * fa.sh_atom[b];
-        e2 = fmax(e2, (A[0] - B[0]) * (A[0] - B[0]) + (A[1] - B[1]) * (A[1] - B[1]) + (A[2] - B[2]) * (A[2] - B[2]));
+        e2 = (A[0] - B[0]) * (A[0] - B[0]) + (A[1] - B[1]) * (A[1] - B[1]) + (A[2] - B[2]) * (A[2] - B[2]);
         for (int k = 0; k < ps.np[i]; ++k) p = fmin(p, fa.pp_p[ps.poff[i] + k]);
     }
+    for (int o = bsz / 2; o > 0; o /= 2) {
+        q = fmax(q, __shfl_xor_sync(0xffffffffu, q, o));
+        qd = fmax(qd, __shfl_xor_sync(0xffffffffu, qd, o));
+        m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        e2 = fmax(e2, __shfl_xor_sync(0xffffffffu, e2, o));
+        p = fmin(p, __shfl_xor_sync(0xffffffffu, p, o));
+    }
+    if (i != lo || lo >= ps.n) return;
     SideFeature f;
     f.q = q;
     f.qd = qd;

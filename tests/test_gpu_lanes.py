@@ -1,7 +1,8 @@
 """The lane kernels at the sizes where their splits change: one and many
 primitives per shell (blocks of bra primitive pairs, partly filled passes,
 groups of ket pairs with different counts), a molecule whose gradient no
-longer fits beside the kernels' arrays, two handles at work on two streams.
+longer fits beside the kernels' arrays, two handles at work on two streams,
+and the tile features of the device planner against those of the samples.
 
 Tolerance: fp64 throughout; the gradient agrees with the oracle to 1e-12 of
 the largest component plus 1e-11 (rounding of sums of up to 10^6 fp64 terms of
@@ -44,7 +45,7 @@ def _system(shells, natom=3, seed=5):
 SHAPES = {
     # every shell one primitive: one primitive quartet per contracted quartet
     "one": [(0, 0, 1), (0, 1, 1), (0, 2, 1), (1, 0, 1), (1, 1, 1), (1, 2, 1), (2, 0, 1), (2, 1, 1), (2, 2, 1)],
-    # counts next to the 32 lanes: 31 = 31 x 1 is not reachable, 2 x 16 = 32 and 3 x 11 = 33 are
+    # pair counts at and next to the 32 lanes: 2 x 16 = 32, 3 x 11 = 33
     "near32": [(0, 0, 16), (1, 0, 2), (1, 1, 11), (2, 1, 3), (2, 2, 2), (0, 2, 1)],
     # the largest contraction a shell may have beside single primitives
     "deep": [(0, 1, 16), (1, 2, 5), (2, 0, 16), (2, 1, 1)],
@@ -100,3 +101,26 @@ def test_two_handles_on_two_streams(tg):
         assert len(got[i]) == 5
         for g in got[i]:
             assert np.array_equal(g, alone[i])
+
+
+@pytest.mark.parametrize("size", [(5, 2, 0), (14, 3, 3), (12, 5, 7)])
+def test_planner_features_route_as_the_sampled_ones(tg, size):
+    """The device planner's tile features come from tables, those of
+    tile_samples from the tiles' pairs.  All tiles go to fp32 exactly when the
+    squared upper edges of their routing bins (8 per octave) sum to at most
+    mixed_tol^2, so the threshold computed from the sampled features has to
+    switch the planner's route (ragged tiles and tiles of one class with itself
+    among them)."""
+    import os
+    router = tg.Router(path=os.path.join(os.path.dirname(tg.__file__), "data", "router.bin"))
+    s = synth.molecule(*size)
+    b = tg.Basis(s)
+    X = b.tile_samples(s["pairs"], stride=1, cap=2000000)[0]
+    _, _, _, (margin, eps_rel, _) = router.get()
+    e = float(eps_rel) * 10.0 ** (router.predict(X).astype(np.float64) + float(margin))
+    upper = 2.0 ** ((np.floor(np.log2(e) * 8.0) + 1.0) / 8.0)
+    tol = float(np.sqrt(np.sum(upper ** 2)))
+    for f, all32 in ((1.0 + 1e-6, True), (1.0 - 1e-6, False)):
+        st = b.grad2e(s["pairs"], precision=tg.TG_MIXED_LEARNED, router=router, mixed_tol=tol * f)[1]
+        assert st["tiles"] == len(X)
+        assert (st["fp32_quartets"] == st["quartets"]) == all32
