@@ -83,8 +83,9 @@ extern "C" {
 /* tg_options.kernel_kind: which class-kernel form evaluates a class (every
  * form gives the same result to rounding; a form not compiled for a class
  * falls back to the class default) */
-#define TG_KERNEL_DEFAULT 0   /* per-class default */
-#define TG_KERNEL_THREAD 1    /* one contracted quartet per thread */
+#define TG_KERNEL_DEFAULT 0   /* per-class default: one primitive quartet per lane, but the warp form for
+                                 (dd|pp), (dd|ds) and the group form for (dd|dp), (dd|dd) in fp32 */
+#define TG_KERNEL_THREAD 1    /* one contracted quartet per thread (compiled for no class now) */
 #define TG_KERNEL_GROUP 2     /* a group of 32-128 threads per quartet, arrays in shared memory */
 #define TG_KERNEL_WARP 3      /* one warp per quartet, every phase spread over its 32 lanes */
 
@@ -262,11 +263,10 @@ int tg_fock2e(const tg_basis *b, int npair, const tg_fpair *pairs, const tg_opti
  * every run (their contents may change, the plan does not), otherwise they
  * are copied at creation.  opt->autotune = 1 autotunes every class list
  * on a sample of 2 to 4 x (SM count) of its tiles taken at a fixed stride
- * over the whole list: the kernel form (thread, group or
- * warp), the persistent grid (8, 4 or 2 CTAs per SM) and the work-unit shape
- * (bra primitive splits per tile: automatic, 1 or 4), searched one
- * coordinate at a time (form, then grid, then splits; 7 timed launches per
- * list), keeping the fastest.
+ * over the whole list: the persistent grid (8, 4 or 2 CTAs per SM) and the
+ * work-unit shape (bra primitive splits per tile: automatic, 1 or 4),
+ * searched one coordinate at a time (grid, then splits; 6 timed launches per
+ * list), keeping the fastest; every class and precision has one kernel form.
  * tg_batch_run replays the graph on opt->stream and writes grads[m]
  * (natom_m * 3, host unless device_ptrs).  Not part of the paper, which
  * evaluates one system at a time (Sec. II.C). */

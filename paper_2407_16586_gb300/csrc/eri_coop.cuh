@@ -1,8 +1,8 @@
-// Cooperative derivative-ERI class kernel for the large angular classes.
+// Cooperative derivative-ERI class kernel: the fp32 route of (dd|dp) and (dd|dd).
 //
-// Same integrals and density contraction as quartet_fp64 / quartet_fp32r
-// (eri_grad.cuh), reorganised for a group of GS threads that shares one
-// contracted quartet, with every array in shared memory.  Per bra primitive
+// The integrals and density contraction of eri_lane32.cuh, organised for a group
+// of GS threads that shares one contracted quartet, with every array in shared
+// memory.  Per bra primitive
 // pair p and ket primitive pair q (both operators s = full, lr):
 //
 //   W_s[cd][h1] += sum_h2 (-1)^|h2| E^{cd}_{h2}(q) R_s[h1+h2](p,q)    (over q)
@@ -446,7 +446,7 @@ __device__ void quartet_coop(F *sm, int lane, int bar, const GeoArgs &geo, const
 
 // Persistent cooperative class kernel: 128 threads = 128/GS groups; group g
 // takes quartets g, g + 128/GS, ... of every tile; the tile's 12 x TILE
-// contributions are then added in the same fixed order as k_grad.
+// contributions are then added in a fixed order (tile_reduce).
 template <int LA, int LB, int LC, int LD, typename F, int GS>
 __global__ void __launch_bounds__(TILE) k_grad_coop(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out,
                                                     const double *__restrict__ boys)

@@ -631,7 +631,7 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
 
 // Persistent warp-cooperative class kernel: 4 warps per CTA, warp w takes
 // quartets w, w + 4, ... of each unit (tile, chunk, split); the tile's
-// 12 x TILE contributions are then added in the same fixed order as k_grad.
+// 12 x TILE contributions are then added in a fixed order (tile_reduce).
 template <int LA, int LB, int LC, int LD, typename F>
 __global__ void __launch_bounds__(TILE, 2) k_grad_warp(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out,
                                                     const double *__restrict__ boys)
