@@ -611,8 +611,9 @@ cudaError_t launch_coop(int gcap, size_t smem, cudaStream_t st, const MolDesc *m
                         const OutArgs &out, const double *boys)
 {
     using C = CoopChoice<LA, LB, LC, LD, F>;
-    return launch_units(k_grad_coop<LA, LB, LC, LD, F, C::GS>, TILE / C::GS, gcap, smem + C::bytes_all(), st, mols,
-                        cl, out, boys);
+    OutArgs o = out;
+    const size_t sm = unit_smem(C::bytes_all(), smem, o);
+    return launch_units(k_grad_coop<LA, LB, LC, LD, F, C::GS>, TILE / C::GS, gcap, sm, st, mols, cl, o, boys);
 }
 
 }  // namespace tg

@@ -102,6 +102,23 @@ __device__ __forceinline__ bool keep_quartet(const ScreenArgs &scr, const PairSe
     return true;
 }
 
+// Dynamic shared memory a CTA of a class kernel may take (227 KB less 4 KB for
+// static arrays).
+constexpr size_t kCtaSmem = 223 * 1024;
+
+// Shared memory of a CTA-wide form: its arrays beside smem, the tile staging
+// with, where out.use_smem says so, the gradient of the largest molecule.
+// Where the three together pass the limit (the 99 KB of (dd|pp) from 4 747 atoms)
+// the gradient stays in the CTA's slab.
+inline size_t unit_smem(size_t arrays, size_t smem, OutArgs &out)
+{
+    if (out.use_smem && arrays + smem > kCtaSmem) {
+        out.use_smem = 0;
+        smem -= sizeof(double) * 3 * (size_t)out.natom_max;
+    }
+    return arrays + smem;
+}
+
 // Launch of a persistent class kernel over units: the grid is the smaller of
 // gcap and the kernel's resident CTAs per SM times the SM count, and each
 // tile is cut into nchunk x nsplit units (nchunk only for the cooperative

@@ -1222,9 +1222,6 @@ __global__ void __launch_bounds__(32 * Op::NW * Op::cta_workers, Op::min_ctas)
     }
 }
 
-// Dynamic shared memory a CTA may take beside the static group records.
-constexpr size_t kCtaSmem = 223 * 1024;
-
 // Launch of a kernel over warp units (tile, chunk, split) with at most gmax
 // CTAs of nw workers (warps, or teams of threads / 32 warps), which take groups of
 // up to kets ket pairs.  Tiles are

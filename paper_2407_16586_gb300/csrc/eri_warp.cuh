@@ -811,8 +811,9 @@ template <int LA, int LB, int LC, int LD, typename F>
 cudaError_t launch_warp(int gcap, size_t smem, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl,
                         const OutArgs &out, const double *boys)
 {
-    return launch_units(k_grad_warp<LA, LB, LC, LD, F>, TILE / 32, gcap, smem + warp_kernel_smem<LA, LB, LC, LD, F>(),
-                        st, mols, cl, out, boys);
+    OutArgs o = out;
+    const size_t sm = unit_smem(warp_kernel_smem<LA, LB, LC, LD, F>(), smem, o);
+    return launch_units(k_grad_warp<LA, LB, LC, LD, F>, TILE / 32, gcap, sm, st, mols, cl, o, boys);
 }
 
 }  // namespace tg

@@ -1,0 +1,51 @@
+"""Calls at the limits of what is shared or scarce: molecules whose gradient
+just fits or no longer fits beside a kernel's arrays.
+
+Bounds: the fp32 route to 6e-6 of the largest component, as elsewhere."""
+import numpy as np
+import pytest
+
+from paper_2407_16586_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tg():
+    from paper_2407_16586_gb300 import build
+    build.build()
+    import paper_2407_16586_gb300 as m
+    return m
+
+
+def _system(shells, xyz, seed=5):
+    """shells: (atom, l, primitives); two random density pairs with both operators."""
+    rng = np.random.default_rng(seed)
+    ex = [np.sort(np.exp(rng.uniform(np.log(0.2), np.log(60.0), k)))[::-1] for _a, _l, k in shells]
+    s = dict(natom=len(xyz), xyz=np.asarray(xyz, float), shell_atom=np.array([a for a, _l, _k in shells], np.int32),
+             shell_l=np.array([l for _a, l, _k in shells], np.int32),
+             shell_nprim=np.array([k for _a, _l, k in shells], np.int32),
+             exps=np.concatenate(ex), coefs=np.concatenate([rng.uniform(0.2, 1.0, len(e)) for e in ex]))
+    n = s["nbf"] = synth.nbf_of(s["shell_l"])
+    m = [rng.normal(size=(n, n)) / n for _ in range(3)]
+    s["pairs"] = [(m[0], m[1], 1.0, -0.3, -0.7, 0.35), (m[2], m[2], 0.5, 0.2, 0.0, 0.0)]
+    return s
+
+
+def _padded(natom):
+    """Three atoms with s, p and d shells; the others carry none."""
+    xyz = np.zeros((natom, 3))
+    xyz[:3] = [[0.0, 0.1, -0.2], [1.6, 0.4, 0.3], [-0.5, 1.5, 0.9]]
+    xyz[3:] = 50.0 + np.arange(3 * (natom - 3)).reshape(-1, 3)
+    return _system([(a, l, 1) for a in range(3) for l in range(3)], xyz)
+
+
+@pytest.mark.parametrize("natom", [4746, 4747, 5500, 6173, 6174])
+def test_fp32_gradient_at_the_shared_memory_limit(tg, natom):
+    """From 4747 to 6173 atoms the gradient (111 to 145 KB) fits in a CTA's shared
+    memory, but not beside the arrays of (dd|pp) as well."""
+    ref = tg.Basis(_padded(3)).grad2e(_padded(3)["pairs"], screen_tol=0.0)[0]
+    s = _padded(natom)
+    g = tg.Basis(s).grad2e(s["pairs"], screen_tol=0.0, precision=tg.TG_FP32)[0]
+    assert np.abs(g[:3] - ref).max() <= 6e-6 * np.abs(ref).max()
+    assert not g[3:].any()
