@@ -103,8 +103,18 @@ __device__ __forceinline__ bool keep_quartet(const ScreenArgs &scr, const PairSe
 }
 
 // Dynamic shared memory a CTA of a class kernel may take (227 KB less 4 KB for
-// static arrays).
+// static arrays).  Every launch allows its kernel this much, whatever it needs
+// itself: the attribute belongs to the kernel in the whole context, and a value
+// of the launch's own would refuse a larger molecule's launch of another thread
+// that had set it just before.
 constexpr size_t kCtaSmem = 223 * 1024;
+
+template <typename K>
+cudaError_t allow_cta_smem(K kern, size_t sm)
+{
+    if (sm > kCtaSmem) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCtaSmem);
+}
 
 // Shared memory of a CTA-wide form: its arrays beside smem, the tile staging
 // with, where out.use_smem says so, the gradient of the largest molecule.
@@ -129,7 +139,7 @@ template <typename K>
 cudaError_t launch_units(K kern, int ngroups, int gcap, size_t sm, cudaStream_t st, const MolDesc *mols,
                          ClassLaunch cl, const OutArgs &out, const double *boys, int block = TILE)
 {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_cta_smem(kern, sm);
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 1, per = 1;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

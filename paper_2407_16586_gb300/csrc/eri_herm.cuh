@@ -1239,7 +1239,7 @@ cudaError_t launch_warp_units(K kern, int nw, int threads, size_t per_warp, int 
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const size_t sm = per_warp * nw;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess) return e;
+    if ((e = allow_cta_smem(kern, sm)) != cudaSuccess) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads * nw, sm)) != cudaSuccess) return e;
     if (gmax > (long long)(per > 0 ? per : 1) * nsm) gmax = (long long)(per > 0 ? per : 1) * nsm;
     cl.nchunk = 1;

@@ -1,7 +1,10 @@
 """Calls at the limits of what is shared or scarce: molecules whose gradient
-just fits or no longer fits beside a kernel's arrays.
+just fits or no longer fits beside a kernel's arrays, and kernel attributes
+while two threads work on molecules of different sizes.
 
-Bounds: the fp32 route to 6e-6 of the largest component, as elsewhere."""
+Bounds: the same sums in the same order are bitwise equal; the fp32 route to 6e-6 of the largest component, as elsewhere."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -49,3 +52,31 @@ def test_fp32_gradient_at_the_shared_memory_limit(tg, natom):
     g = tg.Basis(s).grad2e(s["pairs"], screen_tol=0.0, precision=tg.TG_FP32)[0]
     assert np.abs(g[:3] - ref).max() <= 6e-6 * np.abs(ref).max()
     assert not g[3:].any()
+
+
+def test_two_threads_on_molecules_of_different_sizes(tg):
+    """A kernel's shared-memory limit is common to all threads of the process;
+    a launch for 1200 atoms needs more of it than one for three."""
+    systems = [_padded(3), _padded(1200)]
+    bases = [tg.Basis(s) for s in systems]
+    kw = dict(screen_tol=0.0)
+    alone = [[b.grad2e(s["pairs"], precision=p, **kw)[0] for p in (tg.TG_FP64, tg.TG_FP32)]
+             for b, s in zip(bases, systems)]
+    got, errors = [[], []], []
+
+    def work(i):
+        try:
+            for _ in range(100):
+                got[i].append([bases[i].grad2e(systems[i]["pairs"], precision=p, **kw)[0]
+                               for p in (tg.TG_FP64, tg.TG_FP32)])
+        except tg.TGError as e:
+            errors.append(e)
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for i in range(2):
+        for g in got[i]:
+            assert np.array_equal(g[0], alone[i][0]) and np.array_equal(g[1], alone[i][1])
