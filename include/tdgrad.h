@@ -60,8 +60,9 @@ extern "C" {
                                  beyond int32 indexing: nshell (nshell+1)/2 >= 2^31 shell
                                  pairs, or >= 2^31 primitive pairs kept in one call */
 #define TG_ENOMEM (-3)        /* device or host allocation failed (for tests: while the environment
-                                 variable TDGRAD_FAIL_ALLOC=1 is set, every growth of the library's
-                                 device work areas fails this way, without a CUDA call) */
+                                 variable TDGRAD_FAIL_ALLOC is set to a number of bytes, every growth
+                                 of one of the library's device work areas to more than that, with 1
+                                 every growth, fails this way, without a CUDA call) */
 #define TG_ECUDA (-4)         /* a CUDA runtime call failed */
 #define TG_ETIMEOUT (-5)      /* reserved: a bounded device wait expired.  No kernel of this
                                  version waits on another CTA or a flag, so no call returns it. */

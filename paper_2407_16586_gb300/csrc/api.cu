@@ -22,13 +22,15 @@ using namespace tg;
 
 namespace {
 
-// Test hook for the allocation-failure path: while the environment variable
-// TDGRAD_FAIL_ALLOC is set to 1, every arena growth fails as if cudaMalloc had
-// run out of device memory (checked on the host; no CUDA call is made).
-bool alloc_failure_injected()
+// Test hook for the allocation-failure paths: while the environment variable
+// TDGRAD_FAIL_ALLOC is set to a number of bytes, every arena growth to more
+// than that (1: every growth) fails as if cudaMalloc had run out of device
+// memory (checked on the host; no CUDA call is made).
+bool alloc_failure_injected(size_t bytes)
 {
     const char *e = std::getenv("TDGRAD_FAIL_ALLOC");
-    return e && e[0] == '1' && e[1] == 0;
+    const long long limit = e ? std::atoll(e) : 0;
+    return limit > 0 && bytes > (size_t)limit;
 }
 
 struct DevArena {
@@ -38,7 +40,7 @@ struct DevArena {
     cudaError_t reserve(size_t bytes)
     {
         if (bytes <= cap) return cudaSuccess;
-        if (alloc_failure_injected()) return cudaErrorMemoryAllocation;
+        if (alloc_failure_injected(bytes)) return cudaErrorMemoryAllocation;
         if (p) cudaFree(p);
         p = nullptr;
         cap = 0;
@@ -1020,24 +1022,40 @@ int device_tiles(tg_basis *b, const Plan &pl, const tg_options &opt, cudaStream_
     constexpr long long RCHUNK = 1LL << 25;
     const long long nout = snr > 1 ? std::min(ntl, ntl / snr + 2 * NQC) : ntl;  // a class list of n deals <= n/snr + 1
     const long long nch = std::min(ntl, RCHUNK);
-    size_t needB = al(sizeof(uint4) * ntl) + al(sizeof(uint4) * nout) + al(sizeof(float) * ntl) +
-                   al(sizeof(int) * ntl) + 4096;
-    // feature tables per pair class; the rows of density maxima (nshell doubles a
-    // bra tile: 94 MB for 300 atoms, 6.6 GB for 1500) only up to 16 GB, beyond
-    // which every tile gathers its block factors itself
-    size_t mxbytes = 0;
-    for (int c = 0; c < NPC; ++c) mxbytes += al(sizeof(double) * (size_t)ra.t[c].nbt * b->nshell);
-    const bool tables = learned && mxbytes <= ((size_t)16 << 30);
-    if (learned) needB += al(sizeof(float) * nch * NFEAT) + al(sizeof(float) * nch);
-    if (learned && !tables) needB += al(sizeof(TileRef) * nch);
-    if (tables) {
-        needB += mxbytes;
-        for (int c = 0; c < NPC; ++c)
-            needB += al(sizeof(SideFeature) * ra.t[c].nbt) + al(sizeof(SideFeature) * ra.t[c].nkt) +
-                     al(sizeof(double) * 3 * pl.cls[c].size());
-    }
+    const size_t needT = al(sizeof(uint4) * ntl) + al(sizeof(uint4) * nout) + al(sizeof(float) * ntl) +
+                         al(sizeof(int) * ntl) + 4096 +
+                         (learned ? al(sizeof(float) * nch * NFEAT) + al(sizeof(float) * nch) : 0);
+    // The learned route's features come from tables per pair class, whose rows of
+    // density maxima take nshell doubles a bra tile (94 MB for 300 atoms, 6.6 GB for
+    // 1500), or are gathered tile by tile, which takes a TileRef a tile and more time
+    // (features of the 300-atom plan 184 against 50 ms).  The values are the same bit
+    // for bit.  Tables if the work area holds them already or they take at most a
+    // quarter of the memory left beside the tile lists; what is allocated decides, so
+    // that a call which fits without them never fails for them.
     DevArena &B = b->ws4;
-    TG_CUDA(B.reserve(needB));
+    size_t mxbytes = 0, needM = needT;
+    for (int c = 0; c < NPC; ++c) {
+        const size_t mx = al(sizeof(double) * (size_t)ra.t[c].nbt * b->nshell);
+        mxbytes += mx;
+        needM += mx + al(sizeof(SideFeature) * ra.t[c].nbt) + al(sizeof(SideFeature) * ra.t[c].nkt) +
+                 al(sizeof(double) * 3 * pl.cls[c].size());
+    }
+    bool tables = learned;
+    if (learned && needM > B.cap) {
+        size_t avail = 0, total = 0;
+        TG_CUDA(cudaMemGetInfo(&avail, &total));
+        avail += B.cap;  // given back before the area grows
+        tables = needT < avail && mxbytes <= (avail - needT) / 4;
+        if (tables) {
+            const cudaError_t e = B.reserve(needM);
+            if (e != cudaSuccess) {
+                if (e != cudaErrorMemoryAllocation) TG_CUDA(e);
+                cudaGetLastError();
+                tables = false;
+            }
+        }
+    }
+    if (!tables) TG_CUDA(B.reserve(needT + (learned ? al(sizeof(TileRef) * nch) : 0)));
     B.used = 0;
     uint4 *d_raw = B.take<uint4>(ntl), *d_out = B.take<uint4>(nout);
     float *d_bnd = B.take<float>(ntl);

@@ -1,8 +1,10 @@
 """Calls at the limits of what is shared or scarce: molecules whose gradient
-just fits or no longer fits beside a kernel's arrays, and kernel attributes
-while two threads work on molecules of different sizes.
+just fits or no longer fits beside a kernel's arrays, kernel attributes
+while two threads work on molecules of different sizes, and device memory too
+short for the router's tables.
 
 Bounds: the same sums in the same order are bitwise equal; the fp32 route to 6e-6 of the largest component, as elsewhere."""
+import os
 import threading
 
 import numpy as np
@@ -80,3 +82,30 @@ def test_two_threads_on_molecules_of_different_sizes(tg):
     for i in range(2):
         for g in got[i]:
             assert np.array_equal(g[0], alone[i][0]) and np.array_equal(g[1], alone[i][1])
+
+
+def test_learned_route_without_room_for_its_tables(tg, monkeypatch):
+    """Where the router's feature tables do not fit, the tiles gather their
+    features themselves: the same route and the same gradient, bit for bit."""
+    natom = 100
+    xyz = np.zeros((natom, 3))
+    xyz[:, 0] = 30.0 * np.arange(natom)  # pairs on one atom only: few tiles, many shells
+    s = _system([(a, l, k) for a in range(natom) for l, k in ((0, 2), (0, 1), (1, 1))], xyz)
+    router = tg.Router(path=os.path.join(os.path.dirname(tg.__file__), "data", "router.bin"))
+    kw = dict(precision=tg.TG_MIXED_LEARNED, router=router)
+    ample, tight = tg.Basis(s), tg.Basis(s)
+    st = tight.grad2e(s["pairs"])[1]  # the other work areas have their sizes after this
+    # 124 B a tile without tables; with them 108 B and 8 nshell a bra tile of 16 pairs
+    limit = 124 * st["tiles"] + 8192
+    assert 108 * st["tiles"] + 8 * len(s["shell_l"]) * (st["pairs"] // 16) > limit
+    mixed = 0
+    for tol in (1e-5, 1e-6, 1e-7, 1e-8, 1e-9, 1e-10):
+        g, sa = ample.grad2e(s["pairs"], mixed_tol=tol, **kw)
+        monkeypatch.setenv("TDGRAD_FAIL_ALLOC", str(limit))
+        h, sb = tight.grad2e(s["pairs"], mixed_tol=tol, **kw)
+        monkeypatch.delenv("TDGRAD_FAIL_ALLOC")
+        assert sb["launches"] < sa["launches"]  # the tables take launches of their own
+        assert sb["fp32_quartets"] == sa["fp32_quartets"]
+        assert np.array_equal(g, h)
+        mixed += 0 < sa["fp32_quartets"] < sa["quartets"]
+    assert mixed
