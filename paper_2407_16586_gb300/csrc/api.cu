@@ -116,9 +116,25 @@ struct SideStreams {
         *this = SideStreams();
     }
 };
-// sets of partial-gradient slabs: one per side stream, so that concurrent
-// launches never add to the same slab and every sum keeps a fixed order
-constexpr int kSlabSets = SideStreams::N;
+// Partial-gradient slabs (natom x 3 doubles each): a launch of at most per CTAs
+// adds to one set of them, and every side stream in use has a set of its own, so
+// that concurrent launches never add to the same slab and every sum keeps a
+// fixed order.
+struct Slabs {
+    int sets, per;
+    size_t count() const { return (size_t)sets * per; }
+};
+// Six sets of 8 an SM (175 KB an atom on 152 SMs) while they take at most 4 GiB
+// (24 500 atoms), beyond that as many sets as do; where one does not, and where
+// least asks for it because memory is short, one set of 4 an SM (15 KB an atom).
+inline Slabs slab_plan(int nsm, long long natom, bool least)
+{
+    const size_t grad = sizeof(double) * 3 * (size_t)natom, budget = (size_t)4 << 30;
+    Slabs s = {SideStreams::N, std::max(1, 8 * nsm)};
+    while (s.sets > 1 && s.count() * grad > budget) --s.sets;
+    if (least || s.count() * grad > budget) s = {1, std::max(1, 4 * nsm)};
+    return s;
+}
 
 struct tg_router {
     float params[NPARAM];
@@ -427,7 +443,7 @@ struct Plan {
     unsigned class_mask = 0;
     bool fock = false;  // Fock build: linear bounds, Q only
     int launches = 0;
-    int G = 1;
+    Slabs slabs = {1, 1};
     PairSet set(int c) const
     {
         PairSet s;
@@ -479,7 +495,7 @@ int check_pairs(int npair, const tg_pair *pairs, const tg_options &opt, double &
 
 // Densities, block factors, screened pairs, primitive pairs, unrouted tiles.
 int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &opt, cudaStream_t st, Plan &pl,
-              bool host_tiles = true, bool fock = false)
+              bool host_tiles = true, bool fock = false, bool slabs = false)
 {
     double omega;
     int use_lr;
@@ -589,7 +605,7 @@ int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &op
     // primitive-pair offsets are int32 on the device
     if (npp_max > 0x7fffffffLL) return TG_EUNSUPPORTED;
     // ---- arena 2: pair arrays, primitive-pair records, tiles, features, partials
-    pl.G = std::max(1, 8 * b->nsm);  // partial slabs: up to 8 resident CTAs per SM
+    pl.slabs = slab_plan(b->nsm, natom, false);
     {
         const size_t np_k = (size_t)std::max<long long>(nk_all, 1);
         const size_t npp = (size_t)std::max<long long>(npp_max, 1);
@@ -599,13 +615,21 @@ int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &op
             for (int Qc = 0; Qc <= P; ++Qc)
                 ntl_max += (long long)((pl.cls[P].size() + TB - 1) / TB) * ((pl.cls[Qc].size() + TK - 1) / TK);
         const size_t ntl = host_tiles ? (size_t)std::max<long long>(ntl_max, 1) : 1;
-        const size_t need2 = 6 * al(sizeof(int) * np_k) + 2 * al(sizeof(double) * np_k) +
+        const size_t need0 = 6 * al(sizeof(int) * np_k) + 2 * al(sizeof(double) * np_k) +
                              10 * al(sizeof(double) * npp) + 12 * al(sizeof(float) * npp) + al(sizeof(uint4) * ntl) +
                              al(sizeof(MolDesc)) +
                              al(sizeof(TileRef) * ntl) + al(sizeof(float) * ntl * (NFEAT + 1)) +
-                             al(sizeof(double) * (size_t)kSlabSets * pl.G * 3 * natom) + 8192;
+                             8192;
         DevArena &V = b->ws2;
-        TG_CUDA(V.reserve(need2));
+        // with the slabs of a caller that keeps them in this area
+        auto need2 = [&]() { return need0 + (slabs ? al(sizeof(double) * pl.slabs.count() * 3 * natom) : 0); };
+        cudaError_t e = V.reserve(need2());
+        if (slabs && e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            pl.slabs = slab_plan(b->nsm, natom, true);
+            e = V.reserve(need2());
+        }
+        TG_CUDA(e);
         V.used = 0;
         pl.d_sa = V.take<int>(np_k);
         pl.d_sb = V.take<int>(np_k);
@@ -1244,10 +1268,11 @@ void build_exec(const std::vector<const Plan *> &plans, const std::vector<std::v
 // persistent grid of list k; with dump != nullptr every quartet's 12
 // components go to dump[(list position * TILE + thread) * 12 + c].  With side
 // streams the lists are launched over them, the classes with the longest
-// quartets first, list i on stream i mod N into slab set i mod N (the caller
-// has cleared all sets); without, on st into the first set.
+// quartets first, list i on stream i mod sl.sets into slab set i mod sl.sets (the
+// caller has cleared all sets); without, on st into the first set.
 int launch_exec(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, double *d_part,
-                unsigned long long *dcnt, double *dump, const double *boys, int G, const int *grids, bool timing,
+                unsigned long long *dcnt, double *dump, const double *boys, const Slabs &sl, const int *grids,
+                bool timing,
                 cudaStream_t st, tg_stats *stats, int &launches, const int *kinds = nullptr, int kind_all = 0,
                 int tile_rank = 0, int tile_nranks = 1, const int *splits = nullptr, SideStreams *side = nullptr)
 {
@@ -1295,11 +1320,11 @@ int launch_exec(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, dou
             cl.split_req = splits ? splits[k] : 0;
             OutArgs o = out;
             o.counters = dcnt + NCNT * qc;
-            const int on = nlist++ % SideStreams::N;
+            const int on = nlist++ % sl.sets;
             cudaStream_t ls = side ? side->s[on] : st;
-            if (side) o.partials = d_part + (size_t)on * G * 3 * ex.natom_total;
+            if (side) o.partials = d_part + (size_t)on * sl.per * 3 * ex.natom_total;
             if (dump) o.dump = dump + (size_t)ex.off[k] * TILE * 12;
-            const int grid = std::min(G, (grids && grids[k] > 0) ? grids[k] : G);  // cap; the launcher sizes it
+            const int grid = std::min(sl.per, (grids && grids[k] > 0) ? grids[k] : sl.per);  // cap; the launcher sizes it
             if (timing) cudaEventRecord(e0, st);
             cudaError_t e = kClassLaunchers[qc](r, grid, smem, ls, d_mols, cl, o, boys);
             if (e != cudaSuccess) {
@@ -1350,7 +1375,7 @@ void alu_peaks(double &p64, double &p32)
 // The sample launches write into d_part and d_cnt, which the caller clears
 // afterwards.
 int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, double *d_part,
-               unsigned long long *d_cnt, const double *boys, int G, int nsm, cudaStream_t st, int *kinds,
+               unsigned long long *d_cnt, const double *boys, const Slabs &sl, int nsm, cudaStream_t st, int *kinds,
                int *grids, int *splits)
 {
     for (int k = 0; k < 2 * NQC; ++k) kinds[k] = grids[k] = splits[k] = 0;
@@ -1368,10 +1393,10 @@ int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, doub
         const int step = (int)std::max<long long>(1, nt / (2LL * nsm));
         for (int j = 0; j < 2 * NQC + 1; ++j) sub.off[j] = j <= k ? 0 : nt;
         auto time_cfg = [&](int kind, int mult, int split, float &ms) -> int {
-            std::vector<int> gr(2 * NQC, std::min(G, mult * nsm)), kd(2 * NQC, kind), sp(2 * NQC, split);
+            std::vector<int> gr(2 * NQC, std::min(sl.per, mult * nsm)), kd(2 * NQC, kind), sp(2 * NQC, split);
             int dummy = 0;
             cudaEventRecord(e0, st);
-            int rc = launch_exec(sub, d_mols, d_tiles + ex.off[k], d_part, d_cnt, nullptr, boys, G, gr.data(),
+            int rc = launch_exec(sub, d_mols, d_tiles + ex.off[k], d_part, d_cnt, nullptr, boys, sl, gr.data(),
                                  false, st, nullptr, dummy, kd.data(), 0, 0, step, sp.data());
             cudaEventRecord(e1, st);
             if (rc != TG_OK) return rc;
@@ -1399,7 +1424,7 @@ int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, doub
             if (rc != TG_OK) return rc;
             if (ms < best) best = ms, bs = split;
         }
-        grids[k] = std::min(G, bm * nsm);
+        grids[k] = std::min(sl.per, bm * nsm);
         splits[k] = bs;
     }
     return TG_OK;
@@ -1460,7 +1485,7 @@ struct tg_batch {
     double *d_part = nullptr, *d_grad = nullptr;
     unsigned long long *d_cnt = nullptr;
     std::vector<int> grids, kinds, splits;
-    int G = 1;
+    Slabs slabs = {1, 1};
     int device_ptrs = 0;
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
@@ -1485,15 +1510,15 @@ int tg_grad2e(const tg_basis *cb, int npair, const tg_pair *pairs, const tg_opti
     if (opt.precision == TG_MIXED_LEARNED && (!opt.router || !opt.router->trained)) return TG_EROUTER;
     cudaStream_t st = (cudaStream_t)opt.stream;
     Plan pl;
-    int rc = make_plan(b, npair, pairs, opt, st, pl, false);
+    int rc = make_plan(b, npair, pairs, opt, st, pl, false, false, true);
     if (rc != TG_OK) return rc;
     const int natom = b->natom;
     int launches = pl.launches;
     DevArena &V = b->ws2;
     // with per-class timing the lists run one after the other, in one slab set
-    SideStreams *side = opt.timing ? nullptr : &b->side;
-    const size_t nslab = (size_t)(side ? kSlabSets : 1) * pl.G;
-    double *d_part = V.take<double>((size_t)kSlabSets * pl.G * 3 * natom);
+    SideStreams *side = opt.timing || pl.slabs.sets == 1 ? nullptr : &b->side;
+    const size_t nslab = side ? pl.slabs.count() : (size_t)pl.slabs.per;
+    double *d_part = V.take<double>(pl.slabs.count() * 3 * natom);
     MolDesc *d_mol = V.take<MolDesc>(1);
     // the screened tile lists, routed and split per (class, precision), built on the device
     DevTiles dt;
@@ -1512,7 +1537,7 @@ int tg_grad2e(const tg_basis *cb, int npair, const tg_pair *pairs, const tg_opti
     const bool tune = opt.autotune == 1 || opt.autotune == 2;
     if (tune) {
         if (!b->tuned || opt.autotune == 2) {
-            rc = tune_lists(ex, d_mol, d_tiles, d_part, pl.dcnt, b->d_boys, pl.G, b->nsm, st, b->tune_kind,
+            rc = tune_lists(ex, d_mol, d_tiles, d_part, pl.dcnt, b->d_boys, pl.slabs, b->nsm, st, b->tune_kind,
                             b->tune_grid, b->tune_split);
             if (rc != TG_OK) return rc;
             b->tuned = true;
@@ -1529,7 +1554,7 @@ int tg_grad2e(const tg_basis *cb, int npair, const tg_pair *pairs, const tg_opti
         for (int qc = 0; qc < NQC; ++qc) stats->class_ms[qc] = stats->class_ms_fp32[qc] = 0.0;
     const double plan_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     // (a tile shard is already in the lists)
-    rc = launch_exec(ex, d_mol, d_tiles, d_part, pl.dcnt, nullptr, b->d_boys, pl.G, tune ? gr : nullptr,
+    rc = launch_exec(ex, d_mol, d_tiles, d_part, pl.dcnt, nullptr, b->d_boys, pl.slabs, tune ? gr : nullptr,
                      opt.timing != 0, st, stats, launches, tune ? kd : nullptr, opt.kernel_kind, 0, 1,
                      tune ? sp : nullptr, side);
     if (rc != TG_OK) return rc;
@@ -1542,7 +1567,7 @@ int tg_grad2e(const tg_basis *cb, int npair, const tg_pair *pairs, const tg_opti
                             opt.device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
     TG_CUDA(cudaStreamSynchronize(st));
     if (stats) {
-        fill_stats(stats, hc, pl.npairs_kept, (long long)ntl, launches, pl.G, pl.den.use_lr ? 2 : 1);
+        fill_stats(stats, hc, pl.npairs_kept, (long long)ntl, launches, pl.slabs.per, pl.den.use_lr ? 2 : 1);
         stats->plan_ms = plan_ms;
         stats->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     }
@@ -1718,7 +1743,7 @@ int tg_fock2e(const tg_basis *cb, int npair, const tg_fpair *fpairs, const tg_op
         o.fock = dF;
         if (opt.timing) cudaEventRecord(ev.a, st);
         cudaStream_t ls = side ? side->s[nlist++ % SideStreams::N] : st;
-        cudaError_t e = kFockLaunchers[qc](pl.G, ls, d_mol, cl, o, b->d_boys);
+        cudaError_t e = kFockLaunchers[qc](pl.slabs.per, ls, d_mol, cl, o, b->d_boys);
         if (e != cudaSuccess) {
             cudaGetLastError();
             rc = TG_ECUDA;
@@ -1744,7 +1769,7 @@ int tg_fock2e(const tg_basis *cb, int npair, const tg_fpair *fpairs, const tg_op
                             opt.device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
     TG_CUDA(cudaStreamSynchronize(st));
     if (stats) {
-        fill_stats(stats, hc, pl.npairs_kept, dt.ntiles, launches, pl.G, use_lr ? 2 : 1);
+        fill_stats(stats, hc, pl.npairs_kept, dt.ntiles, launches, pl.slabs.per, use_lr ? 2 : 1);
         stats->fp64_flop = 0.0;  // the gradient's FLOP count does not apply
         stats->fp64_frac_peak = 0.0;
         stats->plan_ms = plan_ms;
@@ -1772,7 +1797,7 @@ int tg_tile_samples(const tg_basis *cb, int npair, const tg_pair *pairs, const t
     if (!n) return TG_OK;
     DevArena &V = b->ws2;
     const size_t need = V.used + al(sizeof(uint4) * n) + al(sizeof(TileRef) * n) + al(sizeof(float) * n * (NFEAT + 1)) +
-                        2 * al(sizeof(double) * n * TILE * 12) + al(sizeof(double) * (size_t)pl.G * 3 * b->natom) +
+                        2 * al(sizeof(double) * n * TILE * 12) + al(sizeof(double) * (size_t)pl.slabs.per * 3 * b->natom) +
                         al(sizeof(MolDesc)) + 8192;
     if (need > V.cap) {
         // grow the plan arena, then rebuild the plan inside it
@@ -1787,7 +1812,7 @@ int tg_tile_samples(const tg_basis *cb, int npair, const tg_pair *pairs, const t
     float *d_pred = V.take<float>(n);
     double *d64 = V.take<double>(n * TILE * 12);
     double *d32 = V.take<double>(n * TILE * 12);
-    double *d_part = V.take<double>((size_t)pl.G * 3 * b->natom);
+    double *d_part = V.take<double>((size_t)pl.slabs.per * 3 * b->natom);
     MolDesc *d_mol = V.take<MolDesc>(1);
     int launches = 0;
     std::vector<float> feat;
@@ -1806,7 +1831,7 @@ int tg_tile_samples(const tg_basis *cb, int npair, const tg_pair *pairs, const t
         TG_CUDA(cudaMemsetAsync(pl.dcnt, 0, sizeof(unsigned long long) * NCNT * NQC, st));
         // the dump is written at list positions; lists are class-major with r fixed,
         // so positions run over the samples in class order
-        rc = launch_exec(ex, d_mol, d_tiles, d_part, pl.dcnt, r ? d32 : d64, b->d_boys, pl.G, nullptr, false, st,
+        rc = launch_exec(ex, d_mol, d_tiles, d_part, pl.dcnt, r ? d32 : d64, b->d_boys, pl.slabs, nullptr, false, st,
                          nullptr, launches);
         if (rc != TG_OK) return rc;
         TG_CUDA(cudaStreamSynchronize(st));
@@ -1883,7 +1908,7 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
     cudaStream_t st = (cudaStream_t)opt.stream;
     std::vector<std::vector<uint8_t>> routes(nmol);
     std::vector<const Plan *> pp(nmol);
-    int natom_total = 0, natom_max = 0, G = 1;
+    int natom_total = 0, natom_max = 0;
     for (int m = 0; m < nmol; ++m) {
         tg_basis *b = const_cast<tg_basis *>(bases[m]);
         bt->bases.push_back(b);
@@ -1901,25 +1926,36 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
         bt->atom_off.push_back(natom_total);
         natom_total += b->natom;
         natom_max = std::max(natom_max, b->natom);
-        G = std::max(G, pl.G);
         bt->pairs += pl.npairs_kept;
         pp[m] = &pl;
     }
     build_exec(pp, routes, nullptr, bt->ex);
     bt->ex.natom_total = natom_total;
     bt->ex.natom_max = natom_max;
-    bt->G = G;
+    const int nsm = std::max(1, bt->bases[0]->nsm);
     const size_t ntl = std::max<size_t>(bt->ex.tiles.size(), 1);
-    const size_t need = al(sizeof(MolDesc) * nmol) + al(sizeof(uint4) * ntl) +
-                        al(sizeof(double) * (size_t)kSlabSets * G * 3 * natom_total) + al(sizeof(double) * 3 * natom_total) +
-                        al(sizeof(unsigned long long) * NCNT * NQC) + 4096;
-    TG_CUDA(bt->arena.reserve(need));
-    bt->arena.used = 0;
-    bt->d_mols = bt->arena.take<MolDesc>(nmol);
-    bt->d_tiles = bt->arena.take<uint4>(ntl);
-    bt->d_part = bt->arena.take<double>((size_t)kSlabSets * G * 3 * natom_total);
-    bt->d_grad = bt->arena.take<double>(3 * natom_total);
-    bt->d_cnt = bt->arena.take<unsigned long long>(NCNT * NQC);
+    auto carve = [&](bool least) {
+        bt->slabs = slab_plan(nsm, natom_total, least);
+        const size_t npart = bt->slabs.count() * 3 * natom_total;
+        const size_t need = al(sizeof(MolDesc) * nmol) + al(sizeof(uint4) * ntl) + al(sizeof(double) * npart) +
+                            al(sizeof(double) * 3 * natom_total) + al(sizeof(unsigned long long) * NCNT * NQC) + 4096;
+        const cudaError_t e = bt->arena.reserve(need);
+        if (e != cudaSuccess) return e;
+        bt->arena.used = 0;
+        bt->d_mols = bt->arena.take<MolDesc>(nmol);
+        bt->d_tiles = bt->arena.take<uint4>(ntl);
+        bt->d_part = bt->arena.take<double>(npart);
+        bt->d_grad = bt->arena.take<double>(3 * natom_total);
+        bt->d_cnt = bt->arena.take<unsigned long long>(NCNT * NQC);
+        return e;
+    };
+    cudaError_t fit = carve(false);
+    if (fit == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        fit = carve(true);
+    }
+    TG_CUDA(fit);
+    const Slabs sl = bt->slabs;
     std::vector<MolDesc> mds(nmol);
     for (int m = 0; m < nmol; ++m) mds[m] = make_desc(bt->plans[m], bt->atom_off[m]);
     TG_CUDA(cudaMemcpy(bt->d_mols, mds.data(), sizeof(MolDesc) * nmol, cudaMemcpyHostToDevice));
@@ -1929,13 +1965,12 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
     const double *boys = bt->bases[0]->d_boys;
 
     // ---- autotune every (class, precision) list (tune_lists)
-    bt->grids.assign(2 * NQC, G);
+    bt->grids.assign(2 * NQC, sl.per);
     bt->kinds.assign(2 * NQC, opt.kernel_kind);
     bt->splits.assign(2 * NQC, 0);
-    const int nsm = std::max(1, bt->bases[0]->nsm);
     if (opt.autotune == 1 || opt.autotune == 2) {
         int kd[2 * NQC], gr[2 * NQC], sp[2 * NQC];
-        const int rc = tune_lists(bt->ex, bt->d_mols, bt->d_tiles, bt->d_part, bt->d_cnt, boys, G, nsm, st, kd, gr,
+        const int rc = tune_lists(bt->ex, bt->d_mols, bt->d_tiles, bt->d_part, bt->d_cnt, boys, sl, nsm, st, kd, gr,
                                   sp);
         if (rc != TG_OK) return rc;
         for (int k = 0; k < 2 * NQC; ++k) {
@@ -1944,37 +1979,19 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
             bt->splits[k] = sp[k];
         }
     }
-    // the partial slabs must cover the largest tuned grid
-    if ((size_t)G * 3 * natom_total > (size_t)bt->plans[0].G * 3 * natom_total) {
-        // re-carve with the larger slab count
-        bt->arena.release();
-        const size_t need2 = al(sizeof(MolDesc) * nmol) + al(sizeof(uint4) * ntl) +
-                             al(sizeof(double) * (size_t)kSlabSets * G * 3 * natom_total) + al(sizeof(double) * 3 * natom_total) +
-                             al(sizeof(unsigned long long) * NCNT * NQC) + 4096;
-        TG_CUDA(bt->arena.reserve(need2));
-        bt->arena.used = 0;
-        bt->d_mols = bt->arena.take<MolDesc>(nmol);
-        bt->d_tiles = bt->arena.take<uint4>(ntl);
-        bt->d_part = bt->arena.take<double>((size_t)kSlabSets * G * 3 * natom_total);
-        bt->d_grad = bt->arena.take<double>(3 * natom_total);
-        bt->d_cnt = bt->arena.take<unsigned long long>(NCNT * NQC);
-        TG_CUDA(cudaMemcpy(bt->d_mols, mds.data(), sizeof(MolDesc) * nmol, cudaMemcpyHostToDevice));
-        if (!bt->ex.tiles.empty())
-            TG_CUDA(cudaMemcpy(bt->d_tiles, bt->ex.tiles.data(), sizeof(uint4) * bt->ex.tiles.size(),
-                               cudaMemcpyHostToDevice));
-    }
-
     // ---- capture the launch sequence once (a run first sets kernel attributes)
     TG_CUDA(cudaStreamCreateWithFlags(&bt->cap, cudaStreamNonBlocking));
+    SideStreams *side = sl.sets == 1 ? nullptr : &bt->side;
+    const size_t nslab = sl.count();
     for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) TG_CUDA(cudaStreamBeginCapture(bt->cap, cudaStreamCaptureModeThreadLocal));
         int n = 0;
-        cudaMemsetAsync(bt->d_part, 0, sizeof(double) * (size_t)kSlabSets * G * 3 * natom_total, bt->cap);
+        cudaMemsetAsync(bt->d_part, 0, sizeof(double) * nslab * 3 * natom_total, bt->cap);
         cudaMemsetAsync(bt->d_cnt, 0, sizeof(unsigned long long) * NCNT * NQC, bt->cap);
-        int rc = launch_exec(bt->ex, bt->d_mols, bt->d_tiles, bt->d_part, bt->d_cnt, nullptr, boys, G,
+        int rc = launch_exec(bt->ex, bt->d_mols, bt->d_tiles, bt->d_part, bt->d_cnt, nullptr, boys, sl,
                              bt->grids.data(), false, bt->cap, nullptr, n, bt->kinds.data(), 0, 0, 1,
-                             bt->splits.data(), &bt->side);
-        k_reduce<<<(3 * natom_total + 31) / 32, 1024, 0, bt->cap>>>(3 * natom_total, kSlabSets * G, bt->d_part,
+                             bt->splits.data(), side);
+        k_reduce<<<(3 * natom_total + 31) / 32, 1024, 0, bt->cap>>>(3 * natom_total, (int)nslab, bt->d_part,
                                                                    bt->d_grad);
         ++n;
         if (pass == 1) {
@@ -2017,7 +2034,7 @@ int tg_batch_run(tg_batch *bt, double *const *grads, const tg_options *opt_in, t
         int nops = 1;
         for (const Plan &pl : bt->plans)
             if (pl.den.use_lr) nops = 2;
-        fill_stats(stats, hc, bt->pairs, (long long)bt->ex.tiles.size(), bt->launches, bt->G, nops);
+        fill_stats(stats, hc, bt->pairs, (long long)bt->ex.tiles.size(), bt->launches, bt->slabs.per, nops);
         stats->plan_ms = 0.0;  // planned at tg_batch_create
         stats->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     }

@@ -1,9 +1,11 @@
 """Calls at the limits of what is shared or scarce: molecules whose gradient
 just fits or no longer fits beside a kernel's arrays, kernel attributes
 while two threads work on molecules of different sizes, and device memory too
-short for the router's tables.
+short for the router's tables or for all sets of partial-gradient slabs.
 
-Bounds: the same sums in the same order are bitwise equal; the fp32 route to 6e-6 of the largest component, as elsewhere."""
+Bounds: the same sums in the same order are bitwise equal; fp64 sums in
+another order agree to 1e-13 of the largest component (a few hundred partial
+sums of that size); the fp32 route to 6e-6 of it, as elsewhere."""
 import os
 import threading
 
@@ -109,3 +111,29 @@ def test_learned_route_without_room_for_its_tables(tg, monkeypatch):
         assert np.array_equal(g, h)
         mixed += 0 < sa["fp32_quartets"] < sa["quartets"]
     assert mixed
+
+
+def test_gradient_without_room_for_all_slabs(tg, monkeypatch):
+    """9000 atoms: one set of slabs, 4 an SM, takes 131 MB on 152 SMs, six sets of
+    8 an SM 1.6 GB.  With 200 MB to be had the call works on the smaller set."""
+    ref = tg.Basis(_padded(3)).grad2e(_padded(3)["pairs"], screen_tol=0.0)[0]
+    s = _padded(9000)
+    b = tg.Basis(s)
+    monkeypatch.setenv("TDGRAD_FAIL_ALLOC", str(200 << 20))
+    g = b.grad2e(s["pairs"], screen_tol=0.0)[0]
+    assert np.abs(g[:3] - ref).max() <= 1e-13 * np.abs(ref).max()
+    assert not g[3:].any()
+    timed = b.grad2e(s["pairs"], screen_tol=0.0, timing=True)[0]
+    assert np.abs(timed[:3] - ref).max() <= 1e-13 * np.abs(ref).max()
+
+
+def test_batch_without_room_for_all_slabs(tg, monkeypatch):
+    """The same for a batch of two such molecules (262 MB against 3.2 GB); its
+    molecules' own work areas hold no slabs."""
+    ref = tg.Basis(_padded(3)).grad2e(_padded(3)["pairs"], screen_tol=0.0)[0]
+    monkeypatch.setenv("TDGRAD_FAIL_ALLOC", str(300 << 20))
+    batch = tg.Batch([_padded(9000), _padded(9000)], screen_tol=0.0)
+    for _ in range(2):
+        for g in batch.run()[0]:
+            assert np.abs(g[:3] - ref).max() <= 1e-13 * np.abs(ref).max()
+            assert not g[3:].any()
