@@ -779,7 +779,7 @@ __device__ void group_herm(double *sm, int tid, int k0, int kg, const GroupInfo 
     const auto &TBra = pair_tab<LA, LB>();
     const auto &TKet = pair_tab<LC, LD>();
     const int nops = den.use_lr ? 2 : 1;
-    const bool ominf = isinf(den.omega);
+    const bool ominf = isinf(den.omega * den.omega);  // theta = 1 to the last bit before that
     const double om = ominf ? 1.0 : den.omega;
     if constexpr (KQ == 1) kg = 1;
     const int LG = 32 / kg, kq = lane / LG, sl = lane % LG;

@@ -1,7 +1,8 @@
 """Calls at the limits of what is shared or scarce: molecules whose gradient
 just fits or no longer fits beside a kernel's arrays, kernel attributes
-while two threads work on molecules of different sizes, and device memory too
-short for the router's tables or for all sets of partial-gradient slabs.
+while two threads work on molecules of different sizes, device memory too short
+for the router's tables or for all sets of partial-gradient slabs, and omega so
+large that its square is infinite.
 
 Bounds: the same sums in the same order are bitwise equal; fp64 sums in
 another order agree to 1e-13 of the largest component (a few hundred partial
@@ -137,3 +138,22 @@ def test_batch_without_room_for_all_slabs(tg, monkeypatch):
         for g in batch.run()[0]:
             assert np.abs(g[:3] - ref).max() <= 1e-13 * np.abs(ref).max()
             assert not g[3:].any()
+
+
+def test_omega_whose_square_overflows(tg):
+    """erf(omega r)/r is 1/r to the last bit long before omega^2 leaves the
+    range of fp64 (1e154) or fp32 (1e19): the result is that of omega = inf."""
+    s = _padded(3)
+    b = tg.Basis(s)
+
+    def grad(om, precision):
+        return b.grad2e([(*p[:5], om) for p in s["pairs"]], screen_tol=0.0, precision=precision)[0]
+
+    def fock(om):
+        return b.fock2e([(s["pairs"][0][0], 1.0, -0.3, -0.7, om)])[0]
+    for precision, tol in ((tg.TG_FP64, 1e-13), (tg.TG_FP32, 0.0)):
+        inf = grad(np.inf, precision)
+        assert np.isfinite(inf).all()
+        for om in (1e25, 1e160):
+            assert np.abs(grad(om, precision) - inf).max() <= tol * np.abs(inf).max(), om
+    assert np.abs(fock(1e160) - fock(np.inf)).max() <= 1e-13 * np.abs(fock(np.inf)).max()
