@@ -1988,6 +1988,17 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
         int n = 0;
         cudaMemsetAsync(bt->d_part, 0, sizeof(double) * nslab * 3 * natom_total, bt->cap);
         cudaMemsetAsync(bt->d_cnt, 0, sizeof(unsigned long long) * NCNT * NQC, bt->cap);
+        // densities in the caller's buffers may have changed since the plan: the
+        // Coulomb part's A + A^T and B + B^T are formed again by every run
+        for (int m = 0; m < nmol && opt.device_ptrs; ++m) {
+            const DensArgs &den = bt->plans[m].den;
+            const unsigned gs = (unsigned)(((size_t)den.nbf * den.nbf + 255) / 256);
+            for (int p = 0; p < den.npair; ++p) {
+                k_symm<<<gs, 256, 0, bt->cap>>>(den.nbf, den.A[p], const_cast<double *>(den.S[p]));
+                k_symm<<<gs, 256, 0, bt->cap>>>(den.nbf, den.B[p], const_cast<double *>(den.T[p]));
+                n += 2;
+            }
+        }
         int rc = launch_exec(bt->ex, bt->d_mols, bt->d_tiles, bt->d_part, bt->d_cnt, nullptr, boys, sl,
                              bt->grids.data(), false, bt->cap, nullptr, n, bt->kinds.data(), 0, 0, 1,
                              bt->splits.data(), side);
