@@ -119,7 +119,7 @@ typedef struct {
                                on the basis's first call with autotune = 1 and reuses the
                                choices on later calls (a list empty at that call keeps the
                                defaults); 2 tunes again on this call.  The tuning launches
-                               time sample tiles and do not change the result's definition:
+                               do not change the result's definition:
                                every form computes the same quartets in the same precision. */
     int kernel_kind;        /* TG_KERNEL_DEFAULT (default), _THREAD, _GROUP or _WARP */
     int deterministic;      /* 1 (default): fixed-order fp64 sums, bitwise reproducible on one
@@ -262,12 +262,12 @@ int tg_fock2e(const tg_basis *b, int npair, const tg_fpair *pairs, const tg_opti
  * (a basis holds one plan at a time) and must outlive the batch; with
  * device_ptrs the densities are read from the caller's device buffers at
  * every run (their contents may change, the plan does not), otherwise they
- * are copied at creation.  opt->autotune = 1 autotunes every class list
- * on a sample of 2 to 4 x (SM count) of its tiles taken at a fixed stride
- * over the whole list: the persistent grid (8, 4 or 2 CTAs per SM) and the
- * work-unit shape (bra primitive splits per tile: automatic, 1 or 4),
+ * are copied at creation.  opt->autotune = 1 autotunes every class list of
+ * 1 to 4 x (SM count) tiles: the persistent grid (8, 4 or 2 CTAs per SM) and
+ * the work-unit shape (bra primitive splits per tile: automatic, 1 or 4),
  * searched one coordinate at a time (grid, then splits; 6 timed launches per
- * list), keeping the fastest; every class and precision has one kernel form.
+ * list), keeping what is at least 3 % faster; longer lists keep the automatic
+ * choices, and every class and precision has one kernel form.
  * tg_batch_run replays the graph on opt->stream and writes grads[m]
  * (natom_m * 3, host unless device_ptrs).  Not part of the paper, which
  * evaluates one system at a time (Sec. II.C). */

@@ -1364,16 +1364,20 @@ void alu_peaks(double &p64, double &p32)
     p32 = (double)nsm * 128.0 * 2.0 * khz * 1e3;
 }
 
-// Autotuner of the class launches: for every (class, precision) list of ex
-// with more than nsm tiles, time a sample of 2 to 4 x nsm tiles taken at a
-// fixed stride over the whole list (whose tiles run from the costliest to
-// the cheapest) and search the grid cap (8, 4 or 2 CTAs per SM) and the unit
-// shape (bra primitive splits per tile: automatic, 1 or 4) one coordinate at a
-// time from (8 CTAs per SM, automatic splits); 6 timed launches per list.  Every
-// class and precision has one kernel form, so kinds[k] stays 0 (the default);
-// lists left untimed keep grids[k] = 0 (the persistent grid) and splits[k] = 0.
-// The sample launches write into d_part and d_cnt, which the caller clears
-// afterwards.
+// Autotuner of the class launches: every (class, precision) list of ex with nsm
+// to 4 nsm tiles is launched as it is and the grid cap (8, 4 or 2 CTAs per SM)
+// and the unit shape (bra primitive splits per tile: automatic, 1 or 4) are
+// searched one coordinate at a time from (8 CTAs per SM, automatic splits); 6
+// timed launches per list.  A choice has to be 3 % faster than the one before
+// it, several times what two runs differ.  Longer lists keep the automatic
+// choices.  A sample of such a list does not show what suits the whole: its
+// warps run short of units, so it favours fewer warps and more splits ((ss|ss) of
+// the 32-atom workload was given half the CTAs that way, 14.8 -> 19.7 ms, the
+// whole fp64 call 1 589 -> 1 611 ms).  Timed whole, lists of up to 32 nsm tiles
+// changed no call by more than 1 % and cost that workload six calls.  Every class
+// and precision has one kernel form, so kinds[k] stays 0 (the default); lists
+// left untimed keep grids[k] = 0 (the persistent grid) and splits[k] = 0.  The
+// timed launches write into d_part and d_cnt, which the caller clears afterwards.
 int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, double *d_part,
                unsigned long long *d_cnt, const double *boys, const Slabs &sl, int nsm, cudaStream_t st, int *kinds,
                int *grids, int *splits)
@@ -1384,20 +1388,17 @@ int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, doub
     cudaEvent_t e0 = ev.a, e1 = ev.b;
     for (int k = 0; k < 2 * NQC; ++k) {
         const long long nt = ex.off[k + 1] - ex.off[k];
-        if (nt <= nsm) continue;
+        if (nt <= nsm || nt > 4LL * nsm) continue;
         Exec sub;
         sub.natom_total = ex.natom_total;
         sub.natom_max = ex.natom_max;
-        // the sample: every step-th tile of the list (2 to 4 x nsm tiles spread
-        // over its whole cost range, through the tile-shard stride)
-        const int step = (int)std::max<long long>(1, nt / (2LL * nsm));
         for (int j = 0; j < 2 * NQC + 1; ++j) sub.off[j] = j <= k ? 0 : nt;
         auto time_cfg = [&](int kind, int mult, int split, float &ms) -> int {
             std::vector<int> gr(2 * NQC, std::min(sl.per, mult * nsm)), kd(2 * NQC, kind), sp(2 * NQC, split);
             int dummy = 0;
             cudaEventRecord(e0, st);
             int rc = launch_exec(sub, d_mols, d_tiles + ex.off[k], d_part, d_cnt, nullptr, boys, sl, gr.data(),
-                                 false, st, nullptr, dummy, kd.data(), 0, 0, step, sp.data());
+                                 false, st, nullptr, dummy, kd.data(), 0, 0, 1, sp.data());
             cudaEventRecord(e1, st);
             if (rc != TG_OK) return rc;
             TG_CUDA(cudaEventSynchronize(e1));
@@ -1416,13 +1417,13 @@ int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, doub
             float ms;
             const int rc = time_cfg(kind, mult, bs, ms);
             if (rc != TG_OK) return rc;
-            if (ms < best) best = ms, bm = mult;
+            if (ms < 0.97f * best) best = ms, bm = mult;
         }
         for (int split : {1, 4}) {
             float ms;
             const int rc = time_cfg(kind, bm, split, ms);
             if (rc != TG_OK) return rc;
-            if (ms < best) best = ms, bs = split;
+            if (ms < 0.97f * best) best = ms, bs = split;
         }
         grids[k] = std::min(sl.per, bm * nsm);
         splits[k] = bs;
