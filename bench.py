@@ -272,7 +272,7 @@ def c3_systems(name):
 def run_c3(args, prec, router, torch):
     """Batched uneven molecules: one planned batch (tg_batch_*: per-class
     launches over all molecules, replayed from a captured CUDA graph, the
-    kernel form and grid of every class list autotuned) against single
+    grids and splits of the shorter class lists autotuned) against single
     tg_grad2e calls on the same molecules (host buffers: the end-to-end
     figure)."""
     import numpy as np
@@ -688,8 +688,8 @@ def main():
                        "quartets_per_step": st0["quartets"], "fp32_quartets_per_step": st0["fp32_quartets"],
                        "prim_quartets_per_step": st0["prim_quartets"], "pairs": st0["pairs"], "tiles": st0["tiles"],
                        "l2": "flushed (512 MB write) before each timed step",
-                       "autotune": ("launches tuned per class list on the first warm-up call, reused"
-                                    if args.autotune else "per-class default kernel forms"),
+                       "autotune": ("shorter class lists tuned on the first warm-up call, reused"
+                                    if args.autotune else "automatic grids and work units"),
                        "parallelism": ("one gradient, tile-cyclic shards per rank, NCCL all-reduce of natom x 3"
                                        if world > 1 else "single GPU")},
             "e2e": {"value": e2e_q / (e2e_ms / 1e3), "unit": UNIT, "h2d_bytes_per_step": h2d,

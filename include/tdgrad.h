@@ -81,14 +81,15 @@ extern "C" {
  * of tg_stats. */
 #define TG_ABI_VERSION 2
 
-/* tg_options.kernel_kind: which class-kernel form evaluates a class (every
- * form gives the same result to rounding; a form not compiled for a class
- * falls back to the class default) */
-#define TG_KERNEL_DEFAULT 0   /* per-class default: one primitive quartet per lane, but the warp form for
-                                 (dd|pp), (dd|ds) and the group form for (dd|dp), (dd|dd) in fp32 */
-#define TG_KERNEL_THREAD 1    /* one contracted quartet per thread (compiled for no class now) */
-#define TG_KERNEL_GROUP 2     /* a group of 32-128 threads per quartet, arrays in shared memory */
-#define TG_KERNEL_WARP 3      /* one warp per quartet, every phase spread over its 32 lanes */
+/* tg_options.kernel_kind: values 0 to 3 are accepted and have no effect.  It
+ * chose among kernel forms per angular class; one form per class and precision
+ * is left: one primitive quartet per lane, but in fp32 one warp per quartet for
+ * (dd|pp) and (dd|ds) and a group of 128 threads per quartet for (dd|dp) and
+ * (dd|dd). */
+#define TG_KERNEL_DEFAULT 0
+#define TG_KERNEL_THREAD 1
+#define TG_KERNEL_GROUP 2
+#define TG_KERNEL_WARP 3
 
 typedef struct tg_basis tg_basis;    /* opaque: basis + geometry, device copies */
 typedef struct tg_router tg_router;  /* opaque: block router MLP weights */
@@ -113,15 +114,15 @@ typedef struct {
     void *stream;           /* cudaStream_t; NULL = legacy default stream */
     int rank, nranks;       /* shard; default 0 / 1 */
     int timing;             /* 1: time every class kernel with CUDA events (tg_stats.class_ms) */
-    int autotune;           /* 0 (default): the per-class default kernel forms and grids.
+    int autotune;           /* 0 (default): the automatic grids and work units.
                                tg_batch_create: 1 autotunes every class list (see there).
                                tg_grad2e: 1 tunes every (class, precision) list the same way
                                on the basis's first call with autotune = 1 and reuses the
                                choices on later calls (a list empty at that call keeps the
                                defaults); 2 tunes again on this call.  The tuning launches
                                do not change the result's definition:
-                               every form computes the same quartets in the same precision. */
-    int kernel_kind;        /* TG_KERNEL_DEFAULT (default), _THREAD, _GROUP or _WARP */
+                               every choice computes the same quartets in the same precision. */
+    int kernel_kind;        /* TG_KERNEL_DEFAULT (default), _THREAD, _GROUP or _WARP: no effect */
     int deterministic;      /* 1 (default): fixed-order fp64 sums, bitwise reproducible on one
                                device for one launch configuration.  Every path of this
                                version is deterministic; 0 is accepted and changes nothing. */

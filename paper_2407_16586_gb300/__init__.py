@@ -305,10 +305,9 @@ class Basis:
                timing=False, router=None, mixed_tol=1e-6, kernel=0, class_mask=0, shard_mode=0, autotune=0,
                spherical=False):
         """Gradient (natom x 3) of host numpy pairs [(A, B, c_J, c_K, c_K_lr, omega)], or of
-        torch CUDA tensors (then the densities and ``out`` stay on the device).  ``kernel``
-        asks for a class-kernel form: 0 per-class default, 1 one quartet per thread, 2 a thread
-        group per quartet, 3 a warp per quartet; a form not compiled for a class and
-        precision (tg_options.kernel_kind) falls back to the default.  ``class_mask``
+        torch CUDA tensors (then the densities and ``out`` stay on the device).  ``kernel`` 0 to
+        3 (tg_options.kernel_kind) is accepted and has no effect: every class and precision has
+        one kernel form.  ``class_mask``
         (0 = all) keeps the angular classes whose bits are set.  ``autotune`` 1 tunes the
         launches of every class list on this basis's first such call and reuses them, 2
         tunes again (tg_options.autotune).  ``spherical``: the matrices are nsph x nsph over

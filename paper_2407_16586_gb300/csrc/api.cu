@@ -159,11 +159,11 @@ struct tg_basis {
     DevArena ws5;       // Fock build: densities, combined matrices, F
     float *d_router = nullptr;  // router parameters, mean and std on the device
     int nsm = 0;
-    // tg_grad2e's autotuner (tg_options.autotune = 1): kernel form, grid cap
-    // and bra-primitive splits per (class, precision) list, chosen on the
-    // first such call and kept for the later ones
+    // tg_grad2e's autotuner (tg_options.autotune = 1): grid cap and bra-primitive
+    // splits per (class, precision) list, chosen on the first such call and kept
+    // for the later ones
     bool tuned = false;
-    int tune_kind[2 * NQC], tune_grid[2 * NQC], tune_split[2 * NQC];
+    int tune_grid[2 * NQC], tune_split[2 * NQC];
     // spherical shells: 2l+1 functions per shell; per Cartesian function its
     // shell's first spherical function << 8 | l << 4 | Cartesian component
     int nsph = 0;
@@ -1273,8 +1273,8 @@ void build_exec(const std::vector<const Plan *> &plans, const std::vector<std::v
 int launch_exec(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, double *d_part,
                 unsigned long long *dcnt, double *dump, const double *boys, const Slabs &sl, const int *grids,
                 bool timing,
-                cudaStream_t st, tg_stats *stats, int &launches, const int *kinds = nullptr, int kind_all = 0,
-                int tile_rank = 0, int tile_nranks = 1, const int *splits = nullptr, SideStreams *side = nullptr)
+                cudaStream_t st, tg_stats *stats, int &launches, const int *splits = nullptr,
+                SideStreams *side = nullptr)
 {
     OutArgs out;
     out.partials = d_part;
@@ -1298,9 +1298,7 @@ int launch_exec(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, dou
         const int qc = side ? NQC - 1 - i : i;
         for (int r = 0; r < 2; ++r) {
             const int k = 2 * qc + r;
-            // tile-cyclic shard: tiles tile_rank, tile_rank + tile_nranks, ... of the list
-            long long first = 0, nt = 0, stride = 1;
-            tg_tile_shard(ex.off[k + 1] - ex.off[k], tile_rank, tile_nranks, &first, &nt, &stride);
+            const long long nt = ex.off[k + 1] - ex.off[k];
             if (nt <= 0) continue;
             ClassLaunch cl;
             int Pc = 0, Qc = 0;
@@ -1313,10 +1311,8 @@ int launch_exec(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, dou
             cl.P = Pc;
             cl.Q = Qc;
             cl.ntiles = nt;
-            cl.tiles = d_tiles + ex.off[k] + first;
-            cl.stride = stride;
+            cl.tiles = d_tiles + ex.off[k];
             cl.nsplit = cl.nchunk = 1;
-            cl.kind = kinds ? kinds[k] : kind_all;
             cl.split_req = splits ? splits[k] : 0;
             OutArgs o = out;
             o.counters = dcnt + NCNT * qc;
@@ -1374,15 +1370,14 @@ void alu_peaks(double &p64, double &p32)
 // warps run short of units, so it favours fewer warps and more splits ((ss|ss) of
 // the 32-atom workload was given half the CTAs that way, 14.8 -> 19.7 ms, the
 // whole fp64 call 1 589 -> 1 611 ms).  Timed whole, lists of up to 32 nsm tiles
-// changed no call by more than 1 % and cost that workload six calls.  Every class
-// and precision has one kernel form, so kinds[k] stays 0 (the default); lists
-// left untimed keep grids[k] = 0 (the persistent grid) and splits[k] = 0.  The
-// timed launches write into d_part and d_cnt, which the caller clears afterwards.
+// changed no call by more than 1 % and cost that workload six calls.  Lists left
+// untimed keep grids[k] = 0 (the persistent grid) and splits[k] = 0.  The timed
+// launches write into d_part and d_cnt, which the caller clears afterwards.
 int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, double *d_part,
-               unsigned long long *d_cnt, const double *boys, const Slabs &sl, int nsm, cudaStream_t st, int *kinds,
-               int *grids, int *splits)
+               unsigned long long *d_cnt, const double *boys, const Slabs &sl, int nsm, cudaStream_t st, int *grids,
+               int *splits)
 {
-    for (int k = 0; k < 2 * NQC; ++k) kinds[k] = grids[k] = splits[k] = 0;
+    for (int k = 0; k < 2 * NQC; ++k) grids[k] = splits[k] = 0;
     EventPair ev;
     TG_CUDA(ev.create());
     cudaEvent_t e0 = ev.a, e1 = ev.b;
@@ -1393,12 +1388,12 @@ int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, doub
         sub.natom_total = ex.natom_total;
         sub.natom_max = ex.natom_max;
         for (int j = 0; j < 2 * NQC + 1; ++j) sub.off[j] = j <= k ? 0 : nt;
-        auto time_cfg = [&](int kind, int mult, int split, float &ms) -> int {
-            std::vector<int> gr(2 * NQC, std::min(sl.per, mult * nsm)), kd(2 * NQC, kind), sp(2 * NQC, split);
+        auto time_cfg = [&](int mult, int split, float &ms) -> int {
+            std::vector<int> gr(2 * NQC, std::min(sl.per, mult * nsm)), sp(2 * NQC, split);
             int dummy = 0;
             cudaEventRecord(e0, st);
             int rc = launch_exec(sub, d_mols, d_tiles + ex.off[k], d_part, d_cnt, nullptr, boys, sl, gr.data(),
-                                 false, st, nullptr, dummy, kd.data(), 0, 0, 1, sp.data());
+                                 false, st, nullptr, dummy, sp.data());
             cudaEventRecord(e1, st);
             if (rc != TG_OK) return rc;
             TG_CUDA(cudaEventSynchronize(e1));
@@ -1406,22 +1401,21 @@ int tune_lists(const Exec &ex, const MolDesc *d_mols, const uint4 *d_tiles, doub
             cudaEventElapsedTime(&ms, e0, e1);
             return TG_OK;
         };
-        const int kind = 0;
         int bm = 8, bs = 0;
         float best = -1.f;
         for (int rep = 0; rep < 2; ++rep) {  // the first one loads the kernel
-            const int rc = time_cfg(kind, bm, bs, best);
+            const int rc = time_cfg(bm, bs, best);
             if (rc != TG_OK) return rc;
         }
         for (int mult : {4, 2}) {
             float ms;
-            const int rc = time_cfg(kind, mult, bs, ms);
+            const int rc = time_cfg(mult, bs, ms);
             if (rc != TG_OK) return rc;
             if (ms < 0.97f * best) best = ms, bm = mult;
         }
         for (int split : {1, 4}) {
             float ms;
-            const int rc = time_cfg(kind, bm, split, ms);
+            const int rc = time_cfg(bm, split, ms);
             if (rc != TG_OK) return rc;
             if (ms < 0.97f * best) best = ms, bs = split;
         }
@@ -1485,7 +1479,7 @@ struct tg_batch {
     uint4 *d_tiles = nullptr;
     double *d_part = nullptr, *d_grad = nullptr;
     unsigned long long *d_cnt = nullptr;
-    std::vector<int> grids, kinds, splits;
+    std::vector<int> grids, splits;
     Slabs slabs = {1, 1};
     int device_ptrs = 0;
     cudaStream_t cap = nullptr;
@@ -1534,17 +1528,16 @@ int tg_grad2e(const tg_basis *cb, int npair, const tg_pair *pairs, const tg_opti
     TG_CUDA(cudaMemcpyAsync(d_mol, &md, sizeof(MolDesc), cudaMemcpyHostToDevice, st));
     // autotune = 1: the per-list launch choices of the basis's first tuned
     // call; autotune = 2: tune again on this call and keep the new choices
-    int kd[2 * NQC], gr[2 * NQC], sp[2 * NQC];
+    int gr[2 * NQC], sp[2 * NQC];
     const bool tune = opt.autotune == 1 || opt.autotune == 2;
     if (tune) {
         if (!b->tuned || opt.autotune == 2) {
-            rc = tune_lists(ex, d_mol, d_tiles, d_part, pl.dcnt, b->d_boys, pl.slabs, b->nsm, st, b->tune_kind,
-                            b->tune_grid, b->tune_split);
+            rc = tune_lists(ex, d_mol, d_tiles, d_part, pl.dcnt, b->d_boys, pl.slabs, b->nsm, st, b->tune_grid,
+                            b->tune_split);
             if (rc != TG_OK) return rc;
             b->tuned = true;
         }
         for (int k = 0; k < 2 * NQC; ++k) {
-            kd[k] = b->tune_kind[k] ? b->tune_kind[k] : opt.kernel_kind;
             gr[k] = b->tune_grid[k];
             sp[k] = b->tune_split[k];
         }
@@ -1556,8 +1549,7 @@ int tg_grad2e(const tg_basis *cb, int npair, const tg_pair *pairs, const tg_opti
     const double plan_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     // (a tile shard is already in the lists)
     rc = launch_exec(ex, d_mol, d_tiles, d_part, pl.dcnt, nullptr, b->d_boys, pl.slabs, tune ? gr : nullptr,
-                     opt.timing != 0, st, stats, launches, tune ? kd : nullptr, opt.kernel_kind, 0, 1,
-                     tune ? sp : nullptr, side);
+                     opt.timing != 0, st, stats, launches, tune ? sp : nullptr, side);
     if (rc != TG_OK) return rc;
     k_reduce<<<(3 * natom + 31) / 32, 1024, 0, st>>>(3 * natom, (int)nslab, d_part, pl.dgrad);
     ++launches;
@@ -1735,7 +1727,6 @@ int tg_fock2e(const tg_basis *cb, int npair, const tg_fpair *fpairs, const tg_op
         cl.Q = pl.qc_Q[qc];
         cl.ntiles = nt;
         cl.tiles = dt.tiles + dt.off[2 * qc];
-        cl.stride = 1;
         cl.nsplit = cl.nchunk = 1;
         OutArgs o;
         std::memset(&o, 0, sizeof(o));
@@ -1967,15 +1958,12 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
 
     // ---- autotune every (class, precision) list (tune_lists)
     bt->grids.assign(2 * NQC, sl.per);
-    bt->kinds.assign(2 * NQC, opt.kernel_kind);
     bt->splits.assign(2 * NQC, 0);
     if (opt.autotune == 1 || opt.autotune == 2) {
-        int kd[2 * NQC], gr[2 * NQC], sp[2 * NQC];
-        const int rc = tune_lists(bt->ex, bt->d_mols, bt->d_tiles, bt->d_part, bt->d_cnt, boys, sl, nsm, st, kd, gr,
-                                  sp);
+        int gr[2 * NQC], sp[2 * NQC];
+        const int rc = tune_lists(bt->ex, bt->d_mols, bt->d_tiles, bt->d_part, bt->d_cnt, boys, sl, nsm, st, gr, sp);
         if (rc != TG_OK) return rc;
         for (int k = 0; k < 2 * NQC; ++k) {
-            if (kd[k]) bt->kinds[k] = kd[k];
             if (gr[k]) bt->grids[k] = gr[k];
             bt->splits[k] = sp[k];
         }
@@ -2001,8 +1989,7 @@ int tg_batch_create(int nmol, const tg_basis *const *bases, const int *npair, co
             }
         }
         int rc = launch_exec(bt->ex, bt->d_mols, bt->d_tiles, bt->d_part, bt->d_cnt, nullptr, boys, sl,
-                             bt->grids.data(), false, bt->cap, nullptr, n, bt->kinds.data(), 0, 0, 1,
-                             bt->splits.data(), side);
+                             bt->grids.data(), false, bt->cap, nullptr, n, bt->splits.data(), side);
         k_reduce<<<(3 * natom_total + 31) / 32, 1024, 0, bt->cap>>>(3 * natom_total, (int)nslab, bt->d_part,
                                                                    bt->d_grad);
         ++n;

@@ -31,7 +31,7 @@ __device__ __forceinline__ void group_sync(int id, int nthreads)
     }
 }
 
-template <int LA, int LB, int LC, int LD, typename F>
+template <int LA, int LB, int LC, int LD>
 struct CoopLayout {
     static constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD);
     static constexpr int NAB = NA * NB, NCD = NC * ND;
@@ -40,7 +40,7 @@ struct CoopLayout {
     static constexpr int NR = nherm(L + 1);
     static constexpr int NEB = (LA + 2) * (LB + 1) * (L1 + 2);
     static constexpr int NEK = (LC + 2) * (LD + 1) * (L2 + 2);
-    // element offsets (in F units) of the per-group regions
+    // element offsets (in floats) of the per-group regions
     static constexpr int o_gam = 0;
     static constexpr int o_gaml = o_gam + NAB * NCD;
     static constexpr int o_F = o_gaml + NAB * NCD;          // [2][NCD][NH1], per bra primitive pair
@@ -55,7 +55,7 @@ struct CoopLayout {
     static constexpr int o_sc = o_Ek + 3 * NEK;             // scalars and powers of s
     static constexpr int NSC = 16 + L + 3;
     static constexpr int TOTAL = o_sc + NSC;
-    static constexpr size_t bytes() { return sizeof(F) * (size_t)TOTAL; }
+    static constexpr size_t bytes() { return sizeof(float) * (size_t)TOTAL; }
 };
 
 __device__ __forceinline__ int ebi(int i, int j, int t, int J1, int T1) { return (i * J1 + j) * T1 + t; }
@@ -88,18 +88,18 @@ __device__ __forceinline__ void cdecode(int c, int l, int &x, int &y, int &z)
 // the group), bra primitive pairs ib0, ib0 + ibs, ...  Adds this lane's
 // partial sums of d/dA (acc[0..2]), d/dA + d/dB (acc[3..5]) and d/dC
 // (acc[6..8]); the caller reduces them over the group.
-template <int LA, int LB, int LC, int LD, typename F, int GS>
-__device__ void quartet_coop(F *sm, int lane, int bar, const GeoArgs &geo, const DensArgs &den, const PrimPairs &pp,
+template <int LA, int LB, int LC, int LD, int GS>
+__device__ void quartet_coop(float *sm, int lane, int bar, const GeoArgs &geo, const DensArgs &den, const PrimPairs &pp,
                              int sa, int sb, int sc, int sd, int pb0, int nbp, int ib0, int ibs, int pk0, int nkp,
                              double scale, const double *boys, double (&acc)[9])
 {
-    using Lay = CoopLayout<LA, LB, LC, LD, F>;
+    using F = float;
+    using Lay = CoopLayout<LA, LB, LC, LD>;
     constexpr int NB = Lay::NB, ND = Lay::ND, NAB = Lay::NAB, NCD = Lay::NCD;
     constexpr int L1 = Lay::L1, L2 = Lay::L2, L = Lay::L;
     constexpr int NH1 = Lay::NH1, NH1P = Lay::NH1P, NH2 = Lay::NH2, NH2P = Lay::NH2P;
     constexpr int BJ = LB + 1, BT = L1 + 2, KJ = LD + 1, KT = L2 + 2;
     constexpr int S = Lay::S, NCUBE = Lay::NCUBE;
-    constexpr bool FP32 = sizeof(F) == 4;
     F *gam = sm + Lay::o_gam, *gaml = sm + Lay::o_gaml, *Fr = sm + Lay::o_F, *E3b = sm + Lay::o_E3b;
     F *W = sm + Lay::o_W, *E3k = sm + Lay::o_E3k, *Rb = sm + Lay::o_R, *Eb = sm + Lay::o_Eb, *Ek = sm + Lay::o_Ek;
     F *scl = sm + Lay::o_sc;
@@ -109,8 +109,7 @@ __device__ void quartet_coop(F *sm, int lane, int bar, const GeoArgs &geo, const
     const bool ominf = isinf((float)om2);
     const int nbf = den.nbf;
     const int fa = geo.sh_bf[sa], fb = geo.sh_bf[sb], fc = geo.sh_bf[sc], fd = geo.sh_bf[sd];
-    const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xb = geo.xyz + 3 * geo.sh_atom[sb];
-    const double *xc = geo.xyz + 3 * geo.sh_atom[sc], *xd = geo.xyz + 3 * geo.sh_atom[sd];
+    const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xc = geo.xyz + 3 * geo.sh_atom[sc];
 
     // ---- Gamma (8 images, scale = 1/|stabiliser|)
     for (int it = lane; it < NAB * NCD; it += GS) {
@@ -138,15 +137,10 @@ __device__ void quartet_coop(F *sm, int lane, int bar, const GeoArgs &geo, const
 
     for (int ib = ib0; ib < nbp; ib += ibs) {
         const int ip = pb0 + ib;
-        const double p = pp.p[ip], Px = pp.Px[ip], Py = pp.Py[ip], Pz = pp.Pz[ip];
         // 1-D bra Hermite tables, one direction per lane
         if (lane < 3) {
-            const double P = lane == 0 ? Px : (lane == 1 ? Py : Pz);
             F E[LA + 2][LB + 1][L1 + 2];
-            if constexpr (FP32)
-                etab<LA + 1, LB>(E, (F)pp.fPA[lane * pp.n + ip], (F)pp.fPB[lane * pp.n + ip], (F)(0.5f / pp.fp[ip]));
-            else
-                etab<LA + 1, LB>(E, (F)(P - xa[lane]), (F)(P - xb[lane]), (F)(0.5 / p));
+            etab<LA + 1, LB>(E, pp.fPA[lane * pp.n + ip], pp.fPB[lane * pp.n + ip], 0.5f / pp.fp[ip]);
             F *dst = Eb + lane * Lay::NEB;
             for (int i = 0; i <= LA + 1; ++i)
                 for (int j = 0; j <= LB; ++j)
@@ -186,18 +180,13 @@ __device__ void quartet_coop(F *sm, int lane, int bar, const GeoArgs &geo, const
             const int kp = pk0 + jk;
             // ket tables (lanes 0-2), Boys and R bases (lanes 3, 4)
             if (lane < 3) {
-                const double Q = lane == 0 ? pp.Px[kp] : (lane == 1 ? pp.Py[kp] : pp.Pz[kp]);
                 F E[LC + 2][LD + 1][L2 + 2];
-                if constexpr (FP32)
-                    etab<LC + 1, LD>(E, (F)pp.fPA[lane * pp.n + kp], (F)pp.fPB[lane * pp.n + kp],
-                                     (F)(0.5f / pp.fp[kp]));
-                else
-                    etab<LC + 1, LD>(E, (F)(Q - xc[lane]), (F)(Q - xd[lane]), (F)(0.5 / pp.p[kp]));
+                etab<LC + 1, LD>(E, pp.fPA[lane * pp.n + kp], pp.fPB[lane * pp.n + kp], 0.5f / pp.fp[kp]);
                 F *dst = Ek + lane * Lay::NEK;
                 for (int i = 0; i <= LC + 1; ++i)
                     for (int j = 0; j <= LD; ++j)
                         for (int t = 0; t <= L2 + 1; ++t) dst[ebi(i, j, t, KJ, KT)] = E[i][j][t];
-            } else if (FP32 && (lane == 3 || (lane == 4 && lr))) {
+            } else if (lane == 3 || (lane == 4 && lr)) {
                 // fp32 scalars: P - Q = (P - A) - (Q - C) + (A - C)
                 const long long nr = pp.n;
                 const float pf = pp.fp[ip], qf = pp.fp[kp], pq = pf + qf, rho = pf * qf / pq;
@@ -226,26 +215,6 @@ __device__ void quartet_coop(F *sm, int lane, int bar, const GeoArgs &geo, const
                         scl[16 + n] = pw;
                         pw *= (F)s;
                     }
-                }
-            } else if (!FP32 && (lane == 3 || (lane == 4 && lr))) {
-                const double q = pp.p[kp], pq = p + q, rho = p * q / pq;
-                const double X = Px - pp.Px[kp], Y = Py - pp.Py[kp], Z = Pz - pp.Pz[kp];
-                const double T = rho * (X * X + Y * Y + Z * Z);
-                const double pref = 34.986836655249725 / (p * q * sqrt(pq)) * pp.K[ip] * pp.K[kp];
-                const double th2 = (lane == 3) ? 1.0 : (ominf ? 1.0 : om2 / (om2 + rho));
-                double Fm[L + 2];
-                boys_fp64<L + 1>(T * th2, Fm, boys);
-                F *base = Rb + 2 * NCUBE + (lane - 3) * (L + 2);
-                double f = pref * sqrt(th2), m2 = -2.0 * rho * th2;
-                for (int n = 0; n <= L + 1; ++n) {
-                    base[n] = (F)(f * Fm[n]);
-                    f *= m2;
-                }
-                if (lane == 3) {
-                    scl[0] = (F)X;
-                    scl[1] = (F)Y;
-                    scl[2] = (F)Z;
-                    for (int n = 0; n <= L + 2; ++n) scl[16 + n] = F(1);
                 }
             }
             group_sync(bar, GS);
@@ -322,10 +291,8 @@ __device__ void quartet_coop(F *sm, int lane, int bar, const GeoArgs &geo, const
                             w0 += ev * R3[b1 + off];
                             if (lr) w1 += ev * R3l[b1 + off];
                         }
-                if constexpr (FP32) {
-                    w0 *= spow[n1];
-                    w1 *= spow[n1];
-                }
+                w0 *= spow[n1];
+                w1 *= spow[n1];
                 W[it] += w0;
                 if (lr) W[NCD * NH1P + it] += w1;
             }
@@ -353,17 +320,12 @@ __device__ void quartet_coop(F *sm, int lane, int bar, const GeoArgs &geo, const
 #pragma unroll
                             for (int v1 = 0; v1 <= L1 - t1 - u1; ++v1) {
                                 const int off = (t1 * S + u1) * S + v1;
-                                if constexpr (FP32) {
-                                    const F sh = spow[t1 + u1 + v1];
-                                    z0 += f0[hidx(t1, u1, v1)] * sh * R3[b2 + off];
-                                    if (lr) z1 += f1[hidx(t1, u1, v1)] * sh * R3l[b2 + off];
-                                } else {
-                                    z0 += f0[hidx(t1, u1, v1)] * R3[b2 + off];
-                                    if (lr) z1 += f1[hidx(t1, u1, v1)] * R3l[b2 + off];
-                                }
+                                const F sh = spow[t1 + u1 + v1];
+                                z0 += f0[hidx(t1, u1, v1)] * sh * R3[b2 + off];
+                                if (lr) z1 += f1[hidx(t1, u1, v1)] * sh * R3l[b2 + off];
                             }
                     F z = z0 + z1;
-                    if constexpr (FP32) z *= spow[n2];
+                    z *= spow[n2];
                     if (n2 & 1) z = -z;
                     const F ex = t2 <= nx ? Ex[ebi(cx, dx, t2, KJ, KT)] : F(0);
                     const F ey = u2 <= ny ? Ey[ebi(cy, dy, u2, KJ, KT)] : F(0);
@@ -447,11 +409,11 @@ __device__ void quartet_coop(F *sm, int lane, int bar, const GeoArgs &geo, const
 // Persistent cooperative class kernel: 128 threads = 128/GS groups; group g
 // takes quartets g, g + 128/GS, ... of every tile; the tile's 12 x TILE
 // contributions are then added in a fixed order (tile_reduce).
-template <int LA, int LB, int LC, int LD, typename F, int GS>
+template <int LA, int LB, int LC, int LD, int GS>
 __global__ void __launch_bounds__(TILE) k_grad_coop(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out,
                                                     const double *__restrict__ boys)
 {
-    using Lay = CoopLayout<LA, LB, LC, LD, F>;
+    using Lay = CoopLayout<LA, LB, LC, LD>;
     constexpr int NG = TILE / GS;
     extern __shared__ double smem[];
     const int nacc3 = out.use_smem ? out.natom_max * 3 : 0;
@@ -461,7 +423,7 @@ __global__ void __launch_bounds__(TILE) k_grad_coop(const MolDesc *__restrict__ 
     double *tred = reinterpret_cast<double *>(sat + TILE * 4);
     int *ratom = reinterpret_cast<int *>(tred + 6 * (TB + TK));
     double *red = reinterpret_cast<double *>(ratom + 2 * (TB + TK));  // [NG][GS/32][9]
-    F *gsm = reinterpret_cast<F *>(red + NG * (GS / 32) * 9) + (size_t)(threadIdx.x / GS) * Lay::TOTAL;
+    float *gsm = reinterpret_cast<float *>(red + NG * (GS / 32) * 9) + (size_t)(threadIdx.x / GS) * Lay::TOTAL;
     const int grp = threadIdx.x / GS, lane = threadIdx.x % GS, bar = 1 + grp;
     double *slab = out.partials + (size_t)blockIdx.x * out.natom_total * 3;
     int cur = -1, cur_off3 = 0, cur_n3 = 0;
@@ -472,7 +434,7 @@ __global__ void __launch_bounds__(TILE) k_grad_coop(const MolDesc *__restrict__ 
     for (long long it = blockIdx.x; it < cl.ntiles * C * S; it += gridDim.x) {
         const long long tile = it / (C * S);
         const int chunk = (int)((it / S) % C), split = (int)(it % S);
-        const uint4 tl = cl.tiles[tile * cl.stride];
+        const uint4 tl = cl.tiles[tile];
         const int mol = (int)tl.x;
         if (mol != cur) {
             if (out.use_smem) {
@@ -523,7 +485,7 @@ __global__ void __launch_bounds__(TILE) k_grad_coop(const MolDesc *__restrict__ 
                 double acc[9];
 #pragma unroll
                 for (int k = 0; k < 9; ++k) acc[k] = 0.0;
-                quartet_coop<LA, LB, LC, LD, F, GS>(gsm, lane, bar, geo, md.den, pp, sa, sb, sc, sd, bra.poff[bi],
+                quartet_coop<LA, LB, LC, LD, GS>(gsm, lane, bar, geo, md.den, pp, sa, sb, sc, sd, bra.poff[bi],
                                                     nbp, split, S, ket.poff[ki], nkp, scale, boys, acc);
 #pragma unroll
                 for (int k = 0; k < 9; ++k)
@@ -586,34 +548,30 @@ __global__ void __launch_bounds__(TILE) k_grad_coop(const MolDesc *__restrict__ 
     }
     if ((threadIdx.x & 31) == 0 && (nq || npq)) {  // a split unit may hold primitives only
         atomicAdd(out.counters + 0, nq);
-        atomicAdd(out.counters + (sizeof(F) == 4 ? 3 : 1), npq);
-        atomicAdd(out.counters + (sizeof(F) == 4 ? 5 : 4), nbv);
-        if (sizeof(F) == 4) atomicAdd(out.counters + 2, nq);
+        atomicAdd(out.counters + 2, nq);
+        atomicAdd(out.counters + 3, npq);
+        atomicAdd(out.counters + 5, nbv);
     }
 }
 
 // Group size and shared-memory use of the cooperative kernel for a class.
-template <int LA, int LB, int LC, int LD, typename F>
+template <int LA, int LB, int LC, int LD>
 struct CoopChoice {
-    using Lay = CoopLayout<LA, LB, LC, LD, F>;
+    using Lay = CoopLayout<LA, LB, LC, LD>;
     static constexpr int work = Lay::NAB * Lay::NH1P > Lay::NCD * Lay::NH2P ? Lay::NAB * Lay::NH1P : Lay::NCD * Lay::NH2P;
     static constexpr int GS = work >= 1024 ? 128 : (work >= 320 ? 64 : 32);
     static constexpr size_t group_bytes() { return Lay::bytes(); }
     static constexpr size_t bytes_all() { return (size_t)(TILE / GS) * Lay::bytes() + sizeof(double) * (TILE / GS) * (GS / 32) * 9 + 64; }
 };
 
-}  // namespace tg
-
-namespace tg {
-
-template <int LA, int LB, int LC, int LD, typename F>
+template <int LA, int LB, int LC, int LD>
 cudaError_t launch_coop(int gcap, size_t smem, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl,
                         const OutArgs &out, const double *boys)
 {
-    using C = CoopChoice<LA, LB, LC, LD, F>;
+    using C = CoopChoice<LA, LB, LC, LD>;
     OutArgs o = out;
     const size_t sm = unit_smem(C::bytes_all(), smem, o);
-    return launch_units(k_grad_coop<LA, LB, LC, LD, F, C::GS>, TILE / C::GS, gcap, sm, st, mols, cl, o, boys);
+    return launch_units(k_grad_coop<LA, LB, LC, LD, C::GS>, TILE / C::GS, gcap, sm, st, mols, cl, o, boys);
 }
 
 }  // namespace tg

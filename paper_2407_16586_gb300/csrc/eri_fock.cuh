@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(32, LA + LB + LC + LD <= 3 ? 16 : 8)
         if (it >= units) continue;
         const long long tile = it / (C * S);
         const int chunk = (int)((it / S) % C), split = (int)(it % S);
-        const uint4 tl = cl.tiles[tile * cl.stride];
+        const uint4 tl = cl.tiles[tile];
         const MolDesc &md = mols[tl.x];
         const PairSet &bra = md.sets[cl.P], &ket = md.sets[cl.Q];
         for (int qi = chunk * QPC; qi < (chunk + 1) * QPC; ++qi) {

@@ -1093,7 +1093,7 @@ __global__ void __launch_bounds__(32 * Op::NW * Op::cta_workers, Op::min_ctas)
         if (it >= units) continue;
         const long long tile = it / (C * S);
         const int chunk = (int)((it / S) % C), split = (int)(it % S);
-        const uint4 tl = cl.tiles[tile * cl.stride];
+        const uint4 tl = cl.tiles[tile];
         const MolDesc &md = mols[tl.x];
         const PairSet &bra = md.sets[cl.P], &ket = md.sets[cl.Q];
         for (int qi = chunk * QPC; qi < (chunk + 1) * QPC; qi += KG) {

@@ -386,12 +386,10 @@ struct Lane32Op {
     }
 };
 
-// Kernel forms per class.  fp64: the Hermite-density kernel.  fp32: the lane
+// The kernel form of a class.  fp64: the Hermite-density kernel.  fp32: the lane
 // kernel, but the warp kernel for (dd|pp) and (dd|ds) and the group kernel for
 // (dd|dp) and (dd|dd), whose order of fp32 sums differs from the lane kernel's:
-// the routed results stay what they were.  ClassLaunch::kind 2 / 3 asks for the
-// group / warp kernel; a form not compiled for the class and precision (the
-// thread form is compiled for none) falls back to the default.
+// the routed results stay what they were.
 template <int LA, int LB, int LC, int LD>
 cudaError_t launch_class_kernel(int fp32, int gcap, size_t smem, cudaStream_t st, const MolDesc *mols,
                                 const ClassLaunch &cl, const OutArgs &out, const double *boys)
@@ -400,9 +398,9 @@ cudaError_t launch_class_kernel(int fp32, int gcap, size_t smem, cudaStream_t st
     constexpr bool group = nfq >= 648, warp = (LA + LB == 4) && nfq >= 216 && nfq < 648;
     if (!fp32) return launch_lanes<HermOp<LA, LB, LC, LD>>(gcap, st, mols, cl, out, boys);
     if constexpr (warp)
-        return launch_warp<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
+        return launch_warp<LA, LB, LC, LD>(gcap, smem, st, mols, cl, out, boys);
     else if constexpr (group)
-        return launch_coop<LA, LB, LC, LD, float>(gcap, smem, st, mols, cl, out, boys);
+        return launch_coop<LA, LB, LC, LD>(gcap, smem, st, mols, cl, out, boys);
     else
         return launch_lanes<Lane32Op<LA, LB, LC, LD>>(gcap, st, mols, cl, out, boys);
 }

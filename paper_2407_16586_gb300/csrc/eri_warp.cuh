@@ -50,10 +50,6 @@ __host__ __device__ constexpr HermTriples make_herm_triples()
 static __device__ const HermTriples kHermTriples = make_herm_triples();
 
 // v, negated when odd is 1 (a sign-bit flip on the integer pipe)
-__device__ __forceinline__ double flip_if(double v, int odd)
-{
-    return __longlong_as_double(__double_as_longlong(v) ^ ((long long)(odd & 1) << 63));
-}
 __device__ __forceinline__ float flip_if(float v, int odd)
 {
     return __int_as_float(__float_as_int(v) ^ ((odd & 1) << 31));
@@ -77,30 +73,23 @@ __device__ __forceinline__ void cart_xyz(int l, int c, int &x, int &y, int &z)
     x = l - s;
 }
 
-// F_m(T) for one order m <= BOYS_M - BOYS_TAYLOR, with no recursion over m:
-// for T < BOYS_TMAX the Taylor step of the tabulated F_m, F_{m+1}, ... about
-// the nearest grid point, F_m(T0 - d) = sum_k F_{m+k}(T0) d^k / k!; above,
-// F_0 = sqrt(pi / T) / 2 (erfc(6) < 3e-17) and the m upward steps
-// F_{k+1} = ((2k + 1) F_k - e^-T) / (2T), stable for large T.
+// F_m(T) for one order m <= BOYS_M - BOYS_TAYLOR and T < BOYS_TMAX (here T < 1),
+// with no recursion over m: the Taylor step of the tabulated F_m, F_{m+1}, ...
+// about the nearest grid point, F_m(T0 - d) = sum_k F_{m+k}(T0) d^k / k!.
 __device__ __forceinline__ double boys_order_fp64(double T, int m, const double *__restrict__ tab)
 {
-    if (T < BOYS_TMAX) {
-        const int i = __double2int_rn(T * (1.0 / BOYS_H));
-        const double d = i * BOYS_H - T;
-        const double *row = tab + i * (BOYS_M + 1) + m;
-        double acc = row[BOYS_TAYLOR];
+    const int i = __double2int_rn(T * (1.0 / BOYS_H));
+    const double d = i * BOYS_H - T;
+    const double *row = tab + i * (BOYS_M + 1) + m;
+    double acc = row[BOYS_TAYLOR];
 #pragma unroll
-        for (int k = BOYS_TAYLOR - 1; k >= 0; --k) acc = row[k] + acc * (d * (1.0 / (k + 1)));
-        return acc;
-    }
-    const double it = 1.0 / T;
-    double f = 0.88622692545275801365 * sqrt(it);
-    const double et = exp(-T), h = 0.5 * it;
-    for (int k = 0; k < m; ++k) f = ((2 * k + 1) * f - et) * h;
-    return f;
+    for (int k = BOYS_TAYLOR - 1; k >= 0; --k) acc = row[k] + acc * (d * (1.0 / (k + 1)));
+    return acc;
 }
 
-// The same in fp32, from the fp32 copy of the table that follows the fp64 one.
+// The same in fp32 for any T, from the fp32 copy of the table that follows the
+// fp64 one; above BOYS_TMAX F_0 = sqrt(pi / T) / 2 (erfc(6) < 3e-17) and the m
+// upward steps F_{k+1} = ((2k + 1) F_k - e^-T) / (2T), stable for large T.
 __device__ __forceinline__ float boys_order_fp32(float T, int m, const double *__restrict__ tab)
 {
     if (T < (float)BOYS_TMAX) {
@@ -121,24 +110,24 @@ __device__ __forceinline__ float boys_order_fp32(float T, int m, const double *_
 }
 
 // Shared memory of a warp-kernel CTA (TILE / 32 warps of base_n + q * per_q
-// elements of fsize bytes, the item lists, and the tile staging plus the
+// floats, the item lists, and the tile staging plus the
 // per-CTA gradient slab of a molecule of up to 32 atoms) and the largest
 // q <= q0 (at least 4) with which two such CTAs fit in one SM's 228 KB
 // (1 KB reserved per CTA); 0 if none does.
-constexpr size_t warp_cta_bytes(size_t fsize, int base_n, int per_q, size_t list_bytes, int q)
+constexpr size_t warp_cta_bytes(int base_n, int per_q, size_t list_bytes, int q)
 {
-    return (size_t)(TILE / 32) * ((fsize * (size_t)(base_n + q * per_q) + 15) & ~(size_t)15) + list_bytes + 64 +
+    return (size_t)(TILE / 32) * ((sizeof(float) * (size_t)(base_n + q * per_q) + 15) & ~(size_t)15) + list_bytes + 64 +
            (size_t)TILE * 12 * sizeof(double) + (size_t)TILE * 4 * sizeof(int) + 6 * (TB + TK) * sizeof(double) +
            2 * (TB + TK) * sizeof(int) + 3 * 32 * sizeof(double);
 }
-constexpr int warp_qt_two_ctas(size_t fsize, int base_n, int per_q, size_t list_bytes, int q0)
+constexpr int warp_qt_two_ctas(int base_n, int per_q, size_t list_bytes, int q0)
 {
     for (int q = q0; q >= 4; --q)
-        if (2 * (warp_cta_bytes(fsize, base_n, per_q, list_bytes, q) + 1024) <= 228 * 1024) return q;
+        if (2 * (warp_cta_bytes(base_n, per_q, list_bytes, q) + 1024) <= 228 * 1024) return q;
     return 0;
 }
 
-template <int LA, int LB, int LC, int LD, typename F>
+template <int LA, int LB, int LC, int LD>
 struct WarpLayout {
     static constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD);
     static constexpr int NAB = NA * NB, NCD = NC * ND;
@@ -148,8 +137,8 @@ struct WarpLayout {
     static constexpr int BJ = LB + 1, BT = L1 + 2, KJ = LD + 1, KT = L2 + 2;
     static constexpr int EBN = (LA + 2) * BJ * BT;  // one direction of the bra 1-D table
     static constexpr int EKN = (LC + 2) * KJ * KT;
-    // per ket primitive pair scalars: X, Y, Z (fp32: times s), T, th2, pref0, pref1,
-    // m0, m1 (fp64: -2 rho, -2 rho th2; fp32: -1, -th2), zc2, s, then s^0 .. s^(L+2)
+    // per ket primitive pair scalars: X, Y, Z (times s), T, th2, pref0, pref1,
+    // m0, m1 (-1, -th2), zc2, s, then s^0 .. s^(L+2)
     static constexpr int SC_X = 0, SC_T = 3, SC_TH2 = 4, SC_PREF = 5, SC_MUL = 7, SC_ZC2 = 9, SC_S = 10,
                          SC_POW = 11;
     // then, per operator, the base multipliers pref_op * mul_op^m for m <= L + 1
@@ -161,13 +150,13 @@ struct WarpLayout {
     static constexpr int PER_Q = 3 * EKN + NSC;
     static constexpr int BASE_N = 2 * NAB * NCD + 2 * NCD * NH1 + 2 * NCD * NH1P + NAB * NH1 + NCD * NH2 + 2 * NR +
                                   2 * (L + 2) + 3 * EBN;
-    static constexpr int QT_RAW = (int)((6144 / sizeof(F)) / PER_Q);
+    static constexpr int QT_RAW = (int)((6144 / sizeof(float)) / PER_Q);
     static constexpr int QT0 = QT_RAW < 4 ? 4 : (QT_RAW > 32 ? 32 : QT_RAW);
     static constexpr int ZMAX = NCD * NH2P, YMAX = NAB * NH1P;
     static constexpr size_t LIST_BYTES = (sizeof(unsigned) * (size_t)(ZMAX + YMAX) + 15) & ~(size_t)15;
-    static constexpr int QT_FIT = warp_qt_two_ctas(sizeof(F), BASE_N, PER_Q, LIST_BYTES, QT0);
+    static constexpr int QT_FIT = warp_qt_two_ctas(BASE_N, PER_Q, LIST_BYTES, QT0);
     static constexpr int QT = QT_FIT > 0 ? QT_FIT : QT0;
-    // element offsets (F units)
+    // offsets in floats
     static constexpr int o_gam = 0;                          // [2][NAB][NCD]
     static constexpr int o_F = o_gam + 2 * NAB * NCD;        // [2][NCD][NH1]
     static constexpr int o_W = o_F + 2 * NCD * NH1;          // [2][NCD][NH1P]
@@ -179,7 +168,7 @@ struct WarpLayout {
     static constexpr int o_Ek = o_Eb + 3 * EBN;              // [QT][3][EKN]
     static constexpr int o_sc = o_Ek + QT * 3 * EKN;         // [QT][NSC]
     static constexpr int TOTAL = o_sc + QT * NSC;
-    static constexpr size_t BYTES = (sizeof(F) * (size_t)TOTAL + 15) & ~(size_t)15;
+    static constexpr size_t BYTES = (sizeof(float) * (size_t)TOTAL + 15) & ~(size_t)15;
     static_assert(o_Ek == BASE_N, "BASE_N counts every array ahead of the ket tables");
     // (ZMAX, YMAX, LIST_BYTES above: the CTA-wide lists of the (cd, h2) items of
     // z and the (ab, h1) items of Y that lie in a derivative box, built once per CTA)
@@ -190,17 +179,12 @@ struct WarpLayout {
 
 // 1-D Hermite table of one direction of primitive pair ip, written to dst
 // as [i][j][t] (i <= LX + 1, j <= LY, t <= LX + LY + 1).
-template <int LX, int LY, typename F>
-__device__ __forceinline__ void pair_table(F *dst, const PrimPairs &pp, int ip, int dir, double cen0, double cen1)
+template <int LX, int LY>
+__device__ __forceinline__ void pair_table(float *dst, const PrimPairs &pp, int ip, int dir)
 {
     constexpr int J1 = LY + 1, T1 = LX + LY + 2;
-    F E[LX + 2][LY + 1][LX + LY + 2];
-    if constexpr (sizeof(F) == 4) {
-        etab<LX + 1, LY>(E, pp.fPA[dir * pp.n + ip], pp.fPB[dir * pp.n + ip], 0.5f / pp.fp[ip]);
-    } else {
-        const double P = dir == 0 ? pp.Px[ip] : (dir == 1 ? pp.Py[ip] : pp.Pz[ip]);
-        etab<LX + 1, LY>(E, (F)(P - cen0), (F)(P - cen1), (F)(0.5 / pp.p[ip]));
-    }
+    float E[LX + 2][LY + 1][LX + LY + 2];
+    etab<LX + 1, LY>(E, pp.fPA[dir * pp.n + ip], pp.fPB[dir * pp.n + ip], 0.5f / pp.fp[ip]);
 #pragma unroll
     for (int i = 0; i <= LX + 1; ++i)
 #pragma unroll
@@ -212,19 +196,19 @@ __device__ __forceinline__ void pair_table(F *dst, const PrimPairs &pp, int ip, 
 // One contracted quartet by one warp, bra primitive pairs ib0, ib0 + ibs, ...
 // acc[0..2] += d/dA, acc[3..5] += d/dA + d/dB, acc[6..8] += d/dC (this lane's
 // share; the caller sums the warp).
-template <int LA, int LB, int LC, int LD, typename F>
-__device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *zlist, int nz, const unsigned *ylist, int ny,
+template <int LA, int LB, int LC, int LD>
+__device__ void quartet_warp(float *sm, int lane, const float *smallf, const unsigned *zlist, int nz, const unsigned *ylist, int ny,
                              const GeoArgs &geo, const DensArgs &den, const PrimPairs &pp, int sa, int sb, int sc,
                              int sd, int pb0, int nbp, int ib0, int ibs, int pk0, int nkp, double scale,
                              const double *boys, double (&acc)[9])
 {
-    using Lay = WarpLayout<LA, LB, LC, LD, F>;
+    using F = float;
+    using Lay = WarpLayout<LA, LB, LC, LD>;
     constexpr int NB = Lay::NB, ND = Lay::ND, NAB = Lay::NAB, NCD = Lay::NCD;
     constexpr int L1 = Lay::L1, L = Lay::L;
     constexpr int NH1 = Lay::NH1, NH1P = Lay::NH1P, NH2 = Lay::NH2, NH2P = Lay::NH2P, NR = Lay::NR;
     constexpr int BJ = Lay::BJ, BT = Lay::BT, KJ = Lay::KJ, KT = Lay::KT, EBN = Lay::EBN, EKN = Lay::EKN;
     constexpr int QT = Lay::QT, NSC = Lay::NSC, KW = Lay::KW;
-    constexpr bool FP32 = sizeof(F) == 4;
     F *gam = sm + Lay::o_gam, *Fr = sm + Lay::o_F, *W = sm + Lay::o_W, *E3b = sm + Lay::o_E3b;
     F *E3k = sm + Lay::o_E3k, *R = sm + Lay::o_R, *base = sm + Lay::o_base, *Eb = sm + Lay::o_Eb;
     F *Ekall = sm + Lay::o_Ek, *scall = sm + Lay::o_sc;
@@ -233,8 +217,7 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
     const bool ominf = isinf((float)om2);
     const int nbf = den.nbf;
     const int fa = geo.sh_bf[sa], fb = geo.sh_bf[sb], fc = geo.sh_bf[sc], fd = geo.sh_bf[sd];
-    const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xb = geo.xyz + 3 * geo.sh_atom[sb];
-    const double *xc = geo.xyz + 3 * geo.sh_atom[sc], *xd = geo.xyz + 3 * geo.sh_atom[sd];
+    const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xc = geo.xyz + 3 * geo.sh_atom[sc];
 
     // ---- Gamma_s[ab][cd]: the 8 permutation images of the pair products, times scale
     for (int it = lane; it < NAB * NCD; it += 32) {
@@ -266,14 +249,14 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
     if (ket_once)
         for (int it = lane; it < 3 * nkp; it += 32) {
             const int j = it / 3, dir = it % 3;
-            pair_table<LC, LD, F>(Ekall + (j * 3 + dir) * EKN, pp, pk0 + j, dir, xc[dir], xd[dir]);
+            pair_table<LC, LD>(Ekall + (j * 3 + dir) * EKN, pp, pk0 + j, dir);
         }
     __syncwarp();
 
     for (int ib = ib0; ib < nbp; ib += ibs) {
         const int ip = pb0 + ib;
         // ---- bra tables (lanes 0-2), then E3b[ab][h1] and W = 0
-        if (lane < 3) pair_table<LA, LB, F>(Eb + lane * EBN, pp, ip, lane, xa[lane], xb[lane]);
+        if (lane < 3) pair_table<LA, LB>(Eb + lane * EBN, pp, ip, lane);
         __syncwarp();
         for (int it = lane; it < NAB * NH1; it += 32) {
             const int ab = it / NH1, h = it % NH1;
@@ -303,7 +286,7 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
         }
         __syncwarp();
 
-        // per-p fp32 partial sums of this lane (fp64 route: accumulated directly)
+        // per-p fp32 partial sums of this lane
         F pC0 = F(0), pC1 = F(0), pC2 = F(0);
         // this lane's W items it = lane + 32 k, both operators, in registers
         F w0r[KW], w1r[KW];
@@ -315,73 +298,44 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
             if (!ket_once)
                 for (int it = lane; it < 3 * nq; it += 32) {
                     const int j = it / 3, dir = it % 3;
-                    pair_table<LC, LD, F>(Ekall + (j * 3 + dir) * EKN, pp, pk0 + q0 + j, dir, xc[dir], xd[dir]);
+                    pair_table<LC, LD>(Ekall + (j * 3 + dir) * EKN, pp, pk0 + q0 + j, dir);
                 }
             if (lane < nq) {
                 F *sc_ = scall + lane * NSC;
                 const int kp = pk0 + q0 + lane;
-                if constexpr (FP32) {
-                    const long long nr = pp.n;
-                    const float pf = pp.fp[ip], qf = pp.fp[kp], pq = pf + qf, rho = pf * qf / pq;
-                    const float X = pp.fPA[ip] - pp.fPA[kp] + (float)(xa[0] - xc[0]);
-                    const float Y = pp.fPA[nr + ip] - pp.fPA[nr + kp] + (float)(xa[1] - xc[1]);
-                    const float Z = pp.fPA[2 * nr + ip] - pp.fPA[2 * nr + kp] + (float)(xa[2] - xc[2]);
-                    const float s = sqrtf(2.0f * rho);
-                    const float om2f = (float)om2;
-                    const float th2 = (nops == 2) ? (ominf ? 1.0f : om2f / (om2f + rho)) : 1.0f;
-                    const float pref = 34.986836655249725f * rsqrtf(pq) / (pf * qf) * pp.fK[ip] * pp.fK[kp];
-                    sc_[0] = X * s;
-                    sc_[1] = Y * s;
-                    sc_[2] = Z * s;
-                    sc_[Lay::SC_T] = rho * (X * X + Y * Y + Z * Z);
-                    sc_[Lay::SC_TH2] = th2;
-                    sc_[Lay::SC_PREF] = pref;
-                    sc_[Lay::SC_PREF + 1] = pref * sqrtf(th2);
-                    sc_[Lay::SC_MUL] = -1.0f;
-                    sc_[Lay::SC_MUL + 1] = -th2;
-                    sc_[Lay::SC_ZC2] = 2.0f * pp.fza[kp];
-                    sc_[Lay::SC_S] = s;
-                    float pw = 1.0f;
+                const long long nr = pp.n;
+                const float pf = pp.fp[ip], qf = pp.fp[kp], pq = pf + qf, rho = pf * qf / pq;
+                const float X = pp.fPA[ip] - pp.fPA[kp] + (float)(xa[0] - xc[0]);
+                const float Y = pp.fPA[nr + ip] - pp.fPA[nr + kp] + (float)(xa[1] - xc[1]);
+                const float Z = pp.fPA[2 * nr + ip] - pp.fPA[2 * nr + kp] + (float)(xa[2] - xc[2]);
+                const float s = sqrtf(2.0f * rho);
+                const float om2f = (float)om2;
+                const float th2 = (nops == 2) ? (ominf ? 1.0f : om2f / (om2f + rho)) : 1.0f;
+                const float pref = 34.986836655249725f * rsqrtf(pq) / (pf * qf) * pp.fK[ip] * pp.fK[kp];
+                sc_[0] = X * s;
+                sc_[1] = Y * s;
+                sc_[2] = Z * s;
+                sc_[Lay::SC_T] = rho * (X * X + Y * Y + Z * Z);
+                sc_[Lay::SC_TH2] = th2;
+                sc_[Lay::SC_PREF] = pref;
+                sc_[Lay::SC_PREF + 1] = pref * sqrtf(th2);
+                sc_[Lay::SC_MUL] = -1.0f;
+                sc_[Lay::SC_MUL + 1] = -th2;
+                sc_[Lay::SC_ZC2] = 2.0f * pp.fza[kp];
+                sc_[Lay::SC_S] = s;
+                float pw = 1.0f;
 #pragma unroll
-                    for (int k = 0; k <= L + 2; ++k) {
-                        sc_[Lay::SC_POW + k] = pw;
-                        pw *= s;
-                    }
-                    float b0 = pref, b1 = pref * sqrtf(th2);
+                for (int k = 0; k <= L + 2; ++k) {
+                    sc_[Lay::SC_POW + k] = pw;
+                    pw *= s;
+                }
+                float b0 = pref, b1 = pref * sqrtf(th2);
 #pragma unroll
-                    for (int m = 0; m <= L + 1; ++m) {
-                        sc_[Lay::SC_PW + m] = b0;
-                        sc_[Lay::SC_PW + L + 2 + m] = b1;
-                        b0 = -b0;
-                        b1 *= -th2;
-                    }
-                } else {
-                    const double p = pp.p[ip], q = pp.p[kp], pq = p + q, rho = p * q / pq;
-                    const double X = pp.Px[ip] - pp.Px[kp], Y = pp.Py[ip] - pp.Py[kp], Z = pp.Pz[ip] - pp.Pz[kp];
-                    const double th2 = (nops == 2) ? (ominf ? 1.0 : om2 / (om2 + rho)) : 1.0;
-                    const double pref = 34.986836655249725 / (p * q * sqrt(pq)) * pp.K[ip] * pp.K[kp];
-                    sc_[0] = X;
-                    sc_[1] = Y;
-                    sc_[2] = Z;
-                    sc_[Lay::SC_T] = rho * (X * X + Y * Y + Z * Z);
-                    sc_[Lay::SC_TH2] = th2;
-                    sc_[Lay::SC_PREF] = pref;
-                    sc_[Lay::SC_PREF + 1] = pref * sqrt(th2);
-                    sc_[Lay::SC_MUL] = -2.0 * rho;
-                    sc_[Lay::SC_MUL + 1] = -2.0 * rho * th2;
-                    sc_[Lay::SC_ZC2] = 2.0 * pp.za[kp];
-                    sc_[Lay::SC_S] = 1.0;
-#pragma unroll
-                    for (int k = 0; k <= L + 2; ++k) sc_[Lay::SC_POW + k] = 1.0;
-                    double b0 = pref, b1 = pref * sqrt(th2);
-                    const double m0 = -2.0 * rho, m1 = -2.0 * rho * th2;
-#pragma unroll
-                    for (int m = 0; m <= L + 1; ++m) {
-                        sc_[Lay::SC_PW + m] = b0;
-                        sc_[Lay::SC_PW + L + 2 + m] = b1;
-                        b0 *= m0;
-                        b1 *= m1;
-                    }
+                for (int m = 0; m <= L + 1; ++m) {
+                    sc_[Lay::SC_PW + m] = b0;
+                    sc_[Lay::SC_PW + L + 2 + m] = b1;
+                    b0 = -b0;
+                    b1 *= -th2;
                 }
             }
             __syncwarp();
@@ -395,14 +349,10 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
                     if (op < nops && m <= L + 1) {
                         const F T = sc_[Lay::SC_T] * (op ? sc_[Lay::SC_TH2] : F(1));
                         F fm;
-                        if constexpr (FP32) {
-                            if (T < 1.0f) {
-                                fm = (float)boys_order_fp64((double)T, m, boys);
-                            } else {
-                                fm = boys_order_fp32(T, m, boys);
-                            }
+                        if (T < 1.0f) {
+                            fm = (float)boys_order_fp64((double)T, m, boys);
                         } else {
-                            fm = boys_order_fp64(T, m, boys);
+                            fm = boys_order_fp32(T, m, boys);
                         }
                         base[op * (L + 2) + m] = sc_[Lay::SC_PW + op * (L + 2) + m] * fm;
                     }
@@ -459,7 +409,7 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
                     if (t <= cx + dx && u <= cy + dy && v <= cz + dz) {
                         e = Ek[(cx * KJ + dx) * KT + t] * Ek[EKN + (cy * KJ + dy) * KT + u] *
                             Ek[2 * EKN + (cz * KJ + dz) * KT + v];
-                        if constexpr (FP32) e *= sc_[Lay::SC_POW + t + u + v];
+                        e *= sc_[Lay::SC_POW + t + u + v];
                         e = flip_if(e, t + u + v);
                     }
                     E3k[it] = e;
@@ -478,9 +428,8 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
                     cart_xyz(LD, cd % ND, dx, dy, dz);
                     const int nx = cx + dx, ny = cy + dy, nz = cz + dz;
                     const F *e = E3k + cd * NH2;
-                    // fp64: the terms go straight into the lane's W registers;
-                    // fp32: the item's sum is scaled by s^|h1| first
-                    F w0 = FP32 ? F(0) : w0r[k], w1 = FP32 ? F(0) : w1r[k];
+                    // the item's sum is scaled by s^|h1| first
+                    F w0 = F(0), w1 = F(0);
                     for (int t2 = 0; t2 <= nx; ++t2)
                         for (int u2 = 0; u2 <= ny; ++u2)
                             for (int v2 = 0; v2 <= nz; ++v2) {
@@ -489,14 +438,9 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
                                 w0 += ev * R0[r];
                                 w1 += ev * R1[r];
                             }
-                    if constexpr (FP32) {
-                        const F sh = sc_[Lay::SC_POW + t1 + u1 + v1];
-                        w0r[k] += w0 * sh;
-                        w1r[k] += w1 * sh;
-                    } else {
-                        w0r[k] = w0;
-                        w1r[k] = w1;
-                    }
+                    const F sh = sc_[Lay::SC_POW + t1 + u1 + v1];
+                    w0r[k] += w0 * sh;
+                    w1r[k] += w1 * sh;
                 }
                 // ---- z[cd][h2] over the derivative boxes of cd, contracted with dE^{cd}/dC
                 {
@@ -524,16 +468,11 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
 #pragma unroll
                                 for (int v1 = 0; v1 <= L1 - t1 - u1; ++v1) {
                                     const int r = hidx(t1 + t2, u1 + u2, v1 + v2);
-                                    if constexpr (FP32) {
-                                        const F sh = sc_[Lay::SC_POW + t1 + u1 + v1];
-                                        z += (f0[hidx(t1, u1, v1)] * R0[r] + f1[hidx(t1, u1, v1)] * R1[r]) * sh;
-                                    } else {
-                                        z += f0[hidx(t1, u1, v1)] * R0[r];
-                                        z += f1[hidx(t1, u1, v1)] * R1[r];
-                                    }
+                                    const F sh = sc_[Lay::SC_POW + t1 + u1 + v1];
+                                    z += (f0[hidx(t1, u1, v1)] * R0[r] + f1[hidx(t1, u1, v1)] * R1[r]) * sh;
                                 }
                         const int n2 = t2 + u2 + v2;
-                        if constexpr (FP32) z *= sc_[Lay::SC_POW + n2];
+                        z *= sc_[Lay::SC_POW + n2];
                         z = flip_if(z, n2);
                         const F ex = inx ? Ex[(cx * KJ + dx) * KT + t2] : F(0);
                         const F ey = iny ? Ey[(cy * KJ + dy) * KT + u2] : F(0);
@@ -574,7 +513,7 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
         // ---- Y[ab][h1] = sum_s sum_cd Gamma_s[ab][cd] W_s[cd][h1] with dE/dA and the shifted E
         F a0 = F(0), a1 = F(0), a2 = F(0), t0 = F(0), t1_ = F(0), t2_ = F(0);
         {
-            const F za2 = FP32 ? (F)(2.0f * pp.fza[ip]) : (F)(2.0 * pp.za[ip]);
+            const F za2 = 2.0f * pp.fza[ip];
             const F *Ex = Eb, *Ey = Eb + EBN, *Ez = Eb + 2 * EBN;
             for (int iy = lane; iy < ny; iy += 32) {
                 const unsigned yi = ylist[iy];
@@ -632,11 +571,12 @@ __device__ void quartet_warp(F *sm, int lane, const F *smallf, const unsigned *z
 // Persistent warp-cooperative class kernel: 4 warps per CTA, warp w takes
 // quartets w, w + 4, ... of each unit (tile, chunk, split); the tile's
 // 12 x TILE contributions are then added in a fixed order (tile_reduce).
-template <int LA, int LB, int LC, int LD, typename F>
+template <int LA, int LB, int LC, int LD>
 __global__ void __launch_bounds__(TILE, 2) k_grad_warp(const MolDesc *__restrict__ mols, ClassLaunch cl, OutArgs out,
                                                     const double *__restrict__ boys)
 {
-    using Lay = WarpLayout<LA, LB, LC, LD, F>;
+    using F = float;
+    using Lay = WarpLayout<LA, LB, LC, LD>;
     constexpr int NG = TILE / 32;
     extern __shared__ double smem[];
     const int nacc3 = out.use_smem ? out.natom_max * 3 : 0;
@@ -694,7 +634,7 @@ __global__ void __launch_bounds__(TILE, 2) k_grad_warp(const MolDesc *__restrict
     for (long long it = blockIdx.x; it < cl.ntiles * C * S; it += gridDim.x) {
         const long long tile = it / (C * S);
         const int chunk = (int)((it / S) % C), split = (int)(it % S);
-        const uint4 tl = cl.tiles[tile * cl.stride];
+        const uint4 tl = cl.tiles[tile];
         const int mol = (int)tl.x;
         if (mol != cur) {
             if (out.use_smem) {
@@ -745,7 +685,7 @@ __global__ void __launch_bounds__(TILE, 2) k_grad_warp(const MolDesc *__restrict
                 double acc[9];
 #pragma unroll
                 for (int k = 0; k < 9; ++k) acc[k] = 0.0;
-                quartet_warp<LA, LB, LC, LD, F>(wsm, lane, smallf, zlist, nz, ylist, ny, geo, md.den, pp, sa, sb, sc, sd,
+                quartet_warp<LA, LB, LC, LD>(wsm, lane, smallf, zlist, nz, ylist, ny, geo, md.den, pp, sa, sb, sc, sd,
                                                 bra.poff[bi], nbp, split, S, ket.poff[ki], nkp, scale, boys, acc);
 #pragma unroll
                 for (int k = 0; k < 9; ++k)
@@ -795,25 +735,25 @@ __global__ void __launch_bounds__(TILE, 2) k_grad_warp(const MolDesc *__restrict
     }
     if ((threadIdx.x & 31) == 0 && (nq || npq)) {
         atomicAdd(out.counters + 0, nq);
-        atomicAdd(out.counters + (sizeof(F) == 4 ? 3 : 1), npq);
-        atomicAdd(out.counters + (sizeof(F) == 4 ? 5 : 4), nbv);
-        if (sizeof(F) == 4) atomicAdd(out.counters + 2, nq);
+        atomicAdd(out.counters + 2, nq);
+        atomicAdd(out.counters + 3, npq);
+        atomicAdd(out.counters + 5, nbv);
     }
 }
 
-template <int LA, int LB, int LC, int LD, typename F>
+template <int LA, int LB, int LC, int LD>
 constexpr size_t warp_kernel_smem()
 {
-    return (size_t)(TILE / 32) * WarpLayout<LA, LB, LC, LD, F>::bytes() + WarpLayout<LA, LB, LC, LD, F>::LIST_BYTES + 64;
+    return (size_t)(TILE / 32) * WarpLayout<LA, LB, LC, LD>::bytes() + WarpLayout<LA, LB, LC, LD>::LIST_BYTES + 64;
 }
 
-template <int LA, int LB, int LC, int LD, typename F>
+template <int LA, int LB, int LC, int LD>
 cudaError_t launch_warp(int gcap, size_t smem, cudaStream_t st, const MolDesc *mols, const ClassLaunch &cl,
                         const OutArgs &out, const double *boys)
 {
     OutArgs o = out;
-    const size_t sm = unit_smem(warp_kernel_smem<LA, LB, LC, LD, F>(), smem, o);
-    return launch_units(k_grad_warp<LA, LB, LC, LD, F>, TILE / 32, gcap, sm, st, mols, cl, o, boys);
+    const size_t sm = unit_smem(warp_kernel_smem<LA, LB, LC, LD>(), smem, o);
+    return launch_units(k_grad_warp<LA, LB, LC, LD>, TILE / 32, gcap, sm, st, mols, cl, o, boys);
 }
 
 }  // namespace tg

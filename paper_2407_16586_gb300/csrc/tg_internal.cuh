@@ -102,11 +102,9 @@ struct MolDesc {
 struct ClassLaunch {
     int P, Q;                  // bra and ket pair classes (same list iff P == Q)
     long long ntiles;
-    const uint4 *tiles;        // (molecule, bra tile, ket tile, 0), grouped by molecule; tile t at tiles[t * stride]
-    long long stride;          // 1, or nranks for tile-cyclic shards
+    const uint4 *tiles;        // (molecule, bra tile, ket tile, 0), grouped by molecule
     int nsplit;                // units per tile along the bra primitive pairs (>= 1)
     int nchunk;                // cooperative kernel: quartet chunks per tile (divides TILE / groups)
-    int kind;                  // 0: default form of the class, 1: thread, 2: group, 3: warp
     int split_req;             // bra-primitive splits per tile requested by the autotuner (0: automatic)
 };
 
@@ -162,36 +160,6 @@ __device__ __forceinline__ void tile_reduce(const double *stg, const int *sat, d
             const int a = ratom[r];
             if (a >= 0) tgt[a * 3 + t] += red[r * 3 + t];
         }
-    }
-}
-
-// ---------------------------------------------------------------- Boys
-// F_m(T) for m = 0..M (M <= BOYS_M - BOYS_TAYLOR).  T < 36: Taylor expansion
-// of the top order about the nearest grid point, F_m(T0-d) = sum_k F_{m+k}(T0) d^k/k!,
-// then downward recursion F_{m} = (2T F_{m+1} + e^-T)/(2m+1).  T >= 36: F_0 =
-// sqrt(pi/T)/2 (erfc(6) < 3e-17) and upward recursion.
-template <int M>
-__device__ __forceinline__ void boys_fp64(double T, double (&F)[M + 1], const double *__restrict__ tab)
-{
-    if (T < BOYS_TMAX) {
-        int i = __double2int_rn(T * (1.0 / BOYS_H));
-        double d = i * BOYS_H - T;
-        const double *row = tab + i * (BOYS_M + 1) + M;
-        double acc = row[BOYS_TAYLOR];
-#pragma unroll
-        for (int k = BOYS_TAYLOR - 1; k >= 0; --k) acc = row[k] + acc * d * (1.0 / (k + 1));
-        F[M] = acc;
-        double et = exp(-T);
-        double t2 = 2.0 * T;
-#pragma unroll
-        for (int m = M - 1; m >= 0; --m) F[m] = (t2 * F[m + 1] + et) * (1.0 / (2 * m + 1));
-    } else {
-        double it = 1.0 / T;
-        F[0] = 0.88622692545275801365 * sqrt(it);
-        double et = exp(-T);
-        double h = 0.5 * it;
-#pragma unroll
-        for (int m = 0; m < M; ++m) F[m + 1] = ((2 * m + 1) * F[m] - et) * h;
     }
 }
 
