@@ -3,6 +3,7 @@
 // the final reduction.  Every arithmetic step of the gradient runs in the
 // CUDA kernels; the host only orders work and moves buffers.
 #include <algorithm>
+#include <cfloat>
 #include <cstdio>
 #include <cstdint>
 #include <chrono>
@@ -70,7 +71,12 @@ inline size_t al(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
 // Streams the class launches of one call are spread over.  The 42 lists of a
 // call are independent, and most lists of a small molecule end in a tail of a
 // few long quartets on a few SMs (c1: 21 launches of 0.3 to 3.6 ms each, 27 ms
-// one after the other, with about 5 ms of fp64 work).  Owned by the handle
+// one after the other, with about 5 ms of fp64 work).  Six: with 1 / 3 / 6 / 12
+// streams 3 atoms in fp64 take 4.58 / 2.82 / 2.20 / 2.06 ms, 6 atoms 20.4 / 15.4 /
+// 15.3 / 15.2, 12 atoms 75.3 / 52.5 / 51.5 / 51.6, 1/8 of 32 atoms 222 / 198 / 199 /
+// 200, on the learned route 18.9 / 14.3 / 15.5 / 15.4 (6 atoms) and 176 / 168 / 173 /
+// 169 (1/8 of 32).  Long lists gain nothing: all of 32 atoms learned 1 275 ms here
+// and 1 257 ms of kernels one after the other.  Owned by the handle
 // whose work areas the launches use; every call forks from the caller's
 // stream and joins it again, also on an error.
 struct SideStreams {
@@ -152,6 +158,7 @@ struct tg_basis {
     int *d_sh_atom = nullptr, *d_sh_l = nullptr, *d_sh_nprim = nullptr, *d_sh_poff = nullptr, *d_sh_bf = nullptr;
     std::vector<double> Q, Qd;  // per canonical pair key (x >= y)
     double Qmax = 0.0, Qdmax = 0.0;
+    double exp_max = 0.0;  // largest primitive exponent
     long long *d_bpoff = nullptr;  // per canonical pair key: offset of its primitive-pair bounds
     double *d_bp = nullptr;        // primitive-pair bounds b_kl (larger shell index first)
     DevArena ws1, ws2;
@@ -389,6 +396,7 @@ int tg_basis_create(int natom, const double *xyz, int nshell, const int *shell_a
         so += 2 * shell_l[s] + 1;
     }
     b->nsph = so;
+    b->exp_max = *std::max_element(exps, exps + nprim);
     int rc = basis_setup(b, xyz, exps, coefs);
     if (rc != TG_OK) {
         free_basis(b);
@@ -493,6 +501,15 @@ int check_pairs(int npair, const tg_pair *pairs, const tg_options &opt, double &
     return TG_OK;
 }
 
+// omega as the kernels take it: infinite where its square leaves the range of
+// fp32 (they form it) and theta^2 = omega^2 / (omega^2 + rho) rounds to 1 in fp64
+// for every primitive quartet, whose rho is at most the largest exponent.
+double kernel_omega(const tg_basis *b, double omega)
+{
+    const double w2 = omega * omega;
+    return w2 > FLT_MAX && w2 * 0x1p-54 > b->exp_max ? INFINITY : omega;
+}
+
 // Densities, block factors, screened pairs, primitive pairs, unrouted tiles.
 int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &opt, cudaStream_t st, Plan &pl,
               bool host_tiles = true, bool fock = false, bool slabs = false)
@@ -510,7 +527,7 @@ int make_plan(tg_basis *b, int npair, const tg_pair *pairs, const tg_options &op
     den.npair = npair;
     den.nbf = nbf;
     den.use_lr = use_lr;
-    den.omega = omega;
+    den.omega = kernel_omega(b, omega);
     for (int p = 0; p < npair; ++p) {
         den.cJ[p] = pairs[p].c_J;
         den.cK[p] = pairs[p].c_K;
@@ -1696,7 +1713,7 @@ int tg_fock2e(const tg_basis *cb, int npair, const tg_fpair *fpairs, const tg_op
     int rc = make_plan(b, 2, pseudo, po, st, pl, false, true);
     if (rc != TG_OK) return rc;
     pl.den.use_lr = use_lr;
-    pl.den.omega = omega;
+    pl.den.omega = kernel_omega(b, omega);
     pl.scr.scale = pl.scale;
     int launches = pl.launches + 1;
     DevArena &V = b->ws2;

@@ -106,7 +106,7 @@ __device__ void quartet_coop(float *sm, int lane, int bar, const GeoArgs &geo, c
     const F *spow = scl + 16;
     const bool lr = den.use_lr;
     const double om2 = den.omega * den.omega;
-    const bool ominf = isinf((float)om2);
+    const bool ominf = isinf(den.omega);
     const int nbf = den.nbf;
     const int fa = geo.sh_bf[sa], fb = geo.sh_bf[sb], fc = geo.sh_bf[sc], fd = geo.sh_bf[sd];
     const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xc = geo.xyz + 3 * geo.sh_atom[sc];

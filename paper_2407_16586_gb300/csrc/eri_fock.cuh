@@ -76,7 +76,7 @@ __device__ void quartet_fock_ints(double *sm, int lane, const GeoArgs &geo, cons
     double *vb = sm + Lay::o_X, *vk = vb + Lay::NE1, *half = vk + Lay::NE2;
     const auto &TBra = pair_tab<LA, LB>();
     const auto &TKet = pair_tab<LC, LD>();
-    const bool ominf = isinf(omega * omega);
+    const bool ominf = isinf(omega);
     const double om = ominf ? 1.0 : omega;
     const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xb = geo.xyz + 3 * geo.sh_atom[sb];
     const double *xc = geo.xyz + 3 * geo.sh_atom[sc], *xd = geo.xyz + 3 * geo.sh_atom[sd];

@@ -784,7 +784,7 @@ __device__ void group_herm(double *sm, int tid, int k0, int kg, const GroupInfo 
     const auto &TBra = pair_tab<LA, LB>();
     const auto &TKet = pair_tab<LC, LD>();
     const int nops = den.use_lr ? 2 : 1;
-    const bool ominf = isinf(den.omega * den.omega);  // theta = 1 to the last bit before that
+    const bool ominf = isinf(den.omega);
     const double om = ominf ? 1.0 : den.omega;
     if constexpr (KQ == 1) kg = 1;
     const int LG = 32 / kg, kq = lane / LG, sl = lane % LG;
@@ -1029,13 +1029,16 @@ __device__ void group_herm(double *sm, int tid, int k0, int kg, const GroupInfo 
     }
 }
 
-// Warps of a CTA and CTAs an SM the registers are limited to: 16 warps at 128
-// registers up to L = 2, 12 at 168 for L = 3, 8 at 255 above.  One warp per
-// scheduler already covers most of the fp64 pipe; the others fill the gaps left
-// by the transforms' loads and by dependent steps.  CTAs are small (one or two
-// warps) because a CTA gives its shared memory back only when its last warp
-// ends: with 8 to 16 warps a single long quartet kept a whole SM from the next
-// class's launch.
+// Warps of a CTA, and CTAs an SM that the registers are limited to: 16 warps at
+// 128 registers up to L = 2, 12 at 168 for L = 3, 8 at 255 above (12 at 168 for
+// (dd|dp), of whose three CTAs shared memory holds two).  One warp per scheduler
+// already covers most of the fp64 pipe; the others fill the gaps left by the
+// transforms' loads and by dependent steps.  1/8 of the 32-atom workload in fp64,
+// classes one after the other and as one call: 220 and 199 ms; with 12 warps up to
+// L = 2, 8 for L = 3 and 6 for L = 4: 220 and 195 ms; with 20, 16 and 12: 225 and
+// 231 ms.  CTAs are small (one or two warps) because a CTA gives its shared memory
+// back only when its last warp ends: with 8 to 16 warps a single long quartet kept
+// a whole SM from the next class's launch.
 template <int LA, int LB, int LC, int LD>
 struct HermOp {
     using Lay = HermLay<LA, LB, LC, LD>;
@@ -1045,7 +1048,9 @@ struct HermOp {
     static constexpr int cta_workers = L <= 3 ? 2 : 1, min_ctas = L == 3 ? 6 : (NW == 1 ? 8 : (NW == 2 ? 4 : 10 - L));
     // primitive quartets of a contracted one up to which ket pairs are grouped
     // (kg times it stays below): the smaller the class, the more of a quartet's
-    // work is the density transform that a group shares
+    // work is the density transform that a group shares.  On that shard (ps|ss) takes
+    // 10.4 ms (9.6 at twice these bounds, 11.8 at half, 16.2 ungrouped), (pp|ss) 7.5
+    // (7.2, 8.0, 9.0), (ss|ss) 2.2 (2.2, 2.3, 3.3; 2.6 always grouped)
     static constexpr int group_below = L == 0 ? 512 : (L == 1 ? 256 : (L == 2 ? 128 : 64));
     static __device__ __forceinline__ void group(double *sm, int tid, int k0, int kg, const GroupInfo &gi,
                                                  const MolDesc &md, int sa, int sb, int pb0, int nbp, int ib0, int ibs, const double *boys,
@@ -1057,8 +1062,9 @@ struct HermOp {
 
 // Persistent class kernel; every warp works alone.  Warp w of W takes the
 // units (tile, chunk of cl.nchunk per tile, split) w, 2W - 1 - w, 2W + w, ...:
-// the tile list is in decreasing cost, so the alternating order evens the
-// sums out.  A unit's quartets are taken in groups of up to KQ ket pairs of one
+// a molecule's tiles are in decreasing cost, so the alternating order evens the
+// sums out (in a batch the order starts again with every molecule, and two of
+// 21 and 26 atoms take 634 ms against 601 ms one after the other).  A unit's quartets are taken in groups of up to KQ ket pairs of one
 // bra pair.  Their components are added to the warp's own gradient (shared
 // memory, or with out.use_smem = 0 the warp's slab), so the schedule and the
 // order of all sums are fixed and results are bitwise reproducible.

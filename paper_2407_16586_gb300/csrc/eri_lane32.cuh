@@ -268,7 +268,7 @@ __device__ void quartet_lane32(double *sm, int lane, const GeoArgs &geo, const D
     float *gam = reinterpret_cast<float *>(sm) + Lay::o_gam, *P = reinterpret_cast<float *>(sm) + Lay::o_P;
     const int nbf = den.nbf, nops = den.use_lr ? 2 : 1;
     const float om2f = (float)(den.omega * den.omega);
-    const bool ominf = isinf(om2f);
+    const bool ominf = isinf(den.omega);
     const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xc = geo.xyz + 3 * geo.sh_atom[sc];
     const float ACx = (float)(xa[0] - xc[0]), ACy = (float)(xa[1] - xc[1]), ACz = (float)(xa[2] - xc[2]);
     const long long nr = pp.n;

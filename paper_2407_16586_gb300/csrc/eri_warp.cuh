@@ -214,7 +214,7 @@ __device__ void quartet_warp(float *sm, int lane, const float *smallf, const uns
     F *Ekall = sm + Lay::o_Ek, *scall = sm + Lay::o_sc;
     const int nops = den.use_lr ? 2 : 1;
     const double om2 = den.omega * den.omega;
-    const bool ominf = isinf((float)om2);
+    const bool ominf = isinf(den.omega);
     const int nbf = den.nbf;
     const int fa = geo.sh_bf[sa], fb = geo.sh_bf[sb], fc = geo.sh_bf[sc], fd = geo.sh_bf[sd];
     const double *xa = geo.xyz + 3 * geo.sh_atom[sa], *xc = geo.xyz + 3 * geo.sh_atom[sc];
