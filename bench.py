@@ -539,8 +539,8 @@ def main():
     ap.add_argument("--fock", action="store_true", help="time the Fock-type build (tg_fock2e) instead")
     ap.add_argument("--spherical", action="store_true", help="time tg_grad2e_sph (spherical shells) instead")
     ap.add_argument("--autotune", type=int, default=1, choices=[0, 1],
-                    help="1 (default): tg_options.autotune = 1, launches tuned per class list on the first "
-                         "warm-up call and reused; 0: the per-class default forms")
+                    help="1 (default): tg_options.autotune = 1, launches of the shorter class lists tuned on the "
+                         "first warm-up call and reused; 0: automatic grids and work units")
     ap.add_argument("--shard", type=int, default=1, help="c4, c5: time tile-cyclic shard 0 of this many")
     args = ap.parse_args()
     if args.opcount:

@@ -307,11 +307,11 @@ class Basis:
         """Gradient (natom x 3) of host numpy pairs [(A, B, c_J, c_K, c_K_lr, omega)], or of
         torch CUDA tensors (then the densities and ``out`` stay on the device).  ``kernel`` 0 to
         3 (tg_options.kernel_kind) is accepted and has no effect: every class and precision has
-        one kernel form.  ``class_mask``
-        (0 = all) keeps the angular classes whose bits are set.  ``autotune`` 1 tunes the
-        launches of every class list on this basis's first such call and reuses them, 2
-        tunes again (tg_options.autotune).  ``spherical``: the matrices are nsph x nsph over
-        spherical functions (tg_grad2e_sph)."""
+        one kernel form.  ``class_mask`` (0 = all) keeps the angular classes whose bits are set.
+        ``autotune`` 1 tunes the launches of the shorter class lists on this basis's first such
+        call and reuses them, 2 tunes again (tg_options.autotune).  ``spherical``: the matrices
+        are nsph x nsph over spherical functions (tg_grad2e_sph).  The mixed modes trade accuracy
+        for time on some systems only (tg_options.precision gives figures)."""
         opt = tg_options_default()
         opt.kernel_kind = int(kernel)
         opt.autotune = int(autotune)

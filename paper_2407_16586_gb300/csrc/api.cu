@@ -75,10 +75,10 @@ inline size_t al(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
 // streams 3 atoms in fp64 take 4.58 / 2.82 / 2.20 / 2.06 ms, 6 atoms 20.4 / 15.4 /
 // 15.3 / 15.2, 12 atoms 75.3 / 52.5 / 51.5 / 51.6, 1/8 of 32 atoms 222 / 198 / 199 /
 // 200, on the learned route 18.9 / 14.3 / 15.5 / 15.4 (6 atoms) and 176 / 168 / 173 /
-// 169 (1/8 of 32).  Long lists gain nothing: all of 32 atoms learned 1 275 ms here
-// and 1 257 ms of kernels one after the other.  Owned by the handle
-// whose work areas the launches use; every call forks from the caller's
-// stream and joins it again, also on an error.
+// 169 (1/8 of 32).  Long lists gain nothing: all of 32 atoms learned take 1 258 ms,
+// their kernels one after the other 1 240.  Owned by the handle whose work areas
+// the launches use; every call forks from the caller's stream and joins it again,
+// also on an error.
 struct SideStreams {
     static constexpr int N = 6;
     cudaStream_t s[N] = {};

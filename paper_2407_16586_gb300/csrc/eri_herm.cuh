@@ -1064,7 +1064,7 @@ struct HermOp {
 // units (tile, chunk of cl.nchunk per tile, split) w, 2W - 1 - w, 2W + w, ...:
 // a molecule's tiles are in decreasing cost, so the alternating order evens the
 // sums out (in a batch the order starts again with every molecule, and two of
-// 21 and 26 atoms take 634 ms against 601 ms one after the other).  A unit's quartets are taken in groups of up to KQ ket pairs of one
+// 21 and 26 atoms take 638 ms against 599 ms one after the other).  A unit's quartets are taken in groups of up to KQ ket pairs of one
 // bra pair.  Their components are added to the warp's own gradient (shared
 // memory, or with out.use_smem = 0 the warp's slab), so the schedule and the
 // order of all sums are fixed and results are bitwise reproducible.
